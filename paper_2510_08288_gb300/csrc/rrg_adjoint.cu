@@ -40,19 +40,19 @@ struct ConstAdj {
 // The elementary functions of the reverse sweep.  binary32: MUFU forms
 // (__powf, __logf, approximate reciprocal), relative errors of a few 1e-7,
 // far inside what a binary32 gradient carries anyway; binary64: x^e through
-// the handle's series (pow_m1_series falls back to pow outside [1, 2] or for
+// the handle's table (pow_m1_table falls back to pow outside [1, 2) or for
 // another exponent), log and IEEE division.
 template <typename T> struct VjpMath;
 template <>
 struct VjpMath<float> {
-  static __device__ __forceinline__ float pw(float x, float e, const PowSeries*) { return __powf(x, e); }
+  static __device__ __forceinline__ float pw(float x, float e, const PowTable*) { return __powf(x, e); }
   static __device__ __forceinline__ float ln(float x) { return __logf(x); }
   static __device__ __forceinline__ float inv(float x) { return __fdividef(1.0f, x); }
 };
 template <>
 struct VjpMath<double> {
-  static __device__ __forceinline__ double pw(double x, double e, const PowSeries* S) {
-    return pow_m1_series(S, x, e) + 1.0;
+  static __device__ __forceinline__ double pw(double x, double e, const PowTable* S) {
+    return pow_m1_table(S, x, e) + 1.0;
   }
   static __device__ __forceinline__ double ln(double x) { return log(x); }
   static __device__ __forceinline__ double inv(double x) { return 1.0 / x; }
@@ -203,10 +203,7 @@ __device__ CandK<T> cand_of(const double* P, double I) {
 
 constexpr int kFwdRing = 8;
 
-// The launch's rollout constants in precision T.
-template <typename T> __device__ __forceinline__ RhsU<T> launch_u(const Launch& L);
-template <> __device__ __forceinline__ RhsU<float> launch_u<float>(const Launch& L) { return L.u32; }
-template <> __device__ __forceinline__ RhsU<double> launch_u<double>(const Launch& L) { return L.u64; }
+// The candidate constants in precision T.
 template <typename T> __device__ __forceinline__ RhsC<T> launch_c(const Launch& L, int i);
 template <> __device__ __forceinline__ RhsC<float> launch_c<float>(const Launch& L, int i) { return L.cand_c32[i]; }
 template <> __device__ __forceinline__ RhsC<double> launch_c<double>(const Launch& L, int i) { return L.cand_c64[i]; }
@@ -233,21 +230,23 @@ adjoint_forward_kernel(const Launch L, const DT* __restrict__ d, int checkpoint,
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const int N = L.N, H = L.H;
   if (k >= N) return;
-  RhsU<T> K = launch_u<T>(L);
-  RhsC<T> C = launch_c<T>(L, i);
-  double p_atm = L.params[P_P_ATM];
+  RhsC<T> R = launch_c<T>(L, i);
+  LaneModel<T> M;
+  double p_atm;
   if (L.pmul != nullptr)
-    p_atm = scenario_model<T>(L.params, L.pmul + static_cast<size_t>(k) * RRG_NPARAM, L.cand_v[i],
-                              L.k64.pws, L.y_min, K, C);
+    p_atm = lane_model<T, true>(L, 0, k, L.cand_v[i], R, M);
+  else
+    p_atm = lane_model<T, false>(L, 0, k, 0.0, R, M);
+  const StepU<T>& K = M.U;
+  const StepC<T>& C = M.C;
   T z_ca, z_w, z_sm, w_abs;
-  start_state<T>(C, L.st->x, p_atm, z_ca, z_w, z_sm, w_abs);
-  const double r_ca = static_cast<double>(C.r_ca), r_w = static_cast<double>(C.r_w),
-               r_sm = static_cast<double>(C.r_sm);
-  const StepC<T> S = step_consts<T>(K, static_cast<T>(L.dt));
+  start_state<T>(R, L.st->x, p_atm, z_ca, z_w, z_sm, w_abs);
+  const double r_ca = static_cast<double>(R.r_ca), r_w = static_cast<double>(R.r_w),
+               r_sm = static_cast<double>(R.r_sm);
   const int nseg = H / checkpoint + 1;
   const size_t HN = static_cast<size_t>(H) * N;
   double* ck = ckpt + (static_cast<size_t>(i) * N + k) * nseg * 3;
-  T smin = C.y_scale * (z_sm - z_ca) + C.s_off;
+  T smin = slack_of<T>(C, z_ca, z_sm);
   int arg = 0;
   int next_ck = 0;  // the next step whose state is saved
   if constexpr (sizeof(T) == 4 && sizeof(DT) == 4) {
@@ -283,7 +282,7 @@ adjoint_forward_kernel(const Launch L, const DT* __restrict__ d, int checkpoint,
         c[2] = static_cast<double>(z_sm) + r_sm;
         next_ck += checkpoint;
       }
-      rk4_step_fast<T>(K, C, S, z_ca, z_w, z_sm, w_abs, e0, e1, e2);
+      rk4_step_fast<T>(K, M.pw, C, z_ca, z_w, z_sm, w_abs, e0, e1, e2);
       // the slot is free once its values are in registers: step j + D
       if (j + D < H) {
         cp_async4(e, pf);
@@ -293,7 +292,7 @@ adjoint_forward_kernel(const Launch L, const DT* __restrict__ d, int checkpoint,
       cp_async_commit();
       pf += N;
       slot = (slot + 1) & (D - 1);
-      const T s = C.y_scale * (z_sm - z_ca) + C.s_off;
+      const T s = slack_of<T>(C, z_ca, z_sm);
       if (s < smin) { smin = s; arg = j + 1; }
     }
     cp_async_wait<0>();  // nothing in flight into the ring when the lane ends
@@ -327,8 +326,8 @@ adjoint_forward_kernel(const Launch L, const DT* __restrict__ d, int checkpoint,
         c[2] = static_cast<double>(z_sm) + r_sm;
         next_ck += checkpoint;
       }
-      rk4_step_fast<T>(K, C, S, z_ca, z_w, z_sm, w_abs, e0, e1, e2);
-      const T s = C.y_scale * (z_sm - z_ca) + C.s_off;
+      rk4_step_fast<T>(K, M.pw, C, z_ca, z_w, z_sm, w_abs, e0, e1, e2);
+      const T s = slack_of<T>(C, z_ca, z_sm);
       if (s < smin) { smin = s; arg = j + 1; }
     }
   }
@@ -429,7 +428,8 @@ adjoint_reverse_kernel(const Launch L, const DT* __restrict__ d,
   double P[RRG_NPARAM];
   scenario_params(L, k, P);
   Fc3K<T> K = konst<T>(P);
-  if (sizeof(T) == 8) K.pws = L.k64.pws;  // the series of the model's exponent (checked per call)
+  // the table of the model's exponent
+  if (sizeof(T) == 8) K.pws = (L.k64.pws != nullptr && L.k64.pws->e == static_cast<double>(K.e)) ? L.k64.pws : nullptr;
   const CandK<T> C = cand_of<T>(P, v);
   const T dt = static_cast<T>(L.dt);
   const int nseg = H / checkpoint + 1;

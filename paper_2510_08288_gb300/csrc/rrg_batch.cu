@@ -73,8 +73,8 @@ struct BLaunch {
   const double* params;
   Fc3K<double> k64;
   Fc3K<float> k32;
-  RhsU<double> u64;
-  RhsU<float> u32;
+  StepModel<double> m64;
+  StepModel<float> m32;
   const BInst* inst;
   const int32_t* order;  // instances, longest horizon (then most scenarios) first
   BState* st;
@@ -295,7 +295,7 @@ __global__ void batch_prepare_kernel(const BLaunch B) {
   const double v = governed(st.v_prev, st.r, B.cand_kappa[slot]);
   B.cand_v[slot] = v;
   const double thr = __dadd_rn(B.c.y_min, __dmul_rn(B.c.eps_ss, __dsub_rn(B.c.y_c, B.c.y_min)));
-  const int ok = candidate_setup(B.k64, B.k32, B.params, v, B.c.ss_check, thr, B.c.y_min,
+  const int ok = candidate_setup(B.k64, B.k32, B.m64.c, B.params, v, B.c.ss_check, thr, B.c.y_min,
                                  B.cand_c64 + slot, B.cand_c32 + slot);
   B.cand_ok[slot] = ok;
   B.cand_ss[slot] = ok;
@@ -362,23 +362,29 @@ __device__ __forceinline__ void batch_tile(const BLaunch& B, int s, int i, int k
   if (active) {
     const BState& st = B.st[s];
     const double p_atm = B.params[P_P_ATM];
-    const RhsC<float> C = B.cand_c32[slot];
+    const RhsC<float> R = B.cand_c32[slot];
+    const StepU<float>& U = B.m32.U;
+    const StepC<float> C = step_consts<float>(U, B.m32.F, R);
     float q_ca, w, q_sm, w_abs;  // the deviation from the candidate's reference point
-    start_state<float>(C, st.x, p_atm, q_ca, w, q_sm, w_abs);
+    start_state<float>(R, st.x, p_atm, q_ca, w, q_sm, w_abs);
     int end = LANE_REACHED_END;
     const float* d = (st.cur ? B.d32b : B.d32) + I.off;
-    smin = run_lane<float, PF>(B.u32, C, d, k, I.N, I.H, 0, I.H, q_ca,
-                               w, q_sm, w_abs, inf_v<float>(), static_cast<float>(B.c.dt),
-                               thr, cand_stop ? dead : nullptr,
+    smin = run_lane<float, PF>(U, nullptr, C, d, k, I.N, I.H, 0, I.H, q_ca,
+                               w, q_sm, w_abs, inf_v<float>(), thr, cand_stop ? dead : nullptr,
                                &steps, &end, eps, &jlast);
     if (cand_stop && smin < thr) *dead = 1;
   }
   batch_reduce(B, slot, k, active, smin, steps, jlast, eps, dead);
 }
 
+// Resident threads per SM that the register budget of the one-lane rollout
+// kernels is held to: 168 registers.  Measured on 64 instances (rollouts of an
+// update, default variant): 384 threads 11.3 ms, 512 (128 registers, the
+// coefficients re-read) 11.9, unbounded (up to 187 registers) 14.6.
+constexpr int kBatchThreadsPerSm = 384;
 // Persistent rollout: each CTA takes tiles from the queue until none is left.
 template <int TILE, int PF>
-__global__ void __launch_bounds__(TILE) batch_rollout_kernel(const BLaunch B) {
+__global__ void __launch_bounds__(TILE, kBatchThreadsPerSm / TILE) batch_rollout_kernel(const BLaunch B) {
   __shared__ int sh[3];
   const uint32_t total = B.queue[1];
   for (;;) {
@@ -429,7 +435,7 @@ __device__ __forceinline__ void tile_of(const BLaunch& B, uint32_t t, int tile, 
 }
 
 template <int PF>
-__global__ void __launch_bounds__(128) batch_rollout_warp_kernel(const BLaunch B) {
+__global__ void __launch_bounds__(128, kBatchThreadsPerSm / 128) batch_rollout_warp_kernel(const BLaunch B) {
   const uint32_t total = B.queue[1];
   const int lane = static_cast<int>(threadIdx.x & 31);
   for (;;) {
@@ -480,22 +486,23 @@ __device__ __forceinline__ void batch_tile_pair(const BLaunch& B, int s, int p, 
   if (active) {
     const BState& bs = B.st[s];
     const double p_atm = B.params[P_P_ATM];
-    const RhsC<float> CA = B.cand_c32[slotA], CB = B.cand_c32[slotB];
+    const RhsC<float> RA = B.cand_c32[slotA], RB = B.cand_c32[slotB];
+    const StepU<float>& K = B.m32.U;
+    const StepC<float> CA = step_consts<float>(K, B.m32.F, RA), CB = step_consts<float>(K, B.m32.F, RB);
     float za[4], zb[4];
-    start_state<float>(CA, bs.x, p_atm, za[0], za[1], za[2], za[3]);
-    start_state<float>(CB, bs.x, p_atm, zb[0], zb[1], zb[2], zb[3]);
+    start_state<float>(RA, bs.x, p_atm, za[0], za[1], za[2], za[3]);
+    start_state<float>(RB, bs.x, p_atm, zb[0], zb[1], zb[2], zb[3]);
     const float* d = (bs.cur ? B.d32b : B.d32) + I.off;
-    const float dt = static_cast<float>(B.c.dt);
     if (runA && runB) {
-      run_lane_pair<float, PF>(B.u32, CA, CB, d, k, I.N, I.H, I.H, za, zb, dt, thr, eps,
+      run_lane_pair<float, PF>(K, CA, CB, d, k, I.N, I.H, I.H, za, zb, thr, eps,
                                cand_stop ? deadA : nullptr, cand_stop ? deadB : nullptr, sm, st, en, jl);
     } else if (runA) {
-      sm[0] = run_lane<float, PF>(B.u32, CA, d, k, I.N, I.H, 0, I.H, za[0], za[1], za[2], za[3],
-                                  inf_v<float>(), dt, thr, cand_stop ? deadA : nullptr, &st[0], &en[0], eps,
+      sm[0] = run_lane<float, PF>(K, nullptr, CA, d, k, I.N, I.H, 0, I.H, za[0], za[1], za[2], za[3],
+                                  inf_v<float>(), thr, cand_stop ? deadA : nullptr, &st[0], &en[0], eps,
                                   &jl[0]);
     } else {
-      sm[1] = run_lane<float, PF>(B.u32, CB, d, k, I.N, I.H, 0, I.H, zb[0], zb[1], zb[2], zb[3],
-                                  inf_v<float>(), dt, thr, cand_stop ? deadB : nullptr, &st[1], &en[1], eps,
+      sm[1] = run_lane<float, PF>(K, nullptr, CB, d, k, I.N, I.H, 0, I.H, zb[0], zb[1], zb[2], zb[3],
+                                  inf_v<float>(), thr, cand_stop ? deadB : nullptr, &st[1], &en[1], eps,
                                   &jl[1]);
     }
     if (cand_stop && runA && sm[0] < thr) *deadA = 1;
@@ -528,57 +535,18 @@ __global__ void __launch_bounds__(128) batch_rollout_warp_pair_kernel(const BLau
 // ---------------------------------------------------------------------------
 // Two lanes per trajectory (warp-cooperative): the lanes 2q and 2q + 1 of a
 // warp carry scenario q of a 16-scenario tile.  Both hold the whole state and
-// form the same stage points and RK4 combination; of each right-hand side,
-// role 0 evaluates the two linear flow derivatives (d_ca, d_sm) and role 1 the
-// compressor-speed derivative with its power term and reciprocal (d_w), and
-// the pair swaps them with two shuffles.  Each component is the expression of
-// fc3_rhs_fast, so the trajectory equals the one-lane rollout bit for bit.
-// The warp issues both roles' instructions for half as many trajectories, and
-// the swap sits on every stage's dependency chain: the autotuner measures it
-// against the one-lane variants.
-__device__ __forceinline__ void fc3_rhs_split(const RhsU<float>& U, const RhsC<float>& C, int role,
-                                              float z_ca, float z_w, float z_sm, float w, float x_pw,
-                                              float& d_ca, float& d_w, float& d_sm) {
-  float v0, v1 = 0.0f;
-  if (role == 0) {
-    v0 = U.a1 * z_sm + (C.c_ca - U.a12 * z_ca);
-    v1 = U.g_w * z_w + ((C.c_sm + U.b3 * z_ca) - U.g_sm * z_sm);
-  } else {
-    const float W_cp = U.a_w * z_w + (C.W_r - U.a_p * z_sm);
-    const float f = torque_factor<float>(U, pow_m1<float>(x_pw, U.e, U.pws), w);
-    v0 = (C.e0 - U.e2 * z_w) - W_cp * f;
-  }
-  const float o0 = __shfl_xor_sync(0xffffffffu, v0, 1);
-  const float o1 = __shfl_xor_sync(0xffffffffu, v1, 1);
-  d_ca = role == 0 ? v0 : o0;
-  d_sm = role == 0 ? v1 : o1;
-  d_w = role == 0 ? o0 : v0;
-}
-
-// rk4_step_fast with the split right-hand side (the same stage points and
-// combination, in the same order).  Called by all 32 lanes.
-__device__ __forceinline__ void rk4_step_split(const RhsU<float>& U, const RhsC<float>& C,
-                                               const StepC<float>& S, int role, float& q_ca, float& w,
-                                               float& q_sm, float& w_abs, float e_ca, float e_w,
-                                               float e_sm) {
-  const float dt = S.dt, h2 = S.h2, h6 = S.h6, g2 = S.g2, g1 = S.g1;
-  const float x1 = q_sm * U.inv_p_atm + C.x_r;
-  float a1, b1, c1, a2, b2, c2, a3, b3, c3, a4, b4, c4;
-  fc3_rhs_split(U, C, role, q_ca, w, q_sm, w_abs, x1, a1, b1, c1);
-  fc3_rhs_split(U, C, role, q_ca + h2 * a1, w + h2 * b1, q_sm + h2 * c1, w_abs + h2 * b1, x1 + g2 * c1,
-                a2, b2, c2);
-  fc3_rhs_split(U, C, role, q_ca + h2 * a2, w + h2 * b2, q_sm + h2 * c2, w_abs + h2 * b2, x1 + g2 * c2,
-                a3, b3, c3);
-  const float p_ca = (q_ca + e_ca) + h6 * (a1 + 2.0f * (a2 + a3));
-  const float p_w = (w + e_w) + h6 * (b1 + 2.0f * (b2 + b3));
-  const float p_sm = (q_sm + e_sm) + h6 * (c1 + 2.0f * (c2 + c3));
-  const float p_wa = p_w + C.r_w;
-  fc3_rhs_split(U, C, role, q_ca + dt * a3, w + dt * b3, q_sm + dt * c3, w_abs + dt * b3, x1 + g1 * c3,
-                a4, b4, c4);
-  q_ca = p_ca + h6 * a4;
-  w = p_w + h6 * b4;
-  q_sm = p_sm + h6 * c4;
-  w_abs = p_wa + h6 * b4;
+// form the same combinations; of each torque, role 0 evaluates the power and
+// role 1 the reciprocal, and the pair swaps them with one shuffle.  The
+// operations are rk4_step_fast's, so the trajectory equals the one-lane
+// rollout bit for bit.  The warp issues the combinations for half as many
+// trajectories, and the swap sits on every stage's dependency chain: the
+// autotuner measures it against the one-lane variants.
+__device__ __forceinline__ float torque_split(const StepU<float>& U, int role, float x, float w) {
+  const float v = role == 0 ? __powf(x, U.e) : rcp_approx(w);
+  const float o = __shfl_xor_sync(0xffffffffu, v, 1);
+  const float p = role == 0 ? v : o, r = role == 0 ? o : v;
+  const float t = fma_rn(-fma_rn(U.B, x, -U.B), r, U.A);
+  return fma_rn(p, t, -t);
 }
 
 // run_lane (steps 1..H from step 0) for a lane pair: the same blocks of PF
@@ -588,11 +556,12 @@ __device__ __forceinline__ void rk4_step_split(const RhsU<float>& U, const RhsC<
 // shuffles need every lane); a pair that has stopped, or a lane past the
 // instance's scenarios (on = false), keeps stepping without recording.
 template <int PF>
-__device__ __forceinline__ float run_lane_split(const RhsU<float>& K, const RhsC<float>& C,
+__device__ __forceinline__ float run_lane_split(const StepU<float>& K, const StepC<float>& C,
                                                 const float* __restrict__ d, int k, bool on, int N, int H,
                                                 int role, float& q_ca, float& w, float& q_sm, float& w_abs,
-                                                float dt, float thr, const volatile int32_t* dead,
+                                                float thr, const volatile int32_t* dead,
                                                 unsigned* steps, float band, int* jlast) {
+  const auto tq = [&](float x, float speed) { return torque_split(K, role, x, speed); };
   float smin = inf_v<float>();
   int j = 0, jl = -1, j_stop = 0;
   bool run = on;
@@ -602,7 +571,6 @@ __device__ __forceinline__ float run_lane_split(const RhsU<float>& K, const RhsC
     if (s0 < band) jl = 0;
     if (s0 < thr) run = false;
   }
-  const StepC<float> S = step_consts<float>(K, dt);
   const size_t HN = static_cast<size_t>(H) * N;
   const float* pf = d + (on ? k : 0);  // in bounds for every lane
   float r0[PF], r1[PF], r2[PF];
@@ -619,7 +587,7 @@ __device__ __forceinline__ float run_lane_split(const RhsU<float>& K, const RhsC
   }
   while (j + PF <= H && __any_sync(0xffffffffu, run)) {
     const int dead_now = (run && dead != nullptr) ? *dead : 0;
-    float nf = 0.0f, bmin = inf_v<float>();
+    BlockMin<float> bm;
 #pragma unroll
     for (int u = 0; u < PF; ++u) {
       const float e0 = r0[u], e1 = r1[u], e2 = r2[u];
@@ -629,15 +597,12 @@ __device__ __forceinline__ float run_lane_split(const RhsU<float>& K, const RhsC
         r2[u] = __ldg(pf + 2 * HN);
       }
       pf += N;
-      rk4_step_split(K, C, S, role, q_ca, w, q_sm, w_abs, e0, e1, e2);
+      rk4_step_with(K, C, q_ca, w, q_sm, w_abs, e0, e1, e2, tq);
       ++j;
-      const float s = C.y_scale * (q_sm - q_ca) + C.s_off;
-      bmin = fmin(bmin, s);
-      nf = fma_rn(s, 0.0f, nf);
+      bm.add(slack_of<float>(C, q_ca, q_sm), u);
     }
     if (run) {
-      nf = fma_rn(q_ca, 0.0f, fma_rn(w, 0.0f, fma_rn(q_sm, 0.0f, nf)));
-      if (nf != nf) bmin = -inf_v<float>();
+      const float bmin = bm.result(q_ca, w, q_sm);
       smin = fmin(smin, bmin);
       if (bmin < band) jl = j;
       j_stop = j;
@@ -648,7 +613,7 @@ __device__ __forceinline__ float run_lane_split(const RhsU<float>& K, const RhsC
   while (j < H && __any_sync(0xffffffffu, run)) {
     const float e0 = __ldg(dp), e1 = __ldg(dp + HN), e2 = __ldg(dp + 2 * HN);
     dp += N;
-    rk4_step_split(K, C, S, role, q_ca, w, q_sm, w_abs, e0, e1, e2);
+    rk4_step_with(K, C, q_ca, w, q_sm, w_abs, e0, e1, e2, tq);
     ++j;
     if (run) {
       const float s = checked_slack<float>(C, q_ca, w, q_sm);
@@ -683,14 +648,14 @@ __device__ __forceinline__ void batch_tile_split(const BLaunch& B, int s, int i,
   const float thr = B.c.early_exit != RRG_EXIT_NONE ? -eps : -inf_v<float>();
   const BState& st = B.st[s];
   const double p_atm = B.params[P_P_ATM];
-  const RhsC<float> C = B.cand_c32[slot];
+  const RhsC<float> R = B.cand_c32[slot];
+  const StepC<float> C = step_consts<float>(B.m32.U, B.m32.F, R);
   float q_ca, w, q_sm, w_abs;
-  start_state<float>(C, st.x, p_atm, q_ca, w, q_sm, w_abs);
+  start_state<float>(R, st.x, p_atm, q_ca, w, q_sm, w_abs);
   const float* d = (st.cur ? B.d32b : B.d32) + I.off;
   unsigned steps = 0;
   int jlast = -1;
-  const float smin = run_lane_split<PF>(B.u32, C, d, k, on, I.N, I.H, role, q_ca, w, q_sm, w_abs,
-                                        static_cast<float>(B.c.dt), thr, cand_stop ? dead : nullptr, &steps,
+  const float smin = run_lane_split<PF>(B.m32.U, C, d, k, on, I.N, I.H, role, q_ca, w, q_sm, w_abs, thr, cand_stop ? dead : nullptr, &steps,
                                         eps, &jlast);
   const bool mine = on && role == 0;
   if (cand_stop && mine && smin < thr) *dead = 1;
@@ -735,12 +700,13 @@ __global__ void __launch_bounds__(64) batch_recheck_kernel(const BLaunch B) {
     src.amp[1] = B.c.amp[1];
     src.amp[2] = B.c.amp[2];
     unsigned steps = 0;
-    const RhsC<double> C = B.cand_c64[slot];
+    const RhsC<double> R = B.cand_c64[slot];
+    const StepC<double> C = step_consts<double>(B.m64.U, B.m64.F, R);
     double q_ca, w, q_sm, w_abs;
-    start_state<double>(C, st.x, p_atm, q_ca, w, q_sm, w_abs);
-    const double smin = run_lane_philox(B.u64, C, src, k,
+    start_state<double>(R, st.x, p_atm, q_ca, w, q_sm, w_abs);
+    const double smin = run_lane_philox(B.m64.U, B.m64.pw, C, src, k,
                                         min(static_cast<int>(B.recheck_jlast[e]), B.inst[s].H),
-                                        q_ca, w, q_sm, w_abs, B.c.dt,
+                                        q_ca, w, q_sm, w_abs,
                                         B.c.early_exit != RRG_EXIT_NONE ? 0.0 : -inf_v<double>(),
                                         &steps);
     if (!(smin >= 0.0)) B.cand_ok[slot] = 0;
@@ -829,7 +795,7 @@ batch_plant_kernel(const BLaunch B, uint64_t seed, uint64_t base, const double* 
     const U64x4 r = philox4x64_10(0ull, 0ull, base + t, 1ull, seed + static_cast<uint64_t>(s), 0ull);
     const double x[3] = {st.x[0], st.x[1], st.x[2]};
     double xn[3];
-    plant_step_fast(B.k64, B.u64, B.params, B.c.dt, v, x, uniform_sym(r.w[0], amp[0]),
+    plant_step_fast(B.m64, v, x, uniform_sym(r.w[0], amp[0]),
                     uniform_sym(r.w[1], amp[1]), uniform_sym(r.w[2], amp[2]), xn);
     st.lx[0] = xn[0];
     st.lx[1] = xn[1];
@@ -900,7 +866,7 @@ struct rrg_batch_ctx {
   size_t lanes = 0;            // sum of M N_s
   // device memory
   double* params_dev = nullptr;
-  PowSeries* pws = nullptr;
+  PowTable* pws = nullptr;
   BInst* inst_dev = nullptr;
   int32_t* order_dev = nullptr;
   BState* st = nullptr;
@@ -1205,8 +1171,8 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   });
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->params_dev, h->params, sizeof h->params, cudaMemcpyHostToDevice, h->stream);
-  PowSeries ps;
-  make_pow_series((h->params[P_GAMMA] - 1.0) / h->params[P_GAMMA], &ps);
+  PowTable ps;
+  const bool pws_ok = pow_table((h->params[P_GAMMA] - 1.0) / h->params[P_GAMMA], &ps);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->pws, &ps, sizeof ps, cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->inst_dev, inst.data(), S * sizeof(BInst), cudaMemcpyHostToDevice, h->stream);
@@ -1251,8 +1217,9 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   for (int i = 0; i < 3; ++i) B.c.amp[i] = cfg->dist_amp[i];
   B.params = h->params_dev;
   fold_constants(h->params, &B.k64, &B.k32);
-  B.k64.pws = h->pws;
-  fold_rhs(B.k64, &B.u64, &B.u32);
+  B.k64.pws = pws_ok ? h->pws : nullptr;
+  fold_model(B.k64, h->params, cfg->dt, &B.m64);
+  round_model(B.m64, &B.m32);
   B.inst = h->inst_dev;
   B.order = h->order_dev;
   B.st = h->st;

@@ -5,6 +5,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <utility>
 #include <vector>
@@ -13,6 +14,48 @@
 #include "rrg_internal.h"
 
 using namespace rrg;
+
+namespace rrg {
+
+bool pow_table(double e, PowTable* S) {
+  // the last table built, kept for the next caller of the same exponent (the
+  // allocation-free evaluation builds one per call)
+  static std::mutex mu;
+  static PowTable last;
+  static bool have = false;
+  if (!(std::fabs(e) <= 1.0)) {
+    std::memset(static_cast<void*>(S), 0, sizeof *S);
+    S->e = std::nan("");
+    return false;
+  }
+  std::lock_guard<std::mutex> lock(mu);
+  if (!have || last.e != e) {
+    for (int i = 0; i < kPowCells; ++i) {
+      PowCell& c = last.cell[i];
+      c.inv_cf = static_cast<float>(1.0 / (1.0 + (i + 0.5) / kPowCells));
+      c.inv_c = c.inv_cf;
+      const double l = -e * std::log(c.inv_c);  // log c^e
+      const double ce = std::exp(l);
+      c.a0 = std::expm1(l);
+      double b = e;  // binom(e, n)
+      c.a1 = ce * b;
+      b = b * (e - 1.0) / 2.0;
+      c.a2 = ce * b;
+      b = b * (e - 2.0) / 3.0;
+      c.a3 = static_cast<float>(ce * b);
+      b = b * (e - 3.0) / 4.0;
+      c.a4 = static_cast<float>(ce * b);
+      b = b * (e - 4.0) / 5.0;
+      c.a5 = static_cast<float>(ce * b);
+    }
+    last.e = e;
+    have = true;
+  }
+  *S = last;
+  return true;
+}
+
+}  // namespace rrg
 
 namespace {
 thread_local std::string g_create_error;
@@ -41,9 +84,11 @@ struct rrg_ctx {
   float* d32 = nullptr;
   double* d64b = nullptr;       // second scenario pair, allocated by the first closed loop
   float* d32b = nullptr;
-  PowSeries* pws = nullptr;     // binary64 x^e - 1 series of the model's exponent
+  PowTable* pws = nullptr;      // binary64 x^e - 1 table of the model's exponent
+  bool pws_ok = false;
   double* pmul = nullptr;       // parameter multipliers of each pair (parametric uncertainty)
   double* pmulb = nullptr;
+  ScenFold fold{}, foldb{};     // the folded models of each pair's scenarios
   cudaStream_t side = nullptr;  // samples update t+1 while update t runs
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool cl_next_ready = false;   // the closed loop's next update is already sampled
@@ -204,7 +249,7 @@ void free_all(rrg_ctx* h) {
                   h->cand_min, h->recheck_list, h->recheck_jlast, h->recheck_count, h->stats, h->P_dev, h->io_dev,
                   h->flag_dev, h->kap_dev, h->adm_dev, h->loop, h->cl_dev, h->lane_state,
                   h->adj_ckpt, h->adj_lane_min, h->adj_lane_arg, h->adj_seg, h->adj_out,
-                  h->pmul, h->pmulb, h->pws, h->err_buf};
+                  h->pmul, h->pmulb, h->pws, h->err_buf, h->fold.d, h->fold.f, h->foldb.d, h->foldb.f};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->io_h) cudaFreeHost(h->io_h);
@@ -255,8 +300,9 @@ void fill_launch(rrg_ctx* h) {
   L.scfg = h->scfg;
   L.params = h->params_dev;
   fold_constants(h->params, &L.k64, &L.k32);
-  L.k64.pws = h->pws;
-  fold_rhs(L.k64, &L.u64, &L.u32);
+  L.k64.pws = h->pws_ok ? h->pws : nullptr;
+  fold_model(L.k64, h->params, c.dt, &L.m64);
+  round_model(L.m64, &L.m32);
   L.d64 = h->d64;
   L.d32 = h->d32;
   L.st = h->st;
@@ -279,6 +325,8 @@ void fill_launch(rrg_ctx* h) {
   L.lane_state = h->lane_state;
   L.pmul = h->pmul;
   L.pmulb = h->pmulb;
+  L.fold = h->fold;
+  L.foldb = h->foldb;
   L.punc_rho = c.param_unc_rel;
   L.punc_mask = c.param_unc_mask;
 }
@@ -391,6 +439,10 @@ int enqueue_search(rrg_ctx* h, const double* d_x, const double* d_r,
   return RRG_OK;
 }
 
+// Kernels of one scenario draw (with parametric uncertainty the scenarios'
+// models are folded after it).
+uint64_t sample_launches(const rrg_ctx* h) { return h->pmul ? 2 : 1; }
+
 bool x_ok(const double* x) { return x && is_fin(x[0]) && is_fin(x[1]) && is_fin(x[2]); }
 
 // Launches, rollout launches and rounds of the rounds after a pipelined
@@ -491,7 +543,7 @@ cudaGraph_t capture_conditional_update(rrg_ctx* h, uint64_t seed, uint64_t t0, c
 // device by the kernel that opens it.
 void enqueue_count_only(rrg_ctx* h) {
   const uint64_t rec = h->cfg.precision == RRG_FP32_RECHECK ? 1 : 0;
-  h->launches += 1 + 1 + 1 + 1 + (1 + rec) + 1 + 1;
+  h->launches += sample_launches(h) + 1 + 1 + 1 + (1 + rec) + 1 + 1;
   h->rollout_launches += 2;
   h->rounds += 1;
 }
@@ -753,7 +805,11 @@ int rrg_create(const double* model_params, int n_params, const rrg_config* cfg, 
   ALLOC(kap_dev, 2 * M);
   ALLOC(adm_dev, M);
   ALLOC(loop, 1);
-  if (c.param_unc_rel > 0.0) ALLOC(pmul, N * RRG_NPARAM);
+  if (c.param_unc_rel > 0.0) {
+    ALLOC(pmul, N * RRG_NPARAM);
+    ALLOC(fold.d, N * kFoldDoubles);
+    ALLOC(fold.f, N * kFoldFloats);
+  }
 #undef ALLOC
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&h->io_h), IO_LEN * sizeof(double) + 2 * M * sizeof(double) + M);
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&h->flag_h), 4 * sizeof(int32_t));
@@ -763,13 +819,14 @@ int rrg_create(const double* model_params, int n_params, const rrg_config* cfg, 
   if (e == cudaSuccess) e = cudaMemsetAsync(h->d32, 0, n32 * sizeof(float), h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->params_dev, h->params, sizeof h->params, cudaMemcpyHostToDevice, h->stream);
-  PowSeries ps;
-  make_pow_series((h->params[P_GAMMA] - 1.0) / h->params[P_GAMMA], &ps);
+  PowTable ps;
+  h->pws_ok = pow_table((h->params[P_GAMMA] - 1.0) / h->params[P_GAMMA], &ps);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->pws, &ps, sizeof ps, cudaMemcpyHostToDevice, h->stream);
   fill_launch(h);
   // the zero scenarios are explicit values (marks pair 0's binary64 array valid)
   if (e == cudaSuccess) e = launch_round_scenarios(h->L);
   if (e == cudaSuccess && h->pmul) e = launch_fill(h->L, h->pmul, N * RRG_NPARAM, 1.0);
+  if (e == cudaSuccess) e = launch_scenario_fold(h->L, false);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
     const int code = (e == cudaErrorMemoryAllocation) ? RRG_ENOMEM : RRG_ECUDA;
@@ -820,7 +877,7 @@ int rrg_sample_scenarios(rrg_handle h, uint64_t seed, uint64_t update_index) {
   DeviceGuard g(h->device);
   h->cl_next_ready = false;  // pair 0 may hold a closed loop's next update
   CK(launch_sample(h->L, seed, update_index, nullptr, h->cfg.dist_amp));
-  h->launches++;
+  h->launches += sample_launches(h);
   return RRG_OK;
 }
 
@@ -865,6 +922,8 @@ int rrg_set_param_multipliers(rrg_handle h, const double* m) {
   DeviceGuard g(h->device);
   h->cl_next_ready = false;
   CK(cudaMemcpyAsync(h->pmul, m, n * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+  CK(launch_scenario_fold(h->L, false));
+  h->launches++;
   CK(cudaStreamSynchronize(h->stream));
   return RRG_OK;
 }
@@ -1205,6 +1264,12 @@ int rrg_closed_loop_dev(rrg_handle h, const double* x0, double v0, const double*
       CK(cudaMalloc(reinterpret_cast<void**>(&h->pmulb), np * sizeof(double)));
       CK(launch_fill(h->L, h->pmulb, np, 1.0));
     }
+    if (h->pmul && !h->foldb.f) {
+      const size_t ns = static_cast<size_t>(h->cfg.n_scenarios);
+      if (!h->foldb.d)
+        CK(cudaMalloc(reinterpret_cast<void**>(&h->foldb.d), ns * kFoldDoubles * sizeof(double)));
+      CK(cudaMalloc(reinterpret_cast<void**>(&h->foldb.f), ns * kFoldFloats * sizeof(float)));
+    }
     if (!h->side) CK(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
     if (!h->ev_fork) CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
     if (!h->ev_join) CK(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
@@ -1219,6 +1284,7 @@ int rrg_closed_loop_dev(rrg_handle h, const double* x0, double v0, const double*
     h->L.d64b = h->d64b;
     h->L.d32b = h->d32b;
     h->L.pmulb = h->pmulb;
+    h->L.foldb = h->foldb;
   }
   std::memcpy(h->io_h + IO_AMP, plant_amp, 3 * sizeof(double));
   CK(cudaMemcpyAsync(h->io_dev + IO_AMP, h->io_h + IO_AMP, 3 * sizeof(double),
@@ -1235,7 +1301,7 @@ int rrg_closed_loop_dev(rrg_handle h, const double* x0, double v0, const double*
   // the same run already drew them
   if (!(h->cl_next_ready && h->cl_seed == seed && h->cl_t0 == t0)) {
     CK(launch_sample(L, seed, t0, &h->loop->t, h->cfg.dist_amp, true));
-    h->launches++;
+    h->launches += sample_launches(h);
   }
   // one update: draw update t+1 on the side stream (into the other pair)
   // while update t searches and moves the plant on the main stream
@@ -1244,7 +1310,7 @@ int rrg_closed_loop_dev(rrg_handle h, const double* x0, double v0, const double*
     CK(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
     CK(launch_sample(L, seed, t0 + 1, &h->loop->t, h->cfg.dist_amp, true, h->side));
     CK(cudaEventRecord(h->ev_join, h->side));
-    h->launches++;
+    h->launches += sample_launches(h);
     int rc = enqueue_search(h, h->loop->x, d_r_seq, &h->loop->t, &h->loop->v_prev, nullptr,
                             nullptr, nullptr, static_cast<long long>(t0));
     if (rc != RRG_OK) return rc;

@@ -1,7 +1,8 @@
 // rrg_device.cuh -- device-side building blocks of the robust reference
 // governor: the FC3 closed-loop right-hand side and output, the RK4 step,
 // the Philox4x64-10 scenario generator and order-preserving keys for
-// atomic minima.  Included by rrg_kernels.cu only.
+// atomic minima.  Included by every
+// translation unit with device code.
 #pragma once
 
 #include <cstdint>
@@ -9,40 +10,72 @@
 
 namespace rrg {
 
+// a b + c rounded once; never simplified (x 0 + c is NaN for x = inf or NaN).
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // ---------------------------------------------------------------------------
-// Binomial series of x^e - 1 about c = 3/2, for binary64 (GB300's binary64
-// pow has a dependent latency of about 5,800 cycles, this about 500): with
-// t = x / c - 1, |t| <= 1/3 for x in [1, 2], and
+// x^e - 1 in binary64 for x in [1, 2), from a table of kPowCells cells.
+//
+// A binary64 instruction takes a GB300 warp scheduler 64 cycles (measured: 2
+// lanes per clock and SM, a lone warp's independent DFMAs no faster than its
+// dependent ones), so what counts is their number.  With c the midpoint of
+// x's cell and t = x / c - 1, |t| <= 2^-10,
 //   x^e - 1 = (c^e - 1) + c^e sum_{n >= 1} binom(e, n) t^n,
-// truncated after t^32 (the rest is below 3^-33 c^e / 33 < 1e-17), evaluated by
-// Estrin's scheme.  Built on the host for one exponent (make_pow_series);
-// another exponent or an x outside [1, 2] takes pow.
-struct PowSeries {
-  double e;      // the exponent the coefficients are for
-  double inv_c;  // 1 / c
-  double a[33];  // a[0] = c^e - 1, a[n] = c^e binom(e, n)
+// the terms from t^3 on are below 2^-34 c^e |binom(e, 3)|: formed in binary32
+// (their rounding is below 2^-58) they cost no binary64 instruction, the term
+// t^6 and later ones are below 2^-65.  Four binary64 instructions are left
+// (t and three of Horner's rule) against 38 of one series over [1, 2].
+// 1 / c is a binary32 value, so t is formed with one rounding.  Built on the
+// host for one exponent (pow_table); a nullptr table (another exponent,
+// or one outside [-1, 1]) and an x outside [1, 2) take pow.
+constexpr int kPowCells = 512;
+struct alignas(16) PowCell {
+  double inv_c;       // 1 / c
+  double a0, a1, a2;  // c^e - 1, c^e e, c^e binom(e, 2)
+  float a3, a4, a5;   // c^e binom(e, n)
+  float inv_cf;       // 1 / c
+};
+struct alignas(16) PowTable {
+  PowCell cell[kPowCells];
+  double e;           // the exponent the table is for (NaN: no table)
 };
 
-__device__ __forceinline__ double pow_m1_series(const PowSeries* __restrict__ S, double x,
-                                                double e) {
-  if (S != nullptr && S->e == e) {
-    const double t = fma(x, S->inv_c, -1.0);
-    if (fabs(t) <= 1.0 / 3.0) {
-      const double* a = S->a;
-      const double t2 = t * t, t4 = t2 * t2, t8 = t4 * t4, t16 = t8 * t8, t32 = t16 * t16;
-      double p[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) p[i] = fma(a[2 * i + 1], t, a[2 * i]);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) p[i] = fma(p[2 * i + 1], t2, p[2 * i]);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) p[i] = fma(p[2 * i + 1], t4, p[2 * i]);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) p[i] = fma(p[2 * i + 1], t8, p[2 * i]);
-      return fma(a[32], t32, fma(p[1], t16, p[0]));
-    }
+// A binary32 value widened without the binary64 pipe (0 becomes 2^-127, far
+// below any rounding of its use).
+__device__ __forceinline__ double widen_bits(float f) {
+  const uint32_t u = __float_as_uint(f);
+  const uint32_t hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
+  return __hiloint2double(static_cast<int>(hi), static_cast<int>(u << 29));
+}
+
+__device__ __forceinline__ double pow_m1_table(const PowTable* __restrict__ S, double x, double e) {
+  const int hi = __double2hiint(x);
+  if (S != nullptr && (hi >> 20) == 0x3ff) {
+    const PowCell* __restrict__ c = S->cell + ((hi >> 11) & (kPowCells - 1));
+    const double2 ia = __ldg(reinterpret_cast<const double2*>(c));
+    const double2 a12 = __ldg(reinterpret_cast<const double2*>(c) + 1);
+    const float4 f = __ldg(reinterpret_cast<const float4*>(c) + 2);
+    const double t = fma_rn(x, ia.x, -1.0);
+    // x truncated to binary32 is enough for the binary32 terms
+    const uint32_t m = (static_cast<uint32_t>(hi) & 0xfffffu) << 3 |
+                       static_cast<uint32_t>(__double2loint(x)) >> 29;
+    const float tf = fma_rn(__uint_as_float(0x3f800000u | m), f.w, -1.0f);
+    const double p3 = widen_bits(fma_rn(fma_rn(f.z, tf, f.y), tf, f.x));
+    return fma_rn(t, fma_rn(t, fma_rn(t, p3, a12.y), a12.x), ia.y);
   }
   return pow(x, e) - 1.0;
+}
+
+// 1 / w in binary64: the hardware's approximate reciprocal (about 20 bits),
+// refined by one cubic step of the Newton family, r (1 + d + d^2) with d =
+// 1 - w r (error d^3): three binary64 instructions, within about one unit in
+// the last place.
+__device__ __forceinline__ double rcp_cubic(double w) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(w));
+  const double d = fma_rn(-w, r, 1.0);
+  return fma_rn(r, fma_rn(d, d, d), r);
 }
 
 // ---------------------------------------------------------------------------
@@ -65,7 +98,7 @@ struct Fc3K {
   T RT_Vca;      // R_a T_st / V_ca
   T RT_Vsm;      // R_a T_st / V_sm
   T inv_J;       // 1 / J_cp
-  const PowSeries* pws;  // binary64 x^e - 1 (device memory; nullptr: pow)
+  const PowTable* pws;   // binary64 x^e - 1 (device memory; nullptr: pow)
 };
 
 // Per-candidate constants (functions of the governed setpoint v = I only).
@@ -82,15 +115,15 @@ struct CandK {
 // warp running one trajectory is issue-bound, and the polynomial costs more
 // instructions than the two MUFU operations it would replace.)
 template <typename T>
-__device__ __forceinline__ T pow_e_m1(T e, T u, const PowSeries* S);
+__device__ __forceinline__ T pow_e_m1(T e, T u, const PowTable* S);
 
 template <>
-__device__ __forceinline__ double pow_e_m1<double>(double e, double u, const PowSeries* S) {
-  return pow_m1_series(S, 1.0 + u, e);
+__device__ __forceinline__ double pow_e_m1<double>(double e, double u, const PowTable* S) {
+  return pow_m1_table(S, 1.0 + u, e);
 }
 
 template <>
-__device__ __forceinline__ float pow_e_m1<float>(float e, float u, const PowSeries*) {
+__device__ __forceinline__ float pow_e_m1<float>(float e, float u, const PowTable*) {
   return __powf(1.0f + u, e) - 1.0f;
 }
 
@@ -138,149 +171,224 @@ __device__ __forceinline__ void rk4_step(const Fc3K<T>& K, const CandK<T>& C, T 
 }
 
 // ---------------------------------------------------------------------------
-// The same right-hand side with its constants multiplied out, for the
-// rollouts (the equilibrium solve and the adjoint keep the form above), in
-// deviation coordinates z = q - q_r about a reference point q_r of the
-// candidate (its binary32 equilibrium; 0 gives the gauge form):
-//   d_ca = RT_Vca (k_sm (p_sm - p_ca) - k_ca p_ca - W_o2)
-//        = a1 z_sm - (a1 + a2) z_ca + c_ca
-//   d_sm = RT_Vsm (W_cp - k_sm (p_sm - p_ca))
-//        = RT_Vsm a_w z_w - (RT_Vsm a_p + b3) z_sm + b3 z_ca + c_sm
-//   d_w  = (C_m (V0 - K_p W_cp - k_v w) - C_cp pr W_cp / w) / J
-//        = (e0 - e2 z_w) - W_cp (e1 + e3 pr / w),
-//   W_cp = a_w z_w - a_p z_sm + W_r,  w = w_r + z_w
-// where c_ca, c_sm (the derivatives at q_r), W_r and e0 are folded in
-// binary64 and rounded once.  Near the reference every binary32 term is of
-// the size of the deviation, not of the ~1e4 Pa gauge pressures, so the
-// state's rounding and the cancellations between the flow terms shrink with
-// it (and the terms can be multiplied out without losing digits).  16
-// instructions per evaluation in binary32 (3 of them MUFU), as many as the
-// gauge form, plus five per step that carry the absolute speed w (see
-// rk4_step_fast).
+// The RK4 step of the rollouts, with the linear part of FC3 folded through the
+// four stages (the equilibrium solve and the adjoint's reverse sweep keep the
+// form above).
+//
+// In deviation coordinates z = q - q_r about a reference point q_r of the
+// candidate (its binary32 equilibrium; 0 gives the gauge form) FC3 is linear
+// but for one scalar in the speed's equation, the compressor's torque:
+//   z' = L z + c - N(x, w) e_w,
+//   N = (C_cp / J) W_cp (x^e - 1) / w = (x^e - 1) (A - B (x - 1) / w),
+//   A = C_cp a_w / J, B = C_cp a_p p_atm / J
+// (W_cp / w = a_w - a_p p_atm (x - 1) / w), x = p_sm / p_atm and w the speed.
+// So every stage point and the step's result are fixed linear combinations of
+// z, of c and of the stages' values N_1..N_4:
+//   z_2 = M_2 z + (h/2) c - (h/2) N_1 e_w,   M_2 = I + (h/2) L
+//   z_3 = M_3 z + ...,  M_3 = I + (h/2) L M_2;   M_4 = I + h L M_3
+//   z+  = R z + ...,    R = I + (h/6) (L + 2 L M_2 + 2 L M_3 + L M_4)
+// and a stage needs only its x and w, two rows of the combination.  The
+// coefficients are products of the model's constants and the step size, formed
+// in binary64 once per model and rounded once.
+//
+// Why: against right-hand sides evaluated stage by stage, a step on the TMA
+// ring takes 91 binary32 instructions instead of 110 (4 torque terms of 7, 53
+// multiply-adds, 3 loads, slack and bookkeeping), and its dependent chain
+// shortens: x_{i+1} does not depend on N_i (the torque reaches the pressure one
+// stage later), so the power's lg2 and ex2 of a stage overlap the stage
+// before, and the chain through a stage is N_i -> w_{i+1} -> 1 / w -> N_{i+1}.
+// Measured on GB300: one warp's chain 172 -> 145 cycles a step; launches that
+// fill the SMs 2.3e11 -> 3.5e11 steps/s (nominal model, 114 cycles a step and
+// scheduler: 91 issued, and lg2, rcp and ex2 hold their unit for 80).
+// In binary64 49 multiply-adds and 4 torque terms of 12 instructions are left
+// (pow_m1_table, rcp_cubic): 257 x 8 trajectories 10.8 -> 3.7 us a step.
+//
+// Near the reference every binary32 number is of the size of the deviation,
+// not of the ~1e4 Pa gauge pressures, so the state's rounding shrinks with it;
+// c and the reference are folded in binary64.
 template <typename T>
-struct RhsU {      // constants of the model (per scenario under parametric uncertainty)
-  T a1, a12;       // RT_Vca k_sm, RT_Vca (k_sm + k_ca)
-  T a_w, a_p;      // compressor map
-  T b3;            // RT_Vsm k_sm
-  T g_w, g_sm;     // RT_Vsm a_w, RT_Vsm a_p + b3
-  T inv_p_atm, e;
-  T e1, e2, e3;    // C_m K_p / J, C_m k_v / J, C_cp / J
-  const PowSeries* pws;  // binary64 x^e - 1 (device memory; nullptr: pow)
+struct StepU {  // one model's coefficients (per scenario under parametric uncertainty)
+  T ip;         // 1 / p_atm
+  T e, A, B;    // exponent and torque constants
+  // stage 2..4: rows of x (already over p_atm) and w; nX: coefficient of N_X
+  T x2a, x2w, x2s, w2w, w2s, w2n1;
+  T x3a, x3w, x3s, x3n1, w3a, w3w, w3s, w3n1, w3n2;
+  T x4a, x4w, x4s, x4n1, x4n2, w4a, w4w, w4s, w4n1, w4n2, w4n3;
+  // the step's result: cathode pressure, manifold pressure, speed
+  T faa, faw, fas, fan1, fan2;
+  T fsa, fsw, fss, fsn1, fsn2, fsn3;
+  T fwa, fww, fws, fwn1, fwn2, fwn3, fwn4;
+};
+
+// What multiplies c in the combinations besides StepU's rows: the step sizes
+// and the rows of (h/6) (I + 2 M_2 + 2 M_3 + M_4).
+template <typename T>
+struct StepPhi {
+  T h, h2;
+  T aa, aw, as, sa, sw, ss, wa, ww, ws;
 };
 
 template <typename T>
-struct RhsC {    // constants of the candidate setpoint v (and the scenario's model)
-  T c_ca;        // d_ca at q_r: a1 s_r - a2 ca_r - RT_Vca W_o2
-  T c_sm;        // d_sm at q_r: RT_Vsm W_r - b3 s_r
-  T W_r;         // compressor flow at q_r: a_w w_r - a_p sm_r
-  T e0;          // C_m V0 / J - e2 w_r
-  T x_r;         // 1 + sm_r / p_atm
-  T y_scale;     // x_O2 k_sm / W_o2
-  T s_off;       // slack at q_r: y_scale s_r - y_min
-  T r_ca, r_w, r_sm;  // q_r (binary32 values, so both precisions share it)
+struct RhsC {            // constants of the candidate setpoint v (and the scenario's model)
+  T c_ca, c_w, c_sm;     // the derivative at q_r without the torque: L q_r + b(v)
+  T x_r;                 // 1 + sm_r / p_atm
+  T y_scale;             // x_O2 k_sm / W_o2
+  T s_off;               // slack at q_r: y_scale s_r - y_min
+  T r_ca, r_w, r_sm;     // q_r (binary32 values, so both precisions share it)
 };
 
-// x^e - 1 for the compressor term, x = 1 + q_sm / p_atm formed by the caller.
+// RhsC carried through the stages (formed once per trajectory): the constant
+// of each row.
 template <typename T>
-__device__ __forceinline__ T pow_m1(T x, T e, const PowSeries* S);
-template <>
-__device__ __forceinline__ double pow_m1<double>(double x, double e, const PowSeries* S) {
-  return pow_m1_series(S, x, e);
-}
-template <>
-__device__ __forceinline__ float pow_m1<float>(float x, float e, const PowSeries*) {
-  return __powf(x, e) - 1.0f;
+struct StepC {
+  T x1, x2, w2, x3, w3, x4, w4, fa, fw, fs;
+  T y_scale, s_off, r_w;
+};
+
+template <typename T>
+__device__ __forceinline__ StepC<T> step_consts(const StepU<T>& U, const StepPhi<T>& F, const RhsC<T>& C) {
+  StepC<T> S;
+  const T a = C.c_ca, w = C.c_w, s = C.c_sm;
+  S.x1 = C.x_r;
+  S.x2 = fma_rn(F.h2 * U.ip, s, C.x_r);
+  S.w2 = fma_rn(F.h2, w, C.r_w);
+  S.x3 = fma_rn(F.h2, fma_rn(U.x2a, a, fma_rn(U.x2w, w, U.x2s * s)), C.x_r);
+  S.w3 = fma_rn(F.h2, fma_rn(U.w2w, w, U.w2s * s), C.r_w);
+  S.x4 = fma_rn(F.h, fma_rn(U.x3a, a, fma_rn(U.x3w, w, U.x3s * s)), C.x_r);
+  S.w4 = fma_rn(F.h, fma_rn(U.w3a, a, fma_rn(U.w3w, w, U.w3s * s)), C.r_w);
+  S.fa = fma_rn(F.aa, a, fma_rn(F.aw, w, F.as * s));
+  S.fs = fma_rn(F.sa, a, fma_rn(F.sw, w, F.ss * s));
+  S.fw = fma_rn(F.wa, a, fma_rn(F.ww, w, F.ws * s));
+  S.y_scale = C.y_scale;
+  S.s_off = C.s_off;
+  S.r_w = C.r_w;
+  return S;
 }
 
-// The compressor torque factor f = e1 + e3 pr / w.  binary32: e3 pr is
-// formed on the power term's path and the approximate reciprocal of w feeds
-// the final multiply-add directly (w arrives last, from the previous stage's
-// d_w); binary64: IEEE division.
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-template <typename T> __device__ __forceinline__ T torque_factor(const RhsU<T>& U, T pr, T w);
-template <>
-__device__ __forceinline__ float torque_factor<float>(const RhsU<float>& U, float pr, float w) {
-  return fmaf(U.e3 * pr, rcp_approx(w), U.e1);
+
+// N(x, w).  binary32: x^e by __powf, its - 1 fused with the product.
+__device__ __forceinline__ float torque(const StepU<float>& U, const PowTable*, float x, float w) {
+  const float p = __powf(x, U.e);
+  const float t = fma_rn(-fma_rn(U.B, x, -U.B), rcp_approx(w), U.A);
+  return fma_rn(p, t, -t);
 }
-template <>
-__device__ __forceinline__ double torque_factor<double>(const RhsU<double>& U, double pr, double w) {
-  return U.e1 + (U.e3 / w) * pr;
+__device__ __forceinline__ double torque(const StepU<double>& U, const PowTable* S, double x, double w) {
+  const double t = fma_rn(-fma_rn(U.B, x, -U.B), rcp_cubic(w), U.A);
+  return pow_m1_table(S, x, U.e) * t;
 }
 
-// x_pw = x_r + z_sm / p_atm and the absolute speed w = w_r + z_w are passed
-// in: the caller forms both from the previous stage's derivatives directly
-// (x_pw + (h / p_atm) d_sm, w + h d_w), one dependent operation shorter than
-// through the stage state.  The terms with z_w, the component that arrives
-// last, are added last.
-template <typename T>
-__device__ __forceinline__ void fc3_rhs_fast(const RhsU<T>& U, const RhsC<T>& C, T z_ca, T z_w,
-                                             T z_sm, T w, T x_pw, T& d_ca, T& d_w, T& d_sm) {
-  d_ca = U.a1 * z_sm + (C.c_ca - U.a12 * z_ca);
-  d_sm = U.g_w * z_w + ((C.c_sm + U.b3 * z_ca) - U.g_sm * z_sm);
-  const T W_cp = U.a_w * z_w + (C.W_r - U.a_p * z_sm);
-  const T f = torque_factor<T>(U, pow_m1<T>(x_pw, U.e, U.pws), w);
-  d_w = (C.e0 - U.e2 * z_w) - W_cp * f;
+// One RK4 step followed by the disturbance (e_ca, e_w, e_sm) of Eq. 4, in
+// place, on the deviation z = (q_ca, w, q_sm).  w_abs is the absolute speed
+// r_w + w that the next step's first torque divides by: formed beside w from
+// the same sum, so it never drifts from it by more than a rounding.  The
+// newest N is always added last.  Every operation is spelled out, so each
+// kernel that steps a trajectory gives the same bits.
+// tq(x, w): the torque.
+template <typename T, typename Torque>
+__device__ __forceinline__ void rk4_step_with(const StepU<T>& U, const StepC<T>& C, T& q_ca, T& w, T& q_sm,
+                                              T& w_abs, T e_ca, T e_w, T e_sm, const Torque& tq) {
+  const T a = q_ca, z = w, s = q_sm;
+  const T n1 = tq(fma_rn(U.ip, s, C.x1), w_abs);
+  const T x2 = fma_rn(U.x2w, z, fma_rn(U.x2s, s, fma_rn(U.x2a, a, C.x2)));
+  const T w2 = fma_rn(U.w2n1, n1, fma_rn(U.w2w, z, fma_rn(U.w2s, s, C.w2)));
+  const T n2 = tq(x2, w2);
+  const T x3 = fma_rn(U.x3n1, n1, fma_rn(U.x3w, z, fma_rn(U.x3s, s, fma_rn(U.x3a, a, C.x3))));
+  const T w3 = fma_rn(U.w3n2, n2, fma_rn(U.w3n1, n1, fma_rn(U.w3w, z, fma_rn(U.w3s, s, fma_rn(U.w3a, a, C.w3)))));
+  const T n3 = tq(x3, w3);
+  const T x4 = fma_rn(U.x4n2, n2, fma_rn(U.x4n1, n1, fma_rn(U.x4w, z, fma_rn(U.x4s, s, fma_rn(U.x4a, a, C.x4)))));
+  const T w4 = fma_rn(U.w4n3, n3, fma_rn(U.w4n2, n2, fma_rn(U.w4n1, n1,
+               fma_rn(U.w4w, z, fma_rn(U.w4s, s, fma_rn(U.w4a, a, C.w4))))));
+  const T n4 = tq(x4, w4);
+  q_ca = fma_rn(U.fan2, n2, fma_rn(U.fan1, n1, fma_rn(U.faw, z, fma_rn(U.fas, s, fma_rn(U.faa, a, e_ca + C.fa)))));
+  q_sm = fma_rn(U.fsn3, n3, fma_rn(U.fsn2, n2, fma_rn(U.fsn1, n1,
+         fma_rn(U.fsw, z, fma_rn(U.fss, s, fma_rn(U.fsa, a, e_sm + C.fs))))));
+  const T p = fma_rn(U.fwn3, n3, fma_rn(U.fwn2, n2, fma_rn(U.fwn1, n1,
+              fma_rn(U.fww, z, fma_rn(U.fws, s, fma_rn(U.fwa, a, e_w + C.fw))))));
+  w = fma_rn(U.fwn4, n4, p);
+  w_abs = fma_rn(U.fwn4, n4, p + C.r_w);
 }
 
-// Step-size constants of rk4_step_fast, formed once per trajectory (the
-// division dt / 6 is not left to the compiler to hoist out of the loop).
-template <typename T>
-struct StepC {
-  T dt, h2, h6, g2, g1;  // dt, dt / 2, dt / 6, dt / (2 p_atm), dt / p_atm
-};
-template <typename T>
-__device__ __forceinline__ StepC<T> step_consts(const RhsU<T>& U, T dt) {
-  StepC<T> S;
-  S.dt = dt;
-  S.h2 = T(0.5) * dt;
-  S.h6 = dt / T(6);
-  S.g2 = S.h2 * U.inv_p_atm;
-  S.g1 = dt * U.inv_p_atm;
-  return S;
+// The same step with two binary32 multiply-adds per instruction (the same
+// rounding as two fma_rn, on pairs in adjacent registers): the rows of x and
+// w of a stage, and those of the two pressures, as pairs.  A packed
+// multiply-add occupies its pipe for two cycles, so only issue slots are
+// saved, and the coefficients must sit in registers.  Taken where they do
+// anyway, in the parametric lanes on the TMA ring, which an issue-side
+// conflict of three-register multiply-adds held back (16,384 x 16 x 1,000
+// steps: 892 -> 850 us); the nominal lanes, whose coefficients are
+// constant-bank operands, ran 14 % slower packed (741 -> 843 us), lone warps
+// 6 %.
+__device__ __forceinline__ uint64_t pk(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void upk(uint64_t p, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
 }
 
-// One RK4 step of size dt followed by the disturbance (e_ca, e_w, e_sm) of
-// Eq. 4, in place, on the deviation z = (q_ca, w, q_sm) - q_r.  w_abs is the
-// absolute compressor speed w_r + w that the torque term divides by: it is
-// re-derived from the deviation every step ((p_w + w_r) + h/6 k4 next to
-// p_w + h/6 k4), so it never drifts from it by more than a rounding, and the
-// stage points form it from the previous stage's d_w in one operation.  (A
-// first-order update of one reciprocal per step would not do: in the largest
-// FC3 transients w moves by up to 20 % within half a step.)  The update is
-// summed as ((z + e) + h/6 (k1 + 2 (k2 + k3))) + h/6 k4, so only one
-// operation follows the last stage.
-template <typename T>
-__device__ __forceinline__ void rk4_step_fast(const RhsU<T>& U, const RhsC<T>& C, const StepC<T>& S,
-                                              T& q_ca, T& w, T& q_sm, T& w_abs, T e_ca, T e_w,
-                                              T e_sm) {
-  const T dt = S.dt, h2 = S.h2, h6 = S.h6, g2 = S.g2, g1 = S.g1;
-  const T x1 = q_sm * U.inv_p_atm + C.x_r;
-  T a1, b1, c1, a2, b2, c2, a3, b3, c3, a4, b4, c4;
-  fc3_rhs_fast<T>(U, C, q_ca, w, q_sm, w_abs, x1, a1, b1, c1);
-  fc3_rhs_fast<T>(U, C, q_ca + h2 * a1, w + h2 * b1, q_sm + h2 * c1, w_abs + h2 * b1, x1 + g2 * c1,
-                  a2, b2, c2);
-  fc3_rhs_fast<T>(U, C, q_ca + h2 * a2, w + h2 * b2, q_sm + h2 * c2, w_abs + h2 * b2, x1 + g2 * c2,
-                  a3, b3, c3);
-  const T p_ca = (q_ca + e_ca) + h6 * (a1 + T(2) * (a2 + a3));
-  const T p_w = (w + e_w) + h6 * (b1 + T(2) * (b2 + b3));
-  const T p_sm = (q_sm + e_sm) + h6 * (c1 + T(2) * (c2 + c3));
-  const T p_wa = p_w + C.r_w;
-  fc3_rhs_fast<T>(U, C, q_ca + dt * a3, w + dt * b3, q_sm + dt * c3, w_abs + dt * b3, x1 + g1 * c3,
-                  a4, b4, c4);
-  q_ca = p_ca + h6 * a4;
-  w = p_w + h6 * b4;
-  q_sm = p_sm + h6 * c4;
-  w_abs = p_wa + h6 * b4;
+__device__ __forceinline__ void rk4_step_packed(const StepU<float>& U, const StepC<float>& C, float& q_ca,
+                                                float& w, float& q_sm, float& w_abs, float e_ca, float e_w,
+                                                float e_sm) {
+  const auto tq = [&](float x, float speed) { return torque(U, nullptr, x, speed); };
+  const float a = q_ca, z = w, s = q_sm;
+  const uint64_t aa = pk(a, a), zz = pk(z, z), ss = pk(s, s);
+  const float n1 = tq(fma_rn(U.ip, s, C.x1), w_abs);
+  float x2, w2, x3, w3, x4, w4;
+  upk(fma2(pk(U.x2w, U.w2w), zz, fma2(pk(U.x2s, U.w2s), ss, pk(fma_rn(U.x2a, a, C.x2), C.w2))), x2, w2);
+  uint64_t p3 = fma2(pk(U.x3w, U.w3w), zz, fma2(pk(U.x3s, U.w3s), ss, fma2(pk(U.x3a, U.w3a), aa, pk(C.x3, C.w3))));
+  uint64_t p4 = fma2(pk(U.x4w, U.w4w), zz, fma2(pk(U.x4s, U.w4s), ss, fma2(pk(U.x4a, U.w4a), aa, pk(C.x4, C.w4))));
+  uint64_t pf = fma2(pk(U.faw, U.fsw), zz, fma2(pk(U.fas, U.fss), ss,
+                fma2(pk(U.faa, U.fsa), aa, add2(pk(e_ca, e_sm), pk(C.fa, C.fs)))));
+  float p = fma_rn(U.fww, z, fma_rn(U.fws, s, fma_rn(U.fwa, a, e_w + C.fw)));
+  w2 = fma_rn(U.w2n1, n1, w2);
+  const uint64_t nn1 = pk(n1, n1);
+  p3 = fma2(pk(U.x3n1, U.w3n1), nn1, p3);
+  p4 = fma2(pk(U.x4n1, U.w4n1), nn1, p4);
+  pf = fma2(pk(U.fan1, U.fsn1), nn1, pf);
+  p = fma_rn(U.fwn1, n1, p);
+  const float n2 = tq(x2, w2);
+  upk(p3, x3, w3);
+  w3 = fma_rn(U.w3n2, n2, w3);
+  const uint64_t nn2 = pk(n2, n2);
+  p4 = fma2(pk(U.x4n2, U.w4n2), nn2, p4);
+  pf = fma2(pk(U.fan2, U.fsn2), nn2, pf);
+  p = fma_rn(U.fwn2, n2, p);
+  const float n3 = tq(x3, w3);
+  upk(p4, x4, w4);
+  w4 = fma_rn(U.w4n3, n3, w4);
+  upk(pf, q_ca, q_sm);
+  q_sm = fma_rn(U.fsn3, n3, q_sm);
+  p = fma_rn(U.fwn3, n3, p);
+  const float n4 = tq(x4, w4);
+  w = fma_rn(U.fwn4, n4, p);
+#ifdef RRG_V_WABS1
+  w_abs = w + C.r_w;
+#else
+  w_abs = fma_rn(U.fwn4, n4, p + C.r_w);
+#endif
 }
 
 template <typename T>
-__device__ __forceinline__ void rk4_step_fast(const RhsU<T>& U, const RhsC<T>& C, T dt, T& q_ca,
-                                              T& w, T& q_sm, T& w_abs, T e_ca, T e_w, T e_sm) {
-  rk4_step_fast<T>(U, C, step_consts<T>(U, dt), q_ca, w, q_sm, w_abs, e_ca, e_w, e_sm);
+__device__ __forceinline__ void rk4_step_fast(const StepU<T>& U, const PowTable* pw, const StepC<T>& C,
+                                              T& q_ca, T& w, T& q_sm, T& w_abs, T e_ca, T e_w, T e_sm) {
+  rk4_step_with(U, C, q_ca, w, q_sm, w_abs, e_ca, e_w, e_sm,
+                   [&](T x, T speed) { return torque(U, pw, x, speed); });
 }
 
 // ---------------------------------------------------------------------------

@@ -60,23 +60,20 @@ slack_error_kernel(const Launch L, float band, double* __restrict__ err, int32_t
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= N) return;
   const ScenSrc src = L.st->src[0];
-  RhsU<float> K32 = L.u32;
-  RhsC<float> C32 = L.cand_c32[i];
-  RhsU<double> K64 = L.u64;
-  RhsC<double> C64 = L.cand_c64[i];
-  double p32 = L.params[P_P_ATM], p64 = p32;
-  if constexpr (PU) {
-    const double* mk = L.pmul + static_cast<size_t>(k) * RRG_NPARAM;
-    p32 = scenario_model<float>(L.params, mk, L.cand_v[i], L.k64.pws, L.y_min, K32, C32);
-    p64 = scenario_model<double>(L.params, mk, L.cand_v[i], L.k64.pws, L.y_min, K64, C64);
-  }
+  RhsC<float> R32 = L.cand_c32[i];
+  RhsC<double> R64 = L.cand_c64[i];
+  LaneModel<float> M32;
+  LaneModel<double> M64;
+  const double v = PU ? L.cand_v[i] : 0.0;
+  const double p32 = lane_model<float, PU>(L, 0, k, v, R32, M32);
+  const double p64 = lane_model<double, PU>(L, 0, k, v, R64, M64);
+  const StepC<float>& C32 = M32.C;
+  const StepC<double>& C64 = M64.C;
   // starting states exactly as the rollouts of each precision form them
   float a_ca, a_w, a_sm, a_wa;
   double b_ca, b_w, b_sm, b_wa;
-  start_state<float>(C32, L.st->x, p32, a_ca, a_w, a_sm, a_wa);
-  start_state<double>(C64, L.st->x, p64, b_ca, b_w, b_sm, b_wa);
-  const StepC<float> S32 = step_consts<float>(K32, static_cast<float>(L.dt));
-  const StepC<double> S64 = step_consts<double>(K64, L.dt);
+  start_state<float>(R32, L.st->x, p32, a_ca, a_w, a_sm, a_wa);
+  start_state<double>(R64, L.st->x, p64, b_ca, b_w, b_sm, b_wa);
 
   float s32 = checked_slack<float>(C32, a_ca, a_w, a_sm);
   double s64 = checked_slack<double>(C64, b_ca, b_w, b_sm);
@@ -120,8 +117,8 @@ slack_error_kernel(const Launch L, float band, double* __restrict__ err, int32_t
       e1 = L.d32[HN + q];
       e2 = L.d32[2 * HN + q];
     }
-    rk4_step_fast<float>(K32, C32, S32, a_ca, a_w, a_sm, a_wa, e0, e1, e2);
-    rk4_step_fast<double>(K64, C64, S64, b_ca, b_w, b_sm, b_wa, f0, f1, f2);
+    rk4_step_fast<float>(M32.U, nullptr, C32, a_ca, a_w, a_sm, a_wa, e0, e1, e2);
+    rk4_step_fast<double>(M64.U, M64.pw, C64, b_ca, b_w, b_sm, b_wa, f0, f1, f2);
     s32 = checked_slack<float>(C32, a_ca, a_w, a_sm);
     s64 = checked_slack<double>(C64, b_ca, b_w, b_sm);
     const double e = step_err(s32, s64);

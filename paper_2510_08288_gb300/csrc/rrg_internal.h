@@ -127,6 +127,35 @@ struct SearchCfg {
   double y_min, eps_ss, y_c;
 };
 
+// One model's constants in the form the rollouts use: what the candidate
+// constants need (binary64), the step's coefficients and what carries the
+// candidate constants through the stages (StepU, StepPhi).
+struct ModelC {
+  double l_ca, l_cs;        // d_ca = -l_ca ca + l_cs sm - b_ca v
+  double l_ww, l_ws;        // d_w  = -l_ww w + l_ws sm + d0 + v (d1 + d2 v) - N
+  double l_sa, l_sw, l_ss;  // d_sm = l_sa ca + l_sw w - l_ss sm
+  double b_ca, d0, d1, d2;
+  double ky;                // OER per pascal: ky / v
+  double p_atm, inv_p_atm;
+};
+template <typename T>
+struct StepModel {
+  ModelC c;
+  StepU<T> U;
+  StepPhi<T> F;
+  const PowTable* pw;       // binary64 x^e - 1 (device memory; nullptr: pow)
+};
+
+// The model of every scenario of a pair under parametric uncertainty, folded
+// once per draw for the binary32 rollouts; arrays over the scenarios, so a
+// warp's reads are coalesced: value j of scenario k at [j * N + k].
+constexpr int kFoldDoubles = sizeof(ModelC) / sizeof(double);
+constexpr int kFoldFloats = (sizeof(StepU<float>) + sizeof(StepPhi<float>)) / sizeof(float);
+struct ScenFold {
+  double* d;   // [kFoldDoubles][N]: ModelC
+  float* f;    // [kFoldFloats][N]: StepU<float>, StepPhi<float>
+};
+
 // Everything a launch needs; filled by the host side from the handle.
 struct Launch {
   cudaStream_t stream;
@@ -145,8 +174,8 @@ struct Launch {
   const double* params;         // [RRG_NPARAM] (device)
   Fc3K<double> k64;             // folded model constants, passed by value
   Fc3K<float> k32;
-  RhsU<double> u64;             // the rollout's multiplied-out constants
-  RhsU<float> u32;
+  StepModel<double> m64;        // the rollout step's coefficients
+  StepModel<float> m32;
   double* d64;                  // scenarios [3][H][N]
   float* d32;
   double* d64b;                 // second pair for closed loops (sampling of update t+1
@@ -174,6 +203,7 @@ struct Launch {
   // + p] of each scenario pair (nullptr when off)
   double* pmul;
   double* pmulb;
+  ScenFold fold, foldb;         // the folded models of each pair's scenarios
   double punc_rho;
   uint32_t punc_mask;
   // host: the tensor maps of the two binary32 scenario arrays (the second
@@ -264,91 +294,168 @@ __host__ __device__ inline double add_rn(double a, double b) {
 #endif
 }
 
-// The multiplied-out constants of the rollout right-hand side (products and
-// sums of the folded binary64 constants, each rounded on its own, then
-// rounded once to binary32), the same bits on the host and the device.
-__host__ __device__ inline void fold_rhs(const Fc3K<double>& K, RhsU<double>* u64, RhsU<float>* u32) {
-  RhsU<double> U;
-  U.a1 = mul_rn(K.RT_Vca, K.k_sm);
-  U.a12 = add_rn(U.a1, mul_rn(K.RT_Vca, K.k_ca));
-  U.a_w = K.a_w;
-  U.a_p = K.a_p;
-  U.b3 = mul_rn(K.RT_Vsm, K.k_sm);
-  U.g_w = mul_rn(K.RT_Vsm, K.a_w);
-  U.g_sm = add_rn(mul_rn(K.RT_Vsm, K.a_p), U.b3);
-  U.inv_p_atm = K.inv_p_atm;
-  U.e = K.e;
-  U.e1 = mul_rn(mul_rn(K.C_m, K.K_p), K.inv_J);
-  U.e2 = mul_rn(mul_rn(K.C_m, K.k_v), K.inv_J);
-  U.e3 = mul_rn(K.C_cp, K.inv_J);
-  U.pws = K.pws;
-  *u64 = U;
-  RhsU<float> F;
-  F.a1 = static_cast<float>(U.a1);
-  F.a12 = static_cast<float>(U.a12);
-  F.a_w = static_cast<float>(U.a_w);
-  F.a_p = static_cast<float>(U.a_p);
-  F.b3 = static_cast<float>(U.b3);
-  F.g_w = static_cast<float>(U.g_w);
-  F.g_sm = static_cast<float>(U.g_sm);
-  F.inv_p_atm = static_cast<float>(U.inv_p_atm);
-  F.e = static_cast<float>(U.e);
-  F.e1 = static_cast<float>(U.e1);
-  F.e2 = static_cast<float>(U.e2);
-  F.e3 = static_cast<float>(U.e3);
-  F.pws = nullptr;
-  *u32 = F;
+// L v (components ca, w, sm) of the linear part, each product and sum
+// rounded on its own.
+struct Vec3 { double a, w, s; };
+__host__ __device__ inline Vec3 lin(const ModelC& m, const Vec3& v) {
+  Vec3 r;
+  r.a = add_rn(mul_rn(m.l_cs, v.s), -mul_rn(m.l_ca, v.a));
+  r.w = add_rn(mul_rn(m.l_ws, v.s), -mul_rn(m.l_ww, v.w));
+  r.s = add_rn(add_rn(mul_rn(m.l_sw, v.w), mul_rn(m.l_sa, v.a)), -mul_rn(m.l_ss, v.s));
+  return r;
+}
+// u + c v
+__host__ __device__ inline Vec3 axpy(double c, const Vec3& v, const Vec3& u) {
+  return Vec3{add_rn(u.a, mul_rn(c, v.a)), add_rn(u.w, mul_rn(c, v.w)), add_rn(u.s, mul_rn(c, v.s))};
+}
+__host__ __device__ inline Vec3 scale(double c, const Vec3& v) {
+  return Vec3{mul_rn(c, v.a), mul_rn(c, v.w), mul_rn(c, v.s)};
 }
 
-// Candidate constants of the rollouts about the reference point q_r (gauge
-// coordinates; binary32 values, or 0 for the gauge form), with the output
-// bound y_min folded into the slack offset.  Every operation is rounded on
-// its own in binary64 (no fused multiply-add), so each call site computes the
-// same bits; the products a1, a2, b3, e2 are those of fold_rhs.
-__device__ __forceinline__ void fold_rhs_cand(const Fc3K<double>& K, const CandK<double>& C,
-                                              const double q_r[3], double y_min,
-                                              RhsC<double>* c64, RhsC<float>* c32) {
-  const double a1 = __dmul_rn(K.RT_Vca, K.k_sm), a2 = __dmul_rn(K.RT_Vca, K.k_ca);
-  const double b3 = __dmul_rn(K.RT_Vsm, K.k_sm);
-  const double e2 = __dmul_rn(__dmul_rn(K.C_m, K.k_v), K.inv_J);
-  const double s_r = __dsub_rn(q_r[2], q_r[0]);
+// Folds the model's constants for the rollout step of size h (rk4_step_fast),
+// the same bits on the host and the device.
+__host__ __device__ inline void fold_model(const Fc3K<double>& K, const double* P, double h,
+                                           StepModel<double>* out) {
+  ModelC m;
+  m.l_cs = mul_rn(K.RT_Vca, K.k_sm);
+  m.l_ca = add_rn(m.l_cs, mul_rn(K.RT_Vca, K.k_ca));
+  const double e1 = mul_rn(mul_rn(K.C_m, K.K_p), K.inv_J);
+  const double cj = mul_rn(K.C_m, K.inv_J);
+  m.l_ww = add_rn(mul_rn(cj, K.k_v), mul_rn(e1, K.a_w));
+  m.l_ws = mul_rn(e1, K.a_p);
+  m.l_sa = mul_rn(K.RT_Vsm, K.k_sm);
+  m.l_sw = mul_rn(K.RT_Vsm, K.a_w);
+  m.l_ss = add_rn(mul_rn(K.RT_Vsm, K.a_p), m.l_sa);
+  const double kw = mul_rn(P[P_M_O2], P[P_N_CELL]) / mul_rn(4.0, P[P_FARADAY]);  // W_o2 = kw v
+  m.b_ca = mul_rn(K.RT_Vca, kw);
+  m.d0 = mul_rn(cj, P[P_C0]);
+  m.d1 = mul_rn(cj, add_rn(P[P_C1], mul_rn(K.K_p, mul_rn(P[P_LAM_REF], kw) / P[P_X_O2])));
+  m.d2 = mul_rn(cj, P[P_C2]);
+  m.ky = mul_rn(P[P_X_O2], P[P_K_SM]) / kw;
+  m.p_atm = P[P_P_ATM];
+  m.inv_p_atm = K.inv_p_atm;
+  out->c = m;
+
+  StepU<double>& U = out->U;
+  StepPhi<double>& F = out->F;
+  const double h2 = mul_rn(0.5, h), h6 = h / 6.0, ip = K.inv_p_atm;
+  const double e3 = mul_rn(K.C_cp, K.inv_J);
+  U.ip = ip;
+  U.e = K.e;
+  U.A = mul_rn(e3, K.a_w);
+  U.B = mul_rn(mul_rn(e3, K.a_p), P[P_P_ATM]);
+  F.h = h;
+  F.h2 = h2;
+  // the columns of M_2, M_3, M_4, R and of the combination that carries c
+  Vec3 M2[3], M3[3], M4[3], R[3], Ph[3];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int j = 0; j < 3; ++j) {
+    const Vec3 u{j == 0 ? 1.0 : 0.0, j == 1 ? 1.0 : 0.0, j == 2 ? 1.0 : 0.0};
+    const Vec3 l1 = lin(m, u);
+    M2[j] = axpy(h2, l1, u);
+    const Vec3 l2 = lin(m, M2[j]);
+    M3[j] = axpy(h2, l2, u);
+    const Vec3 l3 = lin(m, M3[j]);
+    M4[j] = axpy(h, l3, u);
+    const Vec3 l4 = lin(m, M4[j]);
+    R[j] = axpy(h6, axpy(2.0, l2, axpy(2.0, l3, axpy(1.0, l1, l4))), u);
+    Ph[j] = scale(h6, axpy(2.0, M2[j], axpy(2.0, M3[j], axpy(1.0, u, M4[j]))));
+  }
+  U.x2a = mul_rn(ip, M2[0].s); U.x2w = mul_rn(ip, M2[1].s); U.x2s = mul_rn(ip, M2[2].s);
+  U.w2w = M2[1].w; U.w2s = M2[2].w;
+  U.x3a = mul_rn(ip, M3[0].s); U.x3w = mul_rn(ip, M3[1].s); U.x3s = mul_rn(ip, M3[2].s);
+  U.w3a = M3[0].w; U.w3w = M3[1].w; U.w3s = M3[2].w;
+  U.x4a = mul_rn(ip, M4[0].s); U.x4w = mul_rn(ip, M4[1].s); U.x4s = mul_rn(ip, M4[2].s);
+  U.w4a = M4[0].w; U.w4w = M4[1].w; U.w4s = M4[2].w;
+  U.faa = R[0].a; U.faw = R[1].a; U.fas = R[2].a;
+  U.fsa = R[0].s; U.fsw = R[1].s; U.fss = R[2].s;
+  U.fwa = R[0].w; U.fww = R[1].w; U.fws = R[2].w;
+  F.aa = Ph[0].a; F.aw = Ph[1].a; F.as = Ph[2].a;
+  F.sa = Ph[0].s; F.sw = Ph[1].s; F.ss = Ph[2].s;
+  F.wa = Ph[0].w; F.ww = Ph[1].w; F.ws = Ph[2].w;
+  // the torque's columns: k_i = L z_i + c - N_i e_w
+  const Vec3 ew{0.0, 1.0, 0.0};
+  const Vec3 le = lin(m, ew);
+  // N_1: z_2 = -h2 e_w, z_3 = h2 L z_2, z_4 = h L z_3
+  const Vec3 p2 = scale(-h2, ew), lp2 = scale(-h2, le);
+  const Vec3 p3 = scale(h2, lp2), lp3 = lin(m, p3);
+  const Vec3 p4 = scale(h, lp3), lp4 = lin(m, p4);
+  const Vec3 f1 = scale(h6, axpy(2.0, lp2, axpy(2.0, lp3, axpy(-1.0, ew, lp4))));
+  // N_2: z_3 = -h2 e_w, z_4 = h L z_3
+  const Vec3 q4 = scale(h, lp2), lq4 = lin(m, q4);
+  const Vec3 f2 = scale(h6, axpy(2.0, lp2, axpy(-2.0, ew, lq4)));
+  // N_3: z_4 = -h e_w
+  const Vec3 f3 = scale(h6, axpy(-2.0, ew, scale(-h, le)));
+  U.w2n1 = p2.w;
+  U.x3n1 = mul_rn(ip, p3.s);
+  U.w3n1 = p3.w;
+  U.w3n2 = p2.w;
+  U.x4n1 = mul_rn(ip, p4.s);
+  U.w4n1 = p4.w;
+  U.x4n2 = mul_rn(ip, q4.s);
+  U.w4n2 = q4.w;
+  U.w4n3 = -h;
+  U.fan1 = f1.a; U.fsn1 = f1.s; U.fwn1 = f1.w;
+  U.fan2 = f2.a; U.fsn2 = f2.s; U.fwn2 = f2.w;
+  U.fsn3 = f3.s; U.fwn3 = f3.w;
+  U.fwn4 = -h6;
+  out->pw = K.pws;
+}
+
+// The coefficients rounded once to binary32 (StepU and StepPhi hold nothing
+// but T values).
+__host__ __device__ inline void round_model(const StepModel<double>& m, StepModel<float>* out) {
+  static_assert(sizeof(StepU<double>) == 2 * sizeof(StepU<float>) &&
+                sizeof(StepPhi<double>) == 2 * sizeof(StepPhi<float>), "arrays of T");
+  out->c = m.c;
+  out->pw = nullptr;
+  const double* u = &m.U.ip;
+  float* uf = &out->U.ip;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (size_t i = 0; i < sizeof(StepU<float>) / sizeof(float); ++i) uf[i] = static_cast<float>(u[i]);
+  const double* p = &m.F.h;
+  float* pf = &out->F.h;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (size_t i = 0; i < sizeof(StepPhi<float>) / sizeof(float); ++i) pf[i] = static_cast<float>(p[i]);
+}
+
+// Candidate constants of the rollouts at setpoint v about the reference point
+// q_r (gauge coordinates; binary32 values, or 0 for the gauge form), with the
+// output bound y_min folded into the slack offset: the derivative at q_r
+// without the torque, c = L q_r + b(v).  Every operation is rounded on its own
+// in binary64, so each call site computes the same bits.
+__device__ __forceinline__ RhsC<double> fold_cand(const ModelC& m, double v, const double q_r[3],
+                                                  double y_min) {
+  const Vec3 l = lin(m, Vec3{q_r[0], q_r[1], q_r[2]});
   RhsC<double> R;
-  R.W_r = __dsub_rn(__dmul_rn(K.a_w, q_r[1]), __dmul_rn(K.a_p, q_r[2]));
-  R.c_ca = __dsub_rn(__dsub_rn(__dmul_rn(a1, s_r), __dmul_rn(a2, q_r[0])), __dmul_rn(K.RT_Vca, C.W_o2));
-  R.c_sm = __dsub_rn(__dmul_rn(K.RT_Vsm, R.W_r), __dmul_rn(b3, s_r));
-  R.e0 = __dsub_rn(__dmul_rn(__dmul_rn(K.C_m, C.V0), K.inv_J), __dmul_rn(e2, q_r[1]));
-  R.x_r = __dadd_rn(1.0, __dmul_rn(q_r[2], K.inv_p_atm));
-  R.y_scale = C.y_scale;
-  R.s_off = __dsub_rn(__dmul_rn(C.y_scale, s_r), y_min);
+  R.c_ca = __dsub_rn(l.a, __dmul_rn(m.b_ca, v));
+  R.c_w = __dadd_rn(l.w, __dadd_rn(m.d0, __dmul_rn(v, __dadd_rn(m.d1, __dmul_rn(m.d2, v)))));
+  R.c_sm = l.s;
+  R.x_r = __dadd_rn(1.0, __dmul_rn(q_r[2], m.inv_p_atm));
+  // 1 / v without the division's instructions, inside its range
+  const unsigned ev = (static_cast<unsigned>(__double2hiint(v)) & 0x7fffffffu) >> 20;
+  R.y_scale = (ev > 24u && ev < 2022u) ? __dmul_rn(m.ky, rcp_cubic(v)) : __ddiv_rn(m.ky, v);
+  R.s_off = __dsub_rn(__dmul_rn(R.y_scale, __dsub_rn(q_r[2], q_r[0])), y_min);
   R.r_ca = q_r[0];
   R.r_w = q_r[1];
   R.r_sm = q_r[2];
-  *c64 = R;
-  c32->c_ca = static_cast<float>(R.c_ca);
-  c32->c_sm = static_cast<float>(R.c_sm);
-  c32->W_r = static_cast<float>(R.W_r);
-  c32->e0 = static_cast<float>(R.e0);
-  c32->x_r = static_cast<float>(R.x_r);
-  c32->y_scale = static_cast<float>(R.y_scale);
-  c32->s_off = static_cast<float>(R.s_off);
-  c32->r_ca = static_cast<float>(R.r_ca);
-  c32->r_w = static_cast<float>(R.r_w);
-  c32->r_sm = static_cast<float>(R.r_sm);
+  return R;
+}
+__device__ __forceinline__ RhsC<float> round_cand(const RhsC<double>& R) {
+  return RhsC<float>{static_cast<float>(R.c_ca), static_cast<float>(R.c_w), static_cast<float>(R.c_sm),
+                     static_cast<float>(R.x_r), static_cast<float>(R.y_scale), static_cast<float>(R.s_off),
+                     static_cast<float>(R.r_ca), static_cast<float>(R.r_w), static_cast<float>(R.r_sm)};
 }
 
-// Coefficients of the binary64 x^e - 1 series (host).
-inline void make_pow_series(double e, PowSeries* S) {
-  const double c = 1.5, lc = std::log(c);
-  const double ce = std::exp(e * lc);
-  S->e = e;
-  S->inv_c = 1.0 / c;
-  S->a[0] = std::expm1(e * lc);
-  double b = 1.0;  // binom(e, n)
-  for (int n = 1; n <= 32; ++n) {
-    b = b * (e - static_cast<double>(n - 1)) / static_cast<double>(n);
-    S->a[n] = ce * b;
-  }
-}
+// Table of the binary64 x^e - 1 (host; rrg_capi.cu); false, and an unusable
+// table, for an exponent outside [-1, 1].
+bool pow_table(double e, PowTable* S);
 
 // ---- kernel launchers (rrg_kernels.cu) --------------------------------
 // dual: write the pair (base + *t_dev) & 1 (closed loops with two pairs).
@@ -356,6 +463,12 @@ inline void make_pow_series(double e, PowSeries* S) {
 cudaError_t launch_sample(const Launch& L, uint64_t seed, uint64_t base,
                           const unsigned long long* t_dev, const double* amp, bool dual = false,
                           cudaStream_t stream = nullptr);
+// The folded models of a pair's scenarios (parametric uncertainty; nothing
+// otherwise) from its multipliers: pair 0, or pair 1 (second), or by the parity
+// of base + *t_dev (dual).  launch_sample runs it after its draw.
+cudaError_t launch_scenario_fold(const Launch& L, bool second, uint64_t base = 0,
+                                 const unsigned long long* t_dev = nullptr, bool dual = false,
+                                 cudaStream_t stream = nullptr);
 // Fills pair 0's binary64 array from its Philox counters if it was sampled
 // lazily (no-op otherwise).
 cudaError_t launch_materialize64(const Launch& L);

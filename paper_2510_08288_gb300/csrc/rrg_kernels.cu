@@ -58,30 +58,25 @@ cudaError_t launch_equilibrium(const Launch& L, double v, double* d_out4, int32_
 // a launch whose lanes each run alone on a scheduler.  out[0] = cycles per
 // step, out[1] keeps the lanes' results alive; *status = the equilibrium's.
 __global__ void __launch_bounds__(32)
-step_latency_kernel(const Launch L, const RhsU<float> U, double v, int steps, double* out,
-                    int32_t* status) {
+step_latency_kernel(const Launch L, double v, int steps, double* out, int32_t* status) {
   const CandK<double> Cd = cand_consts(L.params, v);
-  RhsC<double> c64;
-  RhsC<float> c32;
   float q[3] = {0.0f, 0.0f, 0.0f}, y = 0.0f;
   const int rc = equilibrium_from<float>(L.k32, L.params, Cd, q, &y);
   const double q_r[3] = {q[0], q[1], q[2]};
-  fold_rhs_cand(L.k64, Cd, q_r, L.y_min, &c64, &c32);
+  const StepU<float> U = L.m32.U;
+  const StepC<float> C = step_consts<float>(U, L.m32.F, round_cand(fold_cand(L.m64.c, v, q_r, L.y_min)));
   // deviation coordinates about the equilibrium, lanes slightly apart
-  float q_ca = 1e-3f * static_cast<float>(threadIdx.x), w = 0.0f, q_sm = 0.0f, w_abs = c32.r_w;
-  const StepC<float> S = step_consts<float>(U, static_cast<float>(L.dt));
-  float smin = inf_v<float>(), nf = 0.0f;
+  float q_ca = 1e-3f * static_cast<float>(threadIdx.x), w = 0.0f, q_sm = 0.0f, w_abs = C.r_w;
+  BlockMin<float> bm;
   __syncwarp();
   const long long t0 = clock64();
 #pragma unroll 8
   for (int j = 0; j < steps; ++j) {
-    rk4_step_fast<float>(U, c32, S, q_ca, w, q_sm, w_abs, 0.0f, 0.0f, 0.0f);
-    const float s = c32.y_scale * (q_sm - q_ca) + c32.s_off;
-    smin = fminf(smin, s);
-    nf = fma_rn(s, 0.0f, nf);
+    rk4_step_fast<float>(U, nullptr, C, q_ca, w, q_sm, w_abs, 0.0f, 0.0f, 0.0f);
+    bm.add(slack_of<float>(C, q_ca, q_sm), j);
   }
   const long long t1 = clock64();
-  float r = smin + nf + q_ca + w + q_sm + w_abs;
+  float r = bm.result(q_ca, w, q_sm) + q_ca + w + q_sm + w_abs;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
   if (threadIdx.x == 0) {
@@ -92,7 +87,7 @@ step_latency_kernel(const Launch L, const RhsU<float> U, double v, int steps, do
 }
 
 cudaError_t launch_step_latency(const Launch& L, double v, int steps, double* d_out2, int32_t* d_status) {
-  step_latency_kernel<<<1, 32, 0, L.stream>>>(L, L.u32, v, steps, d_out2, d_status);
+  step_latency_kernel<<<1, 32, 0, L.stream>>>(L, v, steps, d_out2, d_status);
   return cudaGetLastError();
 }
 
@@ -175,6 +170,42 @@ __global__ void sample_kernel(double* __restrict__ d64, float* __restrict__ d32,
   }
 }
 
+// Every scenario's model folded for the binary32 rollouts (ScenFold), one
+// thread per scenario, from the multipliers the draw of update base + *t_dev
+// (the pair by its parity if dual) or the caller wrote.  About 600 binary64
+// instructions a warp, once per draw instead of once per rollout lane.
+__global__ void __launch_bounds__(32)
+scenario_fold_kernel(const Launch L, uint64_t base, const unsigned long long* t_dev, int dual) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= L.N) return;
+  const int pair = (dual && ((base + (t_dev ? *t_dev : 0ull)) & 1ull)) ? 1 : 0;
+  const double* pm = (pair ? L.pmulb : L.pmul) + static_cast<size_t>(k) * RRG_NPARAM;
+  const ScenFold sf = pair ? L.foldb : L.fold;
+  StepModel<double> m;
+  scenario_fold(L.params, pm, L.dt, nullptr, &m);
+  StepModel<float> f;
+  round_model(m, &f);
+  const size_t N = static_cast<size_t>(L.N);
+  const double* d = &m.c.l_ca;
+#pragma unroll
+  for (int j = 0; j < kFoldDoubles; ++j) sf.d[j * N + k] = d[j];
+  constexpr int nu = sizeof(StepU<float>) / sizeof(float);
+  const float* u = &f.U.ip;
+#pragma unroll
+  for (int j = 0; j < nu; ++j) sf.f[j * N + k] = u[j];
+  const float* p = &f.F.h;
+#pragma unroll
+  for (int j = 0; j < kFoldFloats - nu; ++j) sf.f[(nu + j) * N + k] = p[j];
+}
+
+cudaError_t launch_scenario_fold(const Launch& L, bool second, uint64_t base, const unsigned long long* t_dev,
+                                 bool dual, cudaStream_t stream) {
+  if (L.pmul == nullptr) return cudaSuccess;
+  scenario_fold_kernel<<<(L.N + 31) / 32, 32, 0, stream ? stream : L.stream>>>(
+      L, second ? 1ull : base, t_dev, (second || dual) ? 1 : 0);
+  return cudaGetLastError();
+}
+
 static int grid_for(size_t n, int threads, int cap) {
   size_t b = (n + threads - 1) / threads;
   if (b < 1) b = 1;
@@ -196,7 +227,9 @@ cudaError_t launch_sample(const Launch& L, uint64_t seed, uint64_t base,
       L.d64, L.d32, dual ? L.d64b : nullptr, dual ? L.d32b : nullptr, L.N, L.H, seed, base, t_dev,
       amp[0], amp[1], amp[2], write64, L.scen_gen, L.st, L.pmul, dual ? L.pmulb : nullptr, L.punc_rho,
       L.punc_mask, L.kbase);
-  return cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_scenario_fold(L, false, base, t_dev, dual && L.d64b != nullptr, stream);
 }
 
 __global__ void fill_kernel(double* __restrict__ a, size_t n, double v) {
@@ -323,8 +356,7 @@ __device__ __forceinline__ void reduce_lane(const Launch& L, int i, int k, int N
 }
 
 template <typename T, bool PU, int SRC>
-__device__ __forceinline__ void rollout_body(const Launch& L, const RhsU<T>& K0,
-                                             const T* __restrict__ d_pair0,
+__device__ __forceinline__ void rollout_body(const Launch& L, const T* __restrict__ d_pair0,
                                              const T* __restrict__ d_pair1,
                                              const RhsC<T>* __restrict__ cand, int early_exit,
                                              int classify, const void* tm0 = nullptr,
@@ -358,8 +390,8 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const RhsU<T>& K0,
     const int dead0 = __shfl_sync(0xffffffffu, (threadIdx.x & 31) == 0 ? *dead : 0, 0);
     if (dead0) return;
   }
-  RhsC<T> C = cand[i];
-  RhsU<T> K = K0;
+  RhsC<T> R = cand[i];
+  LaneModel<T> M;
   const T eps = static_cast<T>(L.eps_abs);
   const T thr = early_exit != RRG_EXIT_NONE ? (classify ? -eps : T(0)) : -inf_v<T>();
 
@@ -374,14 +406,14 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const RhsU<T>& K0,
   LaneState<T>* ls = nullptr;
   T q_ca = T(0), w = T(0), q_sm = T(0), w_abs = T(0);  // the deviation from the candidate's reference point
   T smin0 = inf_v<T>();
+  // lanes past the scenarios (the TMA ring's, which keep their warp company)
+  // take the last one's model
+  const double p_atm = lane_model<T, PU>(L, L.st->buf, active ? k : N - 1, PU ? L.cand_v[i] : 0.0, R, M);
+  const StepU<T>& K = M.U;
+  const StepC<T>& C = M.C;
   if (active) {
     if (mode != SEG_FULL) ls = static_cast<LaneState<T>*>(L.lane_state) + static_cast<size_t>(i) * N + k;
-    double p_atm = L.params[P_P_ATM];
-    if constexpr (PU)
-      p_atm = scenario_model<T>(L.params,
-                                (L.st->buf ? L.pmulb : L.pmul) + static_cast<size_t>(k) * RRG_NPARAM,
-                                L.cand_v[i], L.k64.pws, L.y_min, K, C);
-    start_state<T>(C, L.st->x, p_atm, q_ca, w, q_sm, w_abs);
+    start_state<T>(R, L.st->x, p_atm, q_ca, w, q_sm, w_abs);
     if (mode == SEG_CONTINUE) {
       const LaneState<T> st = *ls;
       if (st.status != 0) {
@@ -406,8 +438,8 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const RhsU<T>& K0,
                      2 * wid;
     const bool lane_runs = active && final_lane;
     const void* tm = (L.inject & RRG_INJECT_TMA_NO_COPY) ? nullptr : (L.st->buf ? tm1 : tm0);
-    const T s_out = run_lane_tma(K, C, tm, k & ~31, lane_runs, j0, j_end, q_ca, w, q_sm,
-                                 w_abs, smin0, static_cast<T>(L.dt), thr, cand_stop ? dead : nullptr,
+    const T s_out = run_lane_tma<PU>(K, C, tm, k & ~31, lane_runs, j0, j_end, q_ca, w, q_sm,
+                                 w_abs, smin0, thr, cand_stop ? dead : nullptr,
                                  cand_stop ? dead : nullptr, &steps, &end, band, &jlast, stages, bars,
                                  &L.stats->wait_timeouts);
     if (lane_runs) smin = s_out;
@@ -416,18 +448,15 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const RhsU<T>& K0,
       atomicAdd(&L.stats->lane_steps_tma, static_cast<unsigned long long>(wsteps));
   } else if (active && final_lane) {
     if constexpr (SRC == SRC_GEN)
-      smin = run_lane_gen<T>(K, C, L.st->src[L.st->buf], k, j0, j_end, q_ca, w, q_sm, w_abs, smin0,
-                             static_cast<T>(L.dt), thr,
+      smin = run_lane_gen<T>(K, M.pw, C, L.st->src[L.st->buf], k, j0, j_end, q_ca, w, q_sm, w_abs, smin0, thr,
                              cand_stop ? dead : nullptr, &steps, &end, band, &jlast);
     else if constexpr (SRC == SRC_RING) {
       static_assert(sizeof(T) == 4, "the shared-memory ring is binary32");
       __shared__ float ring[RRG_RING_DEPTH * 3 * kRollThreads];
-      smin = run_lane_ring(K, C, d, k, N, L.H, j0, j_end, q_ca, w, q_sm, w_abs, smin0,
-                           static_cast<T>(L.dt), thr,
+      smin = run_lane_ring(K, C, d, k, N, L.H, j0, j_end, q_ca, w, q_sm, w_abs, smin0, thr,
                            cand_stop ? dead : nullptr, &steps, &end, band, &jlast, ring);
     } else
-      smin = run_lane<T>(K, C, d, k, N, L.H, j0, j_end, q_ca, w, q_sm, w_abs, smin0,
-                         static_cast<T>(L.dt), thr,
+      smin = run_lane<T>(K, M.pw, C, d, k, N, L.H, j0, j_end, q_ca, w, q_sm, w_abs, smin0, thr,
                          cand_stop ? dead : nullptr, &steps, &end, band, &jlast);
   }
   if (active && final_lane) {
@@ -451,10 +480,9 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const RhsU<T>& K0,
 // SRC: where the lanes take their disturbances from (RollSrc).
 template <typename T, int SRC>
 __global__ void __launch_bounds__(kRollThreads)
-rollout_kernel(const Launch L, const RhsU<T> K, const T* __restrict__ d_pair0,
-               const T* __restrict__ d_pair1, const RhsC<T>* __restrict__ cand, int early_exit,
-               int classify) {
-  rollout_body<T, false, SRC>(L, K, d_pair0, d_pair1, cand, early_exit, classify);
+rollout_kernel(const Launch L, const T* __restrict__ d_pair0, const T* __restrict__ d_pair1,
+               const RhsC<T>* __restrict__ cand, int early_exit, int classify) {
+  rollout_body<T, false, SRC>(L, d_pair0, d_pair1, cand, early_exit, classify);
 }
 
 // Parametric uncertainty: the per-lane constants need about 30 more
@@ -467,10 +495,9 @@ rollout_kernel(const Launch L, const RhsU<T> K, const T* __restrict__ d_pair0,
 #endif
 template <typename T, int SRC>
 __global__ void __launch_bounds__(kRollThreads, sizeof(T) == 4 ? RRG_PU_MIN_BLOCKS : 1)
-rollout_pu_kernel(const Launch L, const RhsU<T> K, const T* __restrict__ d_pair0,
-                  const T* __restrict__ d_pair1, const RhsC<T>* __restrict__ cand, int early_exit,
-                  int classify) {
-  rollout_body<T, true, SRC>(L, K, d_pair0, d_pair1, cand, early_exit, classify);
+rollout_pu_kernel(const Launch L, const T* __restrict__ d_pair0, const T* __restrict__ d_pair1,
+                  const RhsC<T>* __restrict__ cand, int early_exit, int classify) {
+  rollout_body<T, true, SRC>(L, d_pair0, d_pair1, cand, early_exit, classify);
 }
 
 // Binary32 lanes through the per-warp TMA ring (launches that leave warp
@@ -478,11 +505,10 @@ rollout_pu_kernel(const Launch L, const RhsU<T> K, const T* __restrict__ d_pair0
 // kernel parameters, so a captured graph keeps them.
 template <bool PU>
 __global__ void __launch_bounds__(kRollThreads, PU ? RRG_PU_MIN_BLOCKS : 1)
-rollout_tma_kernel(const Launch L, const RhsU<float> K, const float* __restrict__ d_pair0,
-                   const float* __restrict__ d_pair1, const RhsC<float>* __restrict__ cand, int early_exit,
+rollout_tma_kernel(const Launch L, const float* __restrict__ d_pair0, const float* __restrict__ d_pair1, const RhsC<float>* __restrict__ cand, int early_exit,
                    int classify, const __grid_constant__ CUtensorMap tm0,
                    const __grid_constant__ CUtensorMap tm1) {
-  rollout_body<float, PU, SRC_TMA>(L, K, d_pair0, d_pair1, cand, early_exit, classify, &tm0, &tm1);
+  rollout_body<float, PU, SRC_TMA>(L, d_pair0, d_pair1, cand, early_exit, classify, &tm0, &tm1);
 }
 
 // Two candidates per thread (binary32, register ring): block row y runs the
@@ -505,7 +531,7 @@ rollout_tma_kernel(const Launch L, const RhsU<float> K, const float* __restrict_
 #endif
 template <bool PU>
 __global__ void __launch_bounds__(kRollThreads, PU ? RRG_PAIR_PU_MIN_BLOCKS : RRG_PAIR_MIN_BLOCKS)
-rollout_pair_kernel(const Launch L, const RhsU<float> K0, const float* __restrict__ d_pair0,
+rollout_pair_kernel(const Launch L, const float* __restrict__ d_pair0,
                     const float* __restrict__ d_pair1, const RhsC<float>* __restrict__ cand, int early_exit,
                     int classify) {
   const float* __restrict__ d = L.st->buf ? d_pair1 : d_pair0;
@@ -541,29 +567,27 @@ rollout_pair_kernel(const Launch L, const RhsU<float> K0, const float* __restric
   int jl[2] = {-1, -1}, en[2] = {LANE_REACHED_END, LANE_REACHED_END};
   unsigned paired = 0;  // trajectory steps this lane ran two per thread
   if (active) {
-    RhsU<float> K = K0;
-    RhsC<float> CA = cand[ia], CB = cand[ib >= 0 ? ib : ia];
-    double p_atm = L.params[P_P_ATM];
-    if constexpr (PU) {
-      const double* mk = (L.st->buf ? L.pmulb : L.pmul) + static_cast<size_t>(k) * RRG_NPARAM;
-      if (runa) p_atm = scenario_model<float>(L.params, mk, L.cand_v[ia], L.k64.pws, L.y_min, K, CA);
-      if (runb) p_atm = scenario_model<float>(L.params, mk, L.cand_v[ib], L.k64.pws, L.y_min, K, CB);
-    }
+    RhsC<float> RA = cand[ia], RB = cand[ib >= 0 ? ib : ia];
+    LaneModel<float> MA, MB;
+    // the model is the scenario's, whichever candidate: MA.U serves both
+    const double p_atm = lane_model<float, PU>(L, L.st->buf, k, PU ? L.cand_v[ia] : 0.0, RA, MA);
+    lane_model<float, PU>(L, L.st->buf, k, PU ? L.cand_v[ib >= 0 ? ib : ia] : 0.0, RB, MB);
+    const StepU<float>& K = MA.U;
+    const StepC<float>&CA = MA.C, &CB = MB.C;
     float za[4], zb[4];
-    start_state<float>(CA, L.st->x, p_atm, za[0], za[1], za[2], za[3]);
-    start_state<float>(CB, L.st->x, p_atm, zb[0], zb[1], zb[2], zb[3]);
-    const float dt = static_cast<float>(L.dt);
+    start_state<float>(RA, L.st->x, p_atm, za[0], za[1], za[2], za[3]);
+    start_state<float>(RB, L.st->x, p_atm, zb[0], zb[1], zb[2], zb[3]);
     if (runa && runb) {
       paired = 2u * static_cast<unsigned>(run_lane_pair<float, RRG_PAIR_PF>(
-                            K, CA, CB, d, k, N, L.H, L.H, za, zb, dt, thr, band, cand_stop ? deada : nullptr,
+                            K, CA, CB, d, k, N, L.H, L.H, za, zb, thr, band, cand_stop ? deada : nullptr,
                             cand_stop ? deadb : nullptr, sm, st, en, jl));
     } else if (runa) {
-      sm[0] = run_lane<float, RRG_PAIR_PF>(K, CA, d, k, N, L.H, 0, L.H, za[0], za[1], za[2], za[3],
-                                           inf_v<float>(), dt, thr, cand_stop ? deada : nullptr, &st[0],
+      sm[0] = run_lane<float, RRG_PAIR_PF>(K, nullptr, CA, d, k, N, L.H, 0, L.H, za[0], za[1], za[2], za[3],
+                                           inf_v<float>(), thr, cand_stop ? deada : nullptr, &st[0],
                                            &en[0], band, &jl[0]);
     } else {
-      sm[1] = run_lane<float, RRG_PAIR_PF>(K, CB, d, k, N, L.H, 0, L.H, zb[0], zb[1], zb[2], zb[3],
-                                           inf_v<float>(), dt, thr, cand_stop ? deadb : nullptr, &st[1],
+      sm[1] = run_lane<float, RRG_PAIR_PF>(K, nullptr, CB, d, k, N, L.H, 0, L.H, zb[0], zb[1], zb[2], zb[3],
+                                           inf_v<float>(), thr, cand_stop ? deadb : nullptr, &st[1],
                                            &en[1], band, &jl[1]);
     }
     if (cand_stop && runa && sm[0] < thr) *deada = 1;
@@ -584,7 +608,7 @@ rollout_pair_kernel(const Launch L, const RhsU<float> K0, const float* __restric
 // reduced as in rollout_body.
 template <bool PU>
 __global__ void __launch_bounds__(kRollThreads, PU ? RRG_PAIR_PU_MIN_BLOCKS : RRG_PAIR_MIN_BLOCKS)
-rollout_tma_pair_kernel(const Launch L, const RhsU<float> K0, const RhsC<float>* __restrict__ cand,
+rollout_tma_pair_kernel(const Launch L, const RhsC<float>* __restrict__ cand,
                         int early_exit, int classify, const __grid_constant__ CUtensorMap tm0,
                         const __grid_constant__ CUtensorMap tm1) {
   const Seg s0 = L.st->seg[0], s1 = L.st->seg[1];
@@ -616,17 +640,16 @@ rollout_tma_pair_kernel(const Launch L, const RhsU<float> K0, const RhsC<float>*
   TmaTraj a{}, b{};
   a.smin = b.smin = inf_v<float>();
   a.jl = b.jl = -1;
-  RhsU<float> K = K0;
-  RhsC<float> CA = cand[ia], CB = cand[ib >= 0 ? ib : ia];
+  RhsC<float> RA = cand[ia], RB = cand[ib >= 0 ? ib : ia];
+  LaneModel<float> MA, MB;
+  const int km = active ? k : N - 1;
+  const double p_atm = lane_model<float, PU>(L, L.st->buf, km, PU ? L.cand_v[ia] : 0.0, RA, MA);
+  lane_model<float, PU>(L, L.st->buf, km, PU ? L.cand_v[ib >= 0 ? ib : ia] : 0.0, RB, MB);
+  const StepU<float>& K = MA.U;
+  const StepC<float>&CA = MA.C, &CB = MB.C;
   if (active) {
-    double p_atm = L.params[P_P_ATM];
-    if constexpr (PU) {
-      const double* mk = (L.st->buf ? L.pmulb : L.pmul) + static_cast<size_t>(k) * RRG_NPARAM;
-      if (runa) p_atm = scenario_model<float>(L.params, mk, L.cand_v[ia], L.k64.pws, L.y_min, K, CA);
-      if (runb) p_atm = scenario_model<float>(L.params, mk, L.cand_v[ib], L.k64.pws, L.y_min, K, CB);
-    }
-    start_state<float>(CA, L.st->x, p_atm, a.q_ca, a.w, a.q_sm, a.w_abs);
-    start_state<float>(CB, L.st->x, p_atm, b.q_ca, b.w, b.q_sm, b.w_abs);
+    start_state<float>(RA, L.st->x, p_atm, a.q_ca, a.w, a.q_sm, a.w_abs);
+    start_state<float>(RB, L.st->x, p_atm, b.q_ca, b.w, b.q_sm, b.w_abs);
   }
   const int wid = threadIdx.x >> 5;
   float* stages = reinterpret_cast<float*>(rrg_dyn_smem) + static_cast<size_t>(wid) * 2 * kTmaStageFloats;
@@ -634,7 +657,7 @@ rollout_tma_pair_kernel(const Launch L, const RhsU<float> K0, const RhsC<float>*
   const void* tm = (L.inject & RRG_INJECT_TMA_NO_COPY) ? nullptr : (L.st->buf ? &tm1 : &tm0);
   unsigned paired = 0;
   run_lane_tma_pair(K, CA, CB, tm, k & ~31, active && runa, active && runb, 0, L.H, a, b,
-                    static_cast<float>(L.dt), thr, band, cand_stop ? deada : nullptr,
+                    thr, band, cand_stop ? deada : nullptr,
                     cand_stop ? deadb : nullptr, cand_stop ? deada : nullptr, cand_stop ? deadb : nullptr, stages,
                     bars, &L.stats->wait_timeouts, &paired);
   if (active && cand_stop) {
@@ -703,15 +726,15 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
   const bool filled = !ring && L.pair == RRG_PAIR_FILLED &&
                       pair_blocks >= static_cast<long long>(RRG_PAIR_MIN_WAVES) *
                                          pair_blocks_per_sm(L.pmul != nullptr) * sms;
-#define RRG_ROLLOUT(KERNEL, T, SRC, KK, D0, D1, CAND, CLS) \
-  KERNEL<T, SRC><<<grid, kRollThreads, 0, L.stream>>>(L, KK, D0, D1, CAND, early_exit, CLS)
+#define RRG_ROLLOUT(KERNEL, T, SRC, D0, D1, CAND, CLS) \
+  KERNEL<T, SRC><<<grid, kRollThreads, 0, L.stream>>>(L, D0, D1, CAND, early_exit, CLS)
   if (use_fp64) {
     if (L.pmul) {
-      if (L.scen_gen) RRG_ROLLOUT(rollout_pu_kernel, double, SRC_GEN, L.u64, L.d64, L.d64b, L.cand_c64, 0);
-      else RRG_ROLLOUT(rollout_pu_kernel, double, SRC_REGS, L.u64, L.d64, L.d64b, L.cand_c64, 0);
+      if (L.scen_gen) RRG_ROLLOUT(rollout_pu_kernel, double, SRC_GEN, L.d64, L.d64b, L.cand_c64, 0);
+      else RRG_ROLLOUT(rollout_pu_kernel, double, SRC_REGS, L.d64, L.d64b, L.cand_c64, 0);
     } else {
-      if (L.scen_gen) RRG_ROLLOUT(rollout_kernel, double, SRC_GEN, L.u64, L.d64, L.d64b, L.cand_c64, 0);
-      else RRG_ROLLOUT(rollout_kernel, double, SRC_REGS, L.u64, L.d64, L.d64b, L.cand_c64, 0);
+      if (L.scen_gen) RRG_ROLLOUT(rollout_kernel, double, SRC_GEN, L.d64, L.d64b, L.cand_c64, 0);
+      else RRG_ROLLOUT(rollout_kernel, double, SRC_REGS, L.d64, L.d64b, L.cand_c64, 0);
     }
   } else if (!L.scen_gen && L.tmap != nullptr &&
              (L.tma == RRG_TMA_ALWAYS ||
@@ -727,36 +750,35 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
       const dim3 g2(grid.x, (m_launch + 1) / 2);
       if (L.pmul)
         rollout_tma_pair_kernel<true><<<g2, kRollThreads, kTmaSmemBytes, L.stream>>>(
-            L, L.u32, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
+            L, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
       else
         rollout_tma_pair_kernel<false><<<g2, kRollThreads, kTmaSmemBytes, L.stream>>>(
-            L, L.u32, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
+            L, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
     } else if (L.pmul) {
       rollout_tma_kernel<true><<<grid, kRollThreads, kTmaSmemBytes, L.stream>>>(
-          L, L.u32, L.d32, L.d32b, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
+          L, L.d32, L.d32b, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
     } else {
       rollout_tma_kernel<false><<<grid, kRollThreads, kTmaSmemBytes, L.stream>>>(
-          L, L.u32, L.d32, L.d32b, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
+          L, L.d32, L.d32b, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
     }
   } else if (allow_pair && !L.scen_gen && m_launch > 1 && (L.pair == RRG_PAIR_ALWAYS || filled)) {
     // two candidates per thread (issue-bound launches: one load of each
     // disturbance and one loop's bookkeeping serve both)
     const dim3 g2(grid.x, (m_launch + 1) / 2);
     if (L.pmul)
-      rollout_pair_kernel<true><<<g2, kRollThreads, 0, L.stream>>>(L, L.u32, L.d32, L.d32b, L.cand_c32,
+      rollout_pair_kernel<true><<<g2, kRollThreads, 0, L.stream>>>(L, L.d32, L.d32b, L.cand_c32,
                                                                    early_exit, cls);
     else
-      rollout_pair_kernel<false><<<g2, kRollThreads, 0, L.stream>>>(L, L.u32, L.d32, L.d32b, L.cand_c32,
+      rollout_pair_kernel<false><<<g2, kRollThreads, 0, L.stream>>>(L, L.d32, L.d32b, L.cand_c32,
                                                                     early_exit, cls);
   } else {
     if (L.pmul) {
-      if (L.scen_gen) RRG_ROLLOUT(rollout_pu_kernel, float, SRC_GEN, L.u32, L.d32, L.d32b, L.cand_c32, cls);
-      else if (ring) RRG_ROLLOUT(rollout_pu_kernel, float, SRC_RING, L.u32, L.d32, L.d32b, L.cand_c32, cls);
-      else RRG_ROLLOUT(rollout_pu_kernel, float, SRC_REGS, L.u32, L.d32, L.d32b, L.cand_c32, cls);
+      if (L.scen_gen) RRG_ROLLOUT(rollout_pu_kernel, float, SRC_GEN, L.d32, L.d32b, L.cand_c32, cls);
+      else RRG_ROLLOUT(rollout_pu_kernel, float, SRC_RING, L.d32, L.d32b, L.cand_c32, cls);
     } else {
-      if (L.scen_gen) RRG_ROLLOUT(rollout_kernel, float, SRC_GEN, L.u32, L.d32, L.d32b, L.cand_c32, cls);
-      else if (ring) RRG_ROLLOUT(rollout_kernel, float, SRC_RING, L.u32, L.d32, L.d32b, L.cand_c32, cls);
-      else RRG_ROLLOUT(rollout_kernel, float, SRC_REGS, L.u32, L.d32, L.d32b, L.cand_c32, cls);
+      if (L.scen_gen) RRG_ROLLOUT(rollout_kernel, float, SRC_GEN, L.d32, L.d32b, L.cand_c32, cls);
+      else if (ring) RRG_ROLLOUT(rollout_kernel, float, SRC_RING, L.d32, L.d32b, L.cand_c32, cls);
+      else RRG_ROLLOUT(rollout_kernel, float, SRC_REGS, L.d32, L.d32b, L.cand_c32, cls);
     }
   }
 #undef RRG_ROLLOUT
@@ -766,10 +788,9 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
 // Binary64 re-run of the trajectories the binary32 pass could not decide,
 // over steps 0..jlast of each (the later steps were decided in binary32).
 __global__ void __launch_bounds__(64)
-recheck_kernel(const Launch L, const RhsU<double> K0, int early_exit) {
+recheck_kernel(const Launch L, int early_exit) {
   const uint32_t count = *L.recheck_count;
   const int N = L.N;
-  const double p_atm = L.params[P_P_ATM];
   const double thr = early_exit != RRG_EXIT_NONE ? 0.0 : -inf_v<double>();
   const int buf = L.st->buf;
   const ScenSrc src = L.st->src[buf];
@@ -782,23 +803,23 @@ recheck_kernel(const Launch L, const RhsU<double> K0, int early_exit) {
     if (L.P == nullptr && !L.cand_ok[i]) continue;
     unsigned steps = 0;
     double smin;
-    RhsU<double> K = K0;
-    RhsC<double> C = L.cand_c64[i];
-    double p_atm_k = p_atm;
-    const double* pm = buf ? L.pmulb : L.pmul;
-    if (pm != nullptr)
-      p_atm_k = scenario_model<double>(L.params, pm + static_cast<size_t>(k) * RRG_NPARAM,
-                                       L.cand_v[i], L.k64.pws, L.y_min, K, C);
+    RhsC<double> R = L.cand_c64[i];
+    LaneModel<double> M;
+    double p_atm_k;
+    if (L.pmul != nullptr)
+      p_atm_k = lane_model<double, true>(L, buf, k, L.cand_v[i], R, M);
+    else
+      p_atm_k = lane_model<double, false>(L, buf, k, 0.0, R, M);
     double q_ca, w, q_sm, w_abs;
-    start_state<double>(C, L.st->x, p_atm_k, q_ca, w, q_sm, w_abs);
+    start_state<double>(R, L.st->x, p_atm_k, q_ca, w, q_sm, w_abs);
     if (src.d64_valid) {
       int end = 0;
       int jl = -1;
-      smin = run_lane<double>(K, C, buf ? L.d64b : L.d64, k, N, L.H, 0, j_end, q_ca, w, q_sm,
-                              w_abs, inf_v<double>(), L.dt, thr, nullptr, &steps, &end,
+      smin = run_lane<double>(M.U, M.pw, M.C, buf ? L.d64b : L.d64, k, N, L.H, 0, j_end, q_ca, w, q_sm,
+                              w_abs, inf_v<double>(), thr, nullptr, &steps, &end,
                               -inf_v<double>(), &jl);
     } else {
-      smin = run_lane_philox(K, C, src, k, j_end, q_ca, w, q_sm, w_abs, L.dt, thr, &steps);
+      smin = run_lane_philox(M.U, M.pw, M.C, src, k, j_end, q_ca, w, q_sm, w_abs, thr, &steps);
     }
     const bool ok = smin >= 0.0;
     if (!ok) L.cand_ok[i] = 0;
@@ -873,7 +894,7 @@ int pair_blocks_per_sm(bool pu) {
 }
 
 cudaError_t launch_recheck(const Launch& L, int early_exit) {
-  recheck_kernel<<<L.recheck_blocks, 64, 0, L.stream>>>(L, L.u64, early_exit);
+  recheck_kernel<<<L.recheck_blocks, 64, 0, L.stream>>>(L, early_exit);
   return cudaGetLastError();
 }
 
@@ -1095,7 +1116,7 @@ __device__ void prepare_slot(const Launch& L, int i) {
       __dadd_rn(L.scfg.y_min, __dmul_rn(L.scfg.eps_ss, __dsub_rn(L.scfg.y_c, L.scfg.y_min)));
   const double v = governed(s->v_prev, s->r, L.cand_kappa[i]);
   L.cand_v[i] = v;
-  const int ok = candidate_setup(L.k64, L.k32, L.params, v, L.scfg.ss_check, thr_ss, L.y_min,
+  const int ok = candidate_setup(L.k64, L.k32, L.m64.c, L.params, v, L.scfg.ss_check, thr_ss, L.y_min,
                                  L.cand_c64 + i, L.cand_c32 + i);
   L.cand_ok[i] = ok;
   L.cand_ss[i] = ok;
@@ -1337,89 +1358,13 @@ cudaError_t launch_eval_finish(const Launch& L, int m, uint8_t* d_adm, double* d
 
 // ---------------------------------------------------------------------------
 // Simulated plant of the closed loop (Fig. 1) and the loop bookkeeping.
-// The plant's step runs on one warp.  It is binary64 and sits on the closed
-// loop's critical path, and GB300's binary64 pipe takes a warp instruction at
-// a time however few lanes are active, so a lone thread pays for every
-// instruction of the step.  All 32 lanes run the same step; only the x^e - 1
-// series is shared out: the 16 leaves of pow_m1_series's Estrin tree go to 16
-// lanes, and each level above is one fused multiply-add after two shuffles.
-// The tree, its operands and their order are pow_m1_series's, so every lane
-// gets its value bit for bit (the plant kernel measured 12.8 against 16.8 us).
-// The step around it is rk4_step_fast<double>'s: the same stage points and
-// combination, each right-hand side fc3_rhs_fast's with the shared series.
-// Called by all 32 lanes of the warp with the same arguments.
-__device__ __forceinline__ double pow_m1_warp(const PowSeries* __restrict__ S, double x, double e) {
-  if (S != nullptr && S->e == e) {
-    const double t = fma(x, S->inv_c, -1.0);
-    if (fabs(t) <= 1.0 / 3.0) {
-      const int i = static_cast<int>(threadIdx.x & 15);
-      const double t2 = t * t, t4 = t2 * t2, t8 = t4 * t4, t16 = t8 * t8, t32 = t16 * t16;
-      double p = fma(S->a[2 * i + 1], t, S->a[2 * i]);
-      double hi = __shfl_sync(0xffffffffu, p, 2 * i + 1), lo = __shfl_sync(0xffffffffu, p, 2 * i);
-      p = fma(hi, t2, lo);
-      hi = __shfl_sync(0xffffffffu, p, 2 * i + 1);
-      lo = __shfl_sync(0xffffffffu, p, 2 * i);
-      p = fma(hi, t4, lo);
-      hi = __shfl_sync(0xffffffffu, p, 2 * i + 1);
-      lo = __shfl_sync(0xffffffffu, p, 2 * i);
-      p = fma(hi, t8, lo);
-      const double p1 = __shfl_sync(0xffffffffu, p, 1), p0 = __shfl_sync(0xffffffffu, p, 0);
-      return fma(S->a[32], t32, fma(p1, t16, p0));
-    }
-  }
-  return pow(x, e) - 1.0;
-}
-
-__device__ __forceinline__ void rhs_plant_warp(const RhsU<double>& U, const RhsC<double>& C, double z_ca,
-                                               double z_w, double z_sm, double w, double x_pw, double& d_ca,
-                                               double& d_w, double& d_sm) {
-  d_ca = U.a1 * z_sm + (C.c_ca - U.a12 * z_ca);
-  d_sm = U.g_w * z_w + ((C.c_sm + U.b3 * z_ca) - U.g_sm * z_sm);
-  const double W_cp = U.a_w * z_w + (C.W_r - U.a_p * z_sm);
-  const double f = torque_factor<double>(U, pow_m1_warp(U.pws, x_pw, U.e), w);
-  d_w = (C.e0 - U.e2 * z_w) - W_cp * f;
-}
-
-__device__ __forceinline__ void rk4_plant_warp(const RhsU<double>& U, const RhsC<double>& C, double dt0,
-                                               double& q_ca, double& w, double& q_sm, double& w_abs,
-                                               double e_ca, double e_w, double e_sm) {
-  const StepC<double> S = step_consts<double>(U, dt0);
-  const double dt = S.dt, h2 = S.h2, h6 = S.h6, g2 = S.g2, g1 = S.g1;
-  const double x1 = q_sm * U.inv_p_atm + C.x_r;
-  double a1, b1, c1, a2, b2, c2, a3, b3, c3, a4, b4, c4;
-  rhs_plant_warp(U, C, q_ca, w, q_sm, w_abs, x1, a1, b1, c1);
-  rhs_plant_warp(U, C, q_ca + h2 * a1, w + h2 * b1, q_sm + h2 * c1, w_abs + h2 * b1, x1 + g2 * c1,
-                 a2, b2, c2);
-  rhs_plant_warp(U, C, q_ca + h2 * a2, w + h2 * b2, q_sm + h2 * c2, w_abs + h2 * b2, x1 + g2 * c2,
-                 a3, b3, c3);
-  const double p_ca = (q_ca + e_ca) + h6 * (a1 + 2.0 * (a2 + a3));
-  const double p_w = (w + e_w) + h6 * (b1 + 2.0 * (b2 + b3));
-  const double p_sm = (q_sm + e_sm) + h6 * (c1 + 2.0 * (c2 + c3));
-  const double p_wa = p_w + C.r_w;
-  rhs_plant_warp(U, C, q_ca + dt * a3, w + dt * b3, q_sm + dt * c3, w_abs + dt * b3, x1 + g1 * c3,
-                 a4, b4, c4);
-  q_ca = p_ca + h6 * a4;
-  w = p_w + h6 * b4;
-  q_sm = p_sm + h6 * c4;
-  w_abs = p_wa + h6 * b4;
-}
-
-// x_{t+1} = RK4(x_t, v) + the plant's own draw (plant_step_fast's step, on the
-// warp).
+// x_{t+1} = RK4(x_t, v) + the plant's own draw, by one thread's worth of
+// binary64 instructions (every lane of the warp runs the same step).
 __device__ void plant_step(const Launch& L, const double* x, double v, uint64_t seed, uint64_t upd,
                            const double* amp, double* x_next) {
   const U64x4 r = philox4x64_10(0ull, 0ull, upd, 1ull, seed, 0ull);
-  RhsC<double> c64;
-  RhsC<float> c32;
-  const double q0[3] = {0.0, 0.0, 0.0};
-  fold_rhs_cand(L.k64, cand_consts(L.params, v), q0, 0.0, &c64, &c32);
-  const double p_atm = L.params[P_P_ATM];
-  double q_ca = x[0] - p_atm, w = x[1], q_sm = x[2] - p_atm, w_abs = x[1];
-  rk4_plant_warp(L.u64, c64, L.dt, q_ca, w, q_sm, w_abs, uniform_sym(r.w[0], amp[0]),
-                 uniform_sym(r.w[1], amp[1]), uniform_sym(r.w[2], amp[2]));
-  x_next[0] = q_ca + p_atm;
-  x_next[1] = w;
-  x_next[2] = q_sm + p_atm;
+  plant_step_fast(L.m64, v, x, uniform_sym(r.w[0], amp[0]), uniform_sym(r.w[1], amp[1]),
+                  uniform_sym(r.w[2], amp[2]), x_next);
 }
 
 __global__ void plant_kernel(const Launch L, const double* d_x, const double* d_v, uint64_t seed,
@@ -1466,7 +1411,8 @@ __global__ void loop_end_kernel(const Launch L, LoopState* ls, uint64_t seed, ui
   const double v = s->v_t_out;
   const double x[3] = {ls->x[0], ls->x[1], ls->x[2]};
   double xn[3];
-  plant_step(L, x, v, seed, t0 + t, amp, xn);  // the whole warp (its shuffles order the reads above)
+  plant_step(L, x, v, seed, t0 + t, amp, xn);
+  __syncwarp();  // every lane has read the loop state before it is written
   if (threadIdx.x != 0) return;
   if (v_out) v_out[t] = v;
   if (kappa_out) kappa_out[t] = s->kappa_opt;

@@ -110,6 +110,7 @@ __device__ __forceinline__ int equilibrium_dev(const Fc3K<T>& K, const double* _
 // which case a binary64 solve decides.  Returns the check's outcome (1 when
 // off).
 __device__ __forceinline__ int candidate_setup(const Fc3K<double>& k64, const Fc3K<float>& k32,
+                                               const ModelC& mc,
                                                const double* __restrict__ P, double v, int ss_check,
                                                double thr_ss, double y_min, RhsC<double>* c64,
                                                RhsC<float>* c32) {
@@ -123,7 +124,8 @@ __device__ __forceinline__ int candidate_setup(const Fc3K<double>& k64, const Fc
     q_r[1] = q32[1];
     q_r[2] = q32[2];
   }
-  fold_rhs_cand(k64, C, q_r, y_min, c64, c32);
+  *c64 = fold_cand(mc, v, q_r, y_min);
+  *c32 = round_cand(*c64);
   if (!ss_check) return 1;
   if (rc32 == 0 && fabs(static_cast<double>(y32) - thr_ss) > 1e-4 * (1.0 + fabs(thr_ss)))
     return static_cast<double>(y32) >= thr_ss;
@@ -155,11 +157,10 @@ __device__ __forceinline__ void start_state(const RhsC<T>& C, const double* x, d
 // step on a two-die GB300) overlaps the arithmetic of the steps in between.
 // The candidate's dead flag is read at the start of a block and used at its
 // end, for the same reason.
-// Depth 16 in binary32 (measured on GB300: the closed-loop update ran 24 %
-// faster than with 8, and the 65,536-scenario sweep was unchanged), 8 in
-// binary64 (16 would spill the binary64 state and ring).
+// Depth 8 in binary32 (16,384 x 16 x 1,000 steps: 920 us, 943 at 16, which
+// holds 136 registers, 1,028 at 12), 8 in binary64.
 #ifndef RRG_PREFETCH
-#define RRG_PREFETCH 16
+#define RRG_PREFETCH 8
 #endif
 #ifndef RRG_PREFETCH64
 #define RRG_PREFETCH64 8
@@ -167,18 +168,73 @@ __device__ __forceinline__ void start_state(const RhsC<T>& C, const double* x, d
 template <typename T> struct PrefetchDepth { static constexpr int value = RRG_PREFETCH; };
 template <> struct PrefetchDepth<double> { static constexpr int value = RRG_PREFETCH64; };
 
+// A finite value (the binary64 test by the exponent bits, off the slow
+// binary64 pipe).
+__device__ __forceinline__ bool finite_v(float x) { return fabsf(x) <= FLT_MAX; }
+__device__ __forceinline__ bool finite_v(double x) { return (__double2hiint(x) & 0x7fffffff) < 0x7ff00000; }
+
 // The slack y_j - y_min of the deviation state (y_min is folded into s_off).
 template <typename T>
-__device__ __forceinline__ T checked_slack(const RhsC<T>& C, T q_ca, T w, T q_sm) {
-  const T s = C.y_scale * (q_sm - q_ca) + C.s_off;
-  const bool fin = fabs(q_ca) <= max_finite<T>() && fabs(w) <= max_finite<T>() &&
-                   fabs(q_sm) <= max_finite<T>() && fabs(s) <= max_finite<T>();
-  return fin ? s : -inf_v<T>();
+__device__ __forceinline__ T slack_of(const StepC<T>& C, T q_ca, T q_sm) {
+  return fma_rn(C.y_scale, q_sm - q_ca, C.s_off);
+}
+template <typename T>
+__device__ __forceinline__ T checked_slack(const StepC<T>& C, T q_ca, T w, T q_sm) {
+  const T s = slack_of<T>(C, q_ca, q_sm);
+  return finite_v(q_ca) && finite_v(w) && finite_v(q_sm) && finite_v(s) ? s : -inf_v<T>();
 }
 
-// a b + c rounded once; never simplified (x 0 + c is NaN for x = inf or NaN).
-__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+// The minimum of a block's slacks and whether all of them, and the state at
+// its end, are finite (a block: an even number of steps; step u of it calls
+// add(s, u)).  A non-finite state contaminates every component through the
+// next step and NaN and inf never return to a finite value through +, -, x
+// and / by a finite or NaN operand, so testing each slack and the block's last
+// state finds it; the block's minimum is then -inf, as a per-step test would
+// give.
+//   binary32: the three-operand minimum and maximum take two steps at a time
+// (one instruction a step where a minimum and a finiteness sum took two).
+//   binary64: on the integer pipe (a binary64 compare costs a scheduler 64
+// cycles): the minimum of the order-preserving keys, the maximum of the high
+// words without their signs.
+template <typename T> struct BlockMin;
+template <>
+struct BlockMin<float> {
+  float mn, mx, prev;
+  __device__ __forceinline__ BlockMin() : mn(inf_v<float>()), mx(0.0f), prev(0.0f) {}
+  __device__ __forceinline__ void add(float s, int u) {
+    if (u & 1) {
+      asm("min.f32 %0, %1, %2, %3;" : "=f"(mn) : "f"(mn), "f"(prev), "f"(s));
+      abs3(prev, s);
+    } else {
+      prev = s;
+    }
+  }
+  __device__ __forceinline__ float result(float q_ca, float w, float q_sm) {
+    abs3(q_ca, w);
+    abs3(q_sm, q_sm);
+    return mx <= FLT_MAX ? mn : -inf_v<float>();
+  }
+  __device__ __forceinline__ void abs3(float a, float b) {
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(mx) : "f"(mx), "f"(a), "f"(b));
+  }
+};
+template <>
+struct BlockMin<double> {
+  long long mn;
+  int mx;
+  static __device__ __forceinline__ long long key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffll); }
+  __device__ __forceinline__ BlockMin() : mn(0x7ff0000000000000ll), mx(0) {}
+  __device__ __forceinline__ void add(double s, int) {
+    const long long k = key(__double_as_longlong(s));
+    mn = k < mn ? k : mn;
+    mx = max(mx, __double2hiint(s) & 0x7fffffff);
+  }
+  __device__ __forceinline__ double result(double q_ca, double w, double q_sm) {
+    mx = max(max(mx, __double2hiint(q_ca) & 0x7fffffff),
+             max(__double2hiint(w) & 0x7fffffff, __double2hiint(q_sm) & 0x7fffffff));
+    return mx < 0x7ff00000 ? __longlong_as_double(key(mn)) : -inf_v<double>();
+  }
+};
 
 // Lane outcome of run_lane.
 enum LaneEnd : int { LANE_REACHED_END = 0, LANE_VIOLATED = 1, LANE_STOPPED = 2 };
@@ -195,9 +251,9 @@ enum LaneEnd : int { LANE_REACHED_END = 0, LANE_VIOLATED = 1, LANE_STOPPED = 2 }
 // band, which the band's error bound makes non-negative in binary64.
 // band = -inf tracks nothing.
 template <typename T, int PF = PrefetchDepth<T>::value>
-__device__ __forceinline__ T run_lane(const RhsU<T>& K, const RhsC<T>& C,
+__device__ __forceinline__ T run_lane(const StepU<T>& K, const PowTable* pw, const StepC<T>& C,
                                       const T* __restrict__ d, int k, int N, int H, int j0,
-                                      int j_end, T& q_ca, T& w, T& q_sm, T& w_abs, T smin_in, T dt,
+                                      int j_end, T& q_ca, T& w, T& q_sm, T& w_abs, T smin_in,
                                       T thr, const volatile int32_t* dead, unsigned* steps,
                                       int* end, T band, int* jlast) {
   T smin = smin_in;
@@ -214,7 +270,6 @@ __device__ __forceinline__ T run_lane(const RhsU<T>& K, const RhsC<T>& C,
       go = false;
     }
   }
-  const StepC<T> S = step_consts<T>(K, dt);
   if (go) {
     const size_t HN = static_cast<size_t>(H) * N;
     T r0[PF], r1[PF], r2[PF];
@@ -236,16 +291,10 @@ __device__ __forceinline__ T run_lane(const RhsU<T>& K, const RhsC<T>& C,
     // block runs to the block's end; that only lowers its min slack, so no
     // decision changes.  The last, partial block steps one at a time.
     //
-    // Finiteness is also settled once per block: nf = sum of s_j 0 stays 0
-    // while every slack is finite and turns NaN (for good) at the first that
-    // is not; a non-finite state component is tested at the block's end,
-    // since it contaminates every component through the next right-hand side
-    // (every derivative reads W_cp or s) and NaN and inf never return to a
-    // finite value through +, -, x and / by a finite or NaN operand.  Either
-    // makes the lane's min slack -inf, as a per-step test would.
+    // Finiteness is also settled once per block (BlockMin).
     while (!stop && j + PF <= j_end) {
       const int dead_now = dead != nullptr ? *dead : 0;
-      T nf = T(0), bmin = inf_v<T>();
+      BlockMin<T> bm;
 #pragma unroll
       for (int u = 0; u < PF; ++u) {
         const T e0 = r0[u], e1 = r1[u], e2 = r2[u];
@@ -255,14 +304,11 @@ __device__ __forceinline__ T run_lane(const RhsU<T>& K, const RhsC<T>& C,
           r2[u] = __ldg(pf + 2 * HN);
         }
         pf += N;
-        rk4_step_fast<T>(K, C, S, q_ca, w, q_sm, w_abs, e0, e1, e2);
+        rk4_step_fast<T>(K, pw, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
         ++j;
-        const T s = C.y_scale * (q_sm - q_ca) + C.s_off;
-        bmin = fmin(bmin, s);
-        nf = fma_rn(s, T(0), nf);
+        bm.add(slack_of<T>(C, q_ca, q_sm), u);
       }
-      nf = fma_rn(q_ca, T(0), fma_rn(w, T(0), fma_rn(q_sm, T(0), nf)));
-      if (nf != nf) bmin = -inf_v<T>();
+      const T bmin = bm.result(q_ca, w, q_sm);
       smin = fmin(smin, bmin);
       if (bmin < band) jl = j;
       if (smin < thr) {
@@ -277,7 +323,7 @@ __device__ __forceinline__ T run_lane(const RhsU<T>& K, const RhsC<T>& C,
     while (!stop && j < j_end) {
       const T e0 = __ldg(dp), e1 = __ldg(dp + HN), e2 = __ldg(dp + 2 * HN);
       dp += N;
-      rk4_step_fast<T>(K, C, S, q_ca, w, q_sm, w_abs, e0, e1, e2);
+      rk4_step_fast<T>(K, pw, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
       ++j;
       const T s = checked_slack<T>(C, q_ca, w, q_sm);
       smin = fmin(smin, s);
@@ -317,9 +363,9 @@ __device__ __forceinline__ T run_lane(const RhsU<T>& K, const RhsC<T>& C,
 // w_abs) in and out; smin, steps, end, jlast per trajectory as run_lane's.
 // Returns the steps both trajectories ran together.
 template <typename T, int PF = PrefetchDepth<T>::value>
-__device__ __forceinline__ int run_lane_pair(const RhsU<T>& K, const RhsC<T>& CA, const RhsC<T>& CB,
+__device__ __forceinline__ int run_lane_pair(const StepU<T>& K, const StepC<T>& CA, const StepC<T>& CB,
                                               const T* __restrict__ d, int k, int N, int H, int j_end,
-                                              T* za, T* zb, T dt, T thr, T band,
+                                              T* za, T* zb, T thr, T band,
                                               volatile int32_t* deadA, volatile int32_t* deadB,
                                               T* smin, unsigned* steps, int* end, int* jlast) {
   smin[0] = checked_slack<T>(CA, za[0], za[1], za[2]);
@@ -332,7 +378,6 @@ __device__ __forceinline__ int run_lane_pair(const RhsU<T>& K, const RhsC<T>& CA
   if (how[1] == LANE_VIOLATED && deadB != nullptr) *deadB = 1;
   const bool cand_stop = deadA != nullptr;
   int j = 0;
-  const StepC<T> S = step_consts<T>(K, dt);
   bool pair = how[0] == LANE_REACHED_END && how[1] == LANE_REACHED_END;
   bool stopA = false, stopB = false;  // candidate stopped (dead flag) while not violated
   if (pair && j + PF <= j_end) {
@@ -348,7 +393,7 @@ __device__ __forceinline__ int run_lane_pair(const RhsU<T>& K, const RhsC<T>& CA
     }
     while (pair && j + PF <= j_end) {
       const int dA = cand_stop ? *deadA : 0, dB = cand_stop ? *deadB : 0;
-      T nfa = T(0), nfb = T(0), ba = inf_v<T>(), bb = inf_v<T>();
+      BlockMin<T> bma, bmb;
 #pragma unroll
       for (int u = 0; u < PF; ++u) {
         const T e0 = r0[u], e1 = r1[u], e2 = r2[u];
@@ -358,20 +403,13 @@ __device__ __forceinline__ int run_lane_pair(const RhsU<T>& K, const RhsC<T>& CA
           r2[u] = __ldg(pf + 2 * HN);
         }
         pf += N;
-        rk4_step_fast<T>(K, CA, S, za[0], za[1], za[2], za[3], e0, e1, e2);
-        rk4_step_fast<T>(K, CB, S, zb[0], zb[1], zb[2], zb[3], e0, e1, e2);
+        rk4_step_fast<T>(K, nullptr, CA, za[0], za[1], za[2], za[3], e0, e1, e2);
+        rk4_step_fast<T>(K, nullptr, CB, zb[0], zb[1], zb[2], zb[3], e0, e1, e2);
         ++j;
-        const T sa = CA.y_scale * (za[2] - za[0]) + CA.s_off;
-        const T sb = CB.y_scale * (zb[2] - zb[0]) + CB.s_off;
-        ba = fmin(ba, sa);
-        bb = fmin(bb, sb);
-        nfa = fma_rn(sa, T(0), nfa);
-        nfb = fma_rn(sb, T(0), nfb);
+        bma.add(slack_of<T>(CA, za[0], za[2]), u);
+        bmb.add(slack_of<T>(CB, zb[0], zb[2]), u);
       }
-      nfa = fma_rn(za[0], T(0), fma_rn(za[1], T(0), fma_rn(za[2], T(0), nfa)));
-      nfb = fma_rn(zb[0], T(0), fma_rn(zb[1], T(0), fma_rn(zb[2], T(0), nfb)));
-      if (nfa != nfa) ba = -inf_v<T>();
-      if (nfb != nfb) bb = -inf_v<T>();
+      const T ba = bma.result(za[0], za[1], za[2]), bb = bmb.result(zb[0], zb[1], zb[2]);
       smin[0] = fmin(smin[0], ba);
       smin[1] = fmin(smin[1], bb);
       if (ba < band) jlast[0] = j;
@@ -401,13 +439,13 @@ __device__ __forceinline__ int run_lane_pair(const RhsU<T>& K, const RhsC<T>& CA
   if (how[1] == LANE_REACHED_END && stopB) how[1] = LANE_STOPPED;
   if (how[0] == LANE_REACHED_END && j < j_end) {
     int e = LANE_REACHED_END;
-    smin[0] = run_lane<T, PF>(K, CA, d, k, N, H, j, j_end, za[0], za[1], za[2], za[3], smin[0], dt, thr,
+    smin[0] = run_lane<T, PF>(K, nullptr, CA, d, k, N, H, j, j_end, za[0], za[1], za[2], za[3], smin[0], thr,
                               deadA, &extra[0], &e, band, &jlast[0]);
     how[0] = e;
   }
   if (how[1] == LANE_REACHED_END && j < j_end) {
     int e = LANE_REACHED_END;
-    smin[1] = run_lane<T, PF>(K, CB, d, k, N, H, j, j_end, zb[0], zb[1], zb[2], zb[3], smin[1], dt, thr,
+    smin[1] = run_lane<T, PF>(K, nullptr, CB, d, k, N, H, j, j_end, zb[0], zb[1], zb[2], zb[3], smin[1], thr,
                               deadB, &extra[1], &e, band, &jlast[1]);
     how[1] = e;
   }
@@ -460,10 +498,10 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 template <int D = RRG_RING_DEPTH, int B = RRG_RING_BLOCK, int U = RRG_RING_UNROLL>
-__device__ __forceinline__ float run_lane_ring(const RhsU<float>& K, const RhsC<float>& C,
+__device__ __forceinline__ float run_lane_ring(const StepU<float>& K, const StepC<float>& C,
                                                const float* __restrict__ d, int k, int N, int H,
                                                int j0, int j_end, float& q_ca, float& w,
-                                               float& q_sm, float& w_abs, float smin_in, float dt,
+                                               float& q_sm, float& w_abs, float smin_in,
                                                float thr, const volatile int32_t* dead,
                                                unsigned* steps, int* end, float band, int* jlast,
                                                float* ring) {
@@ -481,7 +519,6 @@ __device__ __forceinline__ float run_lane_ring(const RhsU<float>& K, const RhsC<
       go = false;
     }
   }
-  const StepC<float> S = step_consts<float>(K, dt);
   if (go) {
     const size_t HN = static_cast<size_t>(H) * N;
     const int bd = blockDim.x;
@@ -506,13 +543,13 @@ __device__ __forceinline__ float run_lane_ring(const RhsU<float>& K, const RhsC<
     int dead_prev = 0;
     while (!stop && j + B <= j_end) {
       const int dead_now = dead != nullptr ? *dead : 0;
-      float nf = 0.0f, bmin = inf_v<float>();
+      BlockMin<float> bm;
 #pragma unroll U
       for (int u = 0; u < B; ++u) {
         cp_async_wait<D - 1>();
         float* e = my + (3 * slot) * bd;
         const float e0 = e[0], e1 = e[bd], e2 = e[2 * bd];
-        rk4_step_fast<float>(K, C, S, q_ca, w, q_sm, w_abs, e0, e1, e2);
+        rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
         // the slot is free once its values are in registers: step j + D
         if (j + D < j_end) {
           cp_async4(e, pf);
@@ -523,12 +560,9 @@ __device__ __forceinline__ float run_lane_ring(const RhsU<float>& K, const RhsC<
         pf += N;
         slot = (slot + 1) & (D - 1);
         ++j;
-        const float s = C.y_scale * (q_sm - q_ca) + C.s_off;
-        bmin = fmin(bmin, s);
-        nf = fma_rn(s, 0.0f, nf);
+        bm.add(slack_of<float>(C, q_ca, q_sm), u);
       }
-      nf = fma_rn(q_ca, 0.0f, fma_rn(w, 0.0f, fma_rn(q_sm, 0.0f, nf)));
-      if (nf != nf) bmin = -inf_v<float>();
+      const float bmin = bm.result(q_ca, w, q_sm);
       smin = fmin(smin, bmin);
       if (bmin < band) jl = j;
       if (smin < thr) {
@@ -544,7 +578,7 @@ __device__ __forceinline__ float run_lane_ring(const RhsU<float>& K, const RhsC<
       cp_async_wait<D - 1>();
       float* e = my + (3 * slot) * bd;
       const float e0 = e[0], e1 = e[bd], e2 = e[2 * bd];
-      rk4_step_fast<float>(K, C, S, q_ca, w, q_sm, w_abs, e0, e1, e2);
+      rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
       if (j + D < j_end) {
         cp_async4(e, pf);
         cp_async4(e + bd, pf + HN);
@@ -670,9 +704,11 @@ __device__ __forceinline__ void tma_chunk(const void* tmap, uint32_t dst, uint32
       : "memory");
 }
 
-__device__ __forceinline__ float run_lane_tma(const RhsU<float>& K, const RhsC<float>& C, const void* tmap,
+// PACK: rk4_step_packed (the same bits).
+template <bool PACK>
+__device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC<float>& C, const void* tmap,
                                               int k0, bool on, int j0, int j_end, float& q_ca, float& w,
-                                              float& q_sm, float& w_abs, float smin_in, float dt, float thr,
+                                              float& q_sm, float& w_abs, float smin_in, float thr,
                                               const volatile int32_t* dead, volatile int32_t* mark,
                                               unsigned* steps, int* end, float band, int* jlast,
                                               float* stages, uint64_t* bars,
@@ -694,7 +730,6 @@ __device__ __forceinline__ float run_lane_tma(const RhsU<float>& K, const RhsC<f
       if (mark != nullptr) *mark = 1;
     }
   }
-  const StepC<float> S = step_consts<float>(K, dt);
   const int nchunks = j_end > j0 ? (j_end - j0 + T - 1) / T : 0;
   if (nchunks > 0 && __any_sync(0xffffffffu, run)) {
     const uint32_t st0 = smem_u32(stages), bar0 = smem_u32(bars);
@@ -725,18 +760,16 @@ __device__ __forceinline__ float run_lane_tma(const RhsU<float>& K, const RhsC<f
       const int dead_now = (run && dead != nullptr) ? *dead : 0;
       if (run) {
         if (nst == T) {
-          float nf = 0.0f, bmin = inf_v<float>();
+          BlockMin<float> bm;
 #pragma unroll
           for (int u = 0; u < T; ++u) {
             const float e0 = e[u * 32], e1 = e[(T + u) * 32], e2 = e[(2 * T + u) * 32];
-            rk4_step_fast<float>(K, C, S, q_ca, w, q_sm, w_abs, e0, e1, e2);
-            const float sl = C.y_scale * (q_sm - q_ca) + C.s_off;
-            bmin = fmin(bmin, sl);
-            nf = fma_rn(sl, 0.0f, nf);
+            if constexpr (PACK) rk4_step_packed(K, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
+            else rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
+            bm.add(slack_of<float>(C, q_ca, q_sm), u);
           }
           j += T;
-          nf = fma_rn(q_ca, 0.0f, fma_rn(w, 0.0f, fma_rn(q_sm, 0.0f, nf)));
-          if (nf != nf) bmin = -inf_v<float>();
+          const float bmin = bm.result(q_ca, w, q_sm);
           smin = fmin(smin, bmin);
           if (bmin < band) jl = j;
           if (smin < thr) {
@@ -750,7 +783,7 @@ __device__ __forceinline__ float run_lane_tma(const RhsU<float>& K, const RhsC<f
         } else {
           for (int u = 0; u < nst && run; ++u) {
             const float e0 = e[u * 32], e1 = e[(T + u) * 32], e2 = e[(2 * T + u) * 32];
-            rk4_step_fast<float>(K, C, S, q_ca, w, q_sm, w_abs, e0, e1, e2);
+            rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
             ++j;
             const float sl = checked_slack<float>(C, q_ca, w, q_sm);
             smin = fmin(smin, sl);
@@ -817,7 +850,7 @@ struct TmaTraj {
   bool run;
 };
 
-__device__ __forceinline__ void tma_traj_start(TmaTraj& t, const RhsC<float>& C, bool on, int j0, int j_end,
+__device__ __forceinline__ void tma_traj_start(TmaTraj& t, const StepC<float>& C, bool on, int j0, int j_end,
                                                float thr, float band, volatile int32_t* mark) {
   t.j = j0;
   t.how = LANE_REACHED_END;
@@ -835,11 +868,10 @@ __device__ __forceinline__ void tma_traj_start(TmaTraj& t, const RhsC<float>& C,
 }
 
 // The tests at the end of a whole chunk of T steps (run_lane_tma's).
-__device__ __forceinline__ void tma_traj_chunk_end(TmaTraj& t, float bmin, float nf, int T, int j_end, float thr,
+__device__ __forceinline__ void tma_traj_chunk_end(TmaTraj& t, BlockMin<float>& bm, int T, int j_end, float thr,
                                                    float band, int dead_now, volatile int32_t* mark) {
   t.j += T;
-  nf = fma_rn(t.q_ca, 0.0f, fma_rn(t.w, 0.0f, fma_rn(t.q_sm, 0.0f, nf)));
-  if (nf != nf) bmin = -inf_v<float>();
+  const float bmin = bm.result(t.q_ca, t.w, t.q_sm);
   t.smin = fmin(t.smin, bmin);
   if (bmin < band) t.jl = t.j;
   if (t.smin < thr) {
@@ -854,45 +886,39 @@ __device__ __forceinline__ void tma_traj_chunk_end(TmaTraj& t, float bmin, float
 
 // A whole chunk for one trajectory (e: the lane's column of the stage).
 template <int T>
-__device__ __forceinline__ void tma_traj_chunk(TmaTraj& t, const RhsU<float>& K, const RhsC<float>& C,
-                                               const StepC<float>& S, const float* e, float& bmin, float& nf) {
+__device__ __forceinline__ void tma_traj_chunk(TmaTraj& t, const StepU<float>& K, const StepC<float>& C,
+                                               const float* e, BlockMin<float>& bm) {
 #pragma unroll 8
   for (int u = 0; u < T; ++u) {
     const float e0 = e[u * 32], e1 = e[(T + u) * 32], e2 = e[(2 * T + u) * 32];
-    rk4_step_fast<float>(K, C, S, t.q_ca, t.w, t.q_sm, t.w_abs, e0, e1, e2);
-    const float sl = C.y_scale * (t.q_sm - t.q_ca) + C.s_off;
-    bmin = fmin(bmin, sl);
-    nf = fma_rn(sl, 0.0f, nf);
+    rk4_step_fast<float>(K, nullptr, C, t.q_ca, t.w, t.q_sm, t.w_abs, e0, e1, e2);
+    bm.add(slack_of<float>(C, t.q_ca, t.q_sm), u);
   }
 }
 
 // A whole chunk for both trajectories, one load of each value for the two.
 template <int T>
-__device__ __forceinline__ void tma_pair_chunk(TmaTraj& a, TmaTraj& b, const RhsU<float>& K,
-                                               const RhsC<float>& CA, const RhsC<float>& CB,
-                                               const StepC<float>& S, const float* e, float& bma, float& nfa,
-                                               float& bmb, float& nfb) {
+__device__ __forceinline__ void tma_pair_chunk(TmaTraj& a, TmaTraj& b, const StepU<float>& K,
+                                               const StepC<float>& CA, const StepC<float>& CB,
+                                               const float* e, BlockMin<float>& bma,
+                                               BlockMin<float>& bmb) {
 #pragma unroll 8
   for (int u = 0; u < T; ++u) {
     const float e0 = e[u * 32], e1 = e[(T + u) * 32], e2 = e[(2 * T + u) * 32];
-    rk4_step_fast<float>(K, CA, S, a.q_ca, a.w, a.q_sm, a.w_abs, e0, e1, e2);
-    rk4_step_fast<float>(K, CB, S, b.q_ca, b.w, b.q_sm, b.w_abs, e0, e1, e2);
-    const float sa = CA.y_scale * (a.q_sm - a.q_ca) + CA.s_off;
-    const float sb = CB.y_scale * (b.q_sm - b.q_ca) + CB.s_off;
-    bma = fmin(bma, sa);
-    bmb = fmin(bmb, sb);
-    nfa = fma_rn(sa, 0.0f, nfa);
-    nfb = fma_rn(sb, 0.0f, nfb);
+    rk4_step_fast<float>(K, nullptr, CA, a.q_ca, a.w, a.q_sm, a.w_abs, e0, e1, e2);
+    rk4_step_fast<float>(K, nullptr, CB, b.q_ca, b.w, b.q_sm, b.w_abs, e0, e1, e2);
+    bma.add(slack_of<float>(CA, a.q_ca, a.q_sm), u);
+    bmb.add(slack_of<float>(CB, b.q_ca, b.q_sm), u);
   }
 }
 
 // The last, partial chunk: step by step with the per-step test (run_lane's).
-__device__ __forceinline__ void tma_traj_tail(TmaTraj& t, const RhsU<float>& K, const RhsC<float>& C,
-                                              const StepC<float>& S, const float* e, int T, int nst, float thr,
+__device__ __forceinline__ void tma_traj_tail(TmaTraj& t, const StepU<float>& K, const StepC<float>& C,
+                                              const float* e, int T, int nst, float thr,
                                               float band, volatile int32_t* mark) {
   for (int u = 0; u < nst && t.run; ++u) {
     const float e0 = e[u * 32], e1 = e[(T + u) * 32], e2 = e[(2 * T + u) * 32];
-    rk4_step_fast<float>(K, C, S, t.q_ca, t.w, t.q_sm, t.w_abs, e0, e1, e2);
+    rk4_step_fast<float>(K, nullptr, C, t.q_ca, t.w, t.q_sm, t.w_abs, e0, e1, e2);
     ++t.j;
     const float sl = checked_slack<float>(C, t.q_ca, t.w, t.q_sm);
     t.smin = fmin(t.smin, sl);
@@ -910,9 +936,9 @@ __device__ __forceinline__ void tma_traj_tail(TmaTraj& t, const RhsU<float>& K, 
 // dead_X / mark_X: the candidates' flags (nullptr without a candidate-level
 // exit).  *paired: steps this lane ran for both trajectories at once.  Called
 // by all 32 lanes of the warp.
-__device__ __forceinline__ void run_lane_tma_pair(const RhsU<float>& K, const RhsC<float>& CA,
-                                                  const RhsC<float>& CB, const void* tmap, int k0, bool onA,
-                                                  bool onB, int j0, int j_end, TmaTraj& a, TmaTraj& b, float dt,
+__device__ __forceinline__ void run_lane_tma_pair(const StepU<float>& K, const StepC<float>& CA,
+                                                  const StepC<float>& CB, const void* tmap, int k0, bool onA,
+                                                  bool onB, int j0, int j_end, TmaTraj& a, TmaTraj& b,
                                                   float thr, float band, const volatile int32_t* deadA,
                                                   const volatile int32_t* deadB, volatile int32_t* markA,
                                                   volatile int32_t* markB, float* stages, uint64_t* bars,
@@ -922,7 +948,6 @@ __device__ __forceinline__ void run_lane_tma_pair(const RhsU<float>& K, const Rh
   tma_traj_start(a, CA, onA, j0, j_end, thr, band, markA);
   tma_traj_start(b, CB, onB, j0, j_end, thr, band, markB);
   *paired = 0u;
-  const StepC<float> S = step_consts<float>(K, dt);
   const int nchunks = j_end > j0 ? (j_end - j0 + T - 1) / T : 0;
   if (nchunks > 0 && __any_sync(0xffffffffu, a.run || b.run)) {
     const uint32_t st0 = smem_u32(stages), bar0 = smem_u32(bars);
@@ -953,22 +978,22 @@ __device__ __forceinline__ void run_lane_tma_pair(const RhsU<float>& K, const Rh
       const int da = (a.run && deadA != nullptr) ? *deadA : 0;
       const int db = (b.run && deadB != nullptr) ? *deadB : 0;
       if (nst == T) {
-        float bma = inf_v<float>(), nfa = 0.0f, bmb = inf_v<float>(), nfb = 0.0f;
+        BlockMin<float> bma, bmb;
         if (a.run && b.run) {
-          tma_pair_chunk<T>(a, b, K, CA, CB, S, e, bma, nfa, bmb, nfb);
+          tma_pair_chunk<T>(a, b, K, CA, CB, e, bma, bmb);
           *paired += 2u * T;
-          tma_traj_chunk_end(a, bma, nfa, T, j_end, thr, band, da, markA);
-          tma_traj_chunk_end(b, bmb, nfb, T, j_end, thr, band, db, markB);
+          tma_traj_chunk_end(a, bma, T, j_end, thr, band, da, markA);
+          tma_traj_chunk_end(b, bmb, T, j_end, thr, band, db, markB);
         } else if (a.run) {
-          tma_traj_chunk<T>(a, K, CA, S, e, bma, nfa);
-          tma_traj_chunk_end(a, bma, nfa, T, j_end, thr, band, da, markA);
+          tma_traj_chunk<T>(a, K, CA, e, bma);
+          tma_traj_chunk_end(a, bma, T, j_end, thr, band, da, markA);
         } else if (b.run) {
-          tma_traj_chunk<T>(b, K, CB, S, e, bmb, nfb);
-          tma_traj_chunk_end(b, bmb, nfb, T, j_end, thr, band, db, markB);
+          tma_traj_chunk<T>(b, K, CB, e, bmb);
+          tma_traj_chunk_end(b, bmb, T, j_end, thr, band, db, markB);
         }
       } else {
-        tma_traj_tail(a, K, CA, S, e, T, nst, thr, band, markA);
-        tma_traj_tail(b, K, CB, S, e, T, nst, thr, band, markB);
+        tma_traj_tail(a, K, CA, e, T, nst, thr, band, markA);
+        tma_traj_tail(b, K, CB, e, T, nst, thr, band, markB);
       }
       if (!__any_sync(0xffffffffu, a.run || b.run)) break;
       // every lane is done reading this stage: refill it with chunk c + 2
@@ -1023,9 +1048,10 @@ template <> __device__ __forceinline__ double draw<double>(uint64_t w, double a)
 // same values, so the same trajectory and decisions.  Same contract as
 // run_lane.
 template <typename T, int PF = PrefetchDepth<T>::value>
-__device__ __forceinline__ T run_lane_gen(const RhsU<T>& K, const RhsC<T>& C, const ScenSrc& src,
+__device__ __forceinline__ T run_lane_gen(const StepU<T>& K, const PowTable* pw, const StepC<T>& C,
+                                          const ScenSrc& src,
                                           int k, int j0, int j_end, T& q_ca, T& w, T& q_sm,
-                                          T& w_abs, T smin_in, T dt, T thr,
+                                          T& w_abs, T smin_in, T thr,
                                           const volatile int32_t* dead, unsigned* steps, int* end,
                                           T band, int* jlast) {
   T smin = smin_in;
@@ -1043,23 +1069,19 @@ __device__ __forceinline__ T run_lane_gen(const RhsU<T>& K, const RhsC<T>& C, co
     }
   }
   bool stop = !go;
-  const StepC<T> S = step_consts<T>(K, dt);
   while (!stop && j + PF <= j_end) {
     const int dead_now = dead != nullptr ? *dead : 0;
-    T nf = T(0), bmin = inf_v<T>();
+    BlockMin<T> bm;
 #pragma unroll 4
     for (int u = 0; u < PF; ++u) {
       const U64x4 r = philox4x64_10(static_cast<uint64_t>(j), src.base + static_cast<uint64_t>(k), src.update,
                                     0ull, src.seed, 0ull);
-      rk4_step_fast<T>(K, C, S, q_ca, w, q_sm, w_abs, draw<T>(r.w[0], src.amp[0]),
+      rk4_step_fast<T>(K, pw, C, q_ca, w, q_sm, w_abs, draw<T>(r.w[0], src.amp[0]),
                        draw<T>(r.w[1], src.amp[1]), draw<T>(r.w[2], src.amp[2]));
       ++j;
-      const T s = C.y_scale * (q_sm - q_ca) + C.s_off;
-      bmin = fmin(bmin, s);
-      nf = fma_rn(s, T(0), nf);
+      bm.add(slack_of<T>(C, q_ca, q_sm), u);
     }
-    nf = fma_rn(q_ca, T(0), fma_rn(w, T(0), fma_rn(q_sm, T(0), nf)));
-    if (nf != nf) bmin = -inf_v<T>();
+    const T bmin = bm.result(q_ca, w, q_sm);
     smin = fmin(smin, bmin);
     if (bmin < band) jl = j;
     if (smin < thr) {
@@ -1073,7 +1095,7 @@ __device__ __forceinline__ T run_lane_gen(const RhsU<T>& K, const RhsC<T>& C, co
   while (!stop && j < j_end) {
     const U64x4 r = philox4x64_10(static_cast<uint64_t>(j), src.base + static_cast<uint64_t>(k), src.update, 0ull,
                                   src.seed, 0ull);
-    rk4_step_fast<T>(K, C, S, q_ca, w, q_sm, w_abs, draw<T>(r.w[0], src.amp[0]),
+    rk4_step_fast<T>(K, pw, C, q_ca, w, q_sm, w_abs, draw<T>(r.w[0], src.amp[0]),
                      draw<T>(r.w[1], src.amp[1]), draw<T>(r.w[2], src.amp[2]));
     ++j;
     const T s = checked_slack<T>(C, q_ca, w, q_sm);
@@ -1091,39 +1113,83 @@ __device__ __forceinline__ T run_lane_gen(const RhsU<T>& K, const RhsC<T>& C, co
 }
 
 // Scenario k's model under parametric uncertainty: the parameters theta_p
-// m_p^k folded like the nominal ones, and the candidate constants at v about
-// the reference point of the nominal candidate constants C comes in with
-// (replaced on return).  Returns the scenario's p_atm (the origin of its
-// gauge coordinates).
-template <typename T>
-__device__ __forceinline__ double scenario_model(const double* __restrict__ P,
-                                                 const double* __restrict__ m_k, double v,
-                                                 const PowSeries* pws, double y_min, RhsU<T>& U,
-                                                 RhsC<T>& C) {
-  const double q_r[3] = {static_cast<double>(C.r_ca), static_cast<double>(C.r_w),
-                         static_cast<double>(C.r_sm)};
+// m_p^k folded like the nominal ones (the step of size dt included).
+__device__ __forceinline__ void scenario_fold(const double* __restrict__ P, const double* __restrict__ m_k,
+                                              double dt, const PowTable* pws, StepModel<double>* out) {
   double Pk[RRG_NPARAM];
 #pragma unroll
   for (int p = 0; p < RRG_NPARAM; ++p) Pk[p] = __dmul_rn(P[p], m_k[p]);
   Fc3K<double> k64;
   Fc3K<float> k32;
   fold_constants(Pk, &k64, &k32);
-  k64.pws = pws;  // used only if the scenario's exponent is the table's
-  const CandK<double> c64 = cand_consts(Pk, v);
-  RhsU<double> u64;
-  RhsU<float> u32;
-  RhsC<double> r64;
-  RhsC<float> r32;
-  fold_rhs(k64, &u64, &u32);
-  fold_rhs_cand(k64, c64, q_r, y_min, &r64, &r32);
-  if constexpr (sizeof(T) == 8) {
-    U = u64;
-    C = r64;
+  // the table only if the scenario's exponent is the table's
+  k64.pws = (pws != nullptr && pws->e == k64.e) ? pws : nullptr;
+  fold_model(k64, Pk, dt, out);
+}
+
+// The model a lane integrates: the launch's own, or scenario k's under
+// parametric uncertainty (PU), with the candidate constants at setpoint v
+// about the reference point of the nominal ones that R comes in with
+// (replaced on return).  Returns the origin of the lane's gauge coordinates.
+//   binary32: scenario k's model is read from the arrays that
+// scenario_fold_kernel wrote with the draw; only the candidate constants are
+// formed here (about 20 binary64 instructions; folding the model in every lane
+// took about 600, 1.6 ms of the 65,536-scenario sweep).
+//   binary64 (recheck, binary64 handles): the lane folds it.
+template <typename T>
+struct LaneModel {
+  StepU<T> U;
+  StepC<T> C;
+  const PowTable* pw;
+};
+__device__ __forceinline__ double lane_model_pu(const Launch& L, const ScenFold& sf, const double*, int k,
+                                                double v, RhsC<float>& R, LaneModel<float>& M) {
+  const size_t N = static_cast<size_t>(L.N);
+  ModelC mc;
+  double* d = &mc.l_ca;
+#pragma unroll
+  for (int j = 0; j < kFoldDoubles; ++j) d[j] = __ldg(sf.d + j * N + k);
+  StepPhi<float> F;
+  float* u = &M.U.ip;
+  constexpr int nu = sizeof(StepU<float>) / sizeof(float);
+#pragma unroll
+  for (int j = 0; j < nu; ++j) u[j] = __ldg(sf.f + j * N + k);
+  float* p = &F.h;
+#pragma unroll
+  for (int j = 0; j < kFoldFloats - nu; ++j) p[j] = __ldg(sf.f + (nu + j) * N + k);
+  const double q_r[3] = {static_cast<double>(R.r_ca), static_cast<double>(R.r_w), static_cast<double>(R.r_sm)};
+  R = round_cand(fold_cand(mc, v, q_r, L.y_min));
+  M.C = step_consts<float>(M.U, F, R);
+  M.pw = nullptr;
+  return mc.p_atm;
+}
+__device__ __forceinline__ double lane_model_pu(const Launch& L, const ScenFold&, const double* pm, int k,
+                                                double v, RhsC<double>& R, LaneModel<double>& M) {
+  StepModel<double> sm;
+  scenario_fold(L.params, pm + static_cast<size_t>(k) * RRG_NPARAM, L.dt, L.m64.pw, &sm);
+  const double q_r[3] = {R.r_ca, R.r_w, R.r_sm};
+  R = fold_cand(sm.c, v, q_r, L.y_min);
+  M.U = sm.U;
+  M.C = step_consts<double>(sm.U, sm.F, R);
+  M.pw = sm.pw;
+  return sm.c.p_atm;
+}
+template <typename T> __device__ __forceinline__ const StepModel<T>& launch_model(const Launch& L);
+template <> __device__ __forceinline__ const StepModel<float>& launch_model<float>(const Launch& L) { return L.m32; }
+template <> __device__ __forceinline__ const StepModel<double>& launch_model<double>(const Launch& L) { return L.m64; }
+// pair: the scenario pair the lane reads (0 or 1); pm: its multipliers.
+template <typename T, bool PU>
+__device__ __forceinline__ double lane_model(const Launch& L, int pair, int k, double v, RhsC<T>& R,
+                                             LaneModel<T>& M) {
+  if constexpr (PU) {
+    return lane_model_pu(L, pair ? L.foldb : L.fold, pair ? L.pmulb : L.pmul, k, v, R, M);
   } else {
-    U = u32;
-    C = r32;
+    const StepModel<T>& m = launch_model<T>(L);
+    M.U = m.U;
+    M.C = step_consts<T>(m.U, m.F, R);
+    M.pw = m.pw;
+    return m.c.p_atm;
   }
-  return Pk[P_P_ATM];
 }
 
 // Warp minimum in the lane's own precision (a binary32 lane's value needs no
@@ -1139,18 +1205,17 @@ __device__ __forceinline__ T warp_min(T v) {
 // Philox counters step by step (the pair was sampled in a binary32 mode, so
 // its binary64 array was never written).  Same contract as run_lane over
 // steps 1..H with early exit at s < thr.
-__device__ __forceinline__ double run_lane_philox(const RhsU<double>& K, const RhsC<double>& C,
-                                  const ScenSrc& src, int k, int H, double q_ca, double w,
-                                  double q_sm, double w_abs, double dt, double thr,
+__device__ __forceinline__ double run_lane_philox(const StepU<double>& K, const PowTable* pw,
+                                  const StepC<double>& C, const ScenSrc& src, int k, int H, double q_ca, double w,
+                                  double q_sm, double w_abs, double thr,
                                   unsigned* steps) {
   double smin = checked_slack<double>(C, q_ca, w, q_sm);
   int j = 0;
-  const StepC<double> S = step_consts<double>(K, dt);
   if (!(smin < thr)) {
     while (j < H) {
       const U64x4 r = philox4x64_10(static_cast<uint64_t>(j), src.base + static_cast<uint64_t>(k), src.update,
                                     0ull, src.seed, 0ull);
-      rk4_step_fast<double>(K, C, S, q_ca, w, q_sm, w_abs, uniform_sym(r.w[0], src.amp[0]),
+      rk4_step_fast<double>(K, pw, C, q_ca, w, q_sm, w_abs, uniform_sym(r.w[0], src.amp[0]),
                             uniform_sym(r.w[1], src.amp[1]), uniform_sym(r.w[2], src.amp[2]));
       ++j;
       const double s = checked_slack<double>(C, q_ca, w, q_sm);
@@ -1181,20 +1246,15 @@ __device__ __forceinline__ int interior_points(double* cand_kappa, int M, double
 // ---------------------------------------------------------------------------
 // One step of the simulated plant at setpoint v (Fig. 1): x_{t+1} =
 // RK4(x_t, v) + (e_ca, e_w, e_sm), the plant's own draw added after the step
-// as in Eq. 4.  Binary64, with the rollouts' multiplied-out right-hand side
-// and x^e - 1 series: the plant step sits on the closed loop's critical path,
-// and a binary64 pow() costs thousands of cycles on GB300.
-__device__ __forceinline__ void plant_step_fast(const Fc3K<double>& K, const RhsU<double>& U,
-                                                const double* __restrict__ P, double dt, double v,
-                                                const double x[3], double e_ca, double e_w,
-                                                double e_sm, double x_next[3]) {
-  RhsC<double> c64;
-  RhsC<float> c32;
+// as in Eq. 4.  Binary64, the rollouts' step in gauge coordinates: the plant
+// sits on the closed loop's critical path.
+__device__ __forceinline__ void plant_step_fast(const StepModel<double>& M, double v, const double x[3],
+                                                double e_ca, double e_w, double e_sm, double x_next[3]) {
   const double q0[3] = {0.0, 0.0, 0.0};
-  fold_rhs_cand(K, cand_consts(P, v), q0, 0.0, &c64, &c32);
-  const double p_atm = P[P_P_ATM];
+  const StepC<double> C = step_consts<double>(M.U, M.F, fold_cand(M.c, v, q0, 0.0));
+  const double p_atm = M.c.p_atm;
   double q_ca = x[0] - p_atm, w = x[1], q_sm = x[2] - p_atm, w_abs = x[1];
-  rk4_step_fast<double>(U, c64, dt, q_ca, w, q_sm, w_abs, e_ca, e_w, e_sm);
+  rk4_step_fast<double>(M.U, M.pw, C, q_ca, w, q_sm, w_abs, e_ca, e_w, e_sm);
   x_next[0] = q_ca + p_atm;
   x_next[1] = w;
   x_next[2] = q_sm + p_atm;

@@ -24,7 +24,7 @@ constexpr size_t align256(size_t n) { return (n + 255) & ~static_cast<size_t>(25
 constexpr size_t kOffState = 0;
 constexpr size_t kOffParams = kOffState + align256(sizeof(SearchState));
 constexpr size_t kOffPws = kOffParams + align256(RRG_NPARAM * sizeof(double));
-constexpr size_t kOffKappa = kOffPws + align256(sizeof(PowSeries));
+constexpr size_t kOffKappa = kOffPws + align256(sizeof(PowTable));
 constexpr size_t kOffV = kOffKappa + align256(kStaticMaxCand * sizeof(double));
 constexpr size_t kOffK64 = kOffV + align256(kStaticMaxCand * sizeof(double));
 constexpr size_t kOffK32 = kOffK64 + align256(kStaticMaxCand * sizeof(RhsC<double>));
@@ -43,17 +43,20 @@ static_assert(kScratchBytes <= RRG_STATIC_SCRATCH_BYTES, "scratch layout exceeds
 __device__ __align__(256) unsigned char g_rrg_static_scratch[RRG_STATIC_SCRATCH_BYTES];
 
 struct ParamBlock {
+  PowTable pws;   // binary64 x^e - 1 table of the model's exponent (as rrg_create builds it)
   double v[RRG_NPARAM];
-  PowSeries pws;   // binary64 x^e - 1 series of the model's exponent (as rrg_create builds it)
 };
+static_assert(sizeof(ParamBlock) + 64 <= 32764, "passed by value to a kernel");
 
-// Writes the parameter vector and the x^e - 1 series (passed by value) into
+// Writes the parameter vector and the x^e - 1 table (passed by value) into
 // the scratch and clears the scratch's step counters.
-__global__ void static_params_kernel(ParamBlock pb, double* params, PowSeries* pws,
+__global__ void static_params_kernel(const __grid_constant__ ParamBlock pb, double* params, PowTable* pws,
                                      DevStats* stats, SearchState* st) {
   const int i = threadIdx.x;
   if (i < RRG_NPARAM) params[i] = pb.v[i];
-  if (i == 0) *pws = pb.pws;
+  const uint4* from = reinterpret_cast<const uint4*>(&pb.pws);
+  uint4* to = reinterpret_cast<uint4*>(pws);
+  for (unsigned q = i; q < sizeof(PowTable) / sizeof(uint4); q += blockDim.x) to[q] = from[q];
   if (i == 0) {
     st->src[0].d64_valid = 1;  // the caller's binary64 array holds the values
     st->src[1].d64_valid = 1;
@@ -204,10 +207,13 @@ extern "C" int rrg_eval_candidates_static(const double* model_params, int n_para
   L.scfg.eps_ss = cfg->eps_ss;
   L.scfg.y_c = cfg->y_c;
   fold_constants(model_params, &L.k64, &L.k32);
-  // the binary64 rollouts and the recheck evaluate x^e - 1 by the same series
+  // the binary64 rollouts and the recheck evaluate x^e - 1 by the same table
   // as a handle's, so both give the same bits
-  L.k64.pws = reinterpret_cast<const PowSeries*>(base + kOffPws);
-  fold_rhs(L.k64, &L.u64, &L.u32);
+  ParamBlock pb;
+  PowTable* const pws = reinterpret_cast<PowTable*>(base + kOffPws);
+  if (pow_table(L.k64.e, &pb.pws)) L.k64.pws = pws;
+  fold_model(L.k64, model_params, cfg->dt, &L.m64);
+  round_model(L.m64, &L.m32);
   L.params = reinterpret_cast<double*>(base + kOffParams);
   L.d64 = const_cast<double*>(d_scen64);
   L.d32 = const_cast<float*>(d_scen32);
@@ -228,11 +234,8 @@ extern "C" int rrg_eval_candidates_static(const double* model_params, int n_para
   L.sms = sms;
   L.recheck_blocks = 2 * sms;
 
-  ParamBlock pb;
   std::memcpy(pb.v, model_params, sizeof pb.v);
-  make_pow_series((model_params[P_GAMMA] - 1.0) / model_params[P_GAMMA], &pb.pws);
-  static_params_kernel<<<1, 32, 0, L.stream>>>(pb, const_cast<double*>(L.params),
-                                               const_cast<PowSeries*>(L.k64.pws), L.stats, L.st);
+  static_params_kernel<<<1, 256, 0, L.stream>>>(pb, const_cast<double*>(L.params), pws, L.stats, L.st);
   cudaError_t e = cudaGetLastError();
   // the prepare kernel rewrites every per-candidate flag, key and the recheck
   // count, so nothing left in the scratch by an earlier call is read
