@@ -76,6 +76,7 @@ struct BLaunch {
   StepModel<double> m64;
   StepModel<float> m32;
   const BInst* inst;
+  const int32_t* samp_base;  // [S + 1]: sampler tiles before each instance
   const int32_t* order;  // instances, longest horizon (then most scenarios) first
   BState* st;
   float* d32;
@@ -102,29 +103,36 @@ struct BLaunch {
 // Sampling: instance s draws with key (seed + s, 0) and the counters of the
 // single-problem sampler; only the binary32 copy is stored (the recheck
 // regenerates binary64 values from the same counters).
-__global__ void batch_sample_kernel(const BLaunch B, uint64_t seed, uint64_t base) {
-  const int s = blockIdx.y;
+// One warp per block: block t draws kSampleSteps steps x 64 scenarios (two per
+// thread) of the instance that holds tile t, so instances of all sizes share
+// the SMs evenly (samp_base: tiles before each instance).
+constexpr int kSampleSteps = 32;
+constexpr int sample_tiles_of(int N, int H) { return ((N + 63) / 64) * ((H + kSampleSteps - 1) / kSampleSteps); }
+
+__global__ void __launch_bounds__(32)
+batch_sample_kernel(const BLaunch B, uint64_t seed, uint64_t base) {
+  const int t = static_cast<int>(blockIdx.x);
+  int lo = 0, hi = B.c.S;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (B.samp_base[mid] <= t) lo = mid; else hi = mid;
+  }
+  const int s = lo;
   const BInst I = B.inst[s];
+  const int local = t - B.samp_base[s];
   const uint64_t upd = base + (B.t_dev ? *B.t_dev : 0ull);
   const uint64_t key = seed + static_cast<uint64_t>(s);
   const int pair = (B.d32b != nullptr && (upd & 1ull)) ? 1 : 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (local == 0 && threadIdx.x == 0) {
     B.st[s].seed_p[pair] = key;
     B.st[s].update_p[pair] = upd;
   }
-  const size_t HN = static_cast<size_t>(I.H) * I.N;
-  float* d = (pair ? B.d32b : B.d32) + I.off;
-  const float s0 = static_cast<float>(B.c.amp[0] * 0x1.0p-23),
-              s1 = static_cast<float>(B.c.amp[1] * 0x1.0p-23),
-              s2 = static_cast<float>(B.c.amp[2] * 0x1.0p-23);
-  const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
-  for (size_t q = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < HN; q += stride) {
-    const uint64_t j = q / static_cast<uint64_t>(I.N), k = q - j * static_cast<uint64_t>(I.N);
-    const U64x4 w = philox4x64_10(j, k, upd, 0ull, key, 0ull);
-    d[q] = uniform_sym32(w.w[0], s0);
-    d[HN + q] = uniform_sym32(w.w[1], s1);
-    d[2 * HN + q] = uniform_sym32(w.w[2], s2);
-  }
+  const int nk = (I.N + 63) / 64;
+  const int jt = local / nk, kt = local - jt * nk;
+  const int j0 = jt * kSampleSteps;
+  sample_tile32<2>((pair ? B.d32b : B.d32) + I.off, I.N, I.H, kt * 64 + static_cast<int>(threadIdx.x), j0,
+                   min(j0 + kSampleSteps, I.H), 0ull, upd, key, static_cast<float>(B.c.amp[0] * 0x1.0p-23),
+                   static_cast<float>(B.c.amp[1] * 0x1.0p-23), static_cast<float>(B.c.amp[2] * 0x1.0p-23));
 }
 
 // Tile list of the next round: instance order[o] contributes ceil(m / rows) x
@@ -869,6 +877,8 @@ struct rrg_batch_ctx {
   PowTable* pws = nullptr;
   BInst* inst_dev = nullptr;
   int32_t* order_dev = nullptr;
+  int32_t* samp_base_dev = nullptr;
+  int samp_tiles = 0;
   BState* st = nullptr;
   float* d32 = nullptr;
   float* d32b = nullptr;       // second scenario pair, allocated by the first closed loop
@@ -941,7 +951,7 @@ struct BDeviceGuard {
 };
 
 void bfree_all(rrg_batch_ctx* h) {
-  void* ptrs[] = {h->params_dev, h->pws, h->inst_dev, h->order_dev, h->st, h->d32, h->d32b,
+  void* ptrs[] = {h->params_dev, h->pws, h->inst_dev, h->order_dev, h->samp_base_dev, h->st, h->d32, h->d32b,
                   h->cand_kappa,
                   h->cand_v, h->cand_c64, h->cand_c32, h->cand_ok, h->cand_dead, h->cand_ss,
                   h->cand_min, h->tile_base, h->queue, h->recheck_list, h->recheck_jlast,
@@ -1021,12 +1031,7 @@ int enqueue_rollout(rrg_batch_ctx* h) {
 
 // One update of every instance: sample, then the rounds of the search.
 int enqueue_sample(rrg_batch_ctx* h, uint64_t seed, uint64_t base, cudaStream_t stream) {
-  int blocks = 1;
-  for (const BInst& I : h->inst) {
-    const size_t hn = static_cast<size_t>(I.H) * I.N;
-    blocks = std::max(blocks, static_cast<int>(std::min<size_t>((hn + 255) / 256, 64)));
-  }
-  batch_sample_kernel<<<dim3(blocks, h->B.c.S), 256, 0, stream>>>(h->B, seed, base);
+  batch_sample_kernel<<<h->samp_tiles, 32, 0, stream>>>(h->B, seed, base);
   BCK(cudaGetLastError());
   h->launches++;
   return RRG_OK;
@@ -1113,6 +1118,14 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
     elems += (e + 31ull) & ~31ull;  // 128-byte aligned blocks
     lanes += static_cast<unsigned long long>(M) * static_cast<unsigned long long>(n_scenarios[s]);
   }
+  // the sampler's tiles (32-bit: 2^31 of them would need 50 TB of scenarios)
+  std::vector<int32_t> samp_base(static_cast<size_t>(n_instances) + 1, 0);
+  unsigned long long tiles = 0;
+  for (int s = 0; s < n_instances; ++s) {
+    samp_base[s] = static_cast<int32_t>(tiles);
+    tiles += static_cast<unsigned long long>(sample_tiles_of(inst[s].N, inst[s].H));
+  }
+  samp_base[n_instances] = static_cast<int32_t>(tiles);
   if (lanes >= (1ull << 31)) return bset_err(h, RRG_EINVAL, "sum of max_candidates * n_scenarios >= 2^31");
 
   h = new (std::nothrow) rrg_batch_ctx();
@@ -1141,6 +1154,7 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   alloc(&h->pws, 1);
   alloc(&h->inst_dev, S);
   alloc(&h->order_dev, S);
+  alloc(&h->samp_base_dev, S + 1);
   alloc(&h->st, S);
   alloc(&h->d32, static_cast<size_t>(elems));
   h->d32_elems = static_cast<size_t>(elems);
@@ -1178,6 +1192,9 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
     e = cudaMemcpyAsync(h->inst_dev, inst.data(), S * sizeof(BInst), cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->order_dev, order.data(), S * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h->samp_base_dev, samp_base.data(), (S + 1) * sizeof(int32_t), cudaMemcpyHostToDevice,
+                        h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->st, 0, S * sizeof(BState), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->stats, 0, sizeof(DevStats), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->t_dev, 0, sizeof(unsigned long long), h->stream);
@@ -1222,6 +1239,8 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   round_model(B.m64, &B.m32);
   B.inst = h->inst_dev;
   B.order = h->order_dev;
+  B.samp_base = h->samp_base_dev;
+  h->samp_tiles = static_cast<int>(tiles);
   B.st = h->st;
   B.d32 = h->d32;
   B.d32b = nullptr;

@@ -92,7 +92,8 @@ cudaError_t launch_step_latency(const Launch& L, double v, int steps, double* d_
 }
 
 // ---------------------------------------------------------------------------
-// Scenario sampling: one thread per (j, k), coalesced over k.
+// Scenario sampling: coalesced over the scenarios k, the step j the same for a
+// whole block (philox_tile).
 //
 // binary64 values: d = a (2u - 1), u = (w >> 11) 2^-53 (bit-exact with the
 // definition in rrg.h).  binary32 copy in the binary32 modes: from the top 24
@@ -105,6 +106,7 @@ cudaError_t launch_step_latency(const Launch& L, double v, int steps, double* d_
 // in scenario k for every p set in mask (1 for the rest), u from word p % 4 of
 // the Philox block at counter (p / 4, k, update, 2).
 constexpr int kParamGroups = (RRG_NPARAM + 3) / 4;
+constexpr int kSampleThreads = 128;
 
 __device__ __forceinline__ void sample_param_group(double* __restrict__ pm, uint64_t k, uint64_t kbase,
                                                    int g, uint64_t upd, uint64_t seed, double rho,
@@ -118,54 +120,73 @@ __device__ __forceinline__ void sample_param_group(double* __restrict__ pm, uint
   }
 }
 
-__global__ void sample_kernel(double* __restrict__ d64, float* __restrict__ d32,
-                              double* __restrict__ d64b, float* __restrict__ d32b, int N, int H,
-                              uint64_t seed, uint64_t base, const unsigned long long* t_dev,
-                              double a0, double a1, double a2, int write64, int gen, SearchState* st,
-                              double* __restrict__ pm, double* __restrict__ pmb, double rho,
-                              uint32_t mask, uint64_t kbase) {
-  const uint64_t upd = base + (t_dev ? *t_dev : 0ull);
-  const int pair = (d64b != nullptr && (upd & 1ull)) ? 1 : 0;
-  if (pair) {
-    d64 = d64b;
-    d32 = d32b;
-    pm = pmb;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+// A block draws a tile of steps (blockIdx.y) x scenarios (blockIdx.x), KT
+// scenarios per thread.
+struct SampleArgs {
+  double *d64, *d64b;
+  float *d32, *d32b;
+  int N, H, jc;   // jc: steps per block
+  uint64_t seed, base, kbase;
+  double a0, a1, a2;
+  int write64, gen;
+  SearchState* st;
+  double *pm, *pmb;
+  double rho;
+  uint32_t mask;
+};
+
+template <int KT>
+__device__ __forceinline__ void sample_tile64(double* __restrict__ d, const SampleArgs& A, uint64_t upd) {
+  const int k0 = blockIdx.x * (blockDim.x * KT) + threadIdx.x;
+  const int j0 = blockIdx.y * A.jc, j1 = min(j0 + A.jc, A.H);
+  const size_t N = A.N, HN = static_cast<size_t>(A.H) * N;
+  philox_tile<KT>(A.kbase + static_cast<uint64_t>(k0), blockDim.x, j0, j1, upd, A.seed,
+                  [&](int i, int j, uint64_t w0, uint64_t w1, uint64_t w2) {
+                    const size_t k = static_cast<size_t>(k0) + static_cast<size_t>(i) * blockDim.x;
+                    if (k < N) {
+                      const size_t q = static_cast<size_t>(j) * N + k;
+                      d[q] = uniform_sym(w0, A.a0);
+                      d[HN + q] = uniform_sym(w1, A.a1);
+                      d[2 * HN + q] = uniform_sym(w2, A.a2);
+                    }
+                  });
+}
+
+template <int KT>
+__global__ void __launch_bounds__(kSampleThreads)
+sample_kernel(const SampleArgs A, const unsigned long long* t_dev) {
+  const uint64_t upd = A.base + (t_dev ? *t_dev : 0ull);
+  const int pair = (A.d64b != nullptr && (upd & 1ull)) ? 1 : 0;
+  const size_t blk = static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x;
+  if (blk == 0 && threadIdx.x == 0) {
     ScenSrc src;
-    src.d64_valid = gen ? 0 : write64;
+    src.d64_valid = A.gen ? 0 : A.write64;
     src.pad = 0;
-    src.seed = seed;
+    src.seed = A.seed;
     src.update = upd;
-    src.base = kbase;
-    src.amp[0] = a0;
-    src.amp[1] = a1;
-    src.amp[2] = a2;
-    st->src[pair] = src;
+    src.base = A.kbase;
+    src.amp[0] = A.a0;
+    src.amp[1] = A.a1;
+    src.amp[2] = A.a2;
+    A.st->src[pair] = src;
   }
-  const size_t HN = static_cast<size_t>(H) * N;
-  const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
-  const float s0 = static_cast<float>(a0 * 0x1.0p-23), s1 = static_cast<float>(a1 * 0x1.0p-23),
-              s2 = static_cast<float>(a2 * 0x1.0p-23);
-  for (size_t q = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; !gen && q < HN;
-       q += stride) {
-    const uint64_t j = q / static_cast<uint64_t>(N), k = q - j * static_cast<uint64_t>(N);
-    const U64x4 w = philox4x64_10(j, kbase + k, upd, 0ull, seed, 0ull);
-    if (write64) {
-      d64[q] = uniform_sym(w.w[0], a0);
-      d64[HN + q] = uniform_sym(w.w[1], a1);
-      d64[2 * HN + q] = uniform_sym(w.w[2], a2);
+  if (!A.gen) {
+    if (A.write64) {
+      sample_tile64<KT>(pair ? A.d64b : A.d64, A, upd);
     } else {
-      d32[q] = uniform_sym32(w.w[0], s0);
-      d32[HN + q] = uniform_sym32(w.w[1], s1);
-      d32[2 * HN + q] = uniform_sym32(w.w[2], s2);
+      const int j0 = blockIdx.y * A.jc;
+      sample_tile32<KT>(pair ? A.d32b : A.d32, A.N, A.H, blockIdx.x * (blockDim.x * KT) + threadIdx.x, j0,
+                        min(j0 + A.jc, A.H), A.kbase, upd, A.seed, static_cast<float>(A.a0 * 0x1.0p-23),
+                        static_cast<float>(A.a1 * 0x1.0p-23), static_cast<float>(A.a2 * 0x1.0p-23));
     }
   }
+  double* pm = pair ? A.pmb : A.pm;
   if (pm != nullptr) {
-    const size_t G = static_cast<size_t>(N) * kParamGroups;
-    for (size_t q = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < G; q += stride) {
+    const size_t G = static_cast<size_t>(A.N) * kParamGroups;
+    const size_t stride = static_cast<size_t>(gridDim.x) * gridDim.y * blockDim.x;
+    for (size_t q = blk * blockDim.x + threadIdx.x; q < G; q += stride) {
       const uint64_t k = q / kParamGroups;
-      sample_param_group(pm, k, kbase, static_cast<int>(q - k * kParamGroups), upd, seed, rho, mask);
+      sample_param_group(pm, k, A.kbase, static_cast<int>(q - k * kParamGroups), upd, A.seed, A.rho, A.mask);
     }
   }
 }
@@ -213,20 +234,58 @@ static int grid_for(size_t n, int threads, int cap) {
   return static_cast<int>(b);
 }
 
+// Blocks over (scenarios, steps): about `want` of them, 1 to 64 steps each (more
+// where the grid's height would pass its limit).
+static dim3 sample_grid(int N, int H, int per_block, int want, int* jc) {
+  const long long gx = (static_cast<long long>(N) + per_block - 1) / per_block;
+  long long c = gx * H / want;
+  c = c < 1 ? 1 : (c > 64 ? 64 : c);
+  const long long least = (static_cast<long long>(H) + 65534) / 65535;
+  if (c < least) c = least;
+  *jc = static_cast<int>(c);
+  return dim3(static_cast<unsigned>(gx), static_cast<unsigned>((H + c - 1) / c));
+}
+
 cudaError_t launch_sample(const Launch& L, uint64_t seed, uint64_t base,
                           const unsigned long long* t_dev, const double* amp, bool dual,
                           cudaStream_t stream) {
-  const size_t n = static_cast<size_t>(L.H) * L.N;
-  const int write64 = L.precision == RRG_FP64 ? 1 : 0;
   // Full width also for the next closed-loop update's draw on the side
   // stream: it then finishes while the search's short kernels run.  (One
   // block per SM stretched it over the long rollout and slowed the update by
   // 7 %; stream priorities changed nothing, measured on GB300.)
   if (L.sms <= 0) return cudaErrorInvalidConfiguration;
-  sample_kernel<<<grid_for(n, 256, L.sms * 16), 256, 0, stream ? stream : L.stream>>>(
-      L.d64, L.d32, dual ? L.d64b : nullptr, dual ? L.d32b : nullptr, L.N, L.H, seed, base, t_dev,
-      amp[0], amp[1], amp[2], write64, L.scen_gen, L.st, L.pmul, dual ? L.pmulb : nullptr, L.punc_rho,
-      L.punc_mask, L.kbase);
+  SampleArgs A{};
+  A.d64 = L.d64;
+  A.d32 = L.d32;
+  A.d64b = dual ? L.d64b : nullptr;
+  A.d32b = dual ? L.d32b : nullptr;
+  A.N = L.N;
+  A.H = L.H;
+  A.seed = seed;
+  A.base = base;
+  A.kbase = L.kbase;
+  A.a0 = amp[0];
+  A.a1 = amp[1];
+  A.a2 = amp[2];
+  A.write64 = L.precision == RRG_FP64 ? 1 : 0;
+  A.gen = L.scen_gen;
+  A.st = L.st;
+  A.pm = L.pmul;
+  A.pmb = dual ? L.pmulb : nullptr;
+  A.rho = L.punc_rho;
+  A.mask = L.punc_mask;
+  // two scenarios per thread, but one where that leaves a warp half empty;
+  // blocks of 128 threads (fewer for few scenarios), 16 per SM, of at most 64
+  // steps each
+  const int kt = L.N > 32 ? 2 : 1;
+  const int per = (L.N + kt - 1) / kt;
+  const int threads = per >= kSampleThreads ? kSampleThreads : (per + 31) / 32 * 32;
+  const dim3 tile = sample_grid(L.N, L.scen_gen ? 1 : L.H, threads * kt, L.sms * 16, &A.jc);
+  const cudaStream_t s = stream ? stream : L.stream;
+  if (kt == 2)
+    sample_kernel<2><<<tile, threads, 0, s>>>(A, t_dev);
+  else
+    sample_kernel<1><<<tile, threads, 0, s>>>(A, t_dev);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_scenario_fold(L, false, base, t_dev, dual && L.d64b != nullptr, stream);
@@ -246,19 +305,20 @@ cudaError_t launch_fill(const Launch& L, double* a, size_t n, double v) {
 
 // Writes pair 0's binary64 values from Philox when the pair was sampled in a
 // binary32 mode (its binary64 array is then stale).
-__global__ void materialize64_kernel(double* __restrict__ d64, int N, int H,
-                                     const SearchState* st) {
+__global__ void __launch_bounds__(kSampleThreads)
+materialize64_kernel(double* __restrict__ d64, int N, int H, int jc, const SearchState* st) {
   const ScenSrc src = st->src[0];
   if (src.d64_valid) return;
-  const size_t HN = static_cast<size_t>(H) * N;
-  const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
-  for (size_t q = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < HN; q += stride) {
-    const uint64_t j = q / static_cast<uint64_t>(N), k = q - j * static_cast<uint64_t>(N);
-    const U64x4 w = philox4x64_10(j, src.base + k, src.update, 0ull, src.seed, 0ull);
-    d64[q] = uniform_sym(w.w[0], src.amp[0]);
-    d64[HN + q] = uniform_sym(w.w[1], src.amp[1]);
-    d64[2 * HN + q] = uniform_sym(w.w[2], src.amp[2]);
-  }
+  SampleArgs A{};
+  A.N = N;
+  A.H = H;
+  A.jc = jc;
+  A.seed = src.seed;
+  A.kbase = src.base;
+  A.a0 = src.amp[0];
+  A.a1 = src.amp[1];
+  A.a2 = src.amp[2];
+  sample_tile64<1>(d64, A, src.update);
 }
 
 // Marks pair 0's binary64 array valid once every block of the fill is done
@@ -266,9 +326,10 @@ __global__ void materialize64_kernel(double* __restrict__ d64, int N, int H,
 __global__ void mark64_kernel(SearchState* st) { st->src[0].d64_valid = 1; }
 
 cudaError_t launch_materialize64(const Launch& L) {
-  const size_t n = static_cast<size_t>(L.H) * L.N;
   if (L.sms <= 0) return cudaErrorInvalidConfiguration;
-  materialize64_kernel<<<grid_for(n, 256, L.sms * 16), 256, 0, L.stream>>>(L.d64, L.N, L.H, L.st);
+  int jc = 1;
+  const dim3 tile = sample_grid(L.N, L.H, kSampleThreads, L.sms * 16, &jc);
+  materialize64_kernel<<<tile, kSampleThreads, 0, L.stream>>>(L.d64, L.N, L.H, jc, L.st);
   mark64_kernel<<<1, 1, 0, L.stream>>>(L.st);
   return cudaGetLastError();
 }
