@@ -660,9 +660,10 @@ RRG_API int rrg_step_latency(rrg_handle h, double v, int steps, double *cycles_p
  * instance's result equals rrg_step's for the same inputs and scenarios. */
 #define RRG_BATCH_MAX_INSTANCES 1024
 #define RRG_BATCH_VARIANTS 10  /* rollout variants: lanes per tile {64, 128,
-                                  256} x disturbance prefetch depth {8, 16},
-                                  then warp tiles (32 lanes, each warp takes its
-                                  own) x {8, 16}, then warp tiles of two
+                                  256} x disturbance prefetch depth {8
+                                  (registers), 16 (the per-warp TMA ring's
+                                  chunk)}, then warp tiles (32 lanes, each warp
+                                  takes its own) x {8, 16}, then warp tiles of two
                                   candidates per thread (prefetch 8), then warp
                                   tiles of 16 scenarios at two lanes per
                                   trajectory (prefetch 8; tile_lanes reports
@@ -672,7 +673,7 @@ typedef struct rrg_batch_ctx *rrg_batch_handle;
 /* cfg as for rrg_create (n_scenarios and horizon are ignored); n_scenarios
  * and horizons: host arrays of n_instances values >= 1; sum over instances of
  * max_candidates * N_s must be below 2^31.  Allocates 12 sum(H_s N_s) bytes of
- * scenarios plus O(sum M N_s) bytes of recheck list. */
+ * scenarios (N_s rounded up to a multiple of 4) plus O(sum M N_s) bytes of recheck list. */
 RRG_API int rrg_batch_create(const double *model_params, int n_params, const rrg_config *cfg,
                      int n_instances, const int32_t *n_scenarios, const int32_t *horizons,
                      void *cuda_stream, rrg_batch_handle *out);

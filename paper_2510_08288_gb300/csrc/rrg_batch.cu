@@ -43,7 +43,8 @@ static_assert(kMaxInst <= kDecideThreads, "one decision thread per instance");
 
 struct BInst {
   int32_t N, H;
-  long long off;  // element offset of the instance's [3][H][N] binary32 scenarios
+  int32_t ld, pad;  // row length of its scenario array: N rounded up to 4 (TMA strides)
+  long long off;    // element offset of the instance's [3][H][ld] binary32 scenarios
 };
 
 struct BState {
@@ -81,6 +82,7 @@ struct BLaunch {
   BState* st;
   float* d32;
   float* d32b;         // second scenario pair (closed loops), or nullptr
+  const CUtensorMap* maps;  // [2][S]: tensor map of each pair's instances
   double* cand_kappa;
   double* cand_v;
   RhsC<double>* cand_c64;
@@ -90,7 +92,8 @@ struct BLaunch {
   int32_t* cand_ss;
   unsigned long long* cand_min;
   int32_t* tile_base;  // [S + 1] over `order`
-  uint32_t* queue;     // [0] next tile, [1] tiles of the round
+  uint32_t* queue;     // [0] next tile, [1] tiles of the round, [2] CTAs that take tiles
+  int sms;
   uint2* recheck_list; // (slot, k)
   uint32_t* recheck_jlast;  // the recheck runs steps 0..jlast
   uint32_t* recheck_count;
@@ -130,9 +133,27 @@ batch_sample_kernel(const BLaunch B, uint64_t seed, uint64_t base) {
   const int nk = (I.N + 63) / 64;
   const int jt = local / nk, kt = local - jt * nk;
   const int j0 = jt * kSampleSteps;
-  sample_tile32<2>((pair ? B.d32b : B.d32) + I.off, I.N, I.H, kt * 64 + static_cast<int>(threadIdx.x), j0,
+  sample_tile32<2>((pair ? B.d32b : B.d32) + I.off, I.N, I.ld, I.H, kt * 64 + static_cast<int>(threadIdx.x), j0,
                    min(j0 + kSampleSteps, I.H), 0ull, upd, key, static_cast<float>(B.c.amp[0] * 0x1.0p-23),
                    static_cast<float>(B.c.amp[1] * 0x1.0p-23), static_cast<float>(B.c.amp[2] * 0x1.0p-23));
+}
+
+// CTAs that take tiles in a round of `tiles` tiles: 8 resident warps per SM
+// while the round has fewer than 64 warps of tiles per SM, 12 below 300, every
+// slot of the launch above.  Most tiles end after a few steps, and the ones
+// that run their whole horizon pile up unevenly on the SMs; a round of few
+// tiles then lasts as long as the fullest SM takes per step, and two warps per
+// scheduler step 1.6 times as fast as four.  Measured (rollouts of an update,
+// 8 / 12 / 16 warps per SM): 38 warps of tiles per SM 0.80 / 0.87 / 1.00 ms, 63
+// 1.56 / 1.59 / 1.77, 108 2.75 / 2.45 / 2.58, 152 2.35 / 2.14 / 2.25, 269 7.5 /
+// 6.6 / 6.9, 491 8.7 / 7.4 / 7.3, 657 12.9 / 10.9 / 10.5.
+__device__ uint32_t round_ctas(int sms, uint32_t tiles, int tile) {
+  const uint32_t per_tile = tile <= 32 ? 1u : static_cast<uint32_t>(tile) / 32u;
+  const uint32_t per_cta = tile <= 32 ? 4u : per_tile;
+  const unsigned long long warps = static_cast<unsigned long long>(tiles) * per_tile;
+  if (warps >= 300ull * sms) return 0xffffffffu;
+  const uint32_t want = warps < 64ull * sms ? 8u : 12u;
+  return (static_cast<uint32_t>(sms) * want + per_cta - 1) / per_cta;
 }
 
 // Tile list of the next round: instance order[o] contributes ceil(m / rows) x
@@ -160,6 +181,7 @@ __device__ void build_tiles(const BLaunch& B, int tile, int rows) {
     B.tile_base[0] = 0;
     B.queue[0] = 0u;
     B.queue[1] = static_cast<uint32_t>(sc[B.c.S - 1]);
+    B.queue[2] = round_ctas(B.sms, static_cast<uint32_t>(sc[B.c.S - 1]), tile);
     *B.recheck_count = 0u;
   }
 }
@@ -347,6 +369,18 @@ __device__ __forceinline__ void batch_reduce(const BLaunch& B, size_t slot, int 
   }
 }
 
+// Where a tile's lanes take their disturbances from: PF steps ahead in
+// registers (run_lane), or (PF = 16) each warp's ring of 16-step chunks filled
+// by tensor copies (run_lane_tma), which issues 91 instead of about 100
+// instructions a step and leaves the coefficients as constant-bank operands.
+// Measured on 64 instances (rollouts of an update), ring against registers at
+// the same tile: 64 lanes 11.3 -> 10.2 ms, 128 (the default)
+// 11.3 -> 10.5, 256 11.6 -> 10.9, warp tiles 11.1 -> 10.0.
+template <int PF> constexpr bool kTileRing = PF == kTmaChunk;
+// Dynamic shared memory of a block of `warps` warps with rings.
+constexpr size_t ring_bytes(int warps) { return static_cast<size_t>(warps) * (2 * kTmaStageBytes + 2 * sizeof(uint64_t)); }
+extern __shared__ __align__(128) unsigned char batch_dyn_smem[];
+
 // One tile: lanes k of candidate slot (s, i), binary32 rollouts classified
 // for the binary64 recheck, reduced into the candidate's flags.  Called by
 // every thread of the CTA; returns are warp- or CTA-uniform.
@@ -367,21 +401,31 @@ __device__ __forceinline__ void batch_tile(const BLaunch& B, int s, int i, int k
   float smin = inf_v<float>();
   unsigned steps = 0;
   int jlast = -1;
-  if (active) {
-    const BState& st = B.st[s];
-    const double p_atm = B.params[P_P_ATM];
-    const RhsC<float> R = B.cand_c32[slot];
-    const StepU<float>& U = B.m32.U;
-    const StepC<float> C = step_consts<float>(U, B.m32.F, R);
-    float q_ca, w, q_sm, w_abs;  // the deviation from the candidate's reference point
-    start_state<float>(R, st.x, p_atm, q_ca, w, q_sm, w_abs);
-    int end = LANE_REACHED_END;
+  const BState& st = B.st[s];
+  const RhsC<float> R = B.cand_c32[slot];
+  const StepU<float>& U = B.m32.U;
+  const StepC<float> C = step_consts<float>(U, B.m32.F, R);
+  float q_ca = 0.0f, w = 0.0f, q_sm = 0.0f, w_abs = 0.0f;  // the deviation from the candidate's reference point
+  if (active) start_state<float>(R, st.x, B.params[P_P_ATM], q_ca, w, q_sm, w_abs);
+  int end = LANE_REACHED_END;
+  if constexpr (kTileRing<PF>) {
+    if ((k & ~31) >= I.N) return;  // a warp past the scenarios (the copies serve whole warps)
+    const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    float* stages = reinterpret_cast<float*>(batch_dyn_smem) + static_cast<size_t>(wid) * 2 * kTmaStageFloats;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(batch_dyn_smem + static_cast<size_t>(nw) * 2 * kTmaStageBytes) + 2 * wid;
+    const CUtensorMap* tm = B.maps + (st.cur ? B.c.S : 0) + s;
+    if ((threadIdx.x & 31) == 0) fence_tensormap(tm);
+    const float s_out = run_lane_tma<false>(U, C, tm, k & ~31, active, 0, I.H, q_ca, w, q_sm, w_abs,
+                                            inf_v<float>(), thr, cand_stop ? dead : nullptr,
+                                            cand_stop ? dead : nullptr, &steps, &end, eps, &jlast, stages, bars,
+                                            &B.stats->wait_timeouts);
+    if (active) smin = s_out;
+  } else if (active) {
     const float* d = (st.cur ? B.d32b : B.d32) + I.off;
-    smin = run_lane<float, PF>(U, nullptr, C, d, k, I.N, I.H, 0, I.H, q_ca,
-                               w, q_sm, w_abs, inf_v<float>(), thr, cand_stop ? dead : nullptr,
-                               &steps, &end, eps, &jlast);
-    if (cand_stop && smin < thr) *dead = 1;
+    smin = run_lane<float, PF>(U, nullptr, C, d, k, I.ld, I.H, 0, I.H, q_ca, w, q_sm, w_abs, inf_v<float>(), thr,
+                               cand_stop ? dead : nullptr, &steps, &end, eps, &jlast);
   }
+  if (active && cand_stop && smin < thr) *dead = 1;
   batch_reduce(B, slot, k, active, smin, steps, jlast, eps, dead);
 }
 
@@ -394,6 +438,7 @@ constexpr int kBatchThreadsPerSm = 384;
 template <int TILE, int PF>
 __global__ void __launch_bounds__(TILE, kBatchThreadsPerSm / TILE) batch_rollout_kernel(const BLaunch B) {
   __shared__ int sh[3];
+  if (blockIdx.x >= B.queue[2]) return;
   const uint32_t total = B.queue[1];
   for (;;) {
     if (threadIdx.x == 0) {
@@ -444,6 +489,7 @@ __device__ __forceinline__ void tile_of(const BLaunch& B, uint32_t t, int tile, 
 
 template <int PF>
 __global__ void __launch_bounds__(128, kBatchThreadsPerSm / 128) batch_rollout_warp_kernel(const BLaunch B) {
+  if (blockIdx.x >= B.queue[2]) return;
   const uint32_t total = B.queue[1];
   const int lane = static_cast<int>(threadIdx.x & 31);
   for (;;) {
@@ -502,14 +548,14 @@ __device__ __forceinline__ void batch_tile_pair(const BLaunch& B, int s, int p, 
     start_state<float>(RB, bs.x, p_atm, zb[0], zb[1], zb[2], zb[3]);
     const float* d = (bs.cur ? B.d32b : B.d32) + I.off;
     if (runA && runB) {
-      run_lane_pair<float, PF>(K, CA, CB, d, k, I.N, I.H, I.H, za, zb, thr, eps,
+      run_lane_pair<float, PF>(K, CA, CB, d, k, I.ld, I.H, I.H, za, zb, thr, eps,
                                cand_stop ? deadA : nullptr, cand_stop ? deadB : nullptr, sm, st, en, jl);
     } else if (runA) {
-      sm[0] = run_lane<float, PF>(K, nullptr, CA, d, k, I.N, I.H, 0, I.H, za[0], za[1], za[2], za[3],
+      sm[0] = run_lane<float, PF>(K, nullptr, CA, d, k, I.ld, I.H, 0, I.H, za[0], za[1], za[2], za[3],
                                   inf_v<float>(), thr, cand_stop ? deadA : nullptr, &st[0], &en[0], eps,
                                   &jl[0]);
     } else {
-      sm[1] = run_lane<float, PF>(K, nullptr, CB, d, k, I.N, I.H, 0, I.H, zb[0], zb[1], zb[2], zb[3],
+      sm[1] = run_lane<float, PF>(K, nullptr, CB, d, k, I.ld, I.H, 0, I.H, zb[0], zb[1], zb[2], zb[3],
                                   inf_v<float>(), thr, cand_stop ? deadB : nullptr, &st[1], &en[1], eps,
                                   &jl[1]);
     }
@@ -524,6 +570,7 @@ __device__ __forceinline__ void batch_tile_pair(const BLaunch& B, int s, int p, 
 // instance and scenario block).
 template <int PF>
 __global__ void __launch_bounds__(128) batch_rollout_warp_pair_kernel(const BLaunch B) {
+  if (blockIdx.x >= B.queue[2]) return;
   const uint32_t total = B.queue[1];
   const int lane = static_cast<int>(threadIdx.x & 31);
   for (;;) {
@@ -663,7 +710,7 @@ __device__ __forceinline__ void batch_tile_split(const BLaunch& B, int s, int i,
   const float* d = (st.cur ? B.d32b : B.d32) + I.off;
   unsigned steps = 0;
   int jlast = -1;
-  const float smin = run_lane_split<PF>(B.m32.U, C, d, k, on, I.N, I.H, role, q_ca, w, q_sm, w_abs, thr, cand_stop ? dead : nullptr, &steps,
+  const float smin = run_lane_split<PF>(B.m32.U, C, d, k, on, I.ld, I.H, role, q_ca, w, q_sm, w_abs, thr, cand_stop ? dead : nullptr, &steps,
                                         eps, &jlast);
   const bool mine = on && role == 0;
   if (cand_stop && mine && smin < thr) *dead = 1;
@@ -673,6 +720,7 @@ __device__ __forceinline__ void batch_tile_split(const BLaunch& B, int s, int i,
 // Warp tiles of 16 scenarios at two lanes per trajectory.
 template <int PF>
 __global__ void __launch_bounds__(128) batch_rollout_split_kernel(const BLaunch B) {
+  if (blockIdx.x >= B.queue[2]) return;
   const uint32_t total = B.queue[1];
   const int lane = static_cast<int>(threadIdx.x & 31);
   for (;;) {
@@ -838,7 +886,8 @@ __global__ void batch_loop_init_kernel(const BLaunch B, const double* __restrict
 }
 
 // Rollout variants the autotuner chooses from: threads (= scenario lanes)
-// per tile, the disturbance prefetch depth, and candidate slots per tile.
+// per tile, the disturbance prefetch depth (16: the TMA ring's chunk), and
+// candidate slots per tile.
 struct Variant {
   int tile, pf, rows;
   void (*kernel)(const BLaunch);
@@ -854,6 +903,10 @@ const Variant kVariants[RRG_BATCH_VARIANTS] = {
     {32, 8, 2, batch_rollout_warp_pair_kernel<8>}, {16, 8, 1, batch_rollout_split_kernel<8>},
 };
 constexpr int block_threads(int tile) { return tile <= 32 ? 128 : tile; }
+// Dynamic shared memory of variant v: the rings of its warps.
+size_t variant_smem(const Variant& v) {
+  return v.pf == kTmaChunk ? ring_bytes(block_threads(v.tile) / 32) : 0;
+}
 
 }  // namespace
 }  // namespace rrg
@@ -881,6 +934,7 @@ struct rrg_batch_ctx {
   int samp_tiles = 0;
   BState* st = nullptr;
   float* d32 = nullptr;
+  CUtensorMap* maps_dev = nullptr;  // [2][S]
   float* d32b = nullptr;       // second scenario pair, allocated by the first closed loop
   size_t d32_elems = 0;
   cudaStream_t side = nullptr; // draws update t + 1 while update t searches
@@ -951,7 +1005,7 @@ struct BDeviceGuard {
 };
 
 void bfree_all(rrg_batch_ctx* h) {
-  void* ptrs[] = {h->params_dev, h->pws, h->inst_dev, h->order_dev, h->samp_base_dev, h->st, h->d32, h->d32b,
+  void* ptrs[] = {h->params_dev, h->pws, h->inst_dev, h->order_dev, h->samp_base_dev, h->st, h->d32, h->d32b, h->maps_dev,
                   h->cand_kappa,
                   h->cand_v, h->cand_c64, h->cand_c32, h->cand_ok, h->cand_dead, h->cand_ss,
                   h->cand_min, h->tile_base, h->queue, h->recheck_list, h->recheck_jlast,
@@ -994,6 +1048,17 @@ void bcollect(rrg_batch_ctx* h) {
   h->ev_roll.clear();
 }
 
+// The tensor maps of a pair's scenario arrays (pair 0 or 1).
+cudaError_t upload_maps(rrg_batch_ctx* h, const float* d32, int pair) {
+  std::vector<CUtensorMap> m(h->inst.size());
+  for (size_t s = 0; s < m.size(); ++s) {
+    const BInst& I = h->inst[s];
+    if (!encode_scenario_map(&m[s], d32 + I.off, I.N, I.H, I.ld)) return cudaErrorNotSupported;
+  }
+  return cudaMemcpy(h->maps_dev + static_cast<size_t>(pair) * m.size(), m.data(), m.size() * sizeof(CUtensorMap),
+                    cudaMemcpyHostToDevice);
+}
+
 // Rounds of one update's search: 1 for Alg. 3, n_rounds for the k-section;
 // for the speculative bisection enough trees of the current width to finish
 // Alg. 1's n_bisect iterations from kappa = 1 (instances that finish sooner
@@ -1018,7 +1083,7 @@ int enqueue_rollout(rrg_batch_ctx* h) {
     b = btake_event(h);
     if (a && b) BCK(cudaEventRecord(a, h->stream));
   }
-  v.kernel<<<h->grid[h->variant], block_threads(v.tile), 0, h->stream>>>(h->B);
+  v.kernel<<<h->grid[h->variant], block_threads(v.tile), variant_smem(v), h->stream>>>(h->B);
   BCK(cudaGetLastError());
   if (timed && a && b) {
     BCK(cudaEventRecord(b, h->stream));
@@ -1113,8 +1178,10 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
     inst[s].N = n_scenarios[s];
     inst[s].H = horizons[s];
     inst[s].off = static_cast<long long>(elems);
+    inst[s].ld = static_cast<int32_t>((static_cast<int64_t>(n_scenarios[s]) + 3) & ~int64_t(3));
+    inst[s].pad = 0;
     const unsigned long long e = 3ull * static_cast<unsigned long long>(horizons[s]) *
-                                 static_cast<unsigned long long>(n_scenarios[s]);
+                                 static_cast<unsigned long long>(inst[s].ld);
     elems += (e + 31ull) & ~31ull;  // 128-byte aligned blocks
     lanes += static_cast<unsigned long long>(M) * static_cast<unsigned long long>(n_scenarios[s]);
   }
@@ -1157,6 +1224,7 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   alloc(&h->samp_base_dev, S + 1);
   alloc(&h->st, S);
   alloc(&h->d32, static_cast<size_t>(elems));
+  alloc(&h->maps_dev, 2 * S);
   h->d32_elems = static_cast<size_t>(elems);
   alloc(&h->cand_kappa, SM);
   alloc(&h->cand_v, SM);
@@ -1167,7 +1235,7 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   alloc(&h->cand_ss, SM);
   alloc(&h->cand_min, SM);
   alloc(&h->tile_base, S + 1);
-  alloc(&h->queue, 2);
+  alloc(&h->queue, 3);
   alloc(&h->recheck_list, static_cast<size_t>(lanes));
   alloc(&h->recheck_jlast, static_cast<size_t>(lanes));
   alloc(&h->recheck_count, 1);
@@ -1199,14 +1267,24 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   if (e == cudaSuccess) e = cudaMemsetAsync(h->stats, 0, sizeof(DevStats), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->t_dev, 0, sizeof(unsigned long long), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->d32, 0, static_cast<size_t>(elems) * sizeof(float), h->stream);
+  if (e == cudaSuccess) e = upload_maps(h, h->d32, 0);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   int nsm = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
   h->sms = nsm;
+  // the draw beside the rollouts' rings, as for single problems
+  // (tma_ring_prepare)
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(batch_sample_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared);
   for (int v = 0; v < RRG_BATCH_VARIANTS && e == cudaSuccess; ++v) {
     int per = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kVariants[v].kernel,
-                                                      block_threads(kVariants[v].tile), 0);
+    const size_t sm = variant_smem(kVariants[v]);
+    if (sm > 48 * 1024)
+      e = cudaFuncSetAttribute(kVariants[v].kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm));
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kVariants[v].kernel,
+                                                        block_threads(kVariants[v].tile), sm);
     h->grid[v] = std::max(1, per) * nsm;
   }
   if (e != cudaSuccess) {
@@ -1244,6 +1322,7 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   B.st = h->st;
   B.d32 = h->d32;
   B.d32b = nullptr;
+  B.maps = h->maps_dev;
   B.cand_kappa = h->cand_kappa;
   B.cand_v = h->cand_v;
   B.cand_c64 = h->cand_c64;
@@ -1254,6 +1333,7 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   B.cand_min = h->cand_min;
   B.tile_base = h->tile_base;
   B.queue = h->queue;
+  B.sms = h->sms;
   B.recheck_list = h->recheck_list;
   B.recheck_jlast = h->recheck_jlast;
   B.recheck_count = h->recheck_count;
@@ -1308,6 +1388,7 @@ int rrg_batch_closed_loop_dev(rrg_batch_handle h, const double* d_x0, const doub
     if (!h->side) BCK(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
     if (!h->ev_fork) BCK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
     if (!h->ev_join) BCK(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
+    BCK(upload_maps(h, h->d32b, 1));
     h->B.d32b = h->d32b;
     h->cl_next_ready = false;
     if (h->cl_exec) {
@@ -1565,6 +1646,7 @@ int rrg_batch_get_stats(rrg_batch_handle h, rrg_stats* out) {
   out->timed_rollouts = h->timed_rollouts;
   out->repairs = 0;
   out->graph_conditional = 0;
+  out->wait_timeouts = d.wait_timeouts;
   return RRG_OK;
 }
 

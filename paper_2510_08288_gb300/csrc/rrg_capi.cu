@@ -850,7 +850,7 @@ int rrg_create(const double* model_params, int n_params, const rrg_config* cfg, 
   (void)pair_blocks_per_sm(false);
   (void)pair_blocks_per_sm(true);
   if (!c.scenarios_in_register && tma_ring_prepare() &&
-      encode_scenario_map(&h->tmap[0], h->d32, c.n_scenarios, c.horizon)) {
+      encode_scenario_map(&h->tmap[0], h->d32, c.n_scenarios, c.horizon, c.n_scenarios)) {
     h->tmap[1] = h->tmap[0];
     h->tma_ok = true;
     h->tma_pair_bps = tma_pair_blocks_per_sm(c.param_unc_rel > 0.0);
@@ -1277,7 +1277,8 @@ int rrg_closed_loop_dev(rrg_handle h, const double* x0, double v0, const double*
       cudaGraphExecDestroy(h->st_exec);
       h->st_exec = nullptr;
     }
-    if (h->tma_ok && !encode_scenario_map(&h->tmap[1], h->d32b, h->cfg.n_scenarios, h->cfg.horizon)) {
+    if (h->tma_ok && !encode_scenario_map(&h->tmap[1], h->d32b, h->cfg.n_scenarios, h->cfg.horizon,
+                                          h->cfg.n_scenarios)) {
       h->tma_ok = false;  // the rings fall back to per-lane asynchronous copies
       h->L.tmap = nullptr;
     }

@@ -491,12 +491,12 @@ cudaError_t launch_eval_prepare(const Launch& L, const double* d_x, double v_pre
                                 const double* d_kappas, int m, const double* d_vp = nullptr,
                                 const double* d_r = nullptr);
 cudaError_t launch_eval_finish(const Launch& L, int m, uint8_t* d_adm, double* d_min_slack);
-// Tensor map of a binary32 scenario array [3][H][N] for the TMA ring (boxes
-// of 32 scenarios x one chunk of steps x 3 components); false when N is not a
-// multiple of 4 (row strides must be multiples of 16 bytes) or the driver
-// refuses.  tma_ring_prepare() sets the TMA kernels' shared-memory limit on
+// Tensor map of a binary32 scenario array [3][H][ld] of N <= ld scenarios for
+// the TMA ring (boxes of 32 scenarios x one chunk of steps x 3 components);
+// false when ld is not a multiple of 4 (row strides must be multiples of 16
+// bytes) or the driver refuses.  tma_ring_prepare() sets the TMA kernels' shared-memory limit on
 // the current device (once per device); false if the runtime refuses.
-bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H);
+bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H, int ld);
 bool tma_ring_prepare();
 // Resident blocks per SM of the two-candidates-per-thread TMA kernel (after
 // tma_ring_prepare on the current device; 0 if the runtime does not answer).

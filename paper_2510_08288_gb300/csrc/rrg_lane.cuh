@@ -661,6 +661,11 @@ __device__ __forceinline__ void fence_mbar_init() {
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
+// Makes a tensor map in global memory, written before the launch, visible to
+// this thread's tensor copies.
+__device__ __forceinline__ void fence_tensormap(const void* tmap) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -1043,18 +1048,18 @@ template <> __device__ __forceinline__ double draw<double>(uint64_t w, double a)
   return uniform_sym(w, a);
 }
 
-// The binary32 copy of a tile of steps j0 .. j1 - 1 of an [3][H][N] array, the
+// The binary32 copy of a tile of steps j0 .. j1 - 1 of an [3][H][ld] array, the
 // thread's scenarios k0 + i blockDim.x, i < KT.
 template <int KT>
-__device__ __forceinline__ void sample_tile32(float* __restrict__ d, int N, int H, int k0, int j0, int j1,
-                                              uint64_t kbase, uint64_t upd, uint64_t seed, float s0,
+__device__ __forceinline__ void sample_tile32(float* __restrict__ d, int N, int ld, int H, int k0, int j0,
+                                              int j1, uint64_t kbase, uint64_t upd, uint64_t seed, float s0,
                                               float s1, float s2) {
-  const size_t HN = static_cast<size_t>(H) * N;
+  const size_t HN = static_cast<size_t>(H) * ld;
   philox_tile<KT>(kbase + static_cast<uint64_t>(k0), blockDim.x, j0, j1, upd, seed,
                   [&](int i, int j, uint64_t w0, uint64_t w1, uint64_t w2) {
                     const size_t k = static_cast<size_t>(k0) + static_cast<size_t>(i) * blockDim.x;
                     if (k < static_cast<size_t>(N)) {
-                      const size_t q = static_cast<size_t>(j) * N + k;
+                      const size_t q = static_cast<size_t>(j) * ld + k;
                       d[q] = uniform_sym32(w0, s0);
                       d[HN + q] = uniform_sym32(w1, s1);
                       d[2 * HN + q] = uniform_sym32(w2, s2);
