@@ -406,15 +406,15 @@ RRG_API int rrg_get_pairing(rrg_handle h, int32_t *mode);
 /* How the binary32 rollouts on the stored scenario array bring in their
  * disturbances.  The TMA ring: one tensor copy per warp of a 32-scenario x
  * 16-step x 3-component box into shared memory, completion on an mbarrier, so
- * a step reads its values with three shared loads.  Otherwise: per-lane
- * 4-byte asynchronous copies into a shared-memory ring (launches of at most
- * 16 warps per SM, 64 under parametric uncertainty) or register prefetch
- * (larger launches, optionally two candidates per thread, rrg_set_pairing).
+ * four steps read their values with three shared loads.  Otherwise: per-lane
+ * 16-byte asynchronous copies (four steps of a component each) into a
+ * shared-memory ring, or, for launches that pair (rrg_set_pairing), register
+ * prefetch.
  * RRG_TMA_NEVER: never the TMA; RRG_TMA_AUTO (the default where available):
  * the TMA for launches of at least 24 warps per SM, where warps compete for
  * issue and the saved load instructions pay, ahead of pairing (which it beat
  * where both apply); below, where a warp running alone would pay the
- * chunk's wait and warp votes on its dependency chain, the per-lane forms;
+ * chunk's wait and warp votes on its dependency chain, the per-lane ring;
  * RRG_TMA_ALWAYS: the TMA for every such launch.  The results are identical;
  * only the time changes.  The TMA needs stored binary32 scenarios with
  * n_scenarios a multiple of 4 (the tensor map's row stride must be a multiple
@@ -455,7 +455,9 @@ RRG_API int rrg_autotune_pairing(rrg_handle h, const double *x_t, double r_t, do
  * the steady-state check).  The derivative is taken at the argmin (k*, j*)
  * (first k, then first j, attaining the min; a subgradient where the argmin
  * is not unique) by the discrete adjoint of the RK4 recursion: the forward
- * pass saves every trajectory's state every `checkpoint` steps, the reverse
+ * pass saves every trajectory's state every `checkpoint` steps (rounded up to a
+ * multiple of 16 where binary32 lanes read the stored binary32 array), the
+ * reverse
  * pass recomputes trajectory k*'s segments before j* in parallel and then
  * sweeps them backwards; the handle keeps N * (H / checkpoint + 1) * 3 and
  * (H + 1) * 12 doubles of device scratch for them, allocated on first use.
@@ -673,7 +675,7 @@ typedef struct rrg_batch_ctx *rrg_batch_handle;
 /* cfg as for rrg_create (n_scenarios and horizon are ignored); n_scenarios
  * and horizons: host arrays of n_instances values >= 1; sum over instances of
  * max_candidates * N_s must be below 2^31.  Allocates 12 sum(H_s N_s) bytes of
- * scenarios (N_s rounded up to a multiple of 4) plus O(sum M N_s) bytes of recheck list. */
+ * scenarios (H_s rounded up to a multiple of 4) plus O(sum M N_s) bytes of recheck list. */
 RRG_API int rrg_batch_create(const double *model_params, int n_params, const rrg_config *cfg,
                      int n_instances, const int32_t *n_scenarios, const int32_t *horizons,
                      void *cuda_stream, rrg_batch_handle *out);

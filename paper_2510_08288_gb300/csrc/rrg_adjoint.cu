@@ -208,6 +208,11 @@ template <typename T> __device__ __forceinline__ RhsC<T> launch_c(const Launch& 
 template <> __device__ __forceinline__ RhsC<float> launch_c<float>(const Launch& L, int i) { return L.cand_c32[i]; }
 template <> __device__ __forceinline__ RhsC<double> launch_c<double>(const Launch& L, int i) { return L.cand_c64[i]; }
 
+// The binary32 forward pass on the stored binary32 array saves states between
+// blocks of kAdjBlock steps only: the caller's spacing rounded up.
+constexpr int kAdjBlock = 16;
+constexpr int adj_spacing(int checkpoint) { return (checkpoint + kAdjBlock - 1) / kAdjBlock * kAdjBlock; }
+
 // Forward: one thread per (candidate slot i = blockIdx.y, scenario k), full
 // horizon, with the rollouts' arithmetic (deviation coordinates about the
 // candidate's reference point, the multiplied-out right-hand side, the
@@ -250,52 +255,55 @@ adjoint_forward_kernel(const Launch L, const DT* __restrict__ d, int checkpoint,
   int arg = 0;
   int next_ck = 0;  // the next step whose state is saved
   if constexpr (sizeof(T) == 4 && sizeof(DT) == 4) {
-    // binary32 from the stored binary32 array: the rollouts' shared-memory
-    // ring, one asynchronous copy per lane, component and step, RRG_RING_DEPTH
-    // steps ahead (a warp running its chain alone issues its steps in order,
-    // and the register ring's loads and index arithmetic sit between them)
-    constexpr int D = RRG_RING_DEPTH;
-    __shared__ float sring[D * 3 * 128];
-    const int bd = blockDim.x;
-    float* my = sring + threadIdx.x;
-    const DT* pf = d + k;  // the next step to fetch
-#pragma unroll 1
-    for (int u = 0; u < D; ++u) {
-      if (u < H) {
-        cp_async4(my + (3 * u) * bd, pf);
-        cp_async4(my + (3 * u + 1) * bd, pf + HN);
-        cp_async4(my + (3 * u + 2) * bd, pf + 2 * HN);
-      }
-      cp_async_commit();
-      pf += N;
+    // binary32 from the stored binary32 array: the rollouts' ring of quads in
+    // shared memory, in blocks without a branch (a warp runs its chain alone on
+    // its scheduler; the state is saved between blocks, whose length the
+    // spacing is a multiple of), then the last steps past a whole block
+    __shared__ __align__(16) unsigned char qring[qring_bytes(128)];
+    constexpr int B = kAdjBlock;
+    static_assert(B == 4 * kQringBlock, "saved states lie between blocks");
+    int j = 0;
+    auto save = [&]() {
+      if (j != next_ck) return;
+      double* c = ck + (j / checkpoint) * 3;
+      c[0] = static_cast<double>(z_ca) + r_ca;
+      c[1] = static_cast<double>(z_w) + r_w;
+      c[2] = static_cast<double>(z_sm) + r_sm;
+      next_ck += checkpoint;
+    };
+    if (B <= H) {
+      Qring<128> ring(qring, d, k, N, H, 0, H);
+      do {
+        save();
+        int at = 0;  // step of the block that lowered the minimum last
+        auto step = [&](int u, float e0, float e1, float e2) {
+          rk4_step_fast<T>(K, M.pw, C, z_ca, z_w, z_sm, w_abs, e0, e1, e2);
+          const T s = slack_of<T>(C, z_ca, z_sm);
+          at = s < smin ? u : at;
+          smin = s < smin ? s : smin;
+        };
+#pragma unroll
+        for (int q = 0; q < kQringBlock; ++q) {
+          float4 a, b, c;
+          ring.next(a, b, c, [&](float e0, float e1, float e2) { step(4 * q + 1, e0, e1, e2); });
+          step(4 * q + 2, a.y, b.y, c.y);
+          step(4 * q + 3, a.z, b.z, c.z);
+          step(4 * q + 4, a.w, b.w, c.w);
+        }
+        if (at) arg = j + at;
+        j += B;
+      } while (j + B <= H);
+      ring.drain();
     }
-    int slot = 0;
-#pragma unroll 4
-    for (int j = 0; j < H; ++j) {
-      cp_async_wait<D - 1>();
-      float* e = my + (3 * slot) * bd;
-      const float e0 = e[0], e1 = e[bd], e2 = e[2 * bd];
-      if (j == next_ck) {
-        double* c = ck + (j / checkpoint) * 3;
-        c[0] = static_cast<double>(z_ca) + r_ca;
-        c[1] = static_cast<double>(z_w) + r_w;
-        c[2] = static_cast<double>(z_sm) + r_sm;
-        next_ck += checkpoint;
-      }
-      rk4_step_fast<T>(K, M.pw, C, z_ca, z_w, z_sm, w_abs, e0, e1, e2);
-      // the slot is free once its values are in registers: step j + D
-      if (j + D < H) {
-        cp_async4(e, pf);
-        cp_async4(e + bd, pf + HN);
-        cp_async4(e + 2 * bd, pf + 2 * HN);
-      }
-      cp_async_commit();
-      pf += N;
-      slot = (slot + 1) & (D - 1);
+    if (j < H) save();
+    const size_t comp = quad_rows(H) * 4 * static_cast<size_t>(N);
+    while (j < H) {
+      const size_t o = quad_index(0, j, k, H, N);
+      rk4_step_fast<T>(K, M.pw, C, z_ca, z_w, z_sm, w_abs, __ldg(d + o), __ldg(d + comp + o), __ldg(d + 2 * comp + o));
+      ++j;
       const T s = slack_of<T>(C, z_ca, z_sm);
-      if (s < smin) { smin = s; arg = j + 1; }
+      if (s < smin) { smin = s; arg = j; }
     }
-    cp_async_wait<0>();  // nothing in flight into the ring when the lane ends
     lane_min[static_cast<size_t>(i) * N + k] = static_cast<double>(smin);
     lane_arg[static_cast<size_t>(i) * N + k] = arg;
     return;
@@ -445,11 +453,15 @@ adjoint_reverse_kernel(const Launch L, const DT* __restrict__ d,
       T* sj = seg + static_cast<size_t>(j) * kSegVals;
       sj[0] = a; sj[1] = b; sj[2] = e;
       rk4_stage_points<T>(K, C, dt, a, b, e, sj + 3);
-      const size_t o = static_cast<size_t>(j) * N + k;
+      size_t o = static_cast<size_t>(j) * N + k, cs = HN;
+      if constexpr (sizeof(DT) == 4) {  // the handle's binary32 array
+        o = quad_index(0, j, k, H, N);
+        cs = 4 * quad_rows(H) * static_cast<size_t>(N);
+      }
       rk4_step<T>(K, C, dt, a, b, e);
       a += static_cast<T>(d[o]);
-      b += static_cast<T>(d[HN + o]);
-      e += static_cast<T>(d[2 * HN + o]);
+      b += static_cast<T>(d[cs + o]);
+      e += static_cast<T>(d[2 * cs + o]);
     }
     if (j1 == jstar) {
       T* sj = seg + static_cast<size_t>(jstar) * kSegVals;
@@ -581,7 +593,7 @@ cudaError_t launch_adjoint_forward(const Launch& L, bool fp64, int m, int checkp
     adjoint_forward_kernel<double, double><<<grid, threads, 0, L.stream>>>(L, L.d64, checkpoint, ckpt,
                                                                            lane_min, lane_arg);
   else if (reads32(L, fp64))
-    adjoint_forward_kernel<float, float><<<grid, threads, 0, L.stream>>>(L, L.d32, checkpoint, ckpt,
+    adjoint_forward_kernel<float, float><<<grid, threads, 0, L.stream>>>(L, L.d32, adj_spacing(checkpoint), ckpt,
                                                                          lane_min, lane_arg);
   else
     adjoint_forward_kernel<float, double><<<grid, threads, 0, L.stream>>>(L, L.d64, checkpoint, ckpt,
@@ -605,7 +617,7 @@ cudaError_t launch_adjoint_reverse(const Launch& L, bool fp64, int slot0, int co
         L, L.d64, checkpoint, ckpt, static_cast<double*>(seg), d_out, slot0, lane_min, lane_arg);
   else if (reads32(L, fp64))
     adjoint_reverse_kernel<float, float><<<count, kRevThreads, 0, L.stream>>>(
-        L, L.d32, checkpoint, ckpt, static_cast<float*>(seg), d_out, slot0, lane_min, lane_arg);
+        L, L.d32, adj_spacing(checkpoint), ckpt, static_cast<float*>(seg), d_out, slot0, lane_min, lane_arg);
   else
     adjoint_reverse_kernel<float, double><<<count, kRevThreads, 0, L.stream>>>(
         L, L.d64, checkpoint, ckpt, static_cast<float*>(seg), d_out, slot0, lane_min, lane_arg);

@@ -43,8 +43,7 @@ static_assert(kMaxInst <= kDecideThreads, "one decision thread per instance");
 
 struct BInst {
   int32_t N, H;
-  int32_t ld, pad;  // row length of its scenario array: N rounded up to 4 (TMA strides)
-  long long off;    // element offset of the instance's [3][H][ld] binary32 scenarios
+  long long off;  // element offset of the instance's binary32 scenarios (quad layout)
 };
 
 struct BState {
@@ -106,11 +105,14 @@ struct BLaunch {
 // Sampling: instance s draws with key (seed + s, 0) and the counters of the
 // single-problem sampler; only the binary32 copy is stored (the recheck
 // regenerates binary64 values from the same counters).
-// One warp per block: block t draws kSampleSteps steps x 64 scenarios (two per
-// thread) of the instance that holds tile t, so instances of all sizes share
-// the SMs evenly (samp_base: tiles before each instance).
-constexpr int kSampleSteps = 32;
-constexpr int sample_tiles_of(int N, int H) { return ((N + 63) / 64) * ((H + kSampleSteps - 1) / kSampleSteps); }
+// One warp per block: block t draws kSampleQuads quads of steps x 32 scenarios
+// of the instance that holds tile t, so instances of all sizes share the SMs
+// evenly (samp_base: tiles before each instance).
+constexpr int kSampleQuads = 16;
+inline long long sample_tiles_of(int N, int H) {
+  return static_cast<long long>((static_cast<long long>(N) + 31) / 32) *
+         static_cast<long long>((quad_rows(H) + kSampleQuads - 1) / kSampleQuads);
+}
 
 __global__ void __launch_bounds__(32)
 batch_sample_kernel(const BLaunch B, uint64_t seed, uint64_t base) {
@@ -130,12 +132,13 @@ batch_sample_kernel(const BLaunch B, uint64_t seed, uint64_t base) {
     B.st[s].seed_p[pair] = key;
     B.st[s].update_p[pair] = upd;
   }
-  const int nk = (I.N + 63) / 64;
+  const int nk = (I.N + 31) / 32;
   const int jt = local / nk, kt = local - jt * nk;
-  const int j0 = jt * kSampleSteps;
-  sample_tile32<2>((pair ? B.d32b : B.d32) + I.off, I.N, I.ld, I.H, kt * 64 + static_cast<int>(threadIdx.x), j0,
-                   min(j0 + kSampleSteps, I.H), 0ull, upd, key, static_cast<float>(B.c.amp[0] * 0x1.0p-23),
-                   static_cast<float>(B.c.amp[1] * 0x1.0p-23), static_cast<float>(B.c.amp[2] * 0x1.0p-23));
+  const int q0 = jt * kSampleQuads;
+  sample_quads((pair ? B.d32b : B.d32) + I.off, I.N, I.H, kt * 32 + static_cast<int>(threadIdx.x), q0,
+               min(q0 + kSampleQuads, static_cast<int>(quad_rows(I.H))), 0ull, upd, key,
+               static_cast<float>(B.c.amp[0] * 0x1.0p-23), static_cast<float>(B.c.amp[1] * 0x1.0p-23),
+               static_cast<float>(B.c.amp[2] * 0x1.0p-23));
 }
 
 // CTAs that take tiles in a round of `tiles` tiles: 8 resident warps per SM
@@ -369,22 +372,28 @@ __device__ __forceinline__ void batch_reduce(const BLaunch& B, size_t slot, int 
   }
 }
 
-// Where a tile's lanes take their disturbances from: PF steps ahead in
-// registers (run_lane), or (PF = 16) each warp's ring of 16-step chunks filled
-// by tensor copies (run_lane_tma), which issues 91 instead of about 100
-// instructions a step and leaves the coefficients as constant-bank operands.
-// Measured on 64 instances (rollouts of an update), ring against registers at
-// the same tile: 64 lanes 11.3 -> 10.2 ms, 128 (the default)
-// 11.3 -> 10.5, 256 11.6 -> 10.9, warp tiles 11.1 -> 10.0.
-template <int PF> constexpr bool kTileRing = PF == kTmaChunk;
-// Dynamic shared memory of a block of `warps` warps with rings.
-constexpr size_t ring_bytes(int warps) { return static_cast<size_t>(warps) * (2 * kTmaStageBytes + 2 * sizeof(uint64_t)); }
+// Where a tile's lanes take their disturbances from: FEED_REGS two quads ahead
+// in registers (run_lane_q); FEED_QRING each lane's ring of quads in shared
+// memory (run_lane_qring); FEED_TMA each warp's ring of 16-step chunks filled
+// by tensor copies (run_lane_tma).  Variants of prefetch depth 16 run the TMA
+// form when a round of every candidate has at least kTmaTileWarps warps of
+// tiles per SM, else the ring of quads, which steps a warp alone on its
+// scheduler faster (177 against 198 cycles) and needs no barriers per tile,
+// while the TMA form issues fewer instructions a step (single problems: 112
+// against 116 cycles a step and scheduler).
+enum TileFeed : int { FEED_REGS = 0, FEED_QRING = 1, FEED_TMA = 2 };
+constexpr int kTmaTileWarps = 300;
+// Dynamic shared memory of a block of `threads` lanes.
+constexpr size_t feed_bytes(int feed, int threads) {
+  return feed == FEED_TMA ? static_cast<size_t>(threads / 32) * (2 * kTmaStageBytes + 2 * sizeof(uint64_t))
+                          : feed == FEED_QRING ? qring_bytes(threads) : 0;
+}
 extern __shared__ __align__(128) unsigned char batch_dyn_smem[];
 
 // One tile: lanes k of candidate slot (s, i), binary32 rollouts classified
 // for the binary64 recheck, reduced into the candidate's flags.  Called by
 // every thread of the CTA; returns are warp- or CTA-uniform.
-template <int PF>
+template <int FEED, int THREADS>
 __device__ __forceinline__ void batch_tile(const BLaunch& B, int s, int i, int k) {
   const BInst I = B.inst[s];
   const size_t slot = static_cast<size_t>(s) * B.c.M + i;
@@ -408,22 +417,26 @@ __device__ __forceinline__ void batch_tile(const BLaunch& B, int s, int i, int k
   float q_ca = 0.0f, w = 0.0f, q_sm = 0.0f, w_abs = 0.0f;  // the deviation from the candidate's reference point
   if (active) start_state<float>(R, st.x, B.params[P_P_ATM], q_ca, w, q_sm, w_abs);
   int end = LANE_REACHED_END;
-  if constexpr (kTileRing<PF>) {
+  if constexpr (FEED == FEED_TMA) {
     if ((k & ~31) >= I.N) return;  // a warp past the scenarios (the copies serve whole warps)
     const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     float* stages = reinterpret_cast<float*>(batch_dyn_smem) + static_cast<size_t>(wid) * 2 * kTmaStageFloats;
     uint64_t* bars = reinterpret_cast<uint64_t*>(batch_dyn_smem + static_cast<size_t>(nw) * 2 * kTmaStageBytes) + 2 * wid;
     const CUtensorMap* tm = B.maps + (st.cur ? B.c.S : 0) + s;
     if ((threadIdx.x & 31) == 0) fence_tensormap(tm);
-    const float s_out = run_lane_tma<false>(U, C, tm, k & ~31, active, 0, I.H, q_ca, w, q_sm, w_abs,
+    const float s_out = run_lane_tma<false>(U, C, tm, nullptr, k, I.N, I.H, active, 0, I.H, q_ca, w, q_sm, w_abs,
                                             inf_v<float>(), thr, cand_stop ? dead : nullptr,
                                             cand_stop ? dead : nullptr, &steps, &end, eps, &jlast, stages, bars,
                                             &B.stats->wait_timeouts);
     if (active) smin = s_out;
   } else if (active) {
     const float* d = (st.cur ? B.d32b : B.d32) + I.off;
-    smin = run_lane<float, PF>(U, nullptr, C, d, k, I.ld, I.H, 0, I.H, q_ca, w, q_sm, w_abs, inf_v<float>(), thr,
-                               cand_stop ? dead : nullptr, &steps, &end, eps, &jlast);
+    if constexpr (FEED == FEED_QRING)
+      smin = run_lane_qring<THREADS>(U, C, d, k, I.N, I.H, 0, I.H, q_ca, w, q_sm, w_abs, inf_v<float>(), thr,
+                                     cand_stop ? dead : nullptr, &steps, &end, eps, &jlast, batch_dyn_smem);
+    else
+      smin = run_lane_q(U, C, d, k, I.N, I.H, 0, I.H, q_ca, w, q_sm, w_abs, inf_v<float>(), thr,
+                        cand_stop ? dead : nullptr, &steps, &end, eps, &jlast);
   }
   if (active && cand_stop && smin < thr) *dead = 1;
   batch_reduce(B, slot, k, active, smin, steps, jlast, eps, dead);
@@ -435,7 +448,7 @@ __device__ __forceinline__ void batch_tile(const BLaunch& B, int s, int i, int k
 // coefficients re-read) 11.9, unbounded (up to 187 registers) 14.6.
 constexpr int kBatchThreadsPerSm = 384;
 // Persistent rollout: each CTA takes tiles from the queue until none is left.
-template <int TILE, int PF>
+template <int TILE, int FEED>
 __global__ void __launch_bounds__(TILE, kBatchThreadsPerSm / TILE) batch_rollout_kernel(const BLaunch B) {
   __shared__ int sh[3];
   if (blockIdx.x >= B.queue[2]) return;
@@ -466,7 +479,7 @@ __global__ void __launch_bounds__(TILE, kBatchThreadsPerSm / TILE) batch_rollout
     const int s = sh[0], i = sh[1], b = sh[2];
     __syncthreads();
     if (s < 0) return;
-    batch_tile<PF>(B, s, i, b * TILE + static_cast<int>(threadIdx.x));
+    batch_tile<FEED, TILE>(B, s, i, b * TILE + static_cast<int>(threadIdx.x));
   }
 }
 
@@ -487,7 +500,7 @@ __device__ __forceinline__ void tile_of(const BLaunch& B, uint32_t t, int tile, 
   *b = local - *i * nb;
 }
 
-template <int PF>
+template <int FEED>
 __global__ void __launch_bounds__(128, kBatchThreadsPerSm / 128) batch_rollout_warp_kernel(const BLaunch B) {
   if (blockIdx.x >= B.queue[2]) return;
   const uint32_t total = B.queue[1];
@@ -502,7 +515,7 @@ __global__ void __launch_bounds__(128, kBatchThreadsPerSm / 128) batch_rollout_w
     s = __shfl_sync(0xffffffffu, s, 0);
     i = __shfl_sync(0xffffffffu, i, 0);
     b = __shfl_sync(0xffffffffu, b, 0);
-    batch_tile<PF>(B, s, i, b * 32 + lane);
+    batch_tile<FEED, 128>(B, s, i, b * 32 + lane);
   }
 }
 
@@ -548,14 +561,14 @@ __device__ __forceinline__ void batch_tile_pair(const BLaunch& B, int s, int p, 
     start_state<float>(RB, bs.x, p_atm, zb[0], zb[1], zb[2], zb[3]);
     const float* d = (bs.cur ? B.d32b : B.d32) + I.off;
     if (runA && runB) {
-      run_lane_pair<float, PF>(K, CA, CB, d, k, I.ld, I.H, I.H, za, zb, thr, eps,
+      run_lane_pair(K, CA, CB, d, k, I.N, I.H, I.H, za, zb, thr, eps,
                                cand_stop ? deadA : nullptr, cand_stop ? deadB : nullptr, sm, st, en, jl);
     } else if (runA) {
-      sm[0] = run_lane<float, PF>(K, nullptr, CA, d, k, I.ld, I.H, 0, I.H, za[0], za[1], za[2], za[3],
+      sm[0] = run_lane_q<PF / 4>(K, CA, d, k, I.N, I.H, 0, I.H, za[0], za[1], za[2], za[3],
                                   inf_v<float>(), thr, cand_stop ? deadA : nullptr, &st[0], &en[0], eps,
                                   &jl[0]);
     } else {
-      sm[1] = run_lane<float, PF>(K, nullptr, CB, d, k, I.ld, I.H, 0, I.H, zb[0], zb[1], zb[2], zb[3],
+      sm[1] = run_lane_q<PF / 4>(K, CB, d, k, I.N, I.H, 0, I.H, zb[0], zb[1], zb[2], zb[3],
                                   inf_v<float>(), thr, cand_stop ? deadB : nullptr, &st[1], &en[1], eps,
                                   &jl[1]);
     }
@@ -626,36 +639,38 @@ __device__ __forceinline__ float run_lane_split(const StepU<float>& K, const Ste
     if (s0 < band) jl = 0;
     if (s0 < thr) run = false;
   }
-  const size_t HN = static_cast<size_t>(H) * N;
-  const float* pf = d + (on ? k : 0);  // in bounds for every lane
-  float r0[PF], r1[PF], r2[PF];
+  constexpr int Q = PF / 4;
+  const int kk = on ? k : 0;  // in bounds for every lane
+  const size_t comp = quad_rows(H) * static_cast<size_t>(N);
+  const float4* p = reinterpret_cast<const float4*>(d) + kk;
+  float4 r[Q][3];
 #pragma unroll
-  for (int u = 0; u < PF; ++u) {
-    if (u < H) {
-      r0[u] = __ldg(pf);
-      r1[u] = __ldg(pf + HN);
-      r2[u] = __ldg(pf + 2 * HN);
-    } else {
-      r0[u] = r1[u] = r2[u] = 0.0f;
+  for (int q = 0; q < Q; ++q) {
+    if (PF <= H) {
+      r[q][0] = __ldg(p); r[q][1] = __ldg(p + comp); r[q][2] = __ldg(p + 2 * comp);
     }
-    pf += N;
+    p += N;
   }
   while (j + PF <= H && __any_sync(0xffffffffu, run)) {
     const int dead_now = (run && dead != nullptr) ? *dead : 0;
+    const bool more = j + 2 * PF <= H;
     BlockMin<float> bm;
 #pragma unroll
-    for (int u = 0; u < PF; ++u) {
-      const float e0 = r0[u], e1 = r1[u], e2 = r2[u];
-      if (j + PF < H) {
-        r0[u] = __ldg(pf);
-        r1[u] = __ldg(pf + HN);
-        r2[u] = __ldg(pf + 2 * HN);
+    for (int q = 0; q < Q; ++q) {
+      const float e0[4] = {r[q][0].x, r[q][0].y, r[q][0].z, r[q][0].w},
+                  e1[4] = {r[q][1].x, r[q][1].y, r[q][1].z, r[q][1].w},
+                  e2[4] = {r[q][2].x, r[q][2].y, r[q][2].z, r[q][2].w};
+      if (more) {
+        r[q][0] = __ldg(p); r[q][1] = __ldg(p + comp); r[q][2] = __ldg(p + 2 * comp);
       }
-      pf += N;
-      rk4_step_with(K, C, q_ca, w, q_sm, w_abs, e0, e1, e2, tq);
-      ++j;
-      bm.add(slack_of<float>(C, q_ca, q_sm), u);
+      p += N;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        rk4_step_with(K, C, q_ca, w, q_sm, w_abs, e0[u], e1[u], e2[u], tq);
+        bm.add(slack_of<float>(C, q_ca, q_sm), u);
+      }
     }
+    j += PF;
     if (run) {
       const float bmin = bm.result(q_ca, w, q_sm);
       smin = fmin(smin, bmin);
@@ -664,10 +679,9 @@ __device__ __forceinline__ float run_lane_split(const StepU<float>& K, const Ste
       if (smin < thr || (dead_now != 0 && j < H)) run = false;
     }
   }
-  const float* dp = d + static_cast<size_t>(j) * N + (on ? k : 0);
   while (j < H && __any_sync(0xffffffffu, run)) {
-    const float e0 = __ldg(dp), e1 = __ldg(dp + HN), e2 = __ldg(dp + 2 * HN);
-    dp += N;
+    const float* dp = d + quad_index(0, j, kk, H, N);
+    const float e0 = __ldg(dp), e1 = __ldg(dp + 4 * comp), e2 = __ldg(dp + 8 * comp);
     rk4_step_with(K, C, q_ca, w, q_sm, w_abs, e0, e1, e2, tq);
     ++j;
     if (run) {
@@ -710,7 +724,7 @@ __device__ __forceinline__ void batch_tile_split(const BLaunch& B, int s, int i,
   const float* d = (st.cur ? B.d32b : B.d32) + I.off;
   unsigned steps = 0;
   int jlast = -1;
-  const float smin = run_lane_split<PF>(B.m32.U, C, d, k, on, I.ld, I.H, role, q_ca, w, q_sm, w_abs, thr, cand_stop ? dead : nullptr, &steps,
+  const float smin = run_lane_split<PF>(B.m32.U, C, d, k, on, I.N, I.H, role, q_ca, w, q_sm, w_abs, thr, cand_stop ? dead : nullptr, &steps,
                                         eps, &jlast);
   const bool mine = on && role == 0;
   if (cand_stop && mine && smin < thr) *dead = 1;
@@ -890,23 +904,25 @@ __global__ void batch_loop_init_kernel(const BLaunch B, const double* __restrict
 // candidate slots per tile.
 struct Variant {
   int tile, pf, rows;
-  void (*kernel)(const BLaunch);
+  int feed[2];  // of rounds with few tiles, with many (kTmaTileWarps)
+  void (*kernel[2])(const BLaunch);
 };
 // tile = 32: warp tiles (CTAs of 4 warps, no CTA barrier); rows = 2: two
 // candidates per thread; tile = 16: warp tiles of 16 scenarios, two lanes
 // per trajectory
+#define RRG_TILE8(T) {T, 8, 1, {FEED_REGS, FEED_REGS}, {batch_rollout_kernel<T, FEED_REGS>, batch_rollout_kernel<T, FEED_REGS>}}
+#define RRG_TILE16(T) {T, 16, 1, {FEED_QRING, FEED_TMA}, {batch_rollout_kernel<T, FEED_QRING>, batch_rollout_kernel<T, FEED_TMA>}}
 const Variant kVariants[RRG_BATCH_VARIANTS] = {
-    {64, 8, 1, batch_rollout_kernel<64, 8>},   {64, 16, 1, batch_rollout_kernel<64, 16>},
-    {128, 8, 1, batch_rollout_kernel<128, 8>}, {128, 16, 1, batch_rollout_kernel<128, 16>},
-    {256, 8, 1, batch_rollout_kernel<256, 8>}, {256, 16, 1, batch_rollout_kernel<256, 16>},
-    {32, 8, 1, batch_rollout_warp_kernel<8>},  {32, 16, 1, batch_rollout_warp_kernel<16>},
-    {32, 8, 2, batch_rollout_warp_pair_kernel<8>}, {16, 8, 1, batch_rollout_split_kernel<8>},
+    RRG_TILE8(64), RRG_TILE16(64), RRG_TILE8(128), RRG_TILE16(128), RRG_TILE8(256), RRG_TILE16(256),
+    {32, 8, 1, {FEED_REGS, FEED_REGS}, {batch_rollout_warp_kernel<FEED_REGS>, batch_rollout_warp_kernel<FEED_REGS>}},
+    {32, 16, 1, {FEED_QRING, FEED_TMA}, {batch_rollout_warp_kernel<FEED_QRING>, batch_rollout_warp_kernel<FEED_TMA>}},
+    {32, 8, 2, {FEED_REGS, FEED_REGS}, {batch_rollout_warp_pair_kernel<8>, batch_rollout_warp_pair_kernel<8>}},
+    {16, 8, 1, {FEED_REGS, FEED_REGS}, {batch_rollout_split_kernel<8>, batch_rollout_split_kernel<8>}},
 };
+#undef RRG_TILE8
+#undef RRG_TILE16
 constexpr int block_threads(int tile) { return tile <= 32 ? 128 : tile; }
-// Dynamic shared memory of variant v: the rings of its warps.
-size_t variant_smem(const Variant& v) {
-  return v.pf == kTmaChunk ? ring_bytes(block_threads(v.tile) / 32) : 0;
-}
+size_t variant_smem(const Variant& v, int large) { return feed_bytes(v.feed[large], block_threads(v.tile)); }
 
 }  // namespace
 }  // namespace rrg
@@ -923,7 +939,8 @@ struct rrg_batch_ctx {
   std::vector<BInst> inst;
   int variant = 3;             // 128 lanes per tile, prefetch 16
   int sms = 0;                 // streaming multiprocessors of the device (queried)
-  int grid[RRG_BATCH_VARIANTS]{};
+  int grid[RRG_BATCH_VARIANTS][2]{};
+  unsigned long long scen_warps = 0;  // sum over instances of ceil(N_s / 32)
   size_t lanes = 0;            // sum of M N_s
   // device memory
   double* params_dev = nullptr;
@@ -1053,7 +1070,7 @@ cudaError_t upload_maps(rrg_batch_ctx* h, const float* d32, int pair) {
   std::vector<CUtensorMap> m(h->inst.size());
   for (size_t s = 0; s < m.size(); ++s) {
     const BInst& I = h->inst[s];
-    if (!encode_scenario_map(&m[s], d32 + I.off, I.N, I.H, I.ld)) return cudaErrorNotSupported;
+    if (!encode_scenario_map(&m[s], d32 + I.off, I.N, I.H)) return cudaErrorNotSupported;
   }
   return cudaMemcpy(h->maps_dev + static_cast<size_t>(pair) * m.size(), m.data(), m.size() * sizeof(CUtensorMap),
                     cudaMemcpyHostToDevice);
@@ -1083,7 +1100,9 @@ int enqueue_rollout(rrg_batch_ctx* h) {
     b = btake_event(h);
     if (a && b) BCK(cudaEventRecord(a, h->stream));
   }
-  v.kernel<<<h->grid[h->variant], block_threads(v.tile), variant_smem(v), h->stream>>>(h->B);
+  const unsigned long long cand = h->B.c.search == RRG_SEARCH_SPEC_BISECT ? h->B.c.width : h->B.c.M;
+  const int large = h->scen_warps * cand >= static_cast<unsigned long long>(kTmaTileWarps) * h->sms ? 1 : 0;
+  v.kernel[large]<<<h->grid[h->variant][large], block_threads(v.tile), variant_smem(v, large), h->stream>>>(h->B);
   BCK(cudaGetLastError());
   if (timed && a && b) {
     BCK(cudaEventRecord(b, h->stream));
@@ -1178,10 +1197,7 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
     inst[s].N = n_scenarios[s];
     inst[s].H = horizons[s];
     inst[s].off = static_cast<long long>(elems);
-    inst[s].ld = static_cast<int32_t>((static_cast<int64_t>(n_scenarios[s]) + 3) & ~int64_t(3));
-    inst[s].pad = 0;
-    const unsigned long long e = 3ull * static_cast<unsigned long long>(horizons[s]) *
-                                 static_cast<unsigned long long>(inst[s].ld);
+    const unsigned long long e = quad_elems(horizons[s], n_scenarios[s]);
     elems += (e + 31ull) & ~31ull;  // 128-byte aligned blocks
     lanes += static_cast<unsigned long long>(M) * static_cast<unsigned long long>(n_scenarios[s]);
   }
@@ -1200,6 +1216,7 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   h->cfg = *cfg;
   h->inst = inst;
   h->lanes = lanes;
+  for (const BInst& I : inst) h->scen_warps += (static_cast<unsigned long long>(I.N) + 31) / 32;
   std::memcpy(h->params, model_params, sizeof h->params);
   cudaError_t e = cudaGetDevice(&h->device);
   if (e == cudaSuccess) {
@@ -1279,13 +1296,16 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
                              cudaSharedmemCarveoutMaxShared);
   for (int v = 0; v < RRG_BATCH_VARIANTS && e == cudaSuccess; ++v) {
     int per = 0;
-    const size_t sm = variant_smem(kVariants[v]);
-    if (sm > 48 * 1024)
-      e = cudaFuncSetAttribute(kVariants[v].kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm));
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kVariants[v].kernel,
-                                                        block_threads(kVariants[v].tile), sm);
-    h->grid[v] = std::max(1, per) * nsm;
+    for (int g = 0; g < 2 && e == cudaSuccess; ++g) {
+      const size_t sm = variant_smem(kVariants[v], g);
+      if (sm > 40 * 1024)  // with the kernel's static part past the default limit
+        e = cudaFuncSetAttribute(kVariants[v].kernel[g], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(sm));
+      if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kVariants[v].kernel[g],
+                                                          block_threads(kVariants[v].tile), sm);
+      h->grid[v][g] = std::max(1, per) * nsm;
+    }
   }
   if (e != cudaSuccess) {
     const int code = (e == cudaErrorMemoryAllocation) ? RRG_ENOMEM : RRG_ECUDA;

@@ -304,6 +304,7 @@ void fill_launch(rrg_ctx* h) {
   fold_model(L.k64, h->params, c.dt, &L.m64);
   round_model(L.m64, &L.m32);
   L.d64 = h->d64;
+  L.quads = 1;
   L.d32 = h->d32;
   L.st = h->st;
   L.cand_kappa = h->cand_kappa;
@@ -780,7 +781,7 @@ int rrg_create(const double* model_params, int n_params, const rrg_config* cfg, 
   ALLOC(d64, HN3);
   // in-register scenarios need no binary32 array (the binary64 one stays for
   // rrg_get_scenarios and the adjoint)
-  const size_t n32 = c.scenarios_in_register ? 1 : HN3;
+  const size_t n32 = c.scenarios_in_register ? 1 : quad_elems(c.horizon, c.n_scenarios);
   ALLOC(d32, n32);
   ALLOC(st, 1);
   // two slot ranges: a pipelined round and the round after it run together
@@ -823,8 +824,8 @@ int rrg_create(const double* model_params, int n_params, const rrg_config* cfg, 
   h->pws_ok = pow_table((h->params[P_GAMMA] - 1.0) / h->params[P_GAMMA], &ps);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->pws, &ps, sizeof ps, cudaMemcpyHostToDevice, h->stream);
   fill_launch(h);
-  // the zero scenarios are explicit values (marks pair 0's binary64 array valid)
-  if (e == cudaSuccess) e = launch_round_scenarios(h->L);
+  // the zero scenarios are explicit values
+  if (e == cudaSuccess) e = launch_mark64(h->L);
   if (e == cudaSuccess && h->pmul) e = launch_fill(h->L, h->pmul, N * RRG_NPARAM, 1.0);
   if (e == cudaSuccess) e = launch_scenario_fold(h->L, false);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -849,8 +850,8 @@ int rrg_create(const double* model_params, int n_params, const rrg_config* cfg, 
   // set once here (never inside a capture)
   (void)pair_blocks_per_sm(false);
   (void)pair_blocks_per_sm(true);
-  if (!c.scenarios_in_register && tma_ring_prepare() &&
-      encode_scenario_map(&h->tmap[0], h->d32, c.n_scenarios, c.horizon, c.n_scenarios)) {
+  if (!c.scenarios_in_register && c.n_scenarios % 4 == 0 && tma_ring_prepare() &&
+      encode_scenario_map(&h->tmap[0], h->d32, c.n_scenarios, c.horizon)) {
     h->tmap[1] = h->tmap[0];
     h->tma_ok = true;
     h->tma_pair_bps = tma_pair_blocks_per_sm(c.param_unc_rel > 0.0);
@@ -1257,7 +1258,8 @@ int rrg_closed_loop_dev(rrg_handle h, const double* x0, double v0, const double*
   if (!h->L.d64b) {
     const size_t n = 3 * static_cast<size_t>(h->cfg.horizon) * h->cfg.n_scenarios;
     if (!h->d64b) CK(cudaMalloc(reinterpret_cast<void**>(&h->d64b), n * sizeof(double)));
-    const size_t n32 = h->cfg.scenarios_in_register ? 1 : n;
+    const size_t n32 =
+        h->cfg.scenarios_in_register ? 1 : quad_elems(h->cfg.horizon, h->cfg.n_scenarios);
     if (!h->d32b) CK(cudaMalloc(reinterpret_cast<void**>(&h->d32b), n32 * sizeof(float)));
     if (h->pmul && !h->pmulb) {
       const size_t np = static_cast<size_t>(h->cfg.n_scenarios) * RRG_NPARAM;
@@ -1277,8 +1279,7 @@ int rrg_closed_loop_dev(rrg_handle h, const double* x0, double v0, const double*
       cudaGraphExecDestroy(h->st_exec);
       h->st_exec = nullptr;
     }
-    if (h->tma_ok && !encode_scenario_map(&h->tmap[1], h->d32b, h->cfg.n_scenarios, h->cfg.horizon,
-                                          h->cfg.n_scenarios)) {
+    if (h->tma_ok && !encode_scenario_map(&h->tmap[1], h->d32b, h->cfg.n_scenarios, h->cfg.horizon)) {
       h->tma_ok = false;  // the rings fall back to per-lane asynchronous copies
       h->L.tmap = nullptr;
     }

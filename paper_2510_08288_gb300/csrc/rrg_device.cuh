@@ -421,12 +421,12 @@ __device__ __forceinline__ void mul128(uint64_t m, uint64_t x, uint64_t& hi, uin
   lo = static_cast<uint64_t>(p);
 }
 
-// The blocks (words 0..2) at the counters (j, base + k, upd, 0), key (seed, 0),
-// for steps j0 <= j < j1 and the KT scenarios k = k0 + i kstep of a thread:
-// sink(i, j, w0, w1, w2).  The scenario enters through word 1 and the step
-// through word 0, so of the twenty products of a block one depends on the
-// scenario alone (formed once per thread) and three on the step alone (shared
-// by the thread's scenarios; j is the same for every thread of the block, so
+// Philox blocks at the counters (j, k0 + i kstep, upd, 0), key (seed, 0), for the
+// KT scenarios i of a thread and one step j after the other: step(j, sink) calls
+// sink(i, w0, w1, w2).  The scenario enters through word 1 and the step through
+// word 0, so of the twenty products of a block one depends on the scenario
+// alone (formed once per thread) and three on the step alone (shared by the
+// thread's scenarios; callers keep j the same for every thread of a block, so
 // they may run on the uniform path): 15 + 3 / KT are left per block.
 //
 // The generator is bound by the integer pipes: a 64-bit product is four wide
@@ -434,18 +434,22 @@ __device__ __forceinline__ void mul128(uint64_t m, uint64_t x, uint64_t& hi, uin
 // scheduler's multiply and logic pipes are each half busy.  Measured (16,384 x
 // 5,000 binary32 draws): one block per (j, k) with its index division 892 us,
 // this form 720 us with KT = 1, 700 with 2, 716 with 4.
-template <int KT, typename Sink>
-__device__ __forceinline__ void philox_tile(uint64_t k0, uint64_t kstep, int j0, int j1, uint64_t upd,
-                                            uint64_t seed, const Sink& sink) {
-  constexpr uint64_t kM0 = 0xD2E7470EE14C6C93ull, kM1 = 0xCA5A826395121157ull;
-  constexpr uint64_t kW0 = 0x9E3779B97F4A7C15ull, kW1 = 0xBB67AE8584CAA73Bull;
-  uint64_t u_hi, u_lo;  // round 0 of the update index
-  mul128(kM1, upd, u_hi, u_lo);
-  uint64_t b_hi[KT], b_lo[KT];  // rounds 0 and 1 of the scenario
+template <int KT>
+struct PhiloxCols {
+  static constexpr uint64_t kM0 = 0xD2E7470EE14C6C93ull, kM1 = 0xCA5A826395121157ull;
+  static constexpr uint64_t kW0 = 0x9E3779B97F4A7C15ull, kW1 = 0xBB67AE8584CAA73Bull;
+  uint64_t seed, u_lo, b_hi[KT], b_lo[KT];
+
+  __device__ __forceinline__ PhiloxCols(uint64_t k0, uint64_t kstep, uint64_t upd, uint64_t seed_) : seed(seed_) {
+    uint64_t u_hi;  // round 0 of the update index
+    mul128(kM1, upd, u_hi, u_lo);
 #pragma unroll
-  for (int i = 0; i < KT; ++i)
-    mul128(kM0, u_hi ^ (k0 + static_cast<uint64_t>(i) * kstep) ^ seed, b_hi[i], b_lo[i]);
-  for (int j = j0; j < j1; ++j) {
+    for (int i = 0; i < KT; ++i)  // rounds 0 and 1 of the scenario
+      mul128(kM0, u_hi ^ (k0 + static_cast<uint64_t>(i) * kstep) ^ seed, b_hi[i], b_lo[i]);
+  }
+
+  template <typename Sink>
+  __device__ __forceinline__ void step(int j, const Sink& sink) const {
     uint64_t a_hi, a_lo, c_hi, c_lo, e_hi, e_lo;  // rounds 0, 1 and 2 of the step
     mul128(kM0, static_cast<uint64_t>(j), a_hi, a_lo);
     mul128(kM1, a_hi, c_hi, c_lo);
@@ -467,9 +471,23 @@ __device__ __forceinline__ void philox_tile(uint64_t k0, uint64_t kstep, int j0,
         c2 = h0 ^ c3 ^ kb;
         c3 = l0;
       }
-      sink(i, j, c0, c1, c2);
+      sink(i, c0, c1, c2);
     }
   }
+};
+
+// ---------------------------------------------------------------------------
+// The handles' binary32 scenario arrays hold four consecutive steps of a
+// scenario side by side: [3 components][quads of steps][N scenarios][4 steps],
+// H rounded up to whole quads.  A lane then reads four steps of a component
+// with one 16-byte load (a warp: 512 consecutive bytes), from global memory or
+// from a chunk that the TMA brought, where [3][H][N] took one load (and its
+// share of the address arithmetic) per step and component; and every row is a
+// multiple of 16 bytes whatever N.
+__host__ __device__ inline size_t quad_rows(int H) { return (static_cast<size_t>(H) + 3) / 4; }
+__host__ __device__ inline size_t quad_elems(int H, int N) { return 12 * quad_rows(H) * static_cast<size_t>(N); }
+__host__ __device__ inline size_t quad_index(int c, int j, int k, int H, int N) {
+  return ((c * quad_rows(H) + static_cast<size_t>(j >> 2)) * N + k) * 4 + (j & 3);
 }
 
 // a (2u - 1) with u the top 53 bits of w scaled to [0, 1).  2u - 1 equals

@@ -105,17 +105,17 @@ slack_error_kernel(const Launch L, float band, double* __restrict__ err, int32_t
         e1 = uniform_sym32(r.w[1], sc1);
         e2 = uniform_sym32(r.w[2], sc2);
       } else {
-        e0 = L.d32[q];
-        e1 = L.d32[HN + q];
-        e2 = L.d32[2 * HN + q];
+        e0 = L.d32[quad_index(0, j, k, H, N)];
+        e1 = L.d32[quad_index(1, j, k, H, N)];
+        e2 = L.d32[quad_index(2, j, k, H, N)];
       }
     } else {
       f0 = L.d64[q];
       f1 = L.d64[HN + q];
       f2 = L.d64[2 * HN + q];
-      e0 = L.d32[q];
-      e1 = L.d32[HN + q];
-      e2 = L.d32[2 * HN + q];
+      e0 = L.d32[quad_index(0, j, k, H, N)];
+      e1 = L.d32[quad_index(1, j, k, H, N)];
+      e2 = L.d32[quad_index(2, j, k, H, N)];
     }
     rk4_step_fast<float>(M32.U, nullptr, C32, a_ca, a_w, a_sm, a_wa, e0, e1, e2);
     rk4_step_fast<double>(M64.U, M64.pw, C64, b_ca, b_w, b_sm, b_wa, f0, f1, f2);

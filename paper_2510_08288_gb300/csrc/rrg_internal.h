@@ -177,6 +177,7 @@ struct Launch {
   StepModel<double> m64;        // the rollout step's coefficients
   StepModel<float> m32;
   double* d64;                  // scenarios [3][H][N]
+  int quads;                    // d32 is in the quad layout (0: the caller's [3][H][N])
   float* d32;
   double* d64b;                 // second pair for closed loops (sampling of update t+1
   float* d32b;                  //   overlaps update t), or nullptr
@@ -473,6 +474,8 @@ cudaError_t launch_scenario_fold(const Launch& L, bool second, uint64_t base = 0
 // lazily (no-op otherwise).
 cudaError_t launch_materialize64(const Launch& L);
 cudaError_t launch_round_scenarios(const Launch& L);
+// Marks pair 0's binary64 array as holding its values.
+cudaError_t launch_mark64(const Launch& L);
 cudaError_t launch_fill(const Launch& L, double* a, size_t n, double v);
 // buf_base >= 0: the update index is buf_base + *t_dev and selects the
 // scenario pair by its parity; otherwise pair 0
@@ -491,12 +494,11 @@ cudaError_t launch_eval_prepare(const Launch& L, const double* d_x, double v_pre
                                 const double* d_kappas, int m, const double* d_vp = nullptr,
                                 const double* d_r = nullptr);
 cudaError_t launch_eval_finish(const Launch& L, int m, uint8_t* d_adm, double* d_min_slack);
-// Tensor map of a binary32 scenario array [3][H][ld] of N <= ld scenarios for
-// the TMA ring (boxes of 32 scenarios x one chunk of steps x 3 components);
-// false when ld is not a multiple of 4 (row strides must be multiples of 16
-// bytes) or the driver refuses.  tma_ring_prepare() sets the TMA kernels' shared-memory limit on
-// the current device (once per device); false if the runtime refuses.
-bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H, int ld);
+// Tensor map of a binary32 scenario array in the quad layout for the TMA ring
+// (boxes of 32 scenarios x one chunk of steps x 3 components); false when the
+// driver refuses.  tma_ring_prepare() sets the TMA kernels' shared-memory limit
+// on the current device (once per device); false if the runtime refuses.
+bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H);
 bool tma_ring_prepare();
 // Resident blocks per SM of the two-candidates-per-thread TMA kernel (after
 // tma_ring_prepare on the current device; 0 if the runtime does not answer).

@@ -125,7 +125,7 @@ __device__ __forceinline__ void sample_param_group(double* __restrict__ pm, uint
 struct SampleArgs {
   double *d64, *d64b;
   float *d32, *d32b;
-  int N, H, jc;   // jc: steps per block
+  int N, H, jc;   // jc: steps (binary64) or quads of steps per block
   uint64_t seed, base, kbase;
   double a0, a1, a2;
   int write64, gen;
@@ -135,24 +135,24 @@ struct SampleArgs {
   uint32_t mask;
 };
 
-template <int KT>
+constexpr int kKt64 = 2;  // scenarios per thread of the binary64 draw
 __device__ __forceinline__ void sample_tile64(double* __restrict__ d, const SampleArgs& A, uint64_t upd) {
-  const int k0 = blockIdx.x * (blockDim.x * KT) + threadIdx.x;
+  const int k0 = blockIdx.x * (blockDim.x * kKt64) + threadIdx.x;
   const int j0 = blockIdx.y * A.jc, j1 = min(j0 + A.jc, A.H);
   const size_t N = A.N, HN = static_cast<size_t>(A.H) * N;
-  philox_tile<KT>(A.kbase + static_cast<uint64_t>(k0), blockDim.x, j0, j1, upd, A.seed,
-                  [&](int i, int j, uint64_t w0, uint64_t w1, uint64_t w2) {
-                    const size_t k = static_cast<size_t>(k0) + static_cast<size_t>(i) * blockDim.x;
-                    if (k < N) {
-                      const size_t q = static_cast<size_t>(j) * N + k;
-                      d[q] = uniform_sym(w0, A.a0);
-                      d[HN + q] = uniform_sym(w1, A.a1);
-                      d[2 * HN + q] = uniform_sym(w2, A.a2);
-                    }
-                  });
+  const PhiloxCols<kKt64> P(A.kbase + static_cast<uint64_t>(k0), blockDim.x, upd, A.seed);
+  for (int j = j0; j < j1; ++j)
+    P.step(j, [&](int i, uint64_t w0, uint64_t w1, uint64_t w2) {
+      const size_t k = static_cast<size_t>(k0) + static_cast<size_t>(i) * blockDim.x;
+      if (k < N) {
+        const size_t q = static_cast<size_t>(j) * N + k;
+        d[q] = uniform_sym(w0, A.a0);
+        d[HN + q] = uniform_sym(w1, A.a1);
+        d[2 * HN + q] = uniform_sym(w2, A.a2);
+      }
+    });
 }
 
-template <int KT>
 __global__ void __launch_bounds__(kSampleThreads)
 sample_kernel(const SampleArgs A, const unsigned long long* t_dev) {
   const uint64_t upd = A.base + (t_dev ? *t_dev : 0ull);
@@ -172,12 +172,12 @@ sample_kernel(const SampleArgs A, const unsigned long long* t_dev) {
   }
   if (!A.gen) {
     if (A.write64) {
-      sample_tile64<KT>(pair ? A.d64b : A.d64, A, upd);
+      sample_tile64(pair ? A.d64b : A.d64, A, upd);
     } else {
-      const int j0 = blockIdx.y * A.jc;
-      sample_tile32<KT>(pair ? A.d32b : A.d32, A.N, A.N, A.H, blockIdx.x * (blockDim.x * KT) + threadIdx.x, j0,
-                        min(j0 + A.jc, A.H), A.kbase, upd, A.seed, static_cast<float>(A.a0 * 0x1.0p-23),
-                        static_cast<float>(A.a1 * 0x1.0p-23), static_cast<float>(A.a2 * 0x1.0p-23));
+      const int q0 = blockIdx.y * A.jc, rows = static_cast<int>(quad_rows(A.H));
+      sample_quads(pair ? A.d32b : A.d32, A.N, A.H, blockIdx.x * blockDim.x + threadIdx.x, q0,
+                   min(q0 + A.jc, rows), A.kbase, upd, A.seed, static_cast<float>(A.a0 * 0x1.0p-23),
+                   static_cast<float>(A.a1 * 0x1.0p-23), static_cast<float>(A.a2 * 0x1.0p-23));
     }
   }
   double* pm = pair ? A.pmb : A.pm;
@@ -274,18 +274,13 @@ cudaError_t launch_sample(const Launch& L, uint64_t seed, uint64_t base,
   A.pmb = dual ? L.pmulb : nullptr;
   A.rho = L.punc_rho;
   A.mask = L.punc_mask;
-  // two scenarios per thread, but one where that leaves a warp half empty;
-  // blocks of 128 threads (fewer for few scenarios), 16 per SM, of at most 64
-  // steps each
-  const int kt = L.N > 32 ? 2 : 1;
+  // blocks of 128 threads (fewer for few scenarios), 16 per SM
+  const int kt = A.write64 ? kKt64 : 1;
   const int per = (L.N + kt - 1) / kt;
   const int threads = per >= kSampleThreads ? kSampleThreads : (per + 31) / 32 * 32;
-  const dim3 tile = sample_grid(L.N, L.scen_gen ? 1 : L.H, threads * kt, L.sms * 16, &A.jc);
-  const cudaStream_t s = stream ? stream : L.stream;
-  if (kt == 2)
-    sample_kernel<2><<<tile, threads, 0, s>>>(A, t_dev);
-  else
-    sample_kernel<1><<<tile, threads, 0, s>>>(A, t_dev);
+  const int rows = A.write64 ? L.H : static_cast<int>(quad_rows(L.H));
+  const dim3 tile = sample_grid(L.N, L.scen_gen ? 1 : rows, threads * kt, L.sms * 16, &A.jc);
+  sample_kernel<<<tile, threads, 0, stream ? stream : L.stream>>>(A, t_dev);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_scenario_fold(L, false, base, t_dev, dual && L.d64b != nullptr, stream);
@@ -318,7 +313,7 @@ materialize64_kernel(double* __restrict__ d64, int N, int H, int jc, const Searc
   A.a0 = src.amp[0];
   A.a1 = src.amp[1];
   A.a2 = src.amp[2];
-  sample_tile64<1>(d64, A, src.update);
+  sample_tile64(d64, A, src.update);
 }
 
 // Marks pair 0's binary64 array valid once every block of the fill is done
@@ -328,24 +323,41 @@ __global__ void mark64_kernel(SearchState* st) { st->src[0].d64_valid = 1; }
 cudaError_t launch_materialize64(const Launch& L) {
   if (L.sms <= 0) return cudaErrorInvalidConfiguration;
   int jc = 1;
-  const dim3 tile = sample_grid(L.N, L.H, kSampleThreads, L.sms * 16, &jc);
+  const dim3 tile = sample_grid(L.N, L.H, kSampleThreads * kKt64, L.sms * 16, &jc);
   materialize64_kernel<<<tile, kSampleThreads, 0, L.stream>>>(L.d64, L.N, L.H, jc, L.st);
   mark64_kernel<<<1, 1, 0, L.stream>>>(L.st);
   return cudaGetLastError();
 }
 
-__global__ void round_scenarios_kernel(const double* __restrict__ d64, float* __restrict__ d32,
-                                       size_t n, SearchState* st) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) st->src[0].d64_valid = 1;
-  const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
-  for (size_t q = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < n; q += stride)
-    d32[q] = static_cast<float>(d64[q]);
+// The binary32 copy of explicit scenarios, each value rounded, in the quad
+// layout (block x: scenarios, y and z: quads of steps and components).
+__global__ void round_scenarios_kernel(const double* __restrict__ d64, float* __restrict__ d32, int N, int H,
+                                       SearchState* st) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) st->src[0].d64_valid = 1;
+  const int k = blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.z;
+  if (k >= N || d32 == nullptr) return;
+  const int rows = static_cast<int>(quad_rows(H));
+  for (int q = blockIdx.y; q < rows; q += gridDim.y) {
+    float v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = 4 * q + u;
+      v[u] = j < H ? static_cast<float>(d64[(static_cast<size_t>(c) * H + j) * N + k]) : 0.0f;
+    }
+    *reinterpret_cast<float4*>(d32 + quad_index(c, 4 * q, k, H, N)) = make_float4(v[0], v[1], v[2], v[3]);
+  }
 }
 
 cudaError_t launch_round_scenarios(const Launch& L) {
-  const size_t n = L.scen_gen ? 0 : 3 * static_cast<size_t>(L.H) * L.N;
   if (L.sms <= 0) return cudaErrorInvalidConfiguration;
-  round_scenarios_kernel<<<grid_for(n, 256, L.sms * 16), 256, 0, L.stream>>>(L.d64, L.d32, n, L.st);
+  const size_t rows = quad_rows(L.H);
+  const dim3 grid((L.N + 127) / 128, static_cast<unsigned>(rows < 4096 ? rows : 4096), 3);
+  round_scenarios_kernel<<<grid, 128, 0, L.stream>>>(L.d64, L.scen_gen ? nullptr : L.d32, L.N, L.H, L.st);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_mark64(const Launch& L) {
+  mark64_kernel<<<1, 1, 0, L.stream>>>(L.st);
   return cudaGetLastError();
 }
 
@@ -358,10 +370,11 @@ cudaError_t launch_round_scenarios(const Launch& L) {
 // parametric uncertainty, each lane folds its scenario's own model constants.
 // Where a rollout lane takes its disturbances from.
 enum RollSrc : int {
-  SRC_REGS = 0,  // the stored array through a register prefetch ring (run_lane)
-  SRC_RING = 1,  // the stored array through a shared-memory ring (run_lane_ring, binary32)
+  SRC_REGS = 0,  // an array [3][H][N] through a register prefetch ring (run_lane)
+  SRC_RING = 1,  // an array [3][H][N] through a shared-memory ring (run_lane_ring, binary32)
   SRC_GEN = 2,   // drawn from Philox inside the trajectory loop (run_lane_gen)
-  SRC_TMA = 3    // the stored array through a per-warp TMA ring (run_lane_tma, binary32)
+  SRC_TMA = 3,   // the handle's quads through a per-warp TMA ring (run_lane_tma, binary32)
+  SRC_QRING = 4  // the handle's quads through a shared-memory ring (run_lane_qring, binary32)
 };
 
 // Dynamic shared memory of the TMA-ring rollouts: per warp two stages of
@@ -499,7 +512,7 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
                      2 * wid;
     const bool lane_runs = active && final_lane;
     const void* tm = (L.inject & RRG_INJECT_TMA_NO_COPY) ? nullptr : (L.st->buf ? tm1 : tm0);
-    const T s_out = run_lane_tma<PU>(K, C, tm, k & ~31, lane_runs, j0, j_end, q_ca, w, q_sm,
+    const T s_out = run_lane_tma<PU>(K, C, tm, d, k, N, L.H, lane_runs, j0, j_end, q_ca, w, q_sm,
                                  w_abs, smin0, thr, cand_stop ? dead : nullptr,
                                  cand_stop ? dead : nullptr, &steps, &end, band, &jlast, stages, bars,
                                  &L.stats->wait_timeouts);
@@ -516,6 +529,10 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
       __shared__ float ring[RRG_RING_DEPTH * 3 * kRollThreads];
       smin = run_lane_ring(K, C, d, k, N, L.H, j0, j_end, q_ca, w, q_sm, w_abs, smin0, thr,
                            cand_stop ? dead : nullptr, &steps, &end, band, &jlast, ring);
+    } else if constexpr (SRC == SRC_QRING) {
+      __shared__ __align__(16) unsigned char qring[qring_bytes(kRollThreads)];
+      smin = run_lane_qring<kRollThreads, PU>(K, C, d, k, N, L.H, j0, j_end, q_ca, w, q_sm, w_abs, smin0, thr,
+                                          cand_stop ? dead : nullptr, &steps, &end, band, &jlast, qring);
     } else
       smin = run_lane<T>(K, M.pw, C, d, k, N, L.H, j0, j_end, q_ca, w, q_sm, w_abs, smin0, thr,
                          cand_stop ? dead : nullptr, &steps, &end, band, &jlast);
@@ -584,12 +601,6 @@ rollout_tma_kernel(const Launch L, const float* __restrict__ d_pair0, const floa
 #ifndef RRG_PAIR_MIN_BLOCKS
 #define RRG_PAIR_MIN_BLOCKS 1
 #endif
-// Prefetch depth (and exit block) of a paired thread: each step issues two
-// trajectories' instructions, so half the single lane's depth covers the same
-// load latency with half the unrolled code.
-#ifndef RRG_PAIR_PF
-#define RRG_PAIR_PF 8
-#endif
 template <bool PU>
 __global__ void __launch_bounds__(kRollThreads, PU ? RRG_PAIR_PU_MIN_BLOCKS : RRG_PAIR_MIN_BLOCKS)
 rollout_pair_kernel(const Launch L, const float* __restrict__ d_pair0,
@@ -639,15 +650,15 @@ rollout_pair_kernel(const Launch L, const float* __restrict__ d_pair0,
     start_state<float>(RA, L.st->x, p_atm, za[0], za[1], za[2], za[3]);
     start_state<float>(RB, L.st->x, p_atm, zb[0], zb[1], zb[2], zb[3]);
     if (runa && runb) {
-      paired = 2u * static_cast<unsigned>(run_lane_pair<float, RRG_PAIR_PF>(
+      paired = 2u * static_cast<unsigned>(run_lane_pair(
                             K, CA, CB, d, k, N, L.H, L.H, za, zb, thr, band, cand_stop ? deada : nullptr,
                             cand_stop ? deadb : nullptr, sm, st, en, jl));
     } else if (runa) {
-      sm[0] = run_lane<float, RRG_PAIR_PF>(K, nullptr, CA, d, k, N, L.H, 0, L.H, za[0], za[1], za[2], za[3],
+      sm[0] = run_lane_q(K, CA, d, k, N, L.H, 0, L.H, za[0], za[1], za[2], za[3],
                                            inf_v<float>(), thr, cand_stop ? deada : nullptr, &st[0],
                                            &en[0], band, &jl[0]);
     } else {
-      sm[1] = run_lane<float, RRG_PAIR_PF>(K, nullptr, CB, d, k, N, L.H, 0, L.H, zb[0], zb[1], zb[2], zb[3],
+      sm[1] = run_lane_q(K, CB, d, k, N, L.H, 0, L.H, zb[0], zb[1], zb[2], zb[3],
                                            inf_v<float>(), thr, cand_stop ? deadb : nullptr, &st[1],
                                            &en[1], band, &jl[1]);
     }
@@ -749,19 +760,12 @@ rollout_tma_pair_kernel(const Launch L, const RhsC<float>* __restrict__ cand,
 #endif
 
 // RRG_TMA_AUTO takes the TMA ring for binary32 launches on the stored array
-// of at least this many warps per SM, ahead of the other rings and of
-// pairing.  The TMA saves the per-step load instructions, which pays where
-// many warps compete for issue; a warp running alone pays the chunk's wait,
-// warp votes and fence on its dependency chain instead.  Measured on GB300
-// (k-section sweep, 16 candidates x 5,000 steps, per update), TMA against the
-// per-lane cp.async ring: 16,384 scenarios with uncertain parameters (54
-// warps per SM) 6.28 against 6.75 ms, 8,192 (27) 4.46 against 4.53 ms, 4,096
-// (13.5) 2.78 against 2.70 ms, 1,024 (3.4) 1.85 against 1.64 ms; the
-// 1,024-scenario closed loop (8.8 warps per SM at launch, mostly single
-// survivors) 2,743 against 2,927 updates/s.  Against the register ring and
-// pairing on launches that fill the SMs: 65,536 parametric 21.8 ms against
-// 23.9 (single) and 24.0 (paired), 32,768 10.9 against 11.8; nominal 65,536
-// 27.5 against 30.4 and 30.2.
+// of at least this many warps per SM, ahead of pairing; below, the ring of
+// quads.  Measured on GB300 (no early exit, 1,000 steps), TMA against the ring
+// of quads: nominal 16,384 x 16 scenarios 731 against 753 us, 1,024 x 64 (13.5
+// warps per SM) 229 against 234, x 42 176 against 176, one candidate (each warp
+// alone on its scheduler, where the chunk's wait, votes and refill sit on the
+// chain) 96 against 86; parametric 16,384 x 16 823 against 830.
 #ifndef RRG_TMA_MIN_WARPS_PER_SM
 #define RRG_TMA_MIN_WARPS_PER_SM 24
 #endif
@@ -770,19 +774,15 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
                            bool recheck_classify, bool allow_pair) {
   dim3 grid((L.N + kRollThreads - 1) / kRollThreads, m_launch);
   const int cls = recheck_classify ? 1 : 0;
-  // Binary32 lanes on the stored array: the shared-memory ring when the
-  // launch leaves most warp slots empty (each warp then runs its trajectory
-  // alone on its scheduler, bound by the step's latency), the register ring
-  // when it fills the SMs (bound by issue, where the ring's extra
-  // instructions cost more than they save).  Thresholds measured on GB300:
-  // nominal model, ring up to 16 warps per SM (the 1,024-scenario closed loop
-  // ran 10 % faster, 8,192 x 16 candidates 3 % slower); parametric model
-  // (more registers, fewer resident warps), up to 64 (16,384 x 16 candidates
-  // 2-6 % faster, 65,536 x 16 6 % slower).
+  // Binary32 lanes on a handle's quads that take neither the TMA ring nor
+  // pairing: the shared-memory ring of quads, at every launch size.  The
+  // caller's arrays of the allocation-free call keep the layout [3][H][N] and
+  // its two forms: the per-value ring when the launch leaves most warp slots
+  // empty (up to 16 warps per SM), the register ring above.
   if (L.sms <= 0) return cudaErrorInvalidConfiguration;
   const int sms = L.sms;
   const long long warps = static_cast<long long>(grid.x) * grid.y * (kRollThreads / 32);
-  const bool ring = warps <= (L.pmul ? 64LL : 16LL) * sms;
+  const bool ring = warps <= (L.pmul ? 64LL : 16LL) * sms;  // (also the bound below which launches never pair)
   const long long pair_blocks = static_cast<long long>(grid.x) * ((m_launch + 1) / 2);
   const bool filled = !ring && L.pair == RRG_PAIR_FILLED &&
                       pair_blocks >= static_cast<long long>(RRG_PAIR_MIN_WAVES) *
@@ -835,9 +835,10 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
   } else {
     if (L.pmul) {
       if (L.scen_gen) RRG_ROLLOUT(rollout_pu_kernel, float, SRC_GEN, L.d32, L.d32b, L.cand_c32, cls);
-      else RRG_ROLLOUT(rollout_pu_kernel, float, SRC_RING, L.d32, L.d32b, L.cand_c32, cls);
+      else RRG_ROLLOUT(rollout_pu_kernel, float, SRC_QRING, L.d32, L.d32b, L.cand_c32, cls);
     } else {
       if (L.scen_gen) RRG_ROLLOUT(rollout_kernel, float, SRC_GEN, L.d32, L.d32b, L.cand_c32, cls);
+      else if (L.quads) RRG_ROLLOUT(rollout_kernel, float, SRC_QRING, L.d32, L.d32b, L.cand_c32, cls);
       else if (ring) RRG_ROLLOUT(rollout_kernel, float, SRC_RING, L.d32, L.d32b, L.cand_c32, cls);
       else RRG_ROLLOUT(rollout_kernel, float, SRC_REGS, L.d32, L.d32b, L.cand_c32, cls);
     }
@@ -911,8 +912,7 @@ bool tma_ring_prepare() {
   // neither waits for the other to leave the SM (sixteen closed-loop updates of
   // 1,024 scenarios 4878 -> 4769 us).
   const cudaFuncAttribute c = cudaFuncAttributePreferredSharedMemoryCarveout;
-  cudaFuncSetAttribute(sample_kernel<1>, c, cudaSharedmemCarveoutMaxShared);
-  cudaFuncSetAttribute(sample_kernel<2>, c, cudaSharedmemCarveoutMaxShared);
+  cudaFuncSetAttribute(sample_kernel, c, cudaSharedmemCarveoutMaxShared);
   cudaFuncSetAttribute(scenario_fold_kernel, c, cudaSharedmemCarveoutMaxShared);
   const bool ok = cudaFuncSetAttribute(rollout_tma_kernel<false>, a, sm) == cudaSuccess &&
                   cudaFuncSetAttribute(rollout_tma_kernel<true>, a, sm) == cudaSuccess &&
@@ -922,7 +922,7 @@ bool tma_ring_prepare() {
   return ok;
 }
 
-bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H, int ld) {
+bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H) {
   static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
     void* f = nullptr;
     cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
@@ -932,12 +932,12 @@ bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H, int ld)
       f = nullptr;
     return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
   }();
-  if (encode == nullptr || d32 == nullptr || N <= 0 || H <= 0 || ld < N || ld % 4 != 0) return false;
-  // dims innermost first: scenario k, step j, component c
-  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(N), static_cast<cuuint64_t>(H), 3};
-  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld) * sizeof(float),
-                                 static_cast<cuuint64_t>(H) * ld * sizeof(float)};
-  const cuuint32_t box[3] = {32, static_cast<cuuint32_t>(kTmaChunk), 3};
+  if (encode == nullptr || d32 == nullptr || N <= 0 || H <= 0) return false;
+  // dims innermost first: the four steps of every scenario, quads, components
+  const cuuint64_t rows = quad_rows(H), row = 16 * static_cast<cuuint64_t>(N);
+  const cuuint64_t dims[3] = {4 * static_cast<cuuint64_t>(N), rows, 3};
+  const cuuint64_t strides[2] = {row, rows * row};
+  const cuuint32_t box[3] = {128, static_cast<cuuint32_t>(kTmaChunk / 4), 3};
   const cuuint32_t elem[3] = {1, 1, 1};
   return encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(d32), dims, strides, box, elem,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,

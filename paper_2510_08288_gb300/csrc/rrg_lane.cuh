@@ -341,35 +341,144 @@ __device__ __forceinline__ T run_lane(const StepU<T>& K, const PowTable* pw, con
 }
 
 // ---------------------------------------------------------------------------
+// run_lane on the handles' quad layout: the disturbances of four steps come
+// with one 16-byte load per component, Q quads ahead in registers.  Same
+// contract, arithmetic and results as run_lane<float>; the exit and finiteness
+// tests come every 4 Q steps.  A segment that starts inside a quad
+// (SEG_CONTINUE after an odd probe length) steps to its end one step at a time.
+// The form without shared memory: single problems stage their quads
+// (run_lane_qring), whose deeper look-ahead a lone warp needs (177 against 203
+// cycles a step).
+// The binary32 step, packed or not (the same bits).
+template <bool PACK>
+__device__ __forceinline__ void lane_step(const StepU<float>& K, const StepC<float>& C, float& q_ca, float& w,
+                                          float& q_sm, float& w_abs, float e0, float e1, float e2) {
+  if constexpr (PACK) rk4_step_packed(K, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
+  else rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
+}
+
+// One step with run_lane's per-step tests; false once the lane has violated.
+__device__ __forceinline__ bool lane_step_checked(const StepU<float>& K, const StepC<float>& C, float e0, float e1,
+                                                  float e2, float& q_ca, float& w, float& q_sm, float& w_abs,
+                                                  int& j, float& smin, float thr, float band, int& jl) {
+  rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
+  ++j;
+  const float s = checked_slack<float>(C, q_ca, w, q_sm);
+  smin = fmin(smin, s);
+  if (s < band) jl = j;
+  return !(s < thr);
+}
+
+template <int Q = 2>
+__device__ __forceinline__ float run_lane_q(const StepU<float>& K, const StepC<float>& C,
+                                            const float* __restrict__ d, int k, int N, int H, int j0, int j_end,
+                                            float& q_ca, float& w, float& q_sm, float& w_abs, float smin_in,
+                                            float thr, const volatile int32_t* dead, unsigned* steps, int* end,
+                                            float band, int* jlast) {
+  constexpr int B = 4 * Q;
+  float smin = smin_in;
+  int j = j0;
+  int jl = *jlast;
+  int how = LANE_REACHED_END;
+  bool go = j < j_end;
+  if (j0 == 0) {
+    const float s0 = checked_slack<float>(C, q_ca, w, q_sm);
+    smin = fmin(smin, s0);
+    if (s0 < band) jl = 0;
+    if (s0 < thr) {
+      how = LANE_VIOLATED;
+      go = false;
+    }
+  }
+  const size_t row = 4 * static_cast<size_t>(N), comp = quad_rows(H) * row;
+  auto one = [&]() {
+    const float* p = d + static_cast<size_t>(j >> 2) * row + 4 * static_cast<size_t>(k) + (j & 3);
+    if (!lane_step_checked(K, C, __ldg(p), __ldg(p + comp), __ldg(p + 2 * comp), q_ca, w, q_sm, w_abs, j, smin, thr,
+                           band, jl)) {
+      how = LANE_VIOLATED;
+      go = false;
+    }
+  };
+  while (go && j < j_end && (j & 3) != 0) one();
+  if (go && j + B <= j_end) {
+    const float4* p0 = reinterpret_cast<const float4*>(d + static_cast<size_t>(j >> 2) * row) + k;
+    const float4* p1 = reinterpret_cast<const float4*>(d + comp + static_cast<size_t>(j >> 2) * row) + k;
+    const float4* p2 = reinterpret_cast<const float4*>(d + 2 * comp + static_cast<size_t>(j >> 2) * row) + k;
+    float4 r0[Q], r1[Q], r2[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      r0[q] = __ldg(p0); r1[q] = __ldg(p1); r2[q] = __ldg(p2);
+      p0 += N; p1 += N; p2 += N;
+    }
+    do {
+      const int dead_now = dead != nullptr ? *dead : 0;
+      const bool more = j + 2 * B <= j_end;  // the next block is whole too
+      BlockMin<float> bm;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const float4 e0 = r0[q], e1 = r1[q], e2 = r2[q];
+        if (more) {
+          r0[q] = __ldg(p0); r1[q] = __ldg(p1); r2[q] = __ldg(p2);
+        }
+        p0 += N; p1 += N; p2 += N;
+        rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0.x, e1.x, e2.x);
+        bm.add(slack_of<float>(C, q_ca, q_sm), 0);
+        rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0.y, e1.y, e2.y);
+        bm.add(slack_of<float>(C, q_ca, q_sm), 1);
+        rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0.z, e1.z, e2.z);
+        bm.add(slack_of<float>(C, q_ca, q_sm), 0);
+        rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0.w, e1.w, e2.w);
+        bm.add(slack_of<float>(C, q_ca, q_sm), 1);
+      }
+      j += B;
+      const float bmin = bm.result(q_ca, w, q_sm);
+      smin = fmin(smin, bmin);
+      if (bmin < band) jl = j;
+      if (smin < thr) {
+        how = LANE_VIOLATED;
+        go = false;
+      } else if (dead_now != 0 && j < j_end) {
+        how = LANE_STOPPED;
+        go = false;
+      }
+    } while (go && j + B <= j_end);
+  }
+  while (go && j < j_end) one();
+  *steps = static_cast<unsigned>(j - j0);
+  *end = how;
+  *jlast = jl;
+  return smin;
+}
+
+// ---------------------------------------------------------------------------
 // Two trajectories of one scenario k -- candidates A and B, the same
-// disturbances -- in one thread: each step's three disturbance loads, the
-// ring's addressing and the loop's bookkeeping serve both, and the two step
-// chains are independent work for the scheduler.  Same arithmetic as
-// run_lane for each trajectory: the decisions, and the min slack of a
-// trajectory that does not violate, equal run_lane's bit for bit (a
-// violating one may be integrated a little longer, so its min slack, an upper
-// bound either way, can come out lower).
+// disturbances -- in one thread: each quad's three loads, their addressing and
+// the loop's bookkeeping serve both, and the two step chains are independent
+// work for the scheduler.  Same arithmetic as run_lane_q for each trajectory:
+// the decisions, and the min slack of a trajectory that does not violate,
+// equal its bit for bit (a violating one may be integrated a little longer, so
+// its min slack, an upper bound either way, can come out lower).
 //
 // From step 0 (its slack checked first: a violation there runs nothing in
-// pair) over whole blocks of PF steps while
+// pair) over whole blocks of two quads while
 // neither candidate has been stopped: a trajectory that violates keeps being
 // integrated with its partner (its min slack only falls, so no decision
 // changes) and, when dead_X is given, marks its candidate dead at once, so
 // the stop reaches every lane together at a block end (read at the block's
 // start, as in run_lane) instead of splitting the warp.  Without dead flags
 // (no candidate-level exit) a lane leaves the pair when either trajectory
-// has violated.  The survivor then finishes alone in run_lane from the
+// has violated.  The survivor then finishes alone in run_lane_q from the
 // step reached; the last, partial block too.  z_X[4] = (q_ca, w, q_sm,
 // w_abs) in and out; smin, steps, end, jlast per trajectory as run_lane's.
 // Returns the steps both trajectories ran together.
-template <typename T, int PF = PrefetchDepth<T>::value>
-__device__ __forceinline__ int run_lane_pair(const StepU<T>& K, const StepC<T>& CA, const StepC<T>& CB,
-                                              const T* __restrict__ d, int k, int N, int H, int j_end,
-                                              T* za, T* zb, T thr, T band,
+__device__ __forceinline__ int run_lane_pair(const StepU<float>& K, const StepC<float>& CA, const StepC<float>& CB,
+                                              const float* __restrict__ d, int k, int N, int H, int j_end,
+                                              float* za, float* zb, float thr, float band,
                                               volatile int32_t* deadA, volatile int32_t* deadB,
-                                              T* smin, unsigned* steps, int* end, int* jlast) {
-  smin[0] = checked_slack<T>(CA, za[0], za[1], za[2]);
-  smin[1] = checked_slack<T>(CB, zb[0], zb[1], zb[2]);
+                                              float* smin, unsigned* steps, int* end, int* jlast) {
+  constexpr int Q = 2, B = 4 * Q;
+  smin[0] = checked_slack<float>(CA, za[0], za[1], za[2]);
+  smin[1] = checked_slack<float>(CB, zb[0], zb[1], zb[2]);
   jlast[0] = smin[0] < band ? 0 : -1;
   jlast[1] = smin[1] < band ? 0 : -1;
   int how[2] = {smin[0] < thr ? LANE_VIOLATED : LANE_REACHED_END,
@@ -380,36 +489,39 @@ __device__ __forceinline__ int run_lane_pair(const StepU<T>& K, const StepC<T>& 
   int j = 0;
   bool pair = how[0] == LANE_REACHED_END && how[1] == LANE_REACHED_END;
   bool stopA = false, stopB = false;  // candidate stopped (dead flag) while not violated
-  if (pair && j + PF <= j_end) {
-    const size_t HN = static_cast<size_t>(H) * N;
-    T r0[PF], r1[PF], r2[PF];
-    const T* pf = d + k;
+  if (pair && B <= j_end) {
+    const size_t row = 4 * static_cast<size_t>(N), comp = quad_rows(H) * row;
+    const float4* p0 = reinterpret_cast<const float4*>(d) + k;
+    const float4* p1 = reinterpret_cast<const float4*>(d + comp) + k;
+    const float4* p2 = reinterpret_cast<const float4*>(d + 2 * comp) + k;
+    float4 r0[Q], r1[Q], r2[Q];
 #pragma unroll
-    for (int u = 0; u < PF; ++u) {
-      r0[u] = __ldg(pf);
-      r1[u] = __ldg(pf + HN);
-      r2[u] = __ldg(pf + 2 * HN);
-      pf += N;
+    for (int q = 0; q < Q; ++q) {
+      r0[q] = __ldg(p0); r1[q] = __ldg(p1); r2[q] = __ldg(p2);
+      p0 += N; p1 += N; p2 += N;
     }
-    while (pair && j + PF <= j_end) {
+    while (pair && j + B <= j_end) {
       const int dA = cand_stop ? *deadA : 0, dB = cand_stop ? *deadB : 0;
-      BlockMin<T> bma, bmb;
+      const bool more = j + 2 * B <= j_end;
+      BlockMin<float> bma, bmb;
 #pragma unroll
-      for (int u = 0; u < PF; ++u) {
-        const T e0 = r0[u], e1 = r1[u], e2 = r2[u];
-        if (j + PF < j_end) {
-          r0[u] = __ldg(pf);
-          r1[u] = __ldg(pf + HN);
-          r2[u] = __ldg(pf + 2 * HN);
+      for (int q = 0; q < Q; ++q) {
+        const float e0[4] = {r0[q].x, r0[q].y, r0[q].z, r0[q].w}, e1[4] = {r1[q].x, r1[q].y, r1[q].z, r1[q].w},
+                    e2[4] = {r2[q].x, r2[q].y, r2[q].z, r2[q].w};
+        if (more) {
+          r0[q] = __ldg(p0); r1[q] = __ldg(p1); r2[q] = __ldg(p2);
         }
-        pf += N;
-        rk4_step_fast<T>(K, nullptr, CA, za[0], za[1], za[2], za[3], e0, e1, e2);
-        rk4_step_fast<T>(K, nullptr, CB, zb[0], zb[1], zb[2], zb[3], e0, e1, e2);
-        ++j;
-        bma.add(slack_of<T>(CA, za[0], za[2]), u);
-        bmb.add(slack_of<T>(CB, zb[0], zb[2]), u);
+        p0 += N; p1 += N; p2 += N;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          rk4_step_fast<float>(K, nullptr, CA, za[0], za[1], za[2], za[3], e0[u], e1[u], e2[u]);
+          rk4_step_fast<float>(K, nullptr, CB, zb[0], zb[1], zb[2], zb[3], e0[u], e1[u], e2[u]);
+          bma.add(slack_of<float>(CA, za[0], za[2]), u);
+          bmb.add(slack_of<float>(CB, zb[0], zb[2]), u);
+        }
       }
-      const T ba = bma.result(za[0], za[1], za[2]), bb = bmb.result(zb[0], zb[1], zb[2]);
+      j += B;
+      const float ba = bma.result(za[0], za[1], za[2]), bb = bmb.result(zb[0], zb[1], zb[2]);
       smin[0] = fmin(smin[0], ba);
       smin[1] = fmin(smin[1], bb);
       if (ba < band) jlast[0] = j;
@@ -439,13 +551,13 @@ __device__ __forceinline__ int run_lane_pair(const StepU<T>& K, const StepC<T>& 
   if (how[1] == LANE_REACHED_END && stopB) how[1] = LANE_STOPPED;
   if (how[0] == LANE_REACHED_END && j < j_end) {
     int e = LANE_REACHED_END;
-    smin[0] = run_lane<T, PF>(K, nullptr, CA, d, k, N, H, j, j_end, za[0], za[1], za[2], za[3], smin[0], thr,
+    smin[0] = run_lane_q(K, CA, d, k, N, H, j, j_end, za[0], za[1], za[2], za[3], smin[0], thr,
                               deadA, &extra[0], &e, band, &jlast[0]);
     how[0] = e;
   }
   if (how[1] == LANE_REACHED_END && j < j_end) {
     int e = LANE_REACHED_END;
-    smin[1] = run_lane<T, PF>(K, nullptr, CB, d, k, N, H, j, j_end, zb[0], zb[1], zb[2], zb[3], smin[1], thr,
+    smin[1] = run_lane_q(K, CB, d, k, N, H, j, j_end, zb[0], zb[1], zb[2], zb[3], smin[1], thr,
                               deadB, &extra[1], &e, band, &jlast[1]);
     how[1] = e;
   }
@@ -605,13 +717,151 @@ __device__ __forceinline__ float run_lane_ring(const StepU<float>& K, const Step
 }
 
 // ---------------------------------------------------------------------------
+// run_lane_q with the quads staged through a ring of D in shared memory, filled
+// by 16-byte asynchronous copies D quads ahead (each thread copies and reads
+// its own column, so no thread waits for another).  RING_FIGURES
+__device__ __forceinline__ void cp_async16(uint32_t smem_dst, const float4* gmem_src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ float4 ld_shared16(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
+}
+
+constexpr int kQringDepth = 8;   // quads fetched ahead
+constexpr int kQringBlock = 4;   // quads between exit tests
+// Dynamic or static shared memory of a block of THREADS lanes.
+constexpr size_t qring_bytes(int threads) { return static_cast<size_t>(3 * 16) * kQringDepth * threads; }
+
+// A lane's ring: its column in the block's ring of THREADS columns, and the
+// quads it still has to fetch.
+template <int THREADS>
+struct Qring {
+  static constexpr uint32_t kComp = THREADS * 16, kSlot = 3 * kComp;
+  uint32_t my, slot;   // the lane's column; byte offset of the next quad to read
+  int left;            // whole quads not fetched yet
+  size_t N, comp;      // in 16-byte elements
+  const float4* pf;    // next quad to fetch
+
+  // From quad j / 4 (j a multiple of 4) of scenario k, whole quads before j_end.
+  __device__ __forceinline__ Qring(void* ring, const float* d, int k, int N_, int H, int j, int j_end)
+      : my(static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + threadIdx.x * 16), slot(0u),
+        left((j_end - j) / 4), N(static_cast<size_t>(N_)), comp(quad_rows(H) * static_cast<size_t>(N_)),
+        pf(reinterpret_cast<const float4*>(d) + static_cast<size_t>(j >> 2) * static_cast<size_t>(N_) + k) {
+#pragma unroll 1
+    for (int q = 0; q < kQringDepth; ++q) fetch(my + static_cast<uint32_t>(q) * kSlot);
+  }
+  // One commit group per quad (empty past the last), so that waiting until at
+  // most kQringDepth - 1 groups are pending means the oldest quad has landed.
+  __device__ __forceinline__ void fetch(uint32_t o) {
+    if (left > 0) {
+      cp_async16(o, pf);
+      cp_async16(o + kComp, pf + comp);
+      cp_async16(o + 2 * kComp, pf + 2 * comp);
+    }
+    cp_async_commit();
+    pf += N;
+    --left;
+  }
+  // The next quad's values; first(its first step's) runs between the reads and
+  // the refill of their slot.
+  template <typename First>
+  __device__ __forceinline__ void next(float4& e0, float4& e1, float4& e2, const First& first) {
+    cp_async_wait<kQringDepth - 1>();
+    const uint32_t o = my + slot;
+    e0 = ld_shared16(o);
+    e1 = ld_shared16(o + kComp);
+    e2 = ld_shared16(o + 2 * kComp);
+    first(e0.x, e1.x, e2.x);
+    fetch(o);  // the slot is free once its values are in registers
+    slot = slot + kSlot == kQringDepth * kSlot ? 0u : slot + kSlot;
+  }
+  // Nothing in flight into the ring when the lane ends.
+  __device__ __forceinline__ void drain() { cp_async_wait<0>(); }
+};
+
+// THREADS: threads of the block (at most); ring_mem: its qring_bytes(THREADS).
+template <int THREADS, bool PACK = false>
+__device__ __forceinline__ float run_lane_qring(const StepU<float>& K, const StepC<float>& C,
+                                                const float* __restrict__ d, int k, int N, int H, int j0, int j_end,
+                                                float& q_ca, float& w, float& q_sm, float& w_abs, float smin_in,
+                                                float thr, const volatile int32_t* dead, unsigned* steps, int* end,
+                                                float band, int* jlast, void* ring_mem) {
+  constexpr int B = 4 * kQringBlock;
+  float smin = smin_in;
+  int j = j0;
+  int jl = *jlast;
+  int how = LANE_REACHED_END;
+  bool go = j < j_end;
+  if (j0 == 0) {
+    const float s0 = checked_slack<float>(C, q_ca, w, q_sm);
+    smin = fmin(smin, s0);
+    if (s0 < band) jl = 0;
+    if (s0 < thr) {
+      how = LANE_VIOLATED;
+      go = false;
+    }
+  }
+  const size_t row = 4 * static_cast<size_t>(N), comp = quad_rows(H) * row;
+  auto one = [&]() {
+    const float* p = d + static_cast<size_t>(j >> 2) * row + 4 * static_cast<size_t>(k) + (j & 3);
+    if (!lane_step_checked(K, C, __ldg(p), __ldg(p + comp), __ldg(p + 2 * comp), q_ca, w, q_sm, w_abs, j, smin, thr,
+                           band, jl)) {
+      how = LANE_VIOLATED;
+      go = false;
+    }
+  };
+  while (go && j < j_end && (j & 3) != 0) one();
+  if (go && j + B <= j_end) {
+    Qring<THREADS> ring(ring_mem, d, k, N, H, j, j_end);
+    int dead_prev = 0;  // read at the start of a block, used at the end of the next one
+    do {
+      const int dead_now = dead != nullptr ? *dead : 0;
+      BlockMin<float> bm;
+#pragma unroll
+      for (int q = 0; q < kQringBlock; ++q) {
+        float4 e0, e1, e2;
+        ring.next(e0, e1, e2, [&](float f0, float f1, float f2) {
+          lane_step<PACK>(K, C, q_ca, w, q_sm, w_abs, f0, f1, f2);
+          bm.add(slack_of<float>(C, q_ca, q_sm), 0);
+        });
+        lane_step<PACK>(K, C, q_ca, w, q_sm, w_abs, e0.y, e1.y, e2.y);
+        bm.add(slack_of<float>(C, q_ca, q_sm), 1);
+        lane_step<PACK>(K, C, q_ca, w, q_sm, w_abs, e0.z, e1.z, e2.z);
+        bm.add(slack_of<float>(C, q_ca, q_sm), 0);
+        lane_step<PACK>(K, C, q_ca, w, q_sm, w_abs, e0.w, e1.w, e2.w);
+        bm.add(slack_of<float>(C, q_ca, q_sm), 1);
+      }
+      j += B;
+      const float bmin = bm.result(q_ca, w, q_sm);
+      smin = fmin(smin, bmin);
+      if (bmin < band) jl = j;
+      if (smin < thr) {
+        how = LANE_VIOLATED;
+        go = false;
+      } else if (dead_prev != 0 && j < j_end) {
+        how = LANE_STOPPED;
+        go = false;
+      }
+      dead_prev = dead_now;
+    } while (go && j + B <= j_end);
+    ring.drain();
+  }
+  while (go && j < j_end) one();
+  *steps = static_cast<unsigned>(j - j0);
+  *end = how;
+  *jlast = jl;
+  return smin;
+}
+
+// ---------------------------------------------------------------------------
 // The trajectory loop fed by the Tensor Memory Accelerator.  Each warp owns a
 // two-stage ring of T-step chunks in shared memory; a chunk is one
 // cp.async.bulk.tensor copy of the box (32 scenarios from the warp's first,
-// T steps, 3 components) of the binary32 array [3][H][N], issued by lane 0
-// and counted on the stage's mbarrier, so a step reads its three values with
-// shared loads at fixed offsets instead of issuing three per-lane
-// asynchronous copies, their commit and wait and the address arithmetic.
+// T / 4 quads of steps, 3 components) of the handle's quad layout, issued by
+// lane 0 and counted on the stage's mbarrier, so four steps read their values
+// with three 16-byte shared loads at fixed offsets.
 // Scenarios and steps of a box beyond the array are filled with zeros by the
 // copy (the ragged last warp, the last chunk).
 //
@@ -638,7 +888,9 @@ __device__ __forceinline__ float run_lane_ring(const StepU<float>& K, const Step
 #define RRG_TMA_CHUNK 16
 #endif
 constexpr int kTmaChunk = RRG_TMA_CHUNK;
+static_assert(RRG_TMA_CHUNK % 4 == 0, "whole quads of steps");
 constexpr int kTmaStageFloats = 3 * kTmaChunk * 32;
+constexpr int kTmaComp = kTmaChunk * 32;  // floats of a component in a stage: [quad][32 scenarios][4 steps]
 constexpr unsigned kTmaStageBytes = kTmaStageFloats * 4u;
 constexpr int kTmaWaitLimit = 1 << 22;          // polls
 constexpr unsigned long long kTmaWaitNs = 100000000ull;  // and at most 0.1 s
@@ -694,7 +946,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity)
   }
   return false;
 }
-// Chunk copy: box (x = k0, y = j, z = 0) of the tensor map into `dst`,
+// Chunk copy: box (x = 4 k0, y = j / 4, z = 0) of the tensor map into `dst`,
 // completion counted on `bar` (lane 0 only).  tmap == nullptr (the test
 // switch RRG_INJECT_TMA_NO_COPY): nothing is issued, so the stage's wait runs
 // out.
@@ -705,14 +957,15 @@ __device__ __forceinline__ void tma_chunk(const void* tmap, uint32_t dst, uint32
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(k0), "r"(j), "r"(0), "r"(bar)
+      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(4 * k0), "r"(j >> 2), "r"(0), "r"(bar)
       : "memory");
 }
 
 // PACK: rk4_step_packed (the same bits).
 template <bool PACK>
 __device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC<float>& C, const void* tmap,
-                                              int k0, bool on, int j0, int j_end, float& q_ca, float& w,
+                                              const float* __restrict__ d, int k, int N, int H,
+                                              bool on, int j0, int j_end, float& q_ca, float& w,
                                               float& q_sm, float& w_abs, float smin_in, float thr,
                                               const volatile int32_t* dead, volatile int32_t* mark,
                                               unsigned* steps, int* end, float band, int* jlast,
@@ -735,7 +988,22 @@ __device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC
       if (mark != nullptr) *mark = 1;
     }
   }
-  const int nchunks = j_end > j0 ? (j_end - j0 + T - 1) / T : 0;
+  // a segment that starts inside a quad steps to its end one step at a time
+  const int k0 = k & ~31;
+  int jb = j0;  // the first chunk's step
+  for (; (jb & 3) != 0 && jb < j_end; ++jb) {
+    if (!run) continue;
+    const float* p = d + quad_index(0, jb, k, H, N);
+    const size_t comp = quad_rows(H) * 4 * static_cast<size_t>(N);
+    if (!lane_step_checked(K, C, __ldg(p), __ldg(p + comp), __ldg(p + 2 * comp), q_ca, w, q_sm, w_abs, j, smin, thr,
+                           band, jl)) {
+      how = LANE_VIOLATED;
+      run = false;
+      if (mark != nullptr) *mark = 1;
+    }
+  }
+  if (jb >= j_end) run = false;
+  const int nchunks = j_end > jb ? (j_end - jb + T - 1) / T : 0;
   if (nchunks > 0 && __any_sync(0xffffffffu, run)) {
     const uint32_t st0 = smem_u32(stages), bar0 = smem_u32(bars);
     if (lane == 0) {
@@ -745,8 +1013,8 @@ __device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC
     }
     __syncwarp();
     if (lane == 0) {
-      tma_chunk(tmap, st0, bar0, k0, j0);
-      if (nchunks > 1) tma_chunk(tmap, st0 + kTmaStageBytes, bar0 + 8u, k0, j0 + T);
+      tma_chunk(tmap, st0, bar0, k0, jb);
+      if (nchunks > 1) tma_chunk(tmap, st0 + kTmaStageBytes, bar0 + 8u, k0, jb + T);
     }
     int issued = nchunks > 1 ? 2 : 1;  // chunks whose copy was issued
     int waited = 0;                     // chunks whose copy has landed
@@ -760,18 +1028,26 @@ __device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC
         break;
       }
       waited = c + 1;
-      const float* e = stages + sg * kTmaStageFloats + lane;
-      const int nst = j_end - (j0 + c * T) < T ? j_end - (j0 + c * T) : T;
+      const float* e = stages + sg * kTmaStageFloats + 4 * lane;
+      const int nst = j_end - (jb + c * T) < T ? j_end - (jb + c * T) : T;
       const int dead_now = (run && dead != nullptr) ? *dead : 0;
       if (run) {
         if (nst == T) {
           BlockMin<float> bm;
 #pragma unroll
-          for (int u = 0; u < T; ++u) {
-            const float e0 = e[u * 32], e1 = e[(T + u) * 32], e2 = e[(2 * T + u) * 32];
-            if constexpr (PACK) rk4_step_packed(K, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
-            else rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
-            bm.add(slack_of<float>(C, q_ca, q_sm), u);
+          for (int q = 0; q < T / 4; ++q) {
+            float e0[4], e1[4], e2[4];
+            const float4 f0 = *reinterpret_cast<const float4*>(e + 128 * q),
+                         f1 = *reinterpret_cast<const float4*>(e + kTmaComp + 128 * q),
+                         f2 = *reinterpret_cast<const float4*>(e + 2 * kTmaComp + 128 * q);
+            e0[0] = f0.x; e0[1] = f0.y; e0[2] = f0.z; e0[3] = f0.w;
+            e1[0] = f1.x; e1[1] = f1.y; e1[2] = f1.z; e1[3] = f1.w;
+            e2[0] = f2.x; e2[1] = f2.y; e2[2] = f2.z; e2[3] = f2.w;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              lane_step<PACK>(K, C, q_ca, w, q_sm, w_abs, e0[u], e1[u], e2[u]);
+              bm.add(slack_of<float>(C, q_ca, q_sm), u);
+            }
           }
           j += T;
           const float bmin = bm.result(q_ca, w, q_sm);
@@ -787,13 +1063,9 @@ __device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC
           }
         } else {
           for (int u = 0; u < nst && run; ++u) {
-            const float e0 = e[u * 32], e1 = e[(T + u) * 32], e2 = e[(2 * T + u) * 32];
-            rk4_step_fast<float>(K, nullptr, C, q_ca, w, q_sm, w_abs, e0, e1, e2);
-            ++j;
-            const float sl = checked_slack<float>(C, q_ca, w, q_sm);
-            smin = fmin(smin, sl);
-            if (sl < band) jl = j;
-            if (sl < thr) {
+            const int o = 128 * (u >> 2) + (u & 3);
+            if (!lane_step_checked(K, C, e[o], e[kTmaComp + o], e[2 * kTmaComp + o], q_ca, w, q_sm, w_abs, j, smin,
+                                   thr, band, jl)) {
               how = LANE_VIOLATED;
               run = false;
               if (mark != nullptr) *mark = 1;
@@ -807,7 +1079,7 @@ __device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC
       if (c + 2 < nchunks) {
         if (lane == 0) {
           fence_proxy_async_smem();
-          tma_chunk(tmap, st0 + static_cast<uint32_t>(sg) * kTmaStageBytes, bar, k0, j0 + (c + 2) * T);
+          tma_chunk(tmap, st0 + static_cast<uint32_t>(sg) * kTmaStageBytes, bar, k0, jb + (c + 2) * T);
         }
         issued = c + 3;
       }
@@ -895,8 +1167,8 @@ __device__ __forceinline__ void tma_traj_chunk(TmaTraj& t, const StepU<float>& K
                                                const float* e, BlockMin<float>& bm) {
 #pragma unroll 8
   for (int u = 0; u < T; ++u) {
-    const float e0 = e[u * 32], e1 = e[(T + u) * 32], e2 = e[(2 * T + u) * 32];
-    rk4_step_fast<float>(K, nullptr, C, t.q_ca, t.w, t.q_sm, t.w_abs, e0, e1, e2);
+    const int o = 128 * (u >> 2) + (u & 3);
+    rk4_step_fast<float>(K, nullptr, C, t.q_ca, t.w, t.q_sm, t.w_abs, e[o], e[kTmaComp + o], e[2 * kTmaComp + o]);
     bm.add(slack_of<float>(C, t.q_ca, t.q_sm), u);
   }
 }
@@ -909,7 +1181,8 @@ __device__ __forceinline__ void tma_pair_chunk(TmaTraj& a, TmaTraj& b, const Ste
                                                BlockMin<float>& bmb) {
 #pragma unroll 8
   for (int u = 0; u < T; ++u) {
-    const float e0 = e[u * 32], e1 = e[(T + u) * 32], e2 = e[(2 * T + u) * 32];
+    const int o = 128 * (u >> 2) + (u & 3);
+    const float e0 = e[o], e1 = e[kTmaComp + o], e2 = e[2 * kTmaComp + o];
     rk4_step_fast<float>(K, nullptr, CA, a.q_ca, a.w, a.q_sm, a.w_abs, e0, e1, e2);
     rk4_step_fast<float>(K, nullptr, CB, b.q_ca, b.w, b.q_sm, b.w_abs, e0, e1, e2);
     bma.add(slack_of<float>(CA, a.q_ca, a.q_sm), u);
@@ -919,16 +1192,12 @@ __device__ __forceinline__ void tma_pair_chunk(TmaTraj& a, TmaTraj& b, const Ste
 
 // The last, partial chunk: step by step with the per-step test (run_lane's).
 __device__ __forceinline__ void tma_traj_tail(TmaTraj& t, const StepU<float>& K, const StepC<float>& C,
-                                              const float* e, int T, int nst, float thr,
-                                              float band, volatile int32_t* mark) {
+                                              const float* e, int nst, float thr, float band,
+                                              volatile int32_t* mark) {
   for (int u = 0; u < nst && t.run; ++u) {
-    const float e0 = e[u * 32], e1 = e[(T + u) * 32], e2 = e[(2 * T + u) * 32];
-    rk4_step_fast<float>(K, nullptr, C, t.q_ca, t.w, t.q_sm, t.w_abs, e0, e1, e2);
-    ++t.j;
-    const float sl = checked_slack<float>(C, t.q_ca, t.w, t.q_sm);
-    t.smin = fmin(t.smin, sl);
-    if (sl < band) t.jl = t.j;
-    if (sl < thr) {
+    const int o = 128 * (u >> 2) + (u & 3);
+    if (!lane_step_checked(K, C, e[o], e[kTmaComp + o], e[2 * kTmaComp + o], t.q_ca, t.w, t.q_sm, t.w_abs, t.j,
+                           t.smin, thr, band, t.jl)) {
       t.how = LANE_VIOLATED;
       t.run = false;
       if (mark != nullptr) *mark = 1;
@@ -978,7 +1247,7 @@ __device__ __forceinline__ void run_lane_tma_pair(const StepU<float>& K, const S
         break;
       }
       waited = c + 1;
-      const float* e = stages + sg * kTmaStageFloats + lane;
+      const float* e = stages + sg * kTmaStageFloats + 4 * lane;
       const int nst = j_end - (j0 + c * T) < T ? j_end - (j0 + c * T) : T;
       const int da = (a.run && deadA != nullptr) ? *deadA : 0;
       const int db = (b.run && deadB != nullptr) ? *deadB : 0;
@@ -997,8 +1266,8 @@ __device__ __forceinline__ void run_lane_tma_pair(const StepU<float>& K, const S
           tma_traj_chunk_end(b, bmb, T, j_end, thr, band, db, markB);
         }
       } else {
-        tma_traj_tail(a, K, CA, e, T, nst, thr, band, markA);
-        tma_traj_tail(b, K, CB, e, T, nst, thr, band, markB);
+        tma_traj_tail(a, K, CA, e, nst, thr, band, markA);
+        tma_traj_tail(b, K, CB, e, nst, thr, band, markB);
       }
       if (!__any_sync(0xffffffffu, a.run || b.run)) break;
       // every lane is done reading this stage: refill it with chunk c + 2
@@ -1048,23 +1317,30 @@ template <> __device__ __forceinline__ double draw<double>(uint64_t w, double a)
   return uniform_sym(w, a);
 }
 
-// The binary32 copy of a tile of steps j0 .. j1 - 1 of an [3][H][ld] array, the
-// thread's scenarios k0 + i blockDim.x, i < KT.
-template <int KT>
-__device__ __forceinline__ void sample_tile32(float* __restrict__ d, int N, int ld, int H, int k0, int j0,
-                                              int j1, uint64_t kbase, uint64_t upd, uint64_t seed, float s0,
-                                              float s1, float s2) {
-  const size_t HN = static_cast<size_t>(H) * ld;
-  philox_tile<KT>(kbase + static_cast<uint64_t>(k0), blockDim.x, j0, j1, upd, seed,
-                  [&](int i, int j, uint64_t w0, uint64_t w1, uint64_t w2) {
-                    const size_t k = static_cast<size_t>(k0) + static_cast<size_t>(i) * blockDim.x;
-                    if (k < static_cast<size_t>(N)) {
-                      const size_t q = static_cast<size_t>(j) * ld + k;
-                      d[q] = uniform_sym32(w0, s0);
-                      d[HN + q] = uniform_sym32(w1, s1);
-                      d[2 * HN + q] = uniform_sym32(w2, s2);
-                    }
-                  });
+// The binary32 copy of scenario k's quads q0 .. q1 - 1 (of a block's threads:
+// the same quads).  Steps past the horizon in its last quad are drawn too; no
+// trajectory reads them.
+__device__ __forceinline__ void sample_quads(float* __restrict__ d, int N, int H, int k, int q0, int q1,
+                                             uint64_t kbase, uint64_t upd, uint64_t seed, float s0, float s1,
+                                             float s2) {
+  const PhiloxCols<1> P(kbase + static_cast<uint64_t>(k), 0, upd, seed);
+  const size_t rows = quad_rows(H);
+  for (int q = q0; q < q1; ++q) {
+    float a[4], b[4], c[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      P.step(4 * q + u, [&](int, uint64_t w0, uint64_t w1, uint64_t w2) {
+        a[u] = uniform_sym32(w0, s0);
+        b[u] = uniform_sym32(w1, s1);
+        c[u] = uniform_sym32(w2, s2);
+      });
+    if (k < N) {
+      float4* o = reinterpret_cast<float4*>(d) + static_cast<size_t>(q) * N + k;
+      o[0] = make_float4(a[0], a[1], a[2], a[3]);
+      o[rows * N] = make_float4(b[0], b[1], b[2], b[3]);
+      o[2 * rows * N] = make_float4(c[0], c[1], c[2], c[3]);
+    }
+  }
 }
 
 // run_lane with the disturbances drawn from their Philox counters (j, k,
@@ -1181,6 +1457,12 @@ __device__ __forceinline__ double lane_model_pu(const Launch& L, const ScenFold&
   float* p = &F.h;
 #pragma unroll
   for (int j = 0; j < kFoldFloats - nu; ++j) p[j] = __ldg(sf.f + (nu + j) * N + k);
+  // products of the step size alone: the launch's, constant-bank operands
+  // instead of registers (16,384 x 16 x 1,000 steps: 851 -> 823 us)
+  M.U.w2n1 = L.m32.U.w2n1;
+  M.U.w3n2 = L.m32.U.w3n2;
+  M.U.w4n3 = L.m32.U.w4n3;
+  M.U.fwn4 = L.m32.U.fwn4;
   const double q_r[3] = {static_cast<double>(R.r_ca), static_cast<double>(R.r_w), static_cast<double>(R.r_sm)};
   R = round_cand(fold_cand(mc, v, q_r, L.y_min));
   M.C = step_consts<float>(M.U, F, R);
