@@ -343,6 +343,64 @@ adjoint_forward_kernel(const Launch L, const DT* __restrict__ d, int checkpoint,
   lane_arg[static_cast<size_t>(i) * N + k] = arg;
 }
 
+// The binary64 forward pass with four lanes per trajectory (Coop64): the same
+// states, minima and steps as adjoint_forward_kernel<double, double>.
+__global__ void __launch_bounds__(128)
+adjoint_forward_coop_kernel(const Launch L, const double* __restrict__ d, int checkpoint,
+                            double* __restrict__ ckpt, double* __restrict__ lane_min,
+                            int* __restrict__ lane_arg) {
+  const int i = blockIdx.y;
+  const int N = L.N, H = L.H;
+  const int kt = (blockIdx.x * blockDim.x + threadIdx.x) / 4;
+  const bool on = kt < N;
+  const int k = on ? kt : N - 1;  // a group past the scenarios keeps its warp company
+  RhsC<double> R = L.cand_c64[i];
+  LaneModel<double> M;
+  double p_atm;
+  if (L.pmul != nullptr)
+    p_atm = lane_model<double, true>(L, 0, k, L.cand_v[i], R, M);
+  else
+    p_atm = lane_model<double, false>(L, 0, k, 0.0, R, M);
+  double a, w, s, w_abs;
+  start_state<double>(R, L.st->x, p_atm, a, w, s, w_abs);
+  const Coop64 G(M.U, M.pw, L.m64.pw, M.C);
+  const int nseg = H / checkpoint + 1;
+  const size_t HN = static_cast<size_t>(H) * N;
+  double* ck = ckpt + (static_cast<size_t>(i) * N + k) * nseg * 3;
+  const bool lead = on && G.role == 0;
+  double smin = slack_of<double>(M.C, a, s);
+  int arg = 0, next_ck = 0;
+  const bool ld1 = G.role == 2, ld2 = G.role >= 2;
+  const double* p1 = d + k;
+  const double* p2 = p1 + (G.role == 2 ? 2 * HN : HN);
+  double e1 = ld1 ? __ldg(p1) : 0.0, e2 = ld2 ? __ldg(p2) : 0.0;
+  for (int j = 0; j < H; ++j) {
+    const double f1 = e1, f2 = e2;
+    p1 += N;
+    p2 += N;
+    if (j + 1 < H) {
+      if (ld1) e1 = __ldg(p1);
+      if (ld2) e2 = __ldg(p2);
+    }
+    if (j == next_ck) {
+      if (lead) {
+        double* c = ck + (j / checkpoint) * 3;
+        c[0] = a + R.r_ca;
+        c[1] = w + R.r_w;
+        c[2] = s + R.r_sm;
+      }
+      next_ck += checkpoint;
+    }
+    G.step(a, w, s, w_abs, f1, f2);
+    const double sl = G.slack(a, s);
+    if (sl < smin) { smin = sl; arg = j + 1; }
+  }
+  if (lead) {
+    lane_min[static_cast<size_t>(i) * N + k] = smin;
+    lane_arg[static_cast<size_t>(i) * N + k] = arg;
+  }
+}
+
 // Slot i = blockIdx.x: the first (k, then j) attaining the min of the
 // slot's lanes; out[i * kOutStride + 0] = g, [1], [2] = k*, j* (as long long).
 constexpr int kOutStride = kAdjOutStride;
@@ -589,7 +647,12 @@ cudaError_t launch_adjoint_forward(const Launch& L, bool fp64, int m, int checkp
     const cudaError_t er = cudaEventRecord(fwd_begin, L.stream);
     if (er != cudaSuccess) return er;
   }
-  if (fp64)
+  // four lanes per binary64 trajectory by the rollouts' rule (launch_rollout)
+  const bool coop = fp64 && L.m64.pw != nullptr && static_cast<long long>((L.N + 31) / 32) * m <= 2LL * L.sms;
+  if (coop)
+    adjoint_forward_coop_kernel<<<dim3((L.N + 7) / 8, m), 32, 0, L.stream>>>(L, L.d64, checkpoint, ckpt, lane_min,
+                                                                             lane_arg);
+  else if (fp64)
     adjoint_forward_kernel<double, double><<<grid, threads, 0, L.stream>>>(L, L.d64, checkpoint, ckpt,
                                                                            lane_min, lane_arg);
   else if (reads32(L, fp64))

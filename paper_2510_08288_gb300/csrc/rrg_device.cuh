@@ -68,14 +68,14 @@ __device__ __forceinline__ double pow_m1_table(const PowTable* __restrict__ S, d
 }
 
 // 1 / w in binary64: the hardware's approximate reciprocal (about 20 bits),
-// refined by one cubic step of the Newton family, r (1 + d + d^2) with d =
+// refined by one cubic step of the Newton family, r + d (r + d r) with d =
 // 1 - w r (error d^3): three binary64 instructions, within about one unit in
 // the last place.
 __device__ __forceinline__ double rcp_cubic(double w) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(w));
   const double d = fma_rn(-w, r, 1.0);
-  return fma_rn(r, fma_rn(d, d, d), r);
+  return fma_rn(d, fma_rn(d, r, r), r);
 }
 
 // ---------------------------------------------------------------------------

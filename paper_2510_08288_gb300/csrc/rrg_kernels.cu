@@ -374,6 +374,7 @@ enum RollSrc : int {
   SRC_RING = 1,  // an array [3][H][N] through a shared-memory ring (run_lane_ring, binary32)
   SRC_GEN = 2,   // drawn from Philox inside the trajectory loop (run_lane_gen)
   SRC_TMA = 3,   // the handle's quads through a per-warp TMA ring (run_lane_tma, binary32)
+  SRC_COOP = 5,  // an array [3][H][N], four lanes per trajectory (run_lane_coop64, binary64)
   SRC_QRING = 4  // the handle's quads through a shared-memory ring (run_lane_qring, binary32)
 };
 
@@ -449,8 +450,9 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
     return;
   }
   const int N = L.N;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = k < N;
+  constexpr int kLanes = SRC == SRC_COOP ? 4 : 1;  // lanes of a trajectory
+  const int k = (blockIdx.x * blockDim.x + threadIdx.x) / kLanes;
+  bool active = k < N;
   if (!L.cand_ss[i]) {
     // steady-state check failed: the whole row of P is 0, no rollout
     if (L.P != nullptr && active) L.P[static_cast<size_t>(i) * N + k] = 0;
@@ -520,6 +522,16 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
     const unsigned wsteps = __reduce_add_sync(0xffffffffu, steps);
     if ((threadIdx.x & 31) == 0 && wsteps)
       atomicAdd(&L.stats->lane_steps_tma, static_cast<unsigned long long>(wsteps));
+  } else if constexpr (SRC == SRC_COOP) {
+    static_assert(sizeof(T) == 8, "four lanes per trajectory: binary64");
+    const bool lane_runs = active && final_lane;
+    const T s_out = run_lane_coop64(K, M.pw, L.m64.pw, C, d, active ? k : N - 1, lane_runs, N, L.H, j0, j_end, q_ca, w, q_sm,
+                                    w_abs, smin0, thr, cand_stop ? dead : nullptr, &steps, &end, band, &jlast);
+    // the group's first lane reports it
+    active = active && (threadIdx.x & 3) == 0;
+    final_lane = final_lane && active;
+    if (lane_runs && active) smin = s_out;
+    if (!active) steps = 0;
   } else if (active && final_lane) {
     if constexpr (SRC == SRC_GEN)
       smin = run_lane_gen<T>(K, M.pw, C, L.st->src[L.st->buf], k, j0, j_end, q_ca, w, q_sm, w_abs, smin0, thr,
@@ -790,7 +802,20 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
 #define RRG_ROLLOUT(KERNEL, T, SRC, D0, D1, CAND, CLS) \
   KERNEL<T, SRC><<<grid, kRollThreads, 0, L.stream>>>(L, D0, D1, CAND, early_exit, CLS)
   if (use_fp64) {
-    if (L.pmul) {
+    // four lanes per trajectory while that leaves every scheduler at most two
+    // warps (2 x 42 binary64 instructions a step against 110); 500 steps, one
+    // lane against four: 1.83 -> 0.96 ms with one warp a scheduler, 1.83 -> 1.40
+    // with two, and a third would cost 2.0
+    const long long warps64 = static_cast<long long>((L.N + 31) / 32) * m_launch;
+    if (!L.scen_gen && L.m64.pw != nullptr && warps64 <= 2LL * sms) {
+      const dim3 g4((4 * static_cast<unsigned>(L.N) + kRollThreads - 1) / kRollThreads, m_launch);
+      if (L.pmul)
+        rollout_pu_kernel<double, SRC_COOP><<<g4, kRollThreads, 0, L.stream>>>(L, L.d64, L.d64b, L.cand_c64,
+                                                                               early_exit, 0);
+      else
+        rollout_kernel<double, SRC_COOP><<<g4, kRollThreads, 0, L.stream>>>(L, L.d64, L.d64b, L.cand_c64,
+                                                                            early_exit, 0);
+    } else if (L.pmul) {
       if (L.scen_gen) RRG_ROLLOUT(rollout_pu_kernel, double, SRC_GEN, L.d64, L.d64b, L.cand_c64, 0);
       else RRG_ROLLOUT(rollout_pu_kernel, double, SRC_REGS, L.d64, L.d64b, L.cand_c64, 0);
     } else {

@@ -1498,6 +1498,217 @@ __device__ __forceinline__ double lane_model(const Launch& L, int pair, int k, d
   }
 }
 
+// ---------------------------------------------------------------------------
+// Four lanes per binary64 trajectory.  A binary64 instruction holds a warp
+// scheduler for 64 cycles however many lanes it serves, so while there are
+// fewer warps than schedulers a trajectory's time is its instruction count.
+// The lanes 4 g .. 4 g + 3 of a warp share trajectory g: one instruction forms
+// one multiply-add of up to four rows of rk4_step_fast's combinations (R0: x
+// and w of stage 2, x of stage 1; R1: x and w of stage 3, the cathode
+// pressure; R2: x and w of stage 4, the manifold pressure, the speed), and in
+// a torque lane 0 evaluates the power, lane 1 the reciprocal and lane 2 the
+// factor it multiplies side by side: 42 instead of 110 binary64 instructions a
+// step.  Every row's operations and their order are rk4_step_fast's (a row
+// without a term adds a product with 0), so the trajectory equals the one-lane
+// form's.  The rest of a step is selects and shuffles of operands (446
+// instructions in all); a branch around the power's cell or the reciprocal
+// cost more than all lanes doing both.  Measured on GB300, a step of a lone
+// warp: 7,000 cycles one lane per trajectory, 3,850 here (42 x 64 held by the
+// pipe, the rest shuffle and select latency); 257 x 8 trajectories of 500
+// steps 1.90 -> 1.05 ms a call.
+struct Coop64 {
+  int role, lane0;  // lane in its group, the group's first lane
+  int src1, src2, srcp;  // lane each operand comes from: its own or another's of the group
+  uint32_t neg1, neg2;   // sign flips of lane 1's and lane 2's products
+  bool live = true;      // false: the group's values are not read (no power off the table for them)
+  double r_w, e, A, B, cv;           // r_w: lane 2's, 0 elsewhere
+  double k0[3], k1[3], k2[3];        // rows of (a, s, w)
+  double c0, c1, c2;                 // their constants
+  double n10, n11, n12, n21, n22, n32, n42;
+  double y_scale, s_off;
+  const PowCell* cells;
+  bool table;
+
+  // cells: a table; pw: the trajectory's (nullptr: its exponent has none).
+  __device__ __forceinline__ Coop64(const StepU<double>& U, const PowTable* pw, const PowTable* any,
+                                    const StepC<double>& C)
+      : role(static_cast<int>(threadIdx.x & 3)), lane0(static_cast<int>(threadIdx.x & 28)), e(U.e), A(U.A),
+        B(U.B), y_scale(C.y_scale), s_off(C.s_off), cells(any->cell), table(pw != nullptr) {
+    auto pick = [&](double v0, double v1, double v2, double v3) {
+      return role == 0 ? v0 : role == 1 ? v1 : role == 2 ? v2 : v3;
+    };
+    src1 = role == 1 ? lane0 + 1 : lane0;
+    src2 = role == 2 ? lane0 + 1 : lane0 + role;
+    srcp = role == 2 ? lane0 + 3 : lane0 + role;
+    neg1 = role == 1 ? 0x80000000u : 0u;
+    neg2 = role == 2 ? 0x80000000u : 0u;
+    r_w = pick(0.0, 0.0, C.r_w, 0.0);
+    cv = pick(-1.0, 1.0, -U.B, 0.0);
+    k0[0] = pick(U.x2a, 0.0, 0.0, 0.0);
+    k0[1] = pick(U.x2s, U.w2s, U.ip, 0.0);
+    k0[2] = pick(U.x2w, U.w2w, 0.0, 0.0);
+    c0 = pick(C.x2, C.w2, C.x1, 0.0);
+    k1[0] = pick(U.x3a, U.w3a, U.faa, 0.0);
+    k1[1] = pick(U.x3s, U.w3s, U.fas, 0.0);
+    k1[2] = pick(U.x3w, U.w3w, U.faw, 0.0);
+    c1 = pick(C.x3, C.w3, C.fa, 0.0);
+    k2[0] = pick(U.x4a, U.w4a, U.fsa, U.fwa);
+    k2[1] = pick(U.x4s, U.w4s, U.fss, U.fws);
+    k2[2] = pick(U.x4w, U.w4w, U.fsw, U.fww);
+    c2 = pick(C.x4, C.w4, C.fs, C.fw);
+    n10 = pick(0.0, U.w2n1, 0.0, 0.0);
+    n11 = pick(U.x3n1, U.w3n1, U.fan1, 0.0);
+    n12 = pick(U.x4n1, U.w4n1, U.fsn1, U.fwn1);
+    n21 = pick(0.0, U.w3n2, U.fan2, 0.0);
+    n22 = pick(U.x4n2, U.w4n2, U.fsn2, U.fwn2);
+    n32 = pick(0.0, U.w4n3, U.fsn3, U.fwn3);
+    n42 = U.fwn4;
+  }
+  __device__ __forceinline__ static double get(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+  __device__ __forceinline__ static double flip(double v, uint32_t sign) {
+    return __hiloint2double(__double2hiint(v) ^ static_cast<int>(sign), __double2loint(v));
+  }
+  // N(x, w) in every lane; X: w in lane 1, x in the others.
+  __device__ __forceinline__ double torque4(double X) const {
+    const int hi = __double2hiint(X);
+    const bool in = table && (hi >> 20) == 0x3ff;
+    // pow_m1_table's cell (some cell when x is off the table)
+    const PowCell* __restrict__ c = cells + ((hi >> 11) & (kPowCells - 1));
+    const double2 ia = __ldg(reinterpret_cast<const double2*>(c));
+    const double2 a12 = __ldg(reinterpret_cast<const double2*>(c) + 1);
+    const float4 f = __ldg(reinterpret_cast<const float4*>(c) + 2);
+    double r0;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(X));
+    const uint32_t b = (static_cast<uint32_t>(hi) & 0xfffffu) << 3 |
+                       static_cast<uint32_t>(__double2loint(X)) >> 29;
+    const float tf = fma_rn(__uint_as_float(0x3f800000u | b), f.w, -1.0f);
+    const double p3 = widen_bits(fma_rn(fma_rn(f.z, tf, f.y), tf, f.x));
+    const bool l1 = role == 1, l2 = role == 2;
+    const double v1 = fma_rn(flip(X, neg1), l1 ? r0 : l2 ? B : ia.x, cv);
+    const double v2 = fma_rn(v1, l1 ? r0 : p3, l1 ? r0 : a12.y);
+    const double v3 = fma_rn(v1, v2, l1 ? r0 : a12.x);
+    double v4 = fma_rn(flip(v1, neg2), get(v3, src2), l2 ? A : ia.y);
+    if (__any_sync(0xffffffffu, !in && live && role == 0)) {
+      if (!in && role == 0) v4 = pow(X, e) - 1.0;
+      __syncwarp();
+    }
+    return get(v4, lane0) * get(v4, lane0 + 2);
+  }
+  // One step; every lane of the group holds the state.  e1, e2: lane 2's are
+  // the cathode and manifold pressure's disturbance, lane 3's e2 the speed's,
+  // the others 0.
+  __device__ __forceinline__ void step(double& a, double& w, double& s, double& w_abs, double e1, double e2) const {
+    double R0 = fma_rn(k0[2], w, fma_rn(k0[1], s, fma_rn(k0[0], a, c0)));  // lane 2: x of stage 1
+    const double x = get(R0, lane0 + 2);
+    const double n1 = torque4(role == 1 ? w_abs : x);
+    double R1 = fma_rn(k1[2], w, fma_rn(k1[1], s, fma_rn(k1[0], a, e1 + c1)));
+    double R2 = fma_rn(k2[2], w, fma_rn(k2[1], s, fma_rn(k2[0], a, e2 + c2)));
+    R0 = fma_rn(n10, n1, R0);
+    const double n2 = torque4(get(R0, src1));
+    R1 = fma_rn(n11, n1, R1);
+    R2 = fma_rn(n12, n1, R2);
+    R1 = fma_rn(n21, n2, R1);
+    const double n3 = torque4(get(R1, src1));
+    R2 = fma_rn(n22, n2, R2);
+    R2 = fma_rn(n32, n3, R2);
+    const double n4 = torque4(get(R2, src1));
+    const double V = fma_rn(n42, n4, get(R2, srcp) + r_w);
+    a = get(R1, lane0 + 2);
+    s = get(R2, lane0 + 2);
+    w = get(V, lane0 + 3);
+    w_abs = get(V, lane0 + 2);
+  }
+  __device__ __forceinline__ double slack(double a, double s) const { return fma_rn(y_scale, s - a, s_off); }
+};
+
+// run_lane<double> for a group of four lanes (called by every lane of the warp;
+// on = false: the group only keeps the warp company).  The warp steps together
+// while any of its groups runs; one that has stopped keeps stepping without
+// recording.  Same contract and results as run_lane, in blocks of four steps.
+__device__ __forceinline__ double run_lane_coop64(const StepU<double>& U, const PowTable* pw, const PowTable* any,
+                                                  const StepC<double>& C,
+                                                  const double* __restrict__ d, int k, bool on, int N, int H,
+                                                  int j0, int j_end, double& q_ca, double& w, double& q_sm,
+                                                  double& w_abs, double smin_in, double thr,
+                                                  volatile int32_t* dead, unsigned* steps, int* end,
+                                                  double band, int* jlast) {
+  constexpr int B = 4;
+  Coop64 G(U, pw, any, C);
+  double smin = smin_in;
+  int j = j0, j_stop = j0, jl = *jlast, how = LANE_REACHED_END;
+  bool run = on && j0 < j_end;
+  if (on && j0 == 0) {
+    const double s0 = checked_slack<double>(C, q_ca, w, q_sm);
+    smin = fmin(smin, s0);
+    if (s0 < band) jl = 0;
+    if (s0 < thr) {
+      how = LANE_VIOLATED;
+      run = false;
+    }
+  }
+  const size_t HN = static_cast<size_t>(H) * N;
+  const bool ld1 = on && G.role == 2, ld2 = on && G.role >= 2;
+  const double* p1 = d + static_cast<size_t>(j0) * N + k;
+  const double* p2 = p1 + (G.role == 2 ? 2 * HN : HN);
+  double a = q_ca, v = w, s = q_sm, va = w_abs;
+  double e1 = ld1 && j0 < j_end ? __ldg(p1) : 0.0, e2 = ld2 && j0 < j_end ? __ldg(p2) : 0.0;
+  auto one = [&]() {  // a step, the next one's disturbances on their way
+    const double f1 = e1, f2 = e2;
+    p1 += N;
+    p2 += N;
+    if (j + 1 < j_end) {
+      if (ld1) e1 = __ldg(p1);
+      if (ld2) e2 = __ldg(p2);
+    }
+    G.step(a, v, s, va, f1, f2);
+    ++j;
+  };
+  while (j + B <= j_end && __any_sync(0xffffffffu, run)) {
+    const int dead_now = (run && dead != nullptr) ? *dead : 0;
+    G.live = run;
+    BlockMin<double> bm;
+#pragma unroll 2
+    for (int u = 0; u < B; ++u) {
+      one();
+      bm.add(G.slack(a, s), u);
+    }
+    if (run) {
+      const double bmin = bm.result(a, v, s);
+      smin = fmin(smin, bmin);
+      if (bmin < band) jl = j;
+      j_stop = j;
+      q_ca = a; w = v; q_sm = s; w_abs = va;
+      if (smin < thr) {
+        how = LANE_VIOLATED;
+        run = false;
+        if (dead != nullptr && G.role == 0) *dead = 1;  // the warp's other groups leave at their next look
+      } else if (dead_now != 0 && j < j_end) {
+        how = LANE_STOPPED;
+        run = false;
+      }
+    }
+  }
+  while (j < j_end && __any_sync(0xffffffffu, run)) {
+    G.live = run;
+    one();
+    if (run) {
+      const double sl = checked_slack<double>(C, a, v, s);
+      smin = fmin(smin, sl);
+      if (sl < band) jl = j;
+      j_stop = j;
+      q_ca = a; w = v; q_sm = s; w_abs = va;
+      if (sl < thr) {
+        how = LANE_VIOLATED;
+        run = false;
+      }
+    }
+  }
+  *steps = static_cast<unsigned>(j_stop - j0);
+  *end = how;
+  *jlast = jl;
+  return smin;
+}
+
 // Warp minimum in the lane's own precision (a binary32 lane's value needs no
 // binary64 shuffles or compares on GB300's narrow binary64 pipe).
 template <typename T>
