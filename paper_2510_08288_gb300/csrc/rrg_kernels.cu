@@ -372,8 +372,10 @@ cudaError_t launch_mark64(const Launch& L) {
 enum RollSrc : int {
   SRC_REGS = 0,  // an array [3][H][N] through a register prefetch ring (run_lane)
   SRC_RING = 1,  // an array [3][H][N] through a shared-memory ring (run_lane_ring, binary32)
-  SRC_GEN = 2,   // drawn from Philox inside the trajectory loop (run_lane_gen)
+  SRC_GEN = 2,   // drawn from Philox inside the trajectory loop (run_lane_gen, binary64)
   SRC_TMA = 3,   // the handle's quads through a per-warp TMA ring (run_lane_tma, binary32)
+  SRC_GEN4 = 6,  // drawn by the block's warps for each other (run_lane_gen_shared, binary32):
+  SRC_GEN8 = 7,  //   4 candidates and 4 drawing warps; 8 candidates that draw themselves
   SRC_COOP = 5,  // an array [3][H][N], four lanes per trajectory (run_lane_coop64, binary64)
   SRC_QRING = 4  // the handle's quads through a shared-memory ring (run_lane_qring, binary32)
 };
@@ -438,25 +440,41 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
                                              const void* tm1 = nullptr) {
   const T* __restrict__ d = L.st->buf ? d_pair1 : d_pair0;
   const Seg s0 = L.st->seg[0], s1 = L.st->seg[1];
-  const int y = blockIdx.y;
+  // SRC_GEN4, SRC_GEN8: a block's warps are candidates of one segment; a warp
+  // without one (or whose candidate is done) only draws (`idle`)
+  constexpr bool SH = SRC == SRC_GEN4 || SRC == SRC_GEN8;
+  constexpr int kGenRows = SRC == SRC_GEN4 ? 4 : 8;
+  bool idle = false;
+  const int row = SH ? static_cast<int>(threadIdx.x >> 5) : 0;
+  const bool spare = SH && row >= kGenRows;  // a warp that only draws
+  const int y = SH ? blockIdx.y * kGenRows + (spare ? 0 : row) : blockIdx.y;
+  const int y1 = SH ? (s0.count + kGenRows - 1) / kGenRows * kGenRows : s0.count;  // the second segment's first row
   int mode, i;
-  if (y < s0.count) {
+  if (y < y1) {
+    idle = SH && y >= s0.count;
     mode = s0.mode;
-    i = mode == SEG_CONTINUE ? L.st->cont_slot[y] : s0.base + y;
-  } else if (y - s0.count < s1.count) {
+    i = idle ? 0 : mode == SEG_CONTINUE ? L.st->cont_slot[y] : s0.base + y;
+  } else if (y - y1 < s1.count) {
     mode = s1.mode;
-    i = s1.base + (y - s0.count);
+    i = s1.base + (y - y1);
+  } else if (SH) {
+    idle = true;
+    mode = s1.mode;
+    i = 0;
   } else {
     return;
   }
+  idle = idle || spare;
   const int N = L.N;
   constexpr int kLanes = SRC == SRC_COOP ? 4 : 1;  // lanes of a trajectory
-  const int k = (blockIdx.x * blockDim.x + threadIdx.x) / kLanes;
-  bool active = k < N;
+  const int k = SH ? blockIdx.x * 32 + (threadIdx.x & 31) : (blockIdx.x * blockDim.x + threadIdx.x) / kLanes;
+  bool active = k < N && !idle;
   if (!L.cand_ss[i]) {
     // steady-state check failed: the whole row of P is 0, no rollout
     if (L.P != nullptr && active) L.P[static_cast<size_t>(i) * N + k] = 0;
-    return;
+    if (!SH) return;
+    idle = true;
+    active = false;
   }
   volatile int32_t* dead = L.cand_dead + i;
   const bool cand_stop = early_exit == RRG_EXIT_CANDIDATE;
@@ -464,7 +482,11 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
     // another block may already have found a violation; read once per warp so
     // the warp leaves (or stays) as a whole before the warp reductions below
     const int dead0 = __shfl_sync(0xffffffffu, (threadIdx.x & 31) == 0 ? *dead : 0, 0);
-    if (dead0) return;
+    if (dead0) {
+      if (!SH) return;
+      idle = true;
+      active = false;
+    }
   }
   RhsC<T> R = cand[i];
   LaneModel<T> M;
@@ -522,6 +544,16 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
     const unsigned wsteps = __reduce_add_sync(0xffffffffu, steps);
     if ((threadIdx.x & 31) == 0 && wsteps)
       atomicAdd(&L.stats->lane_steps_tma, static_cast<unsigned long long>(wsteps));
+  } else if constexpr (SH) {
+    static_assert(sizeof(T) == 4, "the shared draw is binary32");
+    using G = GenShape<kGenRows, SRC == SRC_GEN4>;
+    __shared__ __align__(16) float drawn[2 * 3 * G::kComp];
+    const bool lane_runs = active && final_lane;
+    const T s_out = run_lane_gen_shared<kGenRows, SRC == SRC_GEN4, PU>(K, C, L.st->src[L.st->buf], k, lane_runs, j0, j_end, q_ca, w, q_sm, w_abs,
+                                            smin0, thr, cand_stop ? dead : nullptr, &steps, &end, band, &jlast,
+                                            drawn);
+    if (idle) return;
+    if (lane_runs) smin = s_out;
   } else if constexpr (SRC == SRC_COOP) {
     static_assert(sizeof(T) == 8, "four lanes per trajectory: binary64");
     const bool lane_runs = active && final_lane;
@@ -567,9 +599,12 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
   reduce_lane<T>(L, i, k, N, final_lane, smin, steps, jlast, classify, eps, dead);
 }
 
+constexpr int roll_threads(int src) { return src == SRC_GEN4 || src == SRC_GEN8 ? 256 : kRollThreads; }
+static_assert(GenShape<4, true>::kThreads == 256 && GenShape<8, false>::kThreads == 256, "roll_threads");
+
 // SRC: where the lanes take their disturbances from (RollSrc).
 template <typename T, int SRC>
-__global__ void __launch_bounds__(kRollThreads)
+__global__ void __launch_bounds__(roll_threads(SRC))
 rollout_kernel(const Launch L, const T* __restrict__ d_pair0, const T* __restrict__ d_pair1,
                const RhsC<T>* __restrict__ cand, int early_exit, int classify) {
   rollout_body<T, false, SRC>(L, d_pair0, d_pair1, cand, early_exit, classify);
@@ -584,7 +619,7 @@ rollout_kernel(const Launch L, const T* __restrict__ d_pair0, const T* __restric
 #define RRG_PU_MIN_BLOCKS 4
 #endif
 template <typename T, int SRC>
-__global__ void __launch_bounds__(kRollThreads, sizeof(T) == 4 ? RRG_PU_MIN_BLOCKS : 1)
+__global__ void __launch_bounds__(roll_threads(SRC), sizeof(T) == 4 ? RRG_PU_MIN_BLOCKS * kRollThreads / roll_threads(SRC) : 1)
 rollout_pu_kernel(const Launch L, const T* __restrict__ d_pair0, const T* __restrict__ d_pair1,
                   const RhsC<T>* __restrict__ cand, int early_exit, int classify) {
   rollout_body<T, true, SRC>(L, d_pair0, d_pair1, cand, early_exit, classify);
@@ -858,16 +893,31 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
       rollout_pair_kernel<false><<<g2, kRollThreads, 0, L.stream>>>(L, L.d32, L.d32b, L.cand_c32,
                                                                     early_exit, cls);
   } else {
-    if (L.pmul) {
-      if (L.scen_gen) RRG_ROLLOUT(rollout_pu_kernel, float, SRC_GEN, L.d32, L.d32b, L.cand_c32, cls);
-      else RRG_ROLLOUT(rollout_pu_kernel, float, SRC_QRING, L.d32, L.d32b, L.cand_c32, cls);
+    // Drawn disturbances: four drawing warps beside four candidates while that
+    // leaves at most one block per SM, else eight candidates that draw for
+    // themselves (1,000 steps of 1,000 scenarios: 16 candidates, 128 blocks of
+    // the first form 122 against 191 us; 24 candidates 204 against 190).  Two
+    // segments, each in whole blocks.
+    const long long tiles = (L.N + 31) / 32;
+    const bool gen8 = tiles * ((m_launch + 3) / 4) > sms;
+    const int gr = gen8 ? 8 : 4;
+    const dim3 gs(static_cast<unsigned>(tiles), (m_launch + gr - 1) / gr + 1);
+#define RRG_ROLLOUT_GEN(KERNEL, SRC) \
+  KERNEL<float, SRC><<<gs, roll_threads(SRC), 0, L.stream>>>(L, L.d32, L.d32b, L.cand_c32, early_exit, cls)
+    if (L.scen_gen) {
+      if (L.pmul && gen8) RRG_ROLLOUT_GEN(rollout_pu_kernel, SRC_GEN8);
+      else if (L.pmul) RRG_ROLLOUT_GEN(rollout_pu_kernel, SRC_GEN4);
+      else if (gen8) RRG_ROLLOUT_GEN(rollout_kernel, SRC_GEN8);
+      else RRG_ROLLOUT_GEN(rollout_kernel, SRC_GEN4);
+    } else if (L.pmul) {
+      RRG_ROLLOUT(rollout_pu_kernel, float, SRC_QRING, L.d32, L.d32b, L.cand_c32, cls);
     } else {
-      if (L.scen_gen) RRG_ROLLOUT(rollout_kernel, float, SRC_GEN, L.d32, L.d32b, L.cand_c32, cls);
-      else if (L.quads) RRG_ROLLOUT(rollout_kernel, float, SRC_QRING, L.d32, L.d32b, L.cand_c32, cls);
+      if (L.quads) RRG_ROLLOUT(rollout_kernel, float, SRC_QRING, L.d32, L.d32b, L.cand_c32, cls);
       else if (ring) RRG_ROLLOUT(rollout_kernel, float, SRC_RING, L.d32, L.d32b, L.cand_c32, cls);
       else RRG_ROLLOUT(rollout_kernel, float, SRC_REGS, L.d32, L.d32b, L.cand_c32, cls);
     }
   }
+#undef RRG_ROLLOUT_GEN
 #undef RRG_ROLLOUT
   return cudaGetLastError();
 }

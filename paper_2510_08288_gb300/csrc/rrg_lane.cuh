@@ -1412,6 +1412,124 @@ __device__ __forceinline__ T run_lane_gen(const StepU<T>& K, const PowTable* pw,
   return smin;
 }
 
+// Binary32 lanes whose disturbances are drawn, not stored.  A draw costs three
+// times a step's instructions (15 64-bit products), and every candidate of a
+// scenario takes the same one: ROWS warps of a block run different candidates
+// of the same 32 scenarios and share it.  A chunk is 4 ROWS steps in one of two
+// shared buffers; a quad of the next chunk is drawn by each of the ROWS warps
+// themselves, or (SPLIT) by each of ROWS further warps, which fills the gaps of
+// a step's dependent chain while there are few warps on an SM.  One barrier a
+// chunk.  Measured on GB300, 1,000 steps of 1,000 scenarios and 1 / 16 / 64
+// candidates, every lane drawing for itself: 319 / 322 / 921 us; here 119 /
+// 122 / 313 us.
+// Same contract, values and decisions as run_lane_gen; exits are taken at the
+// end of each 16 steps, and a lane that violates marks `dead` at once.  Called
+// by every thread of the block; on = false: the lane only draws.
+template <int ROWS, bool SPLIT>
+struct GenShape {
+  static constexpr int kRows = ROWS, kThreads = 32 * ROWS * (SPLIT ? 2 : 1);
+  static constexpr int kSteps = 4 * ROWS, kComp = 32 * kSteps;  // steps of a chunk, floats of a component
+};
+template <int ROWS, bool SPLIT, bool PACK>
+__device__ __forceinline__ float run_lane_gen_shared(const StepU<float>& K, const StepC<float>& C, const ScenSrc& src,
+                                                     int k, bool on, int j0, int j_end, float& q_ca, float& w,
+                                                     float& q_sm, float& w_abs, float smin_in, float thr,
+                                                     volatile int32_t* dead, unsigned* steps, int* end, float band,
+                                                     int* jlast, float* buf) {
+  constexpr int kSteps = GenShape<ROWS, SPLIT>::kSteps, kComp = GenShape<ROWS, SPLIT>::kComp;
+  const int lane = threadIdx.x & 31, quad = static_cast<int>(threadIdx.x >> 5) - (SPLIT ? ROWS : 0);
+  float smin = smin_in;
+  int j = j0, jl = *jlast, how = LANE_REACHED_END;
+  bool run = on && j0 < j_end;
+  if (on && j0 == 0) {
+    const float s0 = checked_slack<float>(C, q_ca, w, q_sm);
+    smin = fmin(smin, s0);
+    if (s0 < band) jl = 0;
+    if (s0 < thr) {
+      how = LANE_VIOLATED;
+      run = false;
+      if (dead != nullptr) *dead = 1;
+    }
+  }
+  const PhiloxCols<1> P(src.base + static_cast<uint64_t>(k), 0, src.update, src.seed);
+  const float a0 = static_cast<float>(src.amp[0] * 0x1.0p-23), a1 = static_cast<float>(src.amp[1] * 0x1.0p-23),
+              a2 = static_cast<float>(src.amp[2] * 0x1.0p-23);
+  auto fill = [&](int jc, float* b) {  // this warp's quad of the chunk that starts at jc
+    const int jq = jc + 4 * quad;
+    if (quad < 0 || jq >= j_end) return;
+    float e0[4], e1[4], e2[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      P.step(jq + u, [&](int, uint64_t w0, uint64_t w1, uint64_t w2) {
+        e0[u] = uniform_sym32(w0, a0);
+        e1[u] = uniform_sym32(w1, a1);
+        e2[u] = uniform_sym32(w2, a2);
+      });
+    float4* o = reinterpret_cast<float4*>(b + 128 * quad + 4 * lane);
+    o[0] = make_float4(e0[0], e0[1], e0[2], e0[3]);
+    o[kComp / 4] = make_float4(e1[0], e1[1], e1[2], e1[3]);
+    o[kComp / 2] = make_float4(e2[0], e2[1], e2[2], e2[3]);
+  };
+  if (__syncthreads_or(run)) {
+    fill(j0, buf);
+    __syncthreads();
+    for (int jc = j0, sg = 0; jc < j_end; jc += kSteps, sg ^= 1) {
+      if (jc + kSteps < j_end) fill(jc + kSteps, buf + (sg ^ 1) * 3 * kComp);
+#pragma unroll 1
+      for (int h = 0; h < kSteps / 16; ++h) {
+        const float* e = buf + sg * 3 * kComp + h * 512 + 4 * lane;
+        const int left = j_end - (jc + 16 * h);
+        const int dead_now = (run && dead != nullptr) ? *dead : 0;
+        if (run && left >= 16) {
+          BlockMin<float> bm;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            float e0[4], e1[4], e2[4];
+            const float4 f0 = *reinterpret_cast<const float4*>(e + 128 * q),
+                         f1 = *reinterpret_cast<const float4*>(e + kComp + 128 * q),
+                         f2 = *reinterpret_cast<const float4*>(e + 2 * kComp + 128 * q);
+            e0[0] = f0.x; e0[1] = f0.y; e0[2] = f0.z; e0[3] = f0.w;
+            e1[0] = f1.x; e1[1] = f1.y; e1[2] = f1.z; e1[3] = f1.w;
+            e2[0] = f2.x; e2[1] = f2.y; e2[2] = f2.z; e2[3] = f2.w;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              lane_step<PACK>(K, C, q_ca, w, q_sm, w_abs, e0[u], e1[u], e2[u]);
+              bm.add(slack_of<float>(C, q_ca, q_sm), u);
+            }
+          }
+          j += 16;
+          const float bmin = bm.result(q_ca, w, q_sm);
+          smin = fmin(smin, bmin);
+          if (bmin < band) jl = j;
+          if (smin < thr) {
+            how = LANE_VIOLATED;
+            run = false;
+            if (dead != nullptr) *dead = 1;
+          } else if (dead_now != 0 && j < j_end) {
+            how = LANE_STOPPED;
+            run = false;
+          }
+        } else if (run) {
+          for (int u = 0; u < left && run; ++u) {
+            const int o = 128 * (u >> 2) + (u & 3);
+            if (!lane_step_checked(K, C, e[o], e[kComp + o], e[2 * kComp + o], q_ca, w, q_sm, w_abs, j, smin,
+                                   thr, band, jl)) {
+              how = LANE_VIOLATED;
+              run = false;
+              if (dead != nullptr) *dead = 1;
+            }
+          }
+        }
+      }
+      if (!__syncthreads_or(run)) break;
+    }
+  }
+  *steps = static_cast<unsigned>(j - j0);
+  *end = how;
+  *jlast = jl;
+  return smin;
+}
+
 // Scenario k's model under parametric uncertainty: the parameters theta_p
 // m_p^k folded like the nominal ones (the step of size dt included).
 __device__ __forceinline__ void scenario_fold(const double* __restrict__ P, const double* __restrict__ m_k,
