@@ -63,7 +63,7 @@ struct BState {
 struct BCfg {
   int S, M, n_rounds, search, ss_check, early_exit;
   int n_bisect, width;  // speculative bisection: N_kappa, tree nodes per round (<= M)
-  double dt, y_min, eps_ss, y_c, eps_abs;
+  double dt, y_min, eps_abs;
   double amp[3];
 };
 
@@ -73,6 +73,7 @@ struct BLaunch {
   const double* params;
   Fc3K<double> k64;
   Fc3K<float> k32;
+  EqModel eq;
   StepModel<double> m64;
   StepModel<float> m32;
   const BInst* inst;
@@ -327,8 +328,7 @@ __global__ void batch_prepare_kernel(const BLaunch B) {
   const size_t slot = static_cast<size_t>(s) * M + i;
   const double v = governed(st.v_prev, st.r, B.cand_kappa[slot]);
   B.cand_v[slot] = v;
-  const double thr = __dadd_rn(B.c.y_min, __dmul_rn(B.c.eps_ss, __dsub_rn(B.c.y_c, B.c.y_min)));
-  const int ok = candidate_setup(B.k64, B.k32, B.m64.c, B.params, v, B.c.ss_check, thr, B.c.y_min,
+  const int ok = candidate_setup(B.k64, B.k32, B.eq, B.m64.c, B.params, v, B.c.ss_check, B.c.y_min,
                                  B.cand_c64 + slot, B.cand_c32 + slot);
   B.cand_ok[slot] = ok;
   B.cand_ss[slot] = ok;
@@ -1326,14 +1326,13 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   B.c.early_exit = cfg->early_exit;
   B.c.dt = cfg->dt;
   B.c.y_min = cfg->y_min;
-  B.c.eps_ss = cfg->eps_ss;
-  B.c.y_c = cfg->y_c;
   B.c.eps_abs = cfg->recheck_eps_rel * std::fabs(cfg->y_min);
   for (int i = 0; i < 3; ++i) B.c.amp[i] = cfg->dist_amp[i];
   B.params = h->params_dev;
   fold_constants(h->params, &B.k64, &B.k32);
   B.k64.pws = pws_ok ? h->pws : nullptr;
   fold_model(B.k64, h->params, cfg->dt, &B.m64);
+  fold_eq(h->params, cfg->y_min, cfg->eps_ss, cfg->y_c, &B.eq);
   round_model(B.m64, &B.m32);
   B.inst = h->inst_dev;
   B.order = h->order_dev;

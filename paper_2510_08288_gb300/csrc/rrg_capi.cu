@@ -302,6 +302,7 @@ void fill_launch(rrg_ctx* h) {
   fold_constants(h->params, &L.k64, &L.k32);
   L.k64.pws = h->pws_ok ? h->pws : nullptr;
   fold_model(L.k64, h->params, c.dt, &L.m64);
+  fold_eq(h->params, c.y_min, c.eps_ss, c.y_c, &L.eq);
   round_model(L.m64, &L.m32);
   L.d64 = h->d64;
   L.quads = 1;
@@ -382,10 +383,10 @@ int enqueue_round_work(rrg_ctx* h, const Launch& L, int width, int early_exit, b
 // The standard rounds that follow a pipelined pair (they finish the search,
 // after a wrong provisional outcome or when more levels remain; no-ops
 // otherwise).
-int enqueue_extra_rounds(rrg_ctx* h, double* d_vt, double* d_kappa, int32_t* d_flags) {
+int enqueue_extra_rounds(rrg_ctx* h, int extra, double* d_vt, double* d_kappa, int32_t* d_flags) {
   const Launch& L = h->L;
   const SearchCfg& c = h->scfg;
-  const int extra = search_extra_rounds(c), wx = search_extra_width(c);
+  const int wx = search_extra_width(c);
   for (int r = 0; r < extra; ++r) {
     int rc = enqueue_round_work(h, L, wx, h->cfg.early_exit);
     if (rc != RRG_OK) return rc;
@@ -427,7 +428,7 @@ int enqueue_search(rrg_ctx* h, const double* d_x, const double* d_r,
     h->rounds++;
     // after a wrong provisional outcome the search resumes from the level
     // where it went wrong; these rounds do nothing when it went right
-    return with_extra ? enqueue_extra_rounds(h, d_vt, d_kappa, d_flags) : RRG_OK;
+    return with_extra ? enqueue_extra_rounds(h, search_extra_rounds(c), d_vt, d_kappa, d_flags) : RRG_OK;
   }
   for (int r = r0; r < R; ++r) {
     const int width = search_round_width(c, r);
@@ -517,7 +518,7 @@ cudaGraph_t capture_conditional_update(rrg_ctx* h, uint64_t seed, uint64_t t0, c
     cudaGraph_t body = ok ? cp.conditional.phGraph_out[0] : nullptr;
     if (ok) ok = cudaStreamBeginCaptureToGraph(h->stream, body, nullptr, nullptr, 0, mode) == cudaSuccess;
     if (ok) {
-      ok = enqueue_extra_rounds(h, nullptr, nullptr, nullptr) == RRG_OK;
+      ok = enqueue_extra_rounds(h, search_extra_rounds(h->scfg), nullptr, nullptr, nullptr) == RRG_OK;
       ok = (cudaStreamEndCapture(h->stream, &body) == cudaSuccess) && ok;
     }
   }
@@ -844,8 +845,6 @@ int rrg_create(const double* model_params, int n_params, const rrg_config* cfg, 
   s.ss_check = c.ss_check;
   s.probe_steps = c.search == RRG_SEARCH_SPEC_BISECT ? c.probe_steps : 0;
   s.y_min = c.y_min;
-  s.eps_ss = c.eps_ss;
-  s.y_c = c.y_c;
   // occupancy of the paired kernel and the TMA kernels' shared-memory limit,
   // set once here (never inside a capture)
   (void)pair_blocks_per_sm(false);
@@ -1039,8 +1038,10 @@ int rrg_slack_error(rrg_handle h, const double* x_t, double v_prev, double r_t,
 }
 
 // The search of rrg_step, captured once on the handle's fixed io pointers:
-// with a pipelined search the rounds after the pipelined pair sit in a
-// conditional node (as in the closed-loop graph), else, or if the graph API
+// with a pipelined search the rounds after the pipelined pair are a while node
+// whose body is one round (so none runs after the search is done: a control
+// tick of 32 scenarios that needs one of the three takes 130 us, 133 with all
+// three in an if node), else, or if the graph API
 // refuses a step, the plain sequence.  Sets the host counters one replay adds
 // (the conditional body's are added on the device when it runs); nullptr if
 // nothing could be captured.
@@ -1067,7 +1068,8 @@ cudaGraphExec_t capture_step(rrg_ctx* h) {
     if (ok) {
       h->capturing = true;
       h->L.cond = hc;
-      extra_round_counts(h, &h->L.cond_launches, &h->L.cond_rollouts, &h->L.cond_rounds);
+      h->L.cond_launches = h->cfg.precision == RRG_FP32_RECHECK ? 3u : 2u;  // of one round
+      h->L.cond_rollouts = h->L.cond_rounds = 1u;
       ok = enqueue_search(h, io + IO_X, io + IO_R, nullptr, io + IO_V, io + IO_OUT, io + IO_OUT + 1,
                           h->flag_dev, -1, false) == RRG_OK;
       h->L.cond = 0ull;
@@ -1090,7 +1092,7 @@ cudaGraphExec_t capture_step(rrg_ctx* h) {
       cudaGraphNodeParams cp{};
       cp.type = cudaGraphNodeTypeConditional;
       cp.conditional.handle = hc;
-      cp.conditional.type = cudaGraphCondTypeIf;
+      cp.conditional.type = cudaGraphCondTypeWhile;
       cp.conditional.size = 1;
       cudaGraphNode_t cn = nullptr;
       ok = cudaGraphAddNode(&cn, G, sinks.data(), nullptr, sinks.size(), &cp) == cudaSuccess;
@@ -1098,7 +1100,9 @@ cudaGraphExec_t capture_step(rrg_ctx* h) {
       if (ok) ok = cudaStreamBeginCaptureToGraph(h->stream, body, nullptr, nullptr, 0, mode) == cudaSuccess;
       if (ok) {
         h->capturing = true;
-        ok = enqueue_extra_rounds(h, io + IO_OUT, io + IO_OUT + 1, h->flag_dev) == RRG_OK;
+        h->L.cond = hc;
+        ok = enqueue_extra_rounds(h, 1, io + IO_OUT, io + IO_OUT + 1, h->flag_dev) == RRG_OK;
+        h->L.cond = 0ull;
         h->capturing = false;
         ok = (cudaStreamEndCapture(h->stream, &body) == cudaSuccess) && ok;
       }

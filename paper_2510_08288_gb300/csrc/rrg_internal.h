@@ -124,7 +124,7 @@ struct SearchCfg {
   int n_rounds;      // k-section rounds
   int ss_check;
   int probe_steps;   // > 0: pipeline the first two bisection rounds
-  double y_min, eps_ss, y_c;
+  double y_min;
 };
 
 // One model's constants in the form the rollouts use: what the candidate
@@ -137,6 +137,16 @@ struct ModelC {
   double b_ca, d0, d1, d2;
   double ky;                // OER per pascal: ky / v
   double p_atm, inv_p_atm;
+};
+// A setpoint's constants of the equilibrium solve, folded from the parameters
+// (binary64: W_o2 = w1 v, V0 = v0 + v (v1 + v2 v), no division left per
+// candidate), the solve's first guess over W_o2, and the threshold of the
+// steady-state check with the binary32 values outside which a binary32
+// solution decides it.
+struct EqModel {
+  double w1, v0, v1, v2;
+  double thr_ss;
+  float guess, y_fail, y_pass;  // y32 < y_fail: fails, y32 > y_pass: passes
 };
 template <typename T>
 struct StepModel {
@@ -214,6 +224,7 @@ struct Launch {
   int tma;                      // RRG_TMA_*: which ring launches take the TMA
   int inject;                   // RRG_INJECT_* test switches (0 in normal use)
   int tma_pair_bps;             // resident blocks per SM of the paired TMA kernel (0: never paired)
+  EqModel eq;
 };
 
 // Folds the FC3 parameter vector into the constants the kernels use
@@ -426,26 +437,45 @@ __host__ __device__ inline void round_model(const StepModel<double>& m, StepMode
   for (size_t i = 0; i < sizeof(StepPhi<float>) / sizeof(float); ++i) pf[i] = static_cast<float>(p[i]);
 }
 
+// The steady-state threshold is y_min + eps_ss (y_c - y_min); a binary32
+// solution (error about 1e-6) decides it unless it lies within 1e-4 of it.
+inline void fold_eq(const double* P, double y_min, double eps_ss, double y_c, EqModel* E) {
+  E->w1 = P[P_M_O2] * P[P_N_CELL] / (4.0 * P[P_FARADAY]);
+  const double guess = P[P_LAM_REF] / P[P_X_O2];
+  E->v0 = P[P_C0];
+  E->v1 = P[P_C1] + P[P_K_P] * (guess * E->w1);
+  E->v2 = P[P_C2];
+  E->guess = static_cast<float>(guess);
+  const double d = y_c - y_min, p = eps_ss * d;
+  E->thr_ss = y_min + p;
+  const double band = 1e-4 * (1.0 + std::fabs(E->thr_ss));
+  const double hi = E->thr_ss + band, lo = E->thr_ss - band;
+  E->y_pass = static_cast<float>(hi);
+  if (static_cast<double>(E->y_pass) > hi) E->y_pass = std::nextafterf(E->y_pass, -INFINITY);
+  E->y_fail = static_cast<float>(lo);
+  if (static_cast<double>(E->y_fail) < lo) E->y_fail = std::nextafterf(E->y_fail, INFINITY);
+}
+
 // Candidate constants of the rollouts at setpoint v about the reference point
 // q_r (gauge coordinates; binary32 values, or 0 for the gauge form), with the
 // output bound y_min folded into the slack offset: the derivative at q_r
-// without the torque, c = L q_r + b(v).  Every operation is rounded on its own
-// in binary64, so each call site computes the same bits.
+// without the torque, c = L q_r + b(v).  Every operation is spelled out in
+// binary64, so each call site computes the same bits; 18 of them.
 __device__ __forceinline__ RhsC<double> fold_cand(const ModelC& m, double v, const double q_r[3],
                                                   double y_min) {
-  const Vec3 l = lin(m, Vec3{q_r[0], q_r[1], q_r[2]});
+  const double a = q_r[0], w = q_r[1], s = q_r[2];
   RhsC<double> R;
-  R.c_ca = __dsub_rn(l.a, __dmul_rn(m.b_ca, v));
-  R.c_w = __dadd_rn(l.w, __dadd_rn(m.d0, __dmul_rn(v, __dadd_rn(m.d1, __dmul_rn(m.d2, v)))));
-  R.c_sm = l.s;
-  R.x_r = __dadd_rn(1.0, __dmul_rn(q_r[2], m.inv_p_atm));
+  R.c_ca = fma_rn(-m.b_ca, v, fma_rn(m.l_cs, s, __dmul_rn(-m.l_ca, a)));
+  R.c_w = __dadd_rn(fma_rn(m.l_ws, s, __dmul_rn(-m.l_ww, w)), fma_rn(v, fma_rn(m.d2, v, m.d1), m.d0));
+  R.c_sm = fma_rn(-m.l_ss, s, fma_rn(m.l_sw, w, __dmul_rn(m.l_sa, a)));
+  R.x_r = fma_rn(s, m.inv_p_atm, 1.0);
   // 1 / v without the division's instructions, inside its range
   const unsigned ev = (static_cast<unsigned>(__double2hiint(v)) & 0x7fffffffu) >> 20;
   R.y_scale = (ev > 24u && ev < 2022u) ? __dmul_rn(m.ky, rcp_cubic(v)) : __ddiv_rn(m.ky, v);
-  R.s_off = __dsub_rn(__dmul_rn(R.y_scale, __dsub_rn(q_r[2], q_r[0])), y_min);
-  R.r_ca = q_r[0];
-  R.r_w = q_r[1];
-  R.r_sm = q_r[2];
+  R.s_off = fma_rn(R.y_scale, __dsub_rn(s, a), -y_min);
+  R.r_ca = a;
+  R.r_w = w;
+  R.r_sm = s;
   return R;
 }
 __device__ __forceinline__ RhsC<float> round_cand(const RhsC<double>& R) {

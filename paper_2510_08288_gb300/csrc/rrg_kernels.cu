@@ -1057,9 +1057,18 @@ __device__ int tree_count(bool root_is_one, int d) {
   return root_is_one ? (1 << (d - 1)) : ((1 << d) - 1);
 }
 
+// (lo + hi) / 2 of positive numbers and kappa == 1 with one binary64 addition:
+// the halving takes 1 from the exponent (the product below the normal range).
+__device__ __forceinline__ double midpoint(double lo, double hi) {
+  const double t = __dadd_rn(lo, hi);
+  const int e = __double2hiint(t);
+  return e >= 0x00200000 ? __hiloint2double(e - 0x00100000, __double2loint(t)) : __dmul_rn(t, 0.5);
+}
+__device__ __forceinline__ bool is_one(double k) { return __double_as_longlong(k) == 0x3ff0000000000000ll; }
+
 __device__ int choose_depth(const SearchState* s, const SearchCfg& c) {
   const int remaining = c.n_bisect - s->iter;
-  const bool one = s->kappa == 1.0;
+  const bool one = is_one(s->kappa);
   int d = 1;
   while (d + 1 <= remaining && d + 1 <= 11 && tree_count(one, d + 1) <= c.m_cap) ++d;
   return d;
@@ -1084,7 +1093,7 @@ __device__ int build_tree(const SearchState* s, int which, int base, int depth) 
   g_tree_req.lo = s->lo;
   g_tree_req.hi = s->hi;
   g_tree_req.kappa = s->kappa;
-  return tree_count(s->kappa == 1.0, depth);
+  return tree_count(is_one(s->kappa), depth);
 }
 
 // Heap node n of the requested tree goes to slot base + (its rank among the
@@ -1094,7 +1103,7 @@ __device__ void build_tree_block(const Launch& L) {
   const TreeReq r = g_tree_req;
   if (!r.pending) return;
   int32_t* map = r.which ? L.st->slot_of_node1 : L.st->slot_of_node;
-  const bool one = r.kappa == 1.0;
+  const bool one = is_one(r.kappa);
   const int nodes = 1 << r.depth;
   for (int n = threadIdx.x + 1; n < nodes; n += blockDim.x) {
     const int lev = 31 - __clz(n);
@@ -1107,7 +1116,7 @@ __device__ void build_tree_block(const Launch& L) {
     double lo = r.lo, hi = r.hi, k = r.kappa;
     for (int b = lev - 1; b >= 0; --b) {
       if ((n >> b) & 1) lo = k; else hi = k;
-      k = __dmul_rn(__dadd_rn(lo, hi), 0.5);
+      k = midpoint(lo, hi);
     }
     const int rank = !one ? n - 1 : (lev == 0 ? 0 : (1 << (lev - 1)) + off);
     map[n] = r.base + rank;
@@ -1150,14 +1159,14 @@ __device__ void walk_tree(SearchState* s, const SearchCfg& c, const int32_t* slo
       b |= 1u << lev;
       kopt = k;
       any = 1;
-      if (k == 1.0) { done = 1; break; }
+      if (is_one(k)) { done = 1; break; }
       lo = k;
       n = 2 * n + 1;
     } else {
       hi = k;
       n = 2 * n;
     }
-    kap = __dmul_rn(__dadd_rn(lo, hi), 0.5);
+    kap = midpoint(lo, hi);
     if (iter >= c.n_bisect) { done = 1; break; }
   }
   s->kappa = kap; s->lo = lo; s->hi = hi; s->kappa_opt = kopt;
@@ -1258,11 +1267,9 @@ __device__ int next_round(SearchState* s, const SearchCfg& c, double* cand_kappa
 // Eq. 3 and fresh flags.
 __device__ void prepare_slot(const Launch& L, int i) {
   const SearchState* s = L.st;
-  const double thr_ss =
-      __dadd_rn(L.scfg.y_min, __dmul_rn(L.scfg.eps_ss, __dsub_rn(L.scfg.y_c, L.scfg.y_min)));
   const double v = governed(s->v_prev, s->r, L.cand_kappa[i]);
   L.cand_v[i] = v;
-  const int ok = candidate_setup(L.k64, L.k32, L.m64.c, L.params, v, L.scfg.ss_check, thr_ss, L.y_min,
+  const int ok = candidate_setup(L.k64, L.k32, L.eq, L.m64.c, L.params, v, L.scfg.ss_check, L.y_min,
                                  L.cand_c64 + i, L.cand_c32 + i);
   L.cand_ok[i] = ok;
   L.cand_ss[i] = ok;
@@ -1428,8 +1435,11 @@ search_next_kernel(const Launch L, double* v_t, double* kappa, int32_t* flags) {
     s->prep_base = 0;
     s->prep_m = m;
     if (L.cond != 0ull) {
-      cudaGraphSetConditional(L.cond, s->done ? 0u : 1u);
-      if (!s->done) {
+      // (every round decides at least one level, so a loop of rounds ends; the
+      // bound keeps it so)
+      const bool more = !s->done && s->round <= L.scfg.n_bisect;
+      cudaGraphSetConditional(L.cond, more ? 1u : 0u);
+      if (more) {
         L.stats->cond_launches += L.cond_launches;
         L.stats->cond_rollouts += L.cond_rollouts;
         L.stats->cond_rounds += L.cond_rounds;

@@ -47,6 +47,65 @@ template <> __device__ __forceinline__ double eq_tol<double>() { return 1e-15; }
 // and run every iteration.
 template <> __device__ __forceinline__ float eq_tol<float>() { return 1e-6f; }
 
+// Returns 0 and the gauge state q at the equilibrium (C: W_o2 and V0; xs: the
+// first guess), or < 0.  One evaluation site: the stages of the iteration (the
+// sign at W_o2, two points around the target flow, the bracket's upper end,
+// secants) only choose the next flow.
+template <typename T>
+__device__ __forceinline__ int equilibrium_solve(const Fc3K<T>& K, const CandK<T>& C, T guess, T q[3]) {
+  // reciprocals in the solve's own precision (binary32 divisions in the
+  // binary32 screen, none of GB300's slow binary64 ones)
+  const T ikca = T(1) / K.k_ca, iksm = T(1) / K.k_sm;
+  const T a_p = K.a_p, iaw = T(1) / K.a_w;
+  const T big = static_cast<T>(1e30);
+  T lo = C.W_o2, hi = big, x = lo;
+  T x0 = guess, g0 = T(0), x1 = T(0), g1 = T(0);
+  int stage = 0, n = 0;
+#pragma unroll 1
+  for (;;) {
+    const T g = eq_torque<T>(K, C, ikca, iksm, a_p, iaw, x, q);
+    if (stage == 0) {
+      if (!(g > T(0))) return -2;
+      x = x0;
+      stage = 1;
+      continue;
+    }
+    if (stage == 1) {
+      g0 = g;
+      if (g > T(0)) lo = x; else hi = x;
+      x = x0 * (g > T(0) ? T(1.001) : T(0.999));
+      stage = 2;
+      continue;
+    }
+    if (stage == 2) {
+      x1 = x;
+      g1 = g;
+      if (g > T(0)) { if (x > lo) lo = x; } else if (x < hi) hi = x;
+      stage = 3;
+    } else if (stage == 3) {  // closing the bracket before bisection can be needed
+      if (g > T(0)) lo = x; else hi = x;
+      if (++n >= 60 && hi == big) return -2;
+    } else {
+      if (g == T(0)) return 0;
+      if (g > T(0)) lo = x; else hi = x;
+      if (fabs(x - x1) <= eq_tol<T>() * x || hi - lo <= T(0.4) * eq_tol<T>() * hi) return 0;
+      x0 = x1; g0 = g1;
+      x1 = x; g1 = g;
+      if (++n >= 100) return 0;
+    }
+    if (hi == big) {
+      x = T(2) * lo;
+      continue;
+    }
+    if (stage == 3) {
+      stage = 4;
+      n = 0;
+    }
+    x = x1 - g1 * (x1 - x0) / (g1 - g0);
+    if (!(x > lo && x < hi)) x = T(0.5) * (lo + hi);
+  }
+}
+
 // Returns 0 and the gauge state q, output *y_ss at the equilibrium, or < 0.
 template <typename T>
 __device__ __forceinline__ int equilibrium_from(const Fc3K<T>& K, const double* __restrict__ P,
@@ -55,42 +114,9 @@ __device__ __forceinline__ int equilibrium_from(const Fc3K<T>& K, const double* 
   C.W_o2 = static_cast<T>(Cd.W_o2);
   C.V0 = static_cast<T>(Cd.V0);
   C.y_scale = static_cast<T>(Cd.y_scale);
-  // reciprocals in the solve's own precision (binary32 divisions in the
-  // binary32 screen, none of GB300's slow binary64 ones)
-  const T ikca = T(1) / K.k_ca, iksm = T(1) / K.k_sm;
-  const T a_p = K.a_p, iaw = T(1) / K.a_w;
-  const T big = static_cast<T>(1e30);
-  T lo = C.W_o2;
-  if (!(eq_torque<T>(K, C, ikca, iksm, a_p, iaw, lo, q) > T(0))) return -2;
-  T hi = big;
-  // two starting points around the target flow
-  T x0 = static_cast<T>(P[P_LAM_REF] * Cd.W_o2 / P[P_X_O2]);
-  T g0 = eq_torque<T>(K, C, ikca, iksm, a_p, iaw, x0, q);
-  if (g0 > T(0)) lo = x0; else hi = x0;
-  T x1 = x0 * (g0 > T(0) ? T(1.001) : T(0.999));
-  T g1 = eq_torque<T>(K, C, ikca, iksm, a_p, iaw, x1, q);
-  if (g1 > T(0)) { if (x1 > lo) lo = x1; } else if (x1 < hi) hi = x1;
-  // make sure the bracket is closed before bisection can be needed
-  for (int it = 0; it < 60 && hi == big; ++it) {
-    const T xt = T(2) * lo;
-    if (eq_torque<T>(K, C, ikca, iksm, a_p, iaw, xt, q) > T(0)) lo = xt; else hi = xt;
-  }
-  if (hi == big) return -2;
-  T W = x1;
-  for (int it = 0; it < 100; ++it) {
-    T x2 = x1 - g1 * (x1 - x0) / (g1 - g0);
-    if (!(x2 > lo && x2 < hi)) x2 = T(0.5) * (lo + hi);
-    const T g2 = eq_torque<T>(K, C, ikca, iksm, a_p, iaw, x2, q);
-    W = x2;
-    if (g2 == T(0)) break;
-    if (g2 > T(0)) lo = x2; else hi = x2;
-    if (fabs(x2 - x1) <= eq_tol<T>() * x2 || hi - lo <= T(0.4) * eq_tol<T>() * hi) break;
-    x0 = x1; g0 = g1;
-    x1 = x2; g1 = g2;
-  }
-  eq_torque<T>(K, C, ikca, iksm, a_p, iaw, W, q);
-  *y_ss = fc3_output<T>(C, q[0], q[2]);
-  return 0;
+  const int rc = equilibrium_solve<T>(K, C, static_cast<T>(P[P_LAM_REF] * Cd.W_o2 / P[P_X_O2]), q);
+  if (rc == 0) *y_ss = fc3_output<T>(C, q[0], q[2]);
+  return rc;
 }
 
 // The same from the setpoint I alone.
@@ -101,6 +127,11 @@ __device__ __forceinline__ int equilibrium_dev(const Fc3K<T>& K, const double* _
   return equilibrium_from<T>(K, P, cand_consts(P, I), q, y_ss);
 }
 
+__device__ __forceinline__ bool pos_finite(double v) {  // off the binary64 pipe
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v));
+  return b - 1ull < 0x7fefffffffffffffull;
+}
+
 // Candidate set-up shared by the single-problem and batched searches: the
 // binary32 equilibrium of setpoint v (Sec. II-A) is the reference point of
 // the rollouts' deviation coordinates (0 when it cannot be found), the
@@ -109,28 +140,41 @@ __device__ __forceinline__ int equilibrium_dev(const Fc3K<T>& K, const double* _
 // unless y_ss lands within 1e-4 of the threshold (its error is ~1e-6), in
 // which case a binary64 solve decides.  Returns the check's outcome (1 when
 // off).
-__device__ __forceinline__ int candidate_setup(const Fc3K<double>& k64, const Fc3K<float>& k32,
-                                               const ModelC& mc,
-                                               const double* __restrict__ P, double v, int ss_check,
-                                               double thr_ss, double y_min, RhsC<double>* c64,
-                                               RhsC<float>* c32) {
-  const CandK<double> C = cand_consts(P, v);
-  float q32[3] = {0.0f, 0.0f, 0.0f}, y32 = 0.0f;
-  const bool v_ok = v > 0.0 && v <= DBL_MAX;
-  const int rc32 = v_ok ? equilibrium_from<float>(k32, P, C, q32, &y32) : -1;
-  double q_r[3] = {0.0, 0.0, 0.0};
-  if (rc32 == 0 && fabsf(q32[0]) <= FLT_MAX && fabsf(q32[1]) <= FLT_MAX && fabsf(q32[2]) <= FLT_MAX) {
-    q_r[0] = q32[0];
-    q_r[1] = q32[1];
-    q_r[2] = q32[2];
+//
+// One thread's serial chain between two rollouts, so what counts is the number
+// of binary64 instructions (64 cycles each) and of instruction lines fetched
+// once: 29 of them (constants from EqModel, no division; conversions of the
+// reference by bits) and one site of the equilibrium's right-hand side, where
+// every constant was formed from the parameters with three divisions and the
+// right-hand side stood six times in the code.  One candidate's kernel 8.9 -> 5.5
+// us (about 2 of them the launch's).
+__device__ __forceinline__ int candidate_setup(const Fc3K<double>& k64, const Fc3K<float>& k32, const EqModel& eq,
+                                               const ModelC& mc, const double* __restrict__ P, double v,
+                                               int ss_check, double y_min, RhsC<double>* c64, RhsC<float>* c32) {
+  float q32[3] = {0.0f, 0.0f, 0.0f};
+  CandK<float> C;
+  C.W_o2 = static_cast<float>(__dmul_rn(eq.w1, v));
+  C.V0 = static_cast<float>(fma_rn(fma_rn(eq.v2, v, eq.v1), v, eq.v0));
+  C.y_scale = 0.0f;
+  const bool v_ok = pos_finite(v);
+  const int rc32 = v_ok ? equilibrium_solve<float>(k32, C, eq.guess * C.W_o2, q32) : -1;
+  const bool found = rc32 == 0 && fabsf(q32[0]) <= FLT_MAX && fabsf(q32[1]) <= FLT_MAX && fabsf(q32[2]) <= FLT_MAX;
+  double q_r[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const float q = found && fabsf(q32[i]) >= FLT_MIN ? q32[i] : 0.0f;
+    q_r[i] = q == 0.0f ? 0.0 : widen_bits(q);
   }
-  *c64 = fold_cand(mc, v, q_r, y_min);
-  *c32 = round_cand(*c64);
+  const RhsC<double> R = fold_cand(mc, v, q_r, y_min);
+  *c64 = R;
+  const RhsC<float> F = round_cand(R);
+  *c32 = F;
   if (!ss_check) return 1;
-  if (rc32 == 0 && fabs(static_cast<double>(y32) - thr_ss) > 1e-4 * (1.0 + fabs(thr_ss)))
-    return static_cast<double>(y32) >= thr_ss;
+  const float y32 = F.y_scale * (q32[2] - q32[0]);
+  if (rc32 == 0 && y32 > eq.y_pass) return 1;
+  if (rc32 == 0 && y32 < eq.y_fail) return 0;
   double q[3], y_ss = 0.0;
-  return v_ok && equilibrium_from<double>(k64, P, C, q, &y_ss) == 0 && y_ss >= thr_ss;
+  return v_ok && equilibrium_from<double>(k64, P, cand_consts(P, v), q, &y_ss) == 0 && y_ss >= eq.thr_ss;
 }
 
 // Start of a trajectory: the deviation z = q - q_r of the absolute state x

@@ -204,8 +204,6 @@ extern "C" int rrg_eval_candidates_static(const double* model_params, int n_para
   L.scfg.n_rounds = cfg->n_rounds;
   L.scfg.ss_check = cfg->ss_check;
   L.scfg.y_min = cfg->y_min;
-  L.scfg.eps_ss = cfg->eps_ss;
-  L.scfg.y_c = cfg->y_c;
   fold_constants(model_params, &L.k64, &L.k32);
   // the binary64 rollouts and the recheck evaluate x^e - 1 by the same table
   // as a handle's, so both give the same bits
@@ -213,6 +211,7 @@ extern "C" int rrg_eval_candidates_static(const double* model_params, int n_para
   PowTable* const pws = reinterpret_cast<PowTable*>(base + kOffPws);
   if (pow_table(L.k64.e, &pb.pws)) L.k64.pws = pws;
   fold_model(L.k64, model_params, cfg->dt, &L.m64);
+  fold_eq(model_params, cfg->y_min, cfg->eps_ss, cfg->y_c, &L.eq);
   round_model(L.m64, &L.m32);
   L.params = reinterpret_cast<double*>(base + kOffParams);
   L.d64 = const_cast<double*>(d_scen64);
