@@ -13,12 +13,12 @@
 //   argmin   adjoint_argmin_kernel: per kappa, the first (k, then j)
 //            attaining the min;
 //   reverse  adjoint_reverse_kernel: the checkpoint segments before j* are
-//            recomputed in parallel (one thread each), storing every step's
-//            state and RK4 stage points; one thread then sweeps them
-//            backwards with the vector-Jacobian products of the FC3
-//            right-hand side; the adjoints of the folded constants are
-//            mapped to the 27 model parameters, to x_t and (through the
-//            setpoint) to kappa.
+//            recomputed in parallel, storing every step's state; from j* down,
+//            32 steps at a time, every stage's Jacobian in parallel, the
+//            adjoint recursion over them (three multiply-adds a stage, the
+//            only serial part) and every stage's share of the constants'
+//            adjoints in parallel; these are mapped to the 27 model
+//            parameters, to x_t and (through the setpoint) to kappa.
 #include <cfloat>
 #include <cmath>
 
@@ -123,80 +123,19 @@ __device__ void fc3_rhs_vjp(const Fc3K<T>& K, const CandK<T>& C, T q_ca, T w, T 
   qb_sm += qsm_b;
 }
 
-// The RK4 stage points of one step from x: y2 = x + dt/2 k1, y3 = x + dt/2 k2,
-// y4 = x + dt k3 (k_i the right-hand side at the previous stage point);
-// y[0..2] = y2, y[3..5] = y3, y[6..8] = y4.  They do not depend on the adjoint.
+// Stage point `stage` (0: the state itself) of the RK4 step from y, in place.
 template <typename T>
-__device__ __forceinline__ void rk4_stage_points(const Fc3K<T>& K, const CandK<T>& C, T dt, T q_ca, T w,
-                                                 T q_sm, T* y) {
-  const T h2 = T(0.5) * dt;
-  T a, b, c;
-  fc3_rhs<T>(K, C, q_ca, w, q_sm, a, b, c);
-  y[0] = q_ca + h2 * a; y[1] = w + h2 * b; y[2] = q_sm + h2 * c;
-  fc3_rhs<T>(K, C, y[0], y[1], y[2], a, b, c);
-  y[3] = q_ca + h2 * a; y[4] = w + h2 * b; y[5] = q_sm + h2 * c;
-  fc3_rhs<T>(K, C, y[3], y[4], y[5], a, b, c);
-  y[6] = q_ca + dt * a; y[7] = w + dt * b; y[8] = q_sm + dt * c;
-}
-
-// Adjoint of one RK4 step q+ = q + dt/6 (k1 + 2 k2 + 2 k3 + k4) (+ d) at state
-// q with stage points y (rk4_stage_points): given the adjoint (l0, l1, l2) of
-// q+, overwrites it with the adjoint of q; the constants' adjoints accumulate
-// into g.
-template <typename T>
-__device__ void rk4_step_vjp_at(const Fc3K<T>& K, const CandK<T>& C, T dt, T q_ca, T w, T q_sm,
-                                const T* y, T& l0, T& l1, T& l2, ConstAdj<T>& g) {
-  const T h2 = T(0.5) * dt, h6 = dt / T(6);
-  T q0 = l0, q1 = l1, q2 = l2;                  // identity part
-  T k1_0 = h6 * l0, k1_1 = h6 * l1, k1_2 = h6 * l2;
-  T k2_0 = T(2) * h6 * l0, k2_1 = T(2) * h6 * l1, k2_2 = T(2) * h6 * l2;
-  T k3_0 = T(2) * h6 * l0, k3_1 = T(2) * h6 * l1, k3_2 = T(2) * h6 * l2;
-  const T k4_0 = h6 * l0, k4_1 = h6 * l1, k4_2 = h6 * l2;
-  T y0 = 0, y1 = 0, y2 = 0;
-  fc3_rhs_vjp<T>(K, C, y[6], y[7], y[8], k4_0, k4_1, k4_2, y0, y1, y2, g);
-  q0 += y0; q1 += y1; q2 += y2;
-  k3_0 += dt * y0; k3_1 += dt * y1; k3_2 += dt * y2;
-  y0 = y1 = y2 = 0;
-  fc3_rhs_vjp<T>(K, C, y[3], y[4], y[5], k3_0, k3_1, k3_2, y0, y1, y2, g);
-  q0 += y0; q1 += y1; q2 += y2;
-  k2_0 += h2 * y0; k2_1 += h2 * y1; k2_2 += h2 * y2;
-  y0 = y1 = y2 = 0;
-  fc3_rhs_vjp<T>(K, C, y[0], y[1], y[2], k2_0, k2_1, k2_2, y0, y1, y2, g);
-  q0 += y0; q1 += y1; q2 += y2;
-  k1_0 += h2 * y0; k1_1 += h2 * y1; k1_2 += h2 * y2;
-  y0 = y1 = y2 = 0;
-  fc3_rhs_vjp<T>(K, C, q_ca, w, q_sm, k1_0, k1_1, k1_2, y0, y1, y2, g);
-  l0 = q0 + y0;
-  l1 = q1 + y1;
-  l2 = q2 + y2;
-}
-
-// Parameters of scenario k: theta, or theta_p m_p^k under parametric
-// uncertainty (multipliers of scenario pair 0).
-__device__ __forceinline__ void scenario_params(const Launch& L, int k, double* Pk) {
-  for (int p = 0; p < RRG_NPARAM; ++p)
-    Pk[p] = L.pmul ? __dmul_rn(L.params[p], L.pmul[static_cast<size_t>(k) * RRG_NPARAM + p])
-                   : L.params[p];
-}
-
-template <typename T>
-__device__ __forceinline__ Fc3K<T> konst(const double* Pk) {
-  Fc3K<double> k64;
-  Fc3K<float> k32;
-  fold_constants(Pk, &k64, &k32);
-  if constexpr (sizeof(T) == 8) return k64;
-  else return k32;
-}
-
-template <typename T>
-__device__ CandK<T> cand_of(const double* P, double I) {
-  const double W_o2 = P[P_M_O2] * P[P_N_CELL] * I / (4.0 * P[P_FARADAY]);
-  CandK<T> C;
-  C.W_o2 = static_cast<T>(W_o2);
-  C.V0 = static_cast<T>(P[P_C0] + P[P_C1] * I + P[P_C2] * I * I +
-                        P[P_K_P] * P[P_LAM_REF] * W_o2 / P[P_X_O2]);
-  C.y_scale = static_cast<T>(P[P_X_O2] * P[P_K_SM] / W_o2);
-  return C;
+__device__ __forceinline__ void rk4_stage_point(const Fc3K<T>& K, const CandK<T>& C, T dt, int stage, T y[3]) {
+  const T x[3] = {y[0], y[1], y[2]};
+#pragma unroll 1
+  for (int u = 0; u < stage; ++u) {
+    const T h = u < 2 ? T(0.5) * dt : dt;
+    T a, b, c;
+    fc3_rhs<T>(K, C, y[0], y[1], y[2], a, b, c);
+    y[0] = x[0] + h * a;
+    y[1] = x[1] + h * b;
+    y[2] = x[2] + h * c;
+  }
 }
 
 // Register slots of the forward pass's disturbance prefetch ring.
@@ -409,31 +348,37 @@ constexpr int kOutStride = kAdjOutStride;
 // the shared arrays' size): the smallest lane minimum, and among equal ones
 // the smallest k, which the reduction order cannot change; written to
 // o[0..2] by thread 0, visible to the block after its closing barrier.
-__device__ void block_argmin(const double* __restrict__ lm, const int* __restrict__ la, int N, double* o,
-                             double* sv, int* sk) {
-  double best = INFINITY;
+// Compared as integers (a binary64 comparison holds the scheduler 64 cycles);
+// -0 equals 0 and a NaN is never the least.
+constexpr int kArgminWarps = 8;  // of a block, at most
+__device__ void block_argmin(const double* __restrict__ lm, const int* __restrict__ la, int N, double* o) {
+  __shared__ unsigned long long sv[kArgminWarps];
+  __shared__ int sk[kArgminWarps];
+  unsigned long long best = dkey(INFINITY);
   int bk = 0x7fffffff;
-  for (int k = threadIdx.x; k < N; k += blockDim.x) {
-    const double s = lm[k];
-    if (s < best || (s == best && k < bk)) { best = s; bk = k; }
+#pragma unroll 8
+  for (int k = threadIdx.x; k < N; k += blockDim.x) {  // ascending k: the first of equal values stays
+    const long long u = __double_as_longlong(__ldg(lm + k));
+    const unsigned long long mag = static_cast<unsigned long long>(u) & 0x7fffffffffffffffull;
+    const unsigned long long key = mag == 0ull ? dkey(0.0) : dkey(__longlong_as_double(u));
+    if (mag <= 0x7ff0000000000000ull && (key < best || (key == best && k < bk))) { best = key; bk = k; }
   }
-  sv[threadIdx.x] = best;
-  sk[threadIdx.x] = bk;
+  auto fold = [&](unsigned long long key, int kk) {
+    if (key < best || (key == best && kk < bk)) { best = key; bk = kk; }
+  };
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1)
+    fold(__shfl_xor_sync(0xffffffffu, best, w), __shfl_xor_sync(0xffffffffu, bk, w));
+  if ((threadIdx.x & 31) == 0) {
+    sv[threadIdx.x >> 5] = best;
+    sk[threadIdx.x >> 5] = bk;
+  }
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      const double s = sv[threadIdx.x + w];
-      const int kk = sk[threadIdx.x + w];
-      if (s < sv[threadIdx.x] || (s == sv[threadIdx.x] && kk < sk[threadIdx.x])) {
-        sv[threadIdx.x] = s;
-        sk[threadIdx.x] = kk;
-      }
-    }
-    __syncthreads();
-  }
   if (threadIdx.x == 0) {
-    long long kj[2] = {sk[0], (sk[0] >= 0 && sk[0] < N) ? la[sk[0]] : 0};
-    o[0] = sv[0];
+    for (int w = 1; w < static_cast<int>(blockDim.x >> 5); ++w) fold(sv[w], sk[w]);
+    const bool found = bk >= 0 && bk < N;
+    long long kj[2] = {bk, found ? la[bk] : 0};
+    o[0] = found ? lm[bk] : INFINITY;
     memcpy(o + 1, kj, sizeof kj);
   }
   __syncthreads();
@@ -441,26 +386,121 @@ __device__ void block_argmin(const double* __restrict__ lm, const int* __restric
 
 __global__ void adjoint_argmin_kernel(const double* __restrict__ lane_min,
                                       const int* __restrict__ lane_arg, int N, double* out) {
-  __shared__ double sv[256];
-  __shared__ int sk[256];
   const int i = blockIdx.x;
   block_argmin(lane_min + static_cast<size_t>(i) * N, lane_arg + static_cast<size_t>(i) * N, N,
-               out + static_cast<size_t>(i) * kOutStride, sv, sk);
+               out + static_cast<size_t>(i) * kOutStride);
 }
 
-// Values stored per step of the recomputed trajectory: x_j and the three
-// stage points of step j.
-constexpr int kSegVals = 12;
+// Values stored per step of the recomputed trajectory: x_j.
+constexpr int kSegVals = 3;
 constexpr int kRevThreads = 128;
+constexpr int kRevSteps = kRevThreads / 4;  // steps of a sweep's chunk: one thread per stage
+
+// States of segment c of the trajectory (steps j0 .. j1 - 1, and j1 if it is
+// j*) from its checkpoint, by the rollouts' step in deviation coordinates;
+// the disturbances of four steps are fetched while the four before them run.
+template <typename T, typename DT>
+__device__ __forceinline__ void segment_states(const LaneModel<T>& M, const RhsC<T>& R, const DT* __restrict__ d, int k,
+                                               int N, int H, const double* __restrict__ ck, int j0, int j1, bool last,
+                                               T* __restrict__ seg) {
+  T z_ca = static_cast<T>(ck[0] - static_cast<double>(R.r_ca)), z_w = static_cast<T>(ck[1] - static_cast<double>(R.r_w)),
+    z_sm = static_cast<T>(ck[2] - static_cast<double>(R.r_sm));
+  T w_abs = z_w + R.r_w;
+  T e[3][4], f[3][4];
+  auto load = [&](int j) {  // steps j .. j + 3 (those before j1)
+    if constexpr (sizeof(DT) == 4) {  // the handle's binary32 quads; j is a multiple of 4
+      const size_t comp = 4 * quad_rows(H) * static_cast<size_t>(N);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float4 v = j < j1 ? __ldg(reinterpret_cast<const float4*>(d + quad_index(0, j, k, H, N) + c * comp))
+                                : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        f[c][0] = v.x; f[c][1] = v.y; f[c][2] = v.z; f[c][3] = v.w;
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          f[c][u] = j + u < j1 ? static_cast<T>(__ldg(d + (static_cast<size_t>(c) * H + j + u) * N + k)) : T(0);
+    }
+  };
+  auto store = [&](int j) {
+    T* sj = seg + static_cast<size_t>(j) * kSegVals;
+    sj[0] = z_ca + R.r_ca;
+    sj[1] = w_abs;
+    sj[2] = z_sm + R.r_sm;
+  };
+  load(j0);
+#pragma unroll 1
+  for (int j = j0; j < j1; j += 4) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) e[c][u] = f[c][u];
+    load(j + 4);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j + u < j1) {
+        store(j + u);
+        rk4_step_fast<T>(M.U, M.pw, M.C, z_ca, z_w, z_sm, w_abs, e[0][u], e[1][u], e[2][u]);
+      }
+  }
+  if (last) store(j1);
+}
+
+// The same with four lanes per binary64 trajectory (Coop64), by every lane of
+// the warp; `n`: steps the warp runs (its longest segment's).
+__device__ __forceinline__ void segment_states_coop(const LaneModel<double>& M, const PowTable* any,
+                                                    const RhsC<double>& R, const double* __restrict__ d, int k, int N,
+                                                    int H, const double* __restrict__ ck, int j0, int j1, int n, bool on,
+                                                    bool last, double* __restrict__ seg) {
+  Coop64 G(M.U, M.pw, any, M.C);
+  double a = ck[0] - R.r_ca, w = ck[1] - R.r_w, s = ck[2] - R.r_sm;
+  double w_abs = w + R.r_w;
+  const size_t HN = static_cast<size_t>(H) * N;
+  const bool ld1 = G.role == 2, ld2 = G.role >= 2;
+  const double* p1 = d + static_cast<size_t>(j0) * N + k;
+  const double* p2 = p1 + (G.role == 2 ? 2 * HN : HN);
+  double e1 = ld1 && j0 < j1 ? __ldg(p1) : 0.0, e2 = ld2 && j0 < j1 ? __ldg(p2) : 0.0;
+  auto store = [&](int j) {
+    double* sj = seg + static_cast<size_t>(j) * kSegVals;
+    sj[0] = a + R.r_ca;
+    sj[1] = w_abs;
+    sj[2] = s + R.r_sm;
+  };
+#pragma unroll 1
+  for (int j = j0; j < j0 + n; ++j) {
+    const bool mine = on && j < j1;
+    if (mine && G.role == 0) store(j);
+    const double f1 = e1, f2 = e2;
+    p1 += N;
+    p2 += N;
+    if (j + 1 < j1) {
+      if (ld1) e1 = __ldg(p1);
+      if (ld2) e2 = __ldg(p2);
+    }
+    G.live = mine;
+    G.step(a, w, s, w_abs, f1, f2);
+    if (mine && last && j + 1 == j1 && G.role == 0) store(j1);
+  }
+}
 
 // Reverse sweep of trajectory k* from j* to 0, then the chain rule from the
 // folded constants to the model parameters and kappa.  One block:
-//   phase 1, all threads: the checkpoint segments before j* are recomputed
-//     in parallel, one segment per thread, storing for each step j its state
-//     and stage points in seg[j * kSegVals ...], and x_{j*} after the last one;
-//   phase 2, thread 0: the adjoint recursion from j* down to 0 over the
-//     stored steps (the only serial part), each step's values loaded one step
-//     ahead.
+//   phase 1: the checkpoint segments before j* are recomputed in parallel,
+//     one thread (binary64: four lanes) a segment: x_j into seg[3 j ..];
+//   phase 2: 32 steps at a time from j* down, one thread per (step, stage):
+//     the stage point and the two state-dependent entries of its Jacobian
+//     (the others are products of constants); three lanes then run the
+//     adjoint recursion, lane r its component r, leaving every stage's adjoint
+//     in shared memory, from which each thread adds its stage's share of the
+//     constants' adjoints (fc3_rhs_vjp);
+//   phase 3: their sum over the block, and the chain rule with every quotient
+//     on a lane of its own.
+// The recursion is the only serial part: 5 instructions a stage where one
+// thread evaluated power, logarithm and quotients of every stage in turn.
+// Measured on GB300 (a call, two kappas, 512 scenarios of 1,000 steps): j* = 530
+// binary64 10.3 -> 2.66 ms, binary32 587 -> 209 us; j* = 0 binary32 156 -> 146.
 // seg: scratch of (j* + 1) * kSegVals values (at most (H + 1) * kSegVals).
 // out[0] = dg/dkappa, out[1..3] = dg/dx_t, out[4..4+NPARAM) = dg/dtheta.
 template <typename T, typename DT>
@@ -474,61 +514,77 @@ adjoint_reverse_kernel(const Launch L, const DT* __restrict__ d,
   // the inputs of the candidate set-up the forward pass ran on
   const double v_prev = L.st->v_prev, r = L.st->r;
   double* o = out_all + static_cast<size_t>(i) * kOutStride;
-  if (lane_min != nullptr) {
-    // the argmin first, by this block (one launch fewer than a separate pass)
-    __shared__ double sv[kRevThreads];
-    __shared__ int sk[kRevThreads];
-    block_argmin(lane_min + static_cast<size_t>(i) * N, lane_arg + static_cast<size_t>(i) * N, N, o, sv, sk);
-  }
+  // the argmin first, by this block (one launch fewer than a separate pass)
+  if (lane_min != nullptr)
+    block_argmin(lane_min + static_cast<size_t>(i) * N, lane_arg + static_cast<size_t>(i) * N, N, o);
   long long kj[2];
   memcpy(kj, o + 1, sizeof kj);
   double* out = o + 3;
   T* seg = seg_all + static_cast<size_t>(i) * (H + 1) * kSegVals;
-  const double kappa = L.cand_kappa[i];
-  const double v = governed(v_prev, r, kappa);
+  const double v = L.cand_v[i];
   if (kj[0] < 0 || kj[0] >= N || kj[1] < 0 || kj[1] > H) {  // no argmin: same for every thread
     if (threadIdx.x < 4 + RRG_NPARAM) out[threadIdx.x] = NAN;
     return;
   }
   const int k = static_cast<int>(kj[0]), jstar = static_cast<int>(kj[1]);
-  double P[RRG_NPARAM];
-  scenario_params(L, k, P);
-  Fc3K<T> K = konst<T>(P);
-  // the table of the model's exponent
-  if (sizeof(T) == 8) K.pws = (L.k64.pws != nullptr && L.k64.pws->e == static_cast<double>(K.e)) ? L.k64.pws : nullptr;
-  const CandK<T> C = cand_of<T>(P, v);
+  // the scenario's constants: the launch's, folded again under parametric uncertainty
+  __shared__ double P[RRG_NPARAM];
+  if (threadIdx.x < RRG_NPARAM)
+    P[threadIdx.x] = L.pmul ? __dmul_rn(L.params[threadIdx.x], L.pmul[static_cast<size_t>(k) * RRG_NPARAM + threadIdx.x])
+                            : L.params[threadIdx.x];
+  __syncthreads();
+  Fc3K<double> K64 = L.k64;
+  Fc3K<float> K32 = L.k32;
+  CandK<double> C64;
+  RhsC<T> R = launch_c<T>(L, i);
+  LaneModel<T> M;
+  if (L.pmul != nullptr) {
+    fold_constants(P, &K64, &K32);
+    K64.pws = (L.k64.pws != nullptr && L.k64.pws->e == K64.e) ? L.k64.pws : nullptr;
+    C64 = cand_consts(P, v);
+    lane_model<T, true>(L, 0, k, v, R, M);
+  } else {
+    C64.W_o2 = __dmul_rn(L.eq.w1, v);
+    C64.V0 = fma_rn(fma_rn(L.eq.v2, v, L.eq.v1), v, L.eq.v0);
+    C64.y_scale = L.cand_c64[i].y_scale;
+    lane_model<T, false>(L, 0, k, v, R, M);
+  }
+  Fc3K<T> K;
+  CandK<T> C;
+  if constexpr (sizeof(T) == 8) {
+    K = K64;
+    C = C64;
+  } else {
+    K = K32;
+    C = cand_round(C64);
+  }
   const T dt = static_cast<T>(L.dt);
   const int nseg = H / checkpoint + 1;
-  const size_t HN = static_cast<size_t>(H) * N;
   const double* ck = ckpt + (static_cast<size_t>(i) * N + k) * nseg * 3;
   // phase 1: segment c covers steps c * checkpoint .. min((c + 1) * checkpoint, j*) - 1
   const int nc = jstar > 0 ? (jstar - 1) / checkpoint + 1 : 0;
-  for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-    const int j0 = c * checkpoint;
-    const int j1 = (j0 + checkpoint < jstar) ? j0 + checkpoint : jstar;
-    T a = static_cast<T>(ck[c * 3]), b = static_cast<T>(ck[c * 3 + 1]), e = static_cast<T>(ck[c * 3 + 2]);
-    for (int j = j0; j < j1; ++j) {
-      T* sj = seg + static_cast<size_t>(j) * kSegVals;
-      sj[0] = a; sj[1] = b; sj[2] = e;
-      rk4_stage_points<T>(K, C, dt, a, b, e, sj + 3);
-      size_t o = static_cast<size_t>(j) * N + k, cs = HN;
-      if constexpr (sizeof(DT) == 4) {  // the handle's binary32 array
-        o = quad_index(0, j, k, H, N);
-        cs = 4 * quad_rows(H) * static_cast<size_t>(N);
+  bool coop = false;
+  if constexpr (sizeof(T) == 8) {
+    coop = L.m64.pw != nullptr;
+    if (coop) {
+      for (int c0 = static_cast<int>(threadIdx.x >> 5) * 8; c0 < nc; c0 += kRevThreads / 4) {  // the warp's first segment
+        const int c = c0 + static_cast<int>((threadIdx.x & 31) >> 2);
+        const bool on = c < nc;
+        const int j0 = (on ? c : nc - 1) * checkpoint;
+        const int j1 = (j0 + checkpoint < jstar) ? j0 + checkpoint : jstar;
+        const int n = jstar - c0 * checkpoint < checkpoint ? jstar - c0 * checkpoint : checkpoint;
+        segment_states_coop(M, L.m64.pw, R, d, k, N, H, ck + static_cast<size_t>(on ? c : nc - 1) * 3, j0, j1, n, on,
+                            j1 == jstar, seg);
       }
-      rk4_step<T>(K, C, dt, a, b, e);
-      a += static_cast<T>(d[o]);
-      b += static_cast<T>(d[cs + o]);
-      e += static_cast<T>(d[2 * cs + o]);
-    }
-    if (j1 == jstar) {
-      T* sj = seg + static_cast<size_t>(jstar) * kSegVals;
-      sj[0] = a; sj[1] = b; sj[2] = e;
     }
   }
+  if (!coop)
+    for (int c = threadIdx.x; c < nc; c += kRevThreads) {
+      const int j0 = c * checkpoint;
+      const int j1 = (j0 + checkpoint < jstar) ? j0 + checkpoint : jstar;
+      segment_states<T, DT>(M, R, d, k, N, H, ck + static_cast<size_t>(c) * 3, j0, j1, j1 == jstar, seg);
+    }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  ConstAdj<T> g{};
   // output at j*: s = y_scale (q_sm - q_ca) - y_min (x_0 is checkpoint 0)
   T q_ca, q_sm;
   if (jstar == 0) {
@@ -538,82 +594,163 @@ adjoint_reverse_kernel(const Launch L, const DT* __restrict__ d,
     q_ca = seg[static_cast<size_t>(jstar) * kSegVals];
     q_sm = seg[static_cast<size_t>(jstar) * kSegVals + 2];
   }
-  g.y_scale += q_sm - q_ca;
-  T l0 = -C.y_scale, l1 = T(0), l2 = C.y_scale;
-  // phase 2: backwards over the stored steps
-  if (jstar > 0) {
-    T cur[kSegVals];
+  // phase 2
+  __shared__ T jac[kRevThreads][2];  // d(dw)/dw, d(dw)/d(p_sm) of (step, stage) 4 u + stage
+  __shared__ T adj[kRevThreads][3];  // its adjoint
+  const int stage = threadIdx.x & 3, step = threadIdx.x >> 2, comp = threadIdx.x < 3 ? static_cast<int>(threadIdx.x) : 2;
+  const T h2 = T(0.5) * dt, h6 = dt / T(6);
+  const T cA = comp == 0 ? -(K.k_ca + K.k_sm) * K.RT_Vca : comp == 1 ? T(0) : K.k_sm * K.RT_Vca;
+  const T cS = comp == 0 ? K.k_sm * K.RT_Vsm : comp == 1 ? K.a_w * K.RT_Vsm : -(K.k_sm + K.a_p) * K.RT_Vsm;
+  T l = comp == 0 ? -C.y_scale : comp == 1 ? T(0) : C.y_scale;  // warp 0, lane r: the adjoint's component r
+  ConstAdj<T> g{};
+  for (int jt = jstar - 1; jt >= 0; jt -= kRevSteps) {  // chunk of steps jt, jt - 1, ...
+    const int j = jt - step, n = jt + 1 < kRevSteps ? jt + 1 : kRevSteps;
+    T y[3];
+    if (step < n) {
 #pragma unroll
-    for (int u = 0; u < kSegVals; ++u) cur[u] = seg[static_cast<size_t>(jstar - 1) * kSegVals + u];
-    for (int j = jstar - 1; j >= 0; --j) {
-      T nxt[kSegVals];
-      const int jn = j > 0 ? j - 1 : 0;
+      for (int u = 0; u < 3; ++u) y[u] = seg[static_cast<size_t>(j) * kSegVals + u];
+      rk4_stage_point<T>(K, C, dt, stage, y);
+      ConstAdj<T> unused{};
+      T ja = T(0), jw = T(0), js = T(0);
+      fc3_rhs_vjp<T>(K, C, y[0], y[1], y[2], T(0), T(1), T(0), ja, jw, js, unused);
+      jac[threadIdx.x][0] = jw;
+      jac[threadIdx.x][1] = js;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      auto from = [&](T x, int lane) { return __shfl_sync(0xffffffffu, x, lane); };
+#pragma unroll 1
+      for (int u = 0; u < n; ++u) {
+        T cw[4];
 #pragma unroll
-      for (int u = 0; u < kSegVals; ++u) nxt[u] = seg[static_cast<size_t>(jn) * kSegVals + u];
-      rk4_step_vjp_at<T>(K, C, dt, cur[0], cur[1], cur[2], cur + 3, l0, l1, l2, g);
+        for (int st = 0; st < 4; ++st) cw[st] = comp == 0 ? T(0) : jac[4 * u + st][comp - 1 > 0];
+        const T hl = h6 * l;
+        T b = hl, q = l;
 #pragma unroll
-      for (int u = 0; u < kSegVals; ++u) cur[u] = nxt[u];
+        for (int st = 3; st >= 0; --st) {
+          if (threadIdx.x < 3) adj[4 * u + st][threadIdx.x] = b;
+          const T yb = cA * from(b, 0) + (cw[st] * from(b, 1) + cS * from(b, 2));
+          q += yb;
+          if (st == 3) b = T(2) * hl + dt * yb;
+          else if (st == 2) b = T(2) * hl + h2 * yb;
+          else if (st == 1) b = hl + h2 * yb;
+        }
+        l = q;
+      }
+    }
+    __syncthreads();
+    if (step < n) {
+      T ja = T(0), jw = T(0), js = T(0);
+      fc3_rhs_vjp<T>(K, C, y[0], y[1], y[2], adj[threadIdx.x][0], adj[threadIdx.x][1], adj[threadIdx.x][2], ja, jw, js,
+                     g);
     }
   }
-  // chain rule to the parameter vector (binary64)
-  double th[RRG_NPARAM];
-  for (int i = 0; i < RRG_NPARAM; ++i) th[i] = 0.0;
-  const double I = v;
-  const double W_o2 = P[P_M_O2] * P[P_N_CELL] * I / (4.0 * P[P_FARADAY]);
-  const double y_scale = P[P_X_O2] * P[P_K_SM] / W_o2;
-  const double lam = P[P_LAM_REF], xo2 = P[P_X_O2], Kp = P[P_K_P];
-  const double gamma = P[P_GAMMA];
-  th[P_A_W] += g.a_w;
-  th[P_A_P] += g.a_p;
-  th[P_K_SM] += g.k_sm + static_cast<double>(g.y_scale) * y_scale / P[P_K_SM];
-  th[P_K_CA] += g.k_ca;
-  th[P_GAMMA] += static_cast<double>(g.e) / (gamma * gamma);
+  // phase 3: sums over the block, thread (v, s) = (t / 8, t % 8) a part of sum v
+  constexpr int kAdj = 15;  // ConstAdj without y_scale
+  __shared__ T part[kAdj][kRevThreads];
+  __shared__ double tot[16], num[32], den[32], th[RRG_NPARAM], quo[32], lam_x[3];
+  const T gv[kAdj] = {g.a_w, g.a_p, g.k_sm, g.k_ca, g.e, g.C_cp, g.C_m, g.k_v, g.K_p, g.RT_Vca, g.RT_Vsm, g.inv_J,
+                      g.inv_p_atm, g.W_o2, g.V0};
+#pragma unroll
+  for (int u = 0; u < kAdj; ++u) part[u][threadIdx.x] = gv[u];
+  if (threadIdx.x < 3) lam_x[threadIdx.x] = static_cast<double>(l);
+  __syncthreads();
   {
-    const double Ccp = P[P_C_P] * P[P_T_ATM] / P[P_ETA_CP], gc = g.C_cp;
-    th[P_C_P] += gc * P[P_T_ATM] / P[P_ETA_CP];
-    th[P_T_ATM] += gc * P[P_C_P] / P[P_ETA_CP];
-    th[P_ETA_CP] += -gc * Ccp / P[P_ETA_CP];
+    const int u = threadIdx.x >> 3;
+    T s = T(0);
+    if (u < kAdj)
+      for (int t = threadIdx.x & 7; t < kRevThreads; t += 8) s += part[u][t];
+#pragma unroll
+    for (int w = 4; w > 0; w >>= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
+    if ((threadIdx.x & 7) == 0) tot[u] = static_cast<double>(s);
   }
-  {
-    const double Cm = P[P_ETA_CM] * P[P_K_T] / P[P_R_CM], gc = g.C_m;
-    th[P_ETA_CM] += gc * P[P_K_T] / P[P_R_CM];
-    th[P_K_T] += gc * P[P_ETA_CM] / P[P_R_CM];
-    th[P_R_CM] += -gc * Cm / P[P_R_CM];
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  // chain rule to the parameter vector (binary64): numerators and
+  // denominators by lane 0, the quotients by the lanes
+  const double g_a_w = tot[0], g_a_p = tot[1], g_k_sm = tot[2], g_k_ca = tot[3], g_e = tot[4], gc = tot[5], gm = tot[6],
+               g_k_v = tot[7], g_K_p = tot[8], ga = tot[9], gs = tot[10], gJ = tot[11], gp = tot[12], gW_o2 = tot[13],
+               gV0 = tot[14], gy = static_cast<double>(q_sm - q_ca);
+  const double I = v, W_o2 = C64.W_o2, y_scale = C64.y_scale;
+  const double lam = P[P_LAM_REF], xo2 = P[P_X_O2], Kp = P[P_K_P], gamma = P[P_GAMMA];
+  if (threadIdx.x == 0) {
+    auto set = [&](int q, double a, double b) {
+      num[q] = a;
+      den[q] = b;
+    };
+    set(0, gy * y_scale, P[P_K_SM]);
+    set(1, g_e, gamma * gamma);
+    set(2, gc * P[P_T_ATM], P[P_ETA_CP]);
+    set(3, gc * P[P_C_P], P[P_ETA_CP]);
+    set(4, -gc * K64.C_cp, P[P_ETA_CP]);
+    set(5, gm * P[P_K_T], P[P_R_CM]);
+    set(6, gm * P[P_ETA_CM], P[P_R_CM]);
+    set(7, -gm * K64.C_m, P[P_R_CM]);
+    set(8, ga * P[P_T_ST], P[P_V_CA]);
+    set(9, gs * P[P_T_ST], P[P_V_SM]);
+    set(10, ga * P[P_R_A], P[P_V_CA]);
+    set(11, gs * P[P_R_A], P[P_V_SM]);
+    set(12, -ga * K64.RT_Vca, P[P_V_CA]);
+    set(13, -gs * K64.RT_Vsm, P[P_V_SM]);
+    set(14, -gJ, P[P_J_CP] * P[P_J_CP]);
+    set(15, -gp, P[P_P_ATM] * P[P_P_ATM]);
+    const double vk = gV0 * Kp, vl = gV0 * lam * W_o2, yg = gy * y_scale;
+    set(16, vk * lam, xo2);
+    set(17, yg, W_o2);
+    set(18, vl, xo2);
+    set(19, vk * W_o2, xo2);
+    set(20, -vk * lam * W_o2, xo2 * xo2);
+    set(21, yg, xo2);
   }
-  th[P_K_V] += g.k_v;
-  th[P_K_P] += g.K_p;
-  {
-    const double RTa = P[P_R_A] * P[P_T_ST] / P[P_V_CA], RTs = P[P_R_A] * P[P_T_ST] / P[P_V_SM];
-    const double ga = g.RT_Vca, gs = g.RT_Vsm;
-    th[P_R_A] += ga * P[P_T_ST] / P[P_V_CA] + gs * P[P_T_ST] / P[P_V_SM];
-    th[P_T_ST] += ga * P[P_R_A] / P[P_V_CA] + gs * P[P_R_A] / P[P_V_SM];
-    th[P_V_CA] += -ga * RTa / P[P_V_CA];
-    th[P_V_SM] += -gs * RTs / P[P_V_SM];
+  __syncwarp();
+  if (threadIdx.x < 22) quo[threadIdx.x] = num[threadIdx.x] / den[threadIdx.x];
+  __syncwarp();
+  const double gW = gW_o2 + quo[16] - quo[17];
+  if (threadIdx.x < 4) {
+    const double a = threadIdx.x == 2 ? -(gW * W_o2) : gW * W_o2;
+    const double b = threadIdx.x == 0 ? P[P_M_O2] : threadIdx.x == 1 ? P[P_N_CELL] : threadIdx.x == 2 ? P[P_FARADAY] : I;
+    quo[22 + threadIdx.x] = a / b;
   }
-  th[P_J_CP] += -static_cast<double>(g.inv_J) / (P[P_J_CP] * P[P_J_CP]);
-  // p_atm: through 1/p_atm and through q_0 = x_t - p_atm (pressures)
-  th[P_P_ATM] += -static_cast<double>(g.inv_p_atm) / (P[P_P_ATM] * P[P_P_ATM]) -
-                 static_cast<double>(l0) - static_cast<double>(l2);
-  // candidate constants
-  const double gV0 = g.V0, gy = g.y_scale;
-  const double gW = static_cast<double>(g.W_o2) + gV0 * Kp * lam / xo2 - gy * y_scale / W_o2;
-  th[P_M_O2] += gW * W_o2 / P[P_M_O2];
-  th[P_N_CELL] += gW * W_o2 / P[P_N_CELL];
-  th[P_FARADAY] += -gW * W_o2 / P[P_FARADAY];
-  th[P_C0] += gV0;
-  th[P_C1] += gV0 * I;
-  th[P_C2] += gV0 * I * I;
-  th[P_K_P] += gV0 * lam * W_o2 / xo2;
-  th[P_LAM_REF] += gV0 * Kp * W_o2 / xo2;
-  th[P_X_O2] += -gV0 * Kp * lam * W_o2 / (xo2 * xo2) + gy * y_scale / xo2;
-  const double dI = gW * W_o2 / I + gV0 * (P[P_C1] + 2.0 * P[P_C2] * I);
-  out[0] = dI * (r - v_prev);
-  out[1] = l0;
-  out[2] = l1;
-  out[3] = l2;
+  if (threadIdx.x < RRG_NPARAM) th[threadIdx.x] = 0.0;
+  __syncwarp();
+  if (threadIdx.x == 0) {
+    th[P_A_W] = g_a_w;
+    th[P_A_P] = g_a_p;
+    th[P_K_SM] = g_k_sm + quo[0];
+    th[P_K_CA] = g_k_ca;
+    th[P_GAMMA] = quo[1];
+    th[P_C_P] = quo[2];
+    th[P_T_ATM] = quo[3];
+    th[P_ETA_CP] = quo[4];
+    th[P_ETA_CM] = quo[5];
+    th[P_K_T] = quo[6];
+    th[P_R_CM] = quo[7];
+    th[P_K_V] = g_k_v;
+    th[P_K_P] = g_K_p + quo[18];
+    th[P_R_A] = quo[8] + quo[9];
+    th[P_T_ST] = quo[10] + quo[11];
+    th[P_V_CA] = quo[12];
+    th[P_V_SM] = quo[13];
+    th[P_J_CP] = quo[14];
+    // p_atm: through 1/p_atm and through q_0 = x_t - p_atm (pressures)
+    th[P_P_ATM] = quo[15] - lam_x[0] - lam_x[2];
+    th[P_M_O2] = quo[22];
+    th[P_N_CELL] = quo[23];
+    th[P_FARADAY] = quo[24];
+    th[P_C0] = gV0;
+    th[P_C1] = gV0 * I;
+    th[P_C2] = gV0 * I * I;
+    th[P_LAM_REF] = quo[19];
+    th[P_X_O2] = quo[20] + quo[21];
+    const double dI = quo[25] + gV0 * (P[P_C1] + 2.0 * P[P_C2] * I);
+    out[0] = dI * (r - v_prev);
+  }
+  if (threadIdx.x < 3) out[1 + threadIdx.x] = lam_x[threadIdx.x];
+  __syncwarp();
   // theta'_p = theta_p m_p^{k*}: back to the nominal parameters
-  for (int i = 0; i < RRG_NPARAM; ++i)
-    out[4 + i] = L.pmul ? th[i] * L.pmul[static_cast<size_t>(k) * RRG_NPARAM + i] : th[i];
+  if (threadIdx.x < RRG_NPARAM)
+    out[4 + threadIdx.x] =
+        L.pmul ? th[threadIdx.x] * L.pmul[static_cast<size_t>(k) * RRG_NPARAM + threadIdx.x] : th[threadIdx.x];
 }
 
 }  // namespace
@@ -623,7 +760,7 @@ adjoint_reverse_kernel(const Launch L, const DT* __restrict__ d,
 // (kappas in cand_kappa); launch_adjoint_reverse the reverse sweeps of slots
 // slot0 .. slot0 + count - 1 on the states the forward pass saved.
 // ckpt: m N (H / checkpoint + 1) 3 doubles; lane_min / lane_arg: m N each;
-// seg: m (H + 1) 12 values of T; d_out: m kOutStride doubles (per slot: g,
+// seg: m (H + 1) 3 values of T; d_out: m kOutStride doubles (per slot: g,
 // k*, j*, then dg/dkappa, dg/dx_t, dg/dtheta).  fwd_begin / fwd_end (either
 // may be null): events around the forward kernel.  The binary32 gradient
 // reads the stored binary32 disturbances when the handle draws them (the

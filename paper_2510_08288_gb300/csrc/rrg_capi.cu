@@ -575,7 +575,7 @@ namespace {
 int adj_buffers(rrg_ctx* h, size_t M, int checkpoint) {
   const size_t N = h->cfg.n_scenarios, H = h->cfg.horizon;
   const size_t ckpt_need = M * N * (H / checkpoint + 1) * 3;
-  const size_t seg_need = M * (H + 1) * 12;  // every step's state and stage points, per kappa
+  const size_t seg_need = M * (H + 1) * 3;  // every step's state, per kappa
   if (ckpt_need > h->adj_ckpt_cap || seg_need > h->adj_seg_cap || M * N > h->adj_lane_cap)
     CK(cudaStreamSynchronize(h->stream));
   CK(grow(&h->adj_ckpt, &h->adj_ckpt_cap, ckpt_need));
