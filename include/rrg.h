@@ -84,7 +84,11 @@ extern "C" {
 #define RRG_EXIT_LANE       1  /* a trajectory stops at its first violation
                                   (Sec. III-B/C)                             */
 #define RRG_EXIT_CANDIDATE  2  /* additionally, all trajectories of a
-                                  candidate stop once one of them violates   */
+                                  candidate stop once one of them violates,
+                                  and in a grid or k-section search (whose
+                                  result is the largest admissible candidate)
+                                  once a larger candidate has passed all of
+                                  its own                                     */
 
 #define RRG_NPARAM 27         /* length of the FC3 parameter vector          */
 #define RRG_MAX_CANDIDATES 1024

@@ -92,7 +92,8 @@ struct BLaunch {
   int32_t* cand_ss;
   unsigned long long* cand_min;
   int32_t* tile_base;  // [S + 1] over `order`
-  uint32_t* queue;     // [0] next tile, [1] tiles of the round, [2] CTAs that take tiles
+  uint32_t* queue;     // [0] next tile, [1] tiles of the round, [2] CTAs that take tiles, [3] tiles of a row,
+                       // [4] the first tiles' row (top-down; else [3] = [1], [4] = 0)
   int sms;
   uint2* recheck_list; // (slot, k)
   uint32_t* recheck_jlast;  // the recheck runs steps 0..jlast
@@ -100,6 +101,8 @@ struct BLaunch {
   unsigned long long recheck_cap;
   DevStats* stats;
   unsigned long long* t_dev;  // closed-loop update counter
+  int32_t* cand_passed;   // trajectories that passed (top_down)
+  int top_down;           // grid and k-section with RRG_EXIT_CANDIDATE: as Launch::top_down
 };
 
 // ---------------------------------------------------------------------------
@@ -150,19 +153,24 @@ batch_sample_kernel(const BLaunch B, uint64_t seed, uint64_t base) {
 // scheduler step 1.6 times as fast as four.  Measured (rollouts of an update,
 // 8 / 12 / 16 warps per SM): 38 warps of tiles per SM 0.80 / 0.87 / 1.00 ms, 63
 // 1.56 / 1.59 / 1.77, 108 2.75 / 2.45 / 2.58, 152 2.35 / 2.14 / 2.25, 269 7.5 /
-// 6.6 / 6.9, 491 8.7 / 7.4 / 7.3, 657 12.9 / 10.9 / 10.5.
-__device__ uint32_t round_ctas(int sms, uint32_t tiles, int tile) {
+// 6.6 / 6.9, 491 8.7 / 7.4 / 7.3, 657 12.9 / 10.9 / 10.5.  Top-down rounds take
+// 8 whatever their size: the fewer candidates are under way, the fewer run
+// beside the one that passes (64 instances, an update: 4 warps 5.57 ms, 8 5.22,
+// 12 5.36, every slot 5.73; all candidates 12.8; 256 instances 60.3 -> 16.8).
+__device__ uint32_t round_ctas(int sms, uint32_t tiles, int tile, bool top_down) {
   const uint32_t per_tile = tile <= 32 ? 1u : static_cast<uint32_t>(tile) / 32u;
   const uint32_t per_cta = tile <= 32 ? 4u : per_tile;
   const unsigned long long warps = static_cast<unsigned long long>(tiles) * per_tile;
-  if (warps >= 300ull * sms) return 0xffffffffu;
-  const uint32_t want = warps < 64ull * sms ? 8u : 12u;
+  if (!top_down && warps >= 300ull * sms) return 0xffffffffu;
+  const uint32_t want = top_down || warps < 64ull * sms ? 8u : 12u;
   return (static_cast<uint32_t>(sms) * want + per_cta - 1) / per_cta;
 }
 
 // Tile list of the next round: instance order[o] contributes ceil(m / rows) x
 // ceil(N / tile) tiles (rows = 2: two candidate slots per tile); block-wide
-// inclusive scan (blockDim = kDecideThreads >= S).
+// inclusive scan (blockDim = kDecideThreads >= S).  Top-down rounds (every
+// running instance has M candidates): the list is the instances' tiles of the
+// topmost rows, then those of the next rows, and so on (tile_of).
 __device__ void build_tiles(const BLaunch& B, int tile, int rows) {
   __shared__ int sc[kDecideThreads];
   const int o = threadIdx.x;
@@ -170,7 +178,7 @@ __device__ void build_tiles(const BLaunch& B, int tile, int rows) {
   if (o < B.c.S) {
     const int s = B.order[o];
     const BState& st = B.st[s];
-    cnt = (st.done ? 0 : (st.m + rows - 1) / rows) * ((B.inst[s].N + tile - 1) / tile);
+    cnt = (st.done || st.m == 0 ? 0 : B.top_down ? 1 : (st.m + rows - 1) / rows) * ((B.inst[s].N + tile - 1) / tile);
   }
   sc[o] = cnt;
   __syncthreads();
@@ -184,8 +192,13 @@ __device__ void build_tiles(const BLaunch& B, int tile, int rows) {
   if (o == 0) {
     B.tile_base[0] = 0;
     B.queue[0] = 0u;
-    B.queue[1] = static_cast<uint32_t>(sc[B.c.S - 1]);
-    B.queue[2] = round_ctas(B.sms, static_cast<uint32_t>(sc[B.c.S - 1]), tile);
+    const uint32_t per_row = static_cast<uint32_t>(sc[B.c.S - 1]);
+    const uint32_t top = B.top_down ? (B.c.M + rows - 1) / rows - 1 : 0;
+    const uint32_t total = per_row * (top + 1);
+    B.queue[1] = total;
+    B.queue[3] = per_row;
+    B.queue[4] = top;
+    B.queue[2] = round_ctas(B.sms, total, tile, B.top_down != 0);
     *B.recheck_count = 0u;
   }
 }
@@ -334,6 +347,7 @@ __global__ void batch_prepare_kernel(const BLaunch B) {
   B.cand_ss[slot] = ok;
   B.cand_dead[slot] = ok ? 0 : 1;
   B.cand_min[slot] = dkey(inf_v<double>());
+  B.cand_passed[slot] = 0;
 }
 
 // A lane's outcome for candidate slot `slot` (called by every thread of the
@@ -365,8 +379,16 @@ __device__ __forceinline__ void batch_reduce(const BLaunch& B, size_t slot, int 
   const bool all_ok = __all_sync(0xffffffffu, lane_ok);
   const float wmin = warp_min<float>(contrib);
   const unsigned wsteps = __reduce_add_sync(0xffffffffu, steps);
+  // a candidate that every trajectory has passed stops the instance's lower ones
+  // (reduce_lane)
+  const unsigned passed = B.top_down ? __ballot_sync(0xffffffffu, active && lane_ok && !uncertain) : 0u;
   if ((threadIdx.x & 31) == 0) {
     if (!all_ok) B.cand_ok[slot] = 0;
+    if (passed != 0u) {
+      const int n = __popc(passed);
+      if (atomicAdd(B.cand_passed + slot, n) + n == B.inst[slot / B.c.M].N)
+        for (size_t q = slot - slot % B.c.M; q < slot; ++q) *const_cast<volatile int32_t*>(B.cand_dead + q) = 1;
+    }
     if (wmin < inf_v<float>()) atomicMin(B.cand_min + slot, dkey(static_cast<double>(wmin)));
     if (wsteps) atomicAdd(&B.stats->lane_steps, static_cast<unsigned long long>(wsteps));
   }
@@ -442,6 +464,26 @@ __device__ __forceinline__ void batch_tile(const BLaunch& B, int s, int i, int k
   batch_reduce(B, slot, k, active, smin, steps, jlast, eps, dead);
 }
 
+// Tile t of the round: instance s, candidate row i, block b of scenarios.
+__device__ __forceinline__ void tile_of(const BLaunch& B, uint32_t t, int tile, int* s, int* i,
+                                        int* b) {
+  const uint32_t per_row = B.queue[3], down = t / per_row;
+  t -= down * per_row;
+  // tile_base[lo] <= t < tile_base[hi]; instances without tiles have equal
+  // bases and are skipped by taking the last such lo
+  int lo = 0, hi = B.c.S;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (static_cast<uint32_t>(B.tile_base[mid]) <= t) lo = mid; else hi = mid;
+  }
+  *s = B.order[lo];
+  const int nb = (B.inst[*s].N + tile - 1) / tile;
+  const int local = static_cast<int>(t) - B.tile_base[lo];
+  *i = local / nb;
+  *b = local - *i * nb;
+  *i += static_cast<int>(B.queue[4] - down);
+}
+
 // Resident threads per SM that the register budget of the one-lane rollout
 // kernels is held to: 168 registers.  Measured on 64 instances (rollouts of an
 // update, default variant): 384 threads 11.3 ms, 512 (128 registers, the
@@ -457,20 +499,7 @@ __global__ void __launch_bounds__(TILE, kBatchThreadsPerSm / TILE) batch_rollout
     if (threadIdx.x == 0) {
       const uint32_t t = atomicAdd(B.queue, 1u);
       int s = -1, i = 0, b = 0;
-      if (t < total) {
-        // tile_base[lo] <= t < tile_base[hi]; instances without tiles have
-        // equal bases and are skipped by taking the last such lo
-        int lo = 0, hi = B.c.S;
-        while (hi - lo > 1) {
-          const int mid = (lo + hi) >> 1;
-          if (static_cast<uint32_t>(B.tile_base[mid]) <= t) lo = mid; else hi = mid;
-        }
-        s = B.order[lo];
-        const int nb = (B.inst[s].N + TILE - 1) / TILE;
-        const int local = static_cast<int>(t) - B.tile_base[lo];
-        i = local / nb;
-        b = local - i * nb;
-      }
+      if (t < total) tile_of(B, t, TILE, &s, &i, &b);
       sh[0] = s;
       sh[1] = i;
       sh[2] = b;
@@ -486,20 +515,6 @@ __global__ void __launch_bounds__(TILE, kBatchThreadsPerSm / TILE) batch_rollout
 // Persistent rollout with warp-sized tiles: each warp takes its own 32-lane
 // tile from the queue, so a warp whose lanes finish early never waits at a
 // CTA barrier for the others.
-__device__ __forceinline__ void tile_of(const BLaunch& B, uint32_t t, int tile, int* s, int* i,
-                                        int* b) {
-  int lo = 0, hi = B.c.S;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (static_cast<uint32_t>(B.tile_base[mid]) <= t) lo = mid; else hi = mid;
-  }
-  *s = B.order[lo];
-  const int nb = (B.inst[*s].N + tile - 1) / tile;
-  const int local = static_cast<int>(t) - B.tile_base[lo];
-  *i = local / nb;
-  *b = local - *i * nb;
-}
-
 template <int FEED>
 __global__ void __launch_bounds__(128, kBatchThreadsPerSm / 128) batch_rollout_warp_kernel(const BLaunch B) {
   if (blockIdx.x >= B.queue[2]) return;
@@ -757,7 +772,7 @@ __global__ void __launch_bounds__(64) batch_recheck_kernel(const BLaunch B) {
     const uint2 en = B.recheck_list[e];
     const size_t slot = en.x;
     const int k = static_cast<int>(en.y);
-    if (!B.cand_ok[slot]) continue;
+    if (!B.cand_ok[slot] || (B.top_down && B.cand_dead[slot])) continue;
     const int s = static_cast<int>(slot / B.c.M);
     const BState& st = B.st[s];
     ScenSrc src;
@@ -966,6 +981,7 @@ struct rrg_batch_ctx {
   int32_t* cand_dead = nullptr;
   int32_t* cand_ss = nullptr;
   unsigned long long* cand_min = nullptr;
+  int32_t* cand_passed = nullptr;
   int32_t* tile_base = nullptr;
   uint32_t* queue = nullptr;
   uint2* recheck_list = nullptr;
@@ -1025,7 +1041,7 @@ void bfree_all(rrg_batch_ctx* h) {
   void* ptrs[] = {h->params_dev, h->pws, h->inst_dev, h->order_dev, h->samp_base_dev, h->st, h->d32, h->d32b, h->maps_dev,
                   h->cand_kappa,
                   h->cand_v, h->cand_c64, h->cand_c32, h->cand_ok, h->cand_dead, h->cand_ss,
-                  h->cand_min, h->tile_base, h->queue, h->recheck_list, h->recheck_jlast,
+                  h->cand_min, h->cand_passed, h->tile_base, h->queue, h->recheck_list, h->recheck_jlast,
                   h->recheck_count,
                   h->stats, h->t_dev, h->amp_dev};
   for (void* p : ptrs)
@@ -1251,8 +1267,9 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   alloc(&h->cand_dead, SM);
   alloc(&h->cand_ss, SM);
   alloc(&h->cand_min, SM);
+  alloc(&h->cand_passed, SM);
   alloc(&h->tile_base, S + 1);
-  alloc(&h->queue, 3);
+  alloc(&h->queue, 5);
   alloc(&h->recheck_list, static_cast<size_t>(lanes));
   alloc(&h->recheck_jlast, static_cast<size_t>(lanes));
   alloc(&h->recheck_count, 1);
@@ -1324,6 +1341,8 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   B.c.width = M;
   B.c.ss_check = cfg->ss_check;
   B.c.early_exit = cfg->early_exit;
+  B.top_down = cfg->early_exit == RRG_EXIT_CANDIDATE &&
+                 (cfg->search == RRG_SEARCH_GRID || cfg->search == RRG_SEARCH_KSECTION);
   B.c.dt = cfg->dt;
   B.c.y_min = cfg->y_min;
   B.c.eps_abs = cfg->recheck_eps_rel * std::fabs(cfg->y_min);
@@ -1350,6 +1369,7 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
   B.cand_dead = h->cand_dead;
   B.cand_ss = h->cand_ss;
   B.cand_min = h->cand_min;
+  B.cand_passed = h->cand_passed;
   B.tile_base = h->tile_base;
   B.queue = h->queue;
   B.sms = h->sms;

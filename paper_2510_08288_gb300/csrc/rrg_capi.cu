@@ -86,6 +86,7 @@ struct rrg_ctx {
   float* d32b = nullptr;
   PowTable* pws = nullptr;      // binary64 x^e - 1 table of the model's exponent
   bool pws_ok = false;
+  bool smem_ok = false;         // the rollouts' shared-memory limits are set
   double* pmul = nullptr;       // parameter multipliers of each pair (parametric uncertainty)
   double* pmulb = nullptr;
   ScenFold fold{}, foldb{};     // the folded models of each pair's scenarios
@@ -291,6 +292,10 @@ void fill_launch(rrg_ctx* h) {
   L.H = c.horizon;
   L.precision = c.precision;
   L.early_exit = c.early_exit;
+  L.top_down = c.early_exit == RRG_EXIT_CANDIDATE &&
+                       (c.search == RRG_SEARCH_GRID || c.search == RRG_SEARCH_KSECTION)
+                   ? (h->smem_ok ? 2 : 1)
+                   : 0;
   L.m_cap = c.max_candidates;
   L.dt = c.dt;
   L.y_min = c.y_min;
@@ -849,7 +854,8 @@ int rrg_create(const double* model_params, int n_params, const rrg_config* cfg, 
   // set once here (never inside a capture)
   (void)pair_blocks_per_sm(false);
   (void)pair_blocks_per_sm(true);
-  if (!c.scenarios_in_register && c.n_scenarios % 4 == 0 && tma_ring_prepare() &&
+  h->smem_ok = tma_ring_prepare();
+  if (!c.scenarios_in_register && c.n_scenarios % 4 == 0 && h->smem_ok &&
       encode_scenario_map(&h->tmap[0], h->d32, c.n_scenarios, c.horizon)) {
     h->tmap[1] = h->tmap[0];
     h->tma_ok = true;
@@ -960,6 +966,7 @@ int rrg_eval_candidates(rrg_handle h, const double* x_t, double v_prev, double r
   CK(cudaMemcpyAsync(h->io_dev, h->io_h, IO_LEN * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   CK(cudaMemcpyAsync(h->kap_dev, kap_h, m * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   Launch L = h->L;
+  L.top_down = 0;  // every candidate's outcome is asked for
   int early = h->cfg.early_exit;
   if (P) {
     if (!h->P_dev) CK(cudaMalloc(reinterpret_cast<void**>(&h->P_dev),

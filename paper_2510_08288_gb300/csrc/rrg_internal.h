@@ -93,6 +93,7 @@ struct SearchState {
   int32_t w_iter, w_any;
   int32_t slot_of_node[kMaxTreeNodes];   // bisection tree: heap node -> slot
   int32_t slot_of_node1[kMaxTreeNodes];  // tree of the pipelined second round
+  int32_t passed[RRG_MAX_CANDIDATES];  // trajectories that passed, per slot (Launch::top_down)
 };
 
 // Device counters of a handle.
@@ -225,6 +226,12 @@ struct Launch {
   int inject;                   // RRG_INJECT_* test switches (0 in normal use)
   int tma_pair_bps;             // resident blocks per SM of the paired TMA kernel (0: never paired)
   EqModel eq;
+  // Only the largest admissible candidate counts (grid and k-section searches
+  // with RRG_EXIT_CANDIDATE, whose candidates ascend with their slot): rows run
+  // from the largest kappa down, and a candidate that every trajectory has
+  // passed stops those below it.  2: the kernels' shared-memory limits are
+  // set (top_down_pad).
+  int top_down;
 };
 
 // Folds the FC3 parameter vector into the constants the kernels use

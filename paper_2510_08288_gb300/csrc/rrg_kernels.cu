@@ -422,8 +422,18 @@ __device__ __forceinline__ void reduce_lane(const Launch& L, int i, int k, int N
   const bool all_ok = __all_sync(0xffffffffu, lane_ok);
   const T wmin = warp_min<T>(contrib);
   const unsigned wsteps = __reduce_add_sync(0xffffffffu, steps);
+  // Largest-admissible searches (Launch::top_down): a candidate all of
+  // whose trajectories are decided and admissible stops those below it.  (A
+  // lane that was stopped counts too, but then its candidate has a violated
+  // lane, which never does, or is itself below an admissible one.)
+  const unsigned passed = L.top_down ? __ballot_sync(0xffffffffu, final_lane && lane_ok && !uncertain) : 0u;
   if ((threadIdx.x & 31) == 0) {
     if (!all_ok) L.cand_ok[i] = 0;
+    if (passed != 0u) {
+      const int n = __popc(passed);
+      if (atomicAdd(L.st->passed + i, n) + n == N)
+        for (int q = 0; q < i; ++q) *const_cast<volatile int32_t*>(L.cand_dead + q) = 1;
+    }
     if (wmin < inf_v<T>()) atomicMin(L.cand_min + i, dkey(static_cast<double>(wmin)));
     if (wsteps) {
       atomicAdd(&L.stats->lane_steps, static_cast<unsigned long long>(wsteps));
@@ -453,7 +463,7 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
   if (y < y1) {
     idle = SH && y >= s0.count;
     mode = s0.mode;
-    i = idle ? 0 : mode == SEG_CONTINUE ? L.st->cont_slot[y] : s0.base + y;
+    i = idle ? 0 : mode == SEG_CONTINUE ? L.st->cont_slot[y] : s0.base + (L.top_down ? s0.count - 1 - y : y);
   } else if (y - y1 < s1.count) {
     mode = s1.mode;
     i = s1.base + (y - y1);
@@ -817,6 +827,22 @@ rollout_tma_pair_kernel(const Launch L, const RhsC<float>* __restrict__ cand,
 #define RRG_TMA_MIN_WARPS_PER_SM 24
 #endif
 
+// Shared memory a top-down launch's blocks ask for beyond their `own` bytes, so
+// that an SM holds only as many of them as one candidate (and a tenth) takes:
+// candidates below the one that will pass are then not under way beside it.
+// Rollouts of an update, 16 candidates x 5,000 steps, parametric, all
+// candidates / top-down at full residency / held to one candidate: 4,096
+// scenarios 2.37 / 2.04 / 1.46 ms, 16,384 6.06 / 3.41 / 1.86, 32,768 - / 4.23 /
+// 2.46, 65,536 14.4 / 4.71 / 4.50.
+constexpr size_t kSmShared = 227u << 10;
+size_t top_down_pad(const Launch& L, size_t own) {
+  if (L.top_down != 2) return 0;
+  const long long need = ((L.N + 31) / 32 * 11LL + 9) / 10;  // warps of a candidate and a tenth
+  long long b = (need + 4LL * L.sms - 1) / (4LL * L.sms);
+  const size_t per = kSmShared / static_cast<size_t>(b + 1) + 1024;
+  return per > own && per <= kSmShared / static_cast<size_t>(b) - 1024 ? per - own : 0;
+}
+
 cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int early_exit,
                            bool recheck_classify, bool allow_pair) {
   dim3 grid((L.N + kRollThreads - 1) / kRollThreads, m_launch);
@@ -876,10 +902,10 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
         rollout_tma_pair_kernel<false><<<g2, kRollThreads, kTmaSmemBytes, L.stream>>>(
             L, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
     } else if (L.pmul) {
-      rollout_tma_kernel<true><<<grid, kRollThreads, kTmaSmemBytes, L.stream>>>(
+      rollout_tma_kernel<true><<<grid, kRollThreads, kTmaSmemBytes + top_down_pad(L, kTmaSmemBytes), L.stream>>>(
           L, L.d32, L.d32b, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
     } else {
-      rollout_tma_kernel<false><<<grid, kRollThreads, kTmaSmemBytes, L.stream>>>(
+      rollout_tma_kernel<false><<<grid, kRollThreads, kTmaSmemBytes + top_down_pad(L, kTmaSmemBytes), L.stream>>>(
           L, L.d32, L.d32b, L.cand_c32, early_exit, cls, L.tmap[0], L.tmap[1]);
     }
   } else if (allow_pair && !L.scen_gen && m_launch > 1 && (L.pair == RRG_PAIR_ALWAYS || filled)) {
@@ -899,6 +925,7 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
     // the first form 122 against 191 us; 24 candidates 204 against 190).  Two
     // segments, each in whole blocks.
     const long long tiles = (L.N + 31) / 32;
+    const size_t qpad = top_down_pad(L, qring_bytes(kRollThreads));
     const bool gen8 = tiles * ((m_launch + 3) / 4) > sms;
     const int gr = gen8 ? 8 : 4;
     const dim3 gs(static_cast<unsigned>(tiles), (m_launch + gr - 1) / gr + 1);
@@ -910,9 +937,12 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
       else if (gen8) RRG_ROLLOUT_GEN(rollout_kernel, SRC_GEN8);
       else RRG_ROLLOUT_GEN(rollout_kernel, SRC_GEN4);
     } else if (L.pmul) {
-      RRG_ROLLOUT(rollout_pu_kernel, float, SRC_QRING, L.d32, L.d32b, L.cand_c32, cls);
+      rollout_pu_kernel<float, SRC_QRING><<<grid, kRollThreads, qpad, L.stream>>>(L, L.d32, L.d32b, L.cand_c32,
+                                                                                 early_exit, cls);
     } else {
-      if (L.quads) RRG_ROLLOUT(rollout_kernel, float, SRC_QRING, L.d32, L.d32b, L.cand_c32, cls);
+      if (L.quads)
+        rollout_kernel<float, SRC_QRING><<<grid, kRollThreads, qpad, L.stream>>>(L, L.d32, L.d32b, L.cand_c32,
+                                                                                early_exit, cls);
       else if (ring) RRG_ROLLOUT(rollout_kernel, float, SRC_RING, L.d32, L.d32b, L.cand_c32, cls);
       else RRG_ROLLOUT(rollout_kernel, float, SRC_REGS, L.d32, L.d32b, L.cand_c32, cls);
     }
@@ -936,8 +966,9 @@ recheck_kernel(const Launch L, int early_exit) {
     const int j_end = min(static_cast<int>(L.recheck_jlast[e]), L.H);
     const int i = static_cast<int>(idx / static_cast<uint32_t>(N));
     const int k = static_cast<int>(idx - static_cast<uint32_t>(i) * static_cast<uint32_t>(N));
-    // a failed candidate needs no more decisions, unless P asks for every entry
-    if (L.P == nullptr && !L.cand_ok[i]) continue;
+    // a failed candidate, or one below an admissible one, needs no more
+    // decisions, unless P asks for every entry
+    if (L.P == nullptr && (!L.cand_ok[i] || (L.top_down && L.cand_dead[i]))) continue;
     unsigned steps = 0;
     double smin;
     RhsC<double> R = L.cand_c64[i];
@@ -978,7 +1009,7 @@ bool tma_ring_prepare() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return false;
   const int st = state[dev].load();
   if (st != 0) return st == 1;
-  const int sm = static_cast<int>(kTmaSmemBytes);
+  const int sm = static_cast<int>(kSmShared);
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   // An SM runs blocks of two kernels at once only under one division of its
   // memory between L1 and shared memory.  The rollouts' rings want nearly all
@@ -993,7 +1024,10 @@ bool tma_ring_prepare() {
                   cudaFuncSetAttribute(rollout_tma_kernel<true>, a, sm) == cudaSuccess &&
                   cudaFuncSetAttribute(rollout_tma_pair_kernel<false>, a, sm) == cudaSuccess &&
                   cudaFuncSetAttribute(rollout_tma_pair_kernel<true>, a, sm) == cudaSuccess;
-  state[dev].store(ok ? 1 : 2);
+  const int qs = static_cast<int>(kSmShared - qring_bytes(kRollThreads));
+  const bool okq = cudaFuncSetAttribute(rollout_kernel<float, SRC_QRING>, a, qs) == cudaSuccess &&
+                   cudaFuncSetAttribute(rollout_pu_kernel<float, SRC_QRING>, a, qs) == cudaSuccess;
+  state[dev].store(ok && okq ? 1 : 2);
   return ok;
 }
 
@@ -1279,6 +1313,7 @@ __device__ void prepare_slot(const Launch& L, int i) {
   L.cand_ss[i] = ok;
   L.cand_dead[i] = ok ? 0 : 1;
   L.cand_min[i] = dkey(inf_v<double>());
+  if (i < RRG_MAX_CANDIDATES) L.st->passed[i] = 0;
 }
 
 // One block per candidate slot of the round the search kernel just set up;
