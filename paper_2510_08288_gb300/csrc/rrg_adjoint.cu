@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(kRevThreads)
 adjoint_reverse_kernel(const Launch L, const DT* __restrict__ d,
                        int checkpoint, const double* __restrict__ ckpt, T* __restrict__ seg_all,
                        double* __restrict__ out_all, int slot0, const double* __restrict__ lane_min,
-                       const int* __restrict__ lane_arg) {
+                       const int* __restrict__ lane_arg, double* out_h, int32_t* ss_h) {
   const int i = slot0 + static_cast<int>(blockIdx.x);  // candidate slot
   const int N = L.N, H = L.H;
   // the inputs of the candidate set-up the forward pass ran on
@@ -520,10 +520,18 @@ adjoint_reverse_kernel(const Launch L, const DT* __restrict__ d,
   long long kj[2];
   memcpy(kj, o + 1, sizeof kj);
   double* out = o + 3;
+  // the slot's outputs in pinned host memory as well (out_h may be null)
+  auto to_host = [&]() {
+    if (out_h == nullptr) return;
+    for (int u = threadIdx.x; u < kOutStride; u += kRevThreads) out_h[static_cast<size_t>(i) * kOutStride + u] = o[u];
+    if (threadIdx.x == 0) ss_h[i] = L.cand_ss[i];
+  };
   T* seg = seg_all + static_cast<size_t>(i) * (H + 1) * kSegVals;
   const double v = L.cand_v[i];
   if (kj[0] < 0 || kj[0] >= N || kj[1] < 0 || kj[1] > H) {  // no argmin: same for every thread
     if (threadIdx.x < 4 + RRG_NPARAM) out[threadIdx.x] = NAN;
+    __syncthreads();
+    to_host();
     return;
   }
   const int k = static_cast<int>(kj[0]), jstar = static_cast<int>(kj[1]);
@@ -665,92 +673,95 @@ adjoint_reverse_kernel(const Launch L, const DT* __restrict__ d,
     if ((threadIdx.x & 7) == 0) tot[u] = static_cast<double>(s);
   }
   __syncthreads();
-  if (threadIdx.x >= 32) return;
-  // chain rule to the parameter vector (binary64): numerators and
-  // denominators by lane 0, the quotients by the lanes
-  const double g_a_w = tot[0], g_a_p = tot[1], g_k_sm = tot[2], g_k_ca = tot[3], g_e = tot[4], gc = tot[5], gm = tot[6],
-               g_k_v = tot[7], g_K_p = tot[8], ga = tot[9], gs = tot[10], gJ = tot[11], gp = tot[12], gW_o2 = tot[13],
-               gV0 = tot[14], gy = static_cast<double>(q_sm - q_ca);
-  const double I = v, W_o2 = C64.W_o2, y_scale = C64.y_scale;
-  const double lam = P[P_LAM_REF], xo2 = P[P_X_O2], Kp = P[P_K_P], gamma = P[P_GAMMA];
-  if (threadIdx.x == 0) {
-    auto set = [&](int q, double a, double b) {
-      num[q] = a;
-      den[q] = b;
-    };
-    set(0, gy * y_scale, P[P_K_SM]);
-    set(1, g_e, gamma * gamma);
-    set(2, gc * P[P_T_ATM], P[P_ETA_CP]);
-    set(3, gc * P[P_C_P], P[P_ETA_CP]);
-    set(4, -gc * K64.C_cp, P[P_ETA_CP]);
-    set(5, gm * P[P_K_T], P[P_R_CM]);
-    set(6, gm * P[P_ETA_CM], P[P_R_CM]);
-    set(7, -gm * K64.C_m, P[P_R_CM]);
-    set(8, ga * P[P_T_ST], P[P_V_CA]);
-    set(9, gs * P[P_T_ST], P[P_V_SM]);
-    set(10, ga * P[P_R_A], P[P_V_CA]);
-    set(11, gs * P[P_R_A], P[P_V_SM]);
-    set(12, -ga * K64.RT_Vca, P[P_V_CA]);
-    set(13, -gs * K64.RT_Vsm, P[P_V_SM]);
-    set(14, -gJ, P[P_J_CP] * P[P_J_CP]);
-    set(15, -gp, P[P_P_ATM] * P[P_P_ATM]);
-    const double vk = gV0 * Kp, vl = gV0 * lam * W_o2, yg = gy * y_scale;
-    set(16, vk * lam, xo2);
-    set(17, yg, W_o2);
-    set(18, vl, xo2);
-    set(19, vk * W_o2, xo2);
-    set(20, -vk * lam * W_o2, xo2 * xo2);
-    set(21, yg, xo2);
+  if (threadIdx.x < 32) {
+    // chain rule to the parameter vector (binary64): numerators and
+    // denominators by lane 0, the quotients by the lanes
+    const double g_a_w = tot[0], g_a_p = tot[1], g_k_sm = tot[2], g_k_ca = tot[3], g_e = tot[4], gc = tot[5], gm = tot[6],
+                 g_k_v = tot[7], g_K_p = tot[8], ga = tot[9], gs = tot[10], gJ = tot[11], gp = tot[12], gW_o2 = tot[13],
+                 gV0 = tot[14], gy = static_cast<double>(q_sm - q_ca);
+    const double I = v, W_o2 = C64.W_o2, y_scale = C64.y_scale;
+    const double lam = P[P_LAM_REF], xo2 = P[P_X_O2], Kp = P[P_K_P], gamma = P[P_GAMMA];
+    if (threadIdx.x == 0) {
+      auto set = [&](int q, double a, double b) {
+        num[q] = a;
+        den[q] = b;
+      };
+      set(0, gy * y_scale, P[P_K_SM]);
+      set(1, g_e, gamma * gamma);
+      set(2, gc * P[P_T_ATM], P[P_ETA_CP]);
+      set(3, gc * P[P_C_P], P[P_ETA_CP]);
+      set(4, -gc * K64.C_cp, P[P_ETA_CP]);
+      set(5, gm * P[P_K_T], P[P_R_CM]);
+      set(6, gm * P[P_ETA_CM], P[P_R_CM]);
+      set(7, -gm * K64.C_m, P[P_R_CM]);
+      set(8, ga * P[P_T_ST], P[P_V_CA]);
+      set(9, gs * P[P_T_ST], P[P_V_SM]);
+      set(10, ga * P[P_R_A], P[P_V_CA]);
+      set(11, gs * P[P_R_A], P[P_V_SM]);
+      set(12, -ga * K64.RT_Vca, P[P_V_CA]);
+      set(13, -gs * K64.RT_Vsm, P[P_V_SM]);
+      set(14, -gJ, P[P_J_CP] * P[P_J_CP]);
+      set(15, -gp, P[P_P_ATM] * P[P_P_ATM]);
+      const double vk = gV0 * Kp, vl = gV0 * lam * W_o2, yg = gy * y_scale;
+      set(16, vk * lam, xo2);
+      set(17, yg, W_o2);
+      set(18, vl, xo2);
+      set(19, vk * W_o2, xo2);
+      set(20, -vk * lam * W_o2, xo2 * xo2);
+      set(21, yg, xo2);
+    }
+    __syncwarp();
+    if (threadIdx.x < 22) quo[threadIdx.x] = num[threadIdx.x] / den[threadIdx.x];
+    __syncwarp();
+    const double gW = gW_o2 + quo[16] - quo[17];
+    if (threadIdx.x < 4) {
+      const double a = threadIdx.x == 2 ? -(gW * W_o2) : gW * W_o2;
+      const double b = threadIdx.x == 0 ? P[P_M_O2] : threadIdx.x == 1 ? P[P_N_CELL] : threadIdx.x == 2 ? P[P_FARADAY] : I;
+      quo[22 + threadIdx.x] = a / b;
+    }
+    if (threadIdx.x < RRG_NPARAM) th[threadIdx.x] = 0.0;
+    __syncwarp();
+    if (threadIdx.x == 0) {
+      th[P_A_W] = g_a_w;
+      th[P_A_P] = g_a_p;
+      th[P_K_SM] = g_k_sm + quo[0];
+      th[P_K_CA] = g_k_ca;
+      th[P_GAMMA] = quo[1];
+      th[P_C_P] = quo[2];
+      th[P_T_ATM] = quo[3];
+      th[P_ETA_CP] = quo[4];
+      th[P_ETA_CM] = quo[5];
+      th[P_K_T] = quo[6];
+      th[P_R_CM] = quo[7];
+      th[P_K_V] = g_k_v;
+      th[P_K_P] = g_K_p + quo[18];
+      th[P_R_A] = quo[8] + quo[9];
+      th[P_T_ST] = quo[10] + quo[11];
+      th[P_V_CA] = quo[12];
+      th[P_V_SM] = quo[13];
+      th[P_J_CP] = quo[14];
+      // p_atm: through 1/p_atm and through q_0 = x_t - p_atm (pressures)
+      th[P_P_ATM] = quo[15] - lam_x[0] - lam_x[2];
+      th[P_M_O2] = quo[22];
+      th[P_N_CELL] = quo[23];
+      th[P_FARADAY] = quo[24];
+      th[P_C0] = gV0;
+      th[P_C1] = gV0 * I;
+      th[P_C2] = gV0 * I * I;
+      th[P_LAM_REF] = quo[19];
+      th[P_X_O2] = quo[20] + quo[21];
+      const double dI = quo[25] + gV0 * (P[P_C1] + 2.0 * P[P_C2] * I);
+      out[0] = dI * (r - v_prev);
+    }
+    if (threadIdx.x < 3) out[1 + threadIdx.x] = lam_x[threadIdx.x];
+    __syncwarp();
+    // theta'_p = theta_p m_p^{k*}: back to the nominal parameters
+    if (threadIdx.x < RRG_NPARAM)
+      out[4 + threadIdx.x] =
+          L.pmul ? th[threadIdx.x] * L.pmul[static_cast<size_t>(k) * RRG_NPARAM + threadIdx.x] : th[threadIdx.x];
   }
-  __syncwarp();
-  if (threadIdx.x < 22) quo[threadIdx.x] = num[threadIdx.x] / den[threadIdx.x];
-  __syncwarp();
-  const double gW = gW_o2 + quo[16] - quo[17];
-  if (threadIdx.x < 4) {
-    const double a = threadIdx.x == 2 ? -(gW * W_o2) : gW * W_o2;
-    const double b = threadIdx.x == 0 ? P[P_M_O2] : threadIdx.x == 1 ? P[P_N_CELL] : threadIdx.x == 2 ? P[P_FARADAY] : I;
-    quo[22 + threadIdx.x] = a / b;
-  }
-  if (threadIdx.x < RRG_NPARAM) th[threadIdx.x] = 0.0;
-  __syncwarp();
-  if (threadIdx.x == 0) {
-    th[P_A_W] = g_a_w;
-    th[P_A_P] = g_a_p;
-    th[P_K_SM] = g_k_sm + quo[0];
-    th[P_K_CA] = g_k_ca;
-    th[P_GAMMA] = quo[1];
-    th[P_C_P] = quo[2];
-    th[P_T_ATM] = quo[3];
-    th[P_ETA_CP] = quo[4];
-    th[P_ETA_CM] = quo[5];
-    th[P_K_T] = quo[6];
-    th[P_R_CM] = quo[7];
-    th[P_K_V] = g_k_v;
-    th[P_K_P] = g_K_p + quo[18];
-    th[P_R_A] = quo[8] + quo[9];
-    th[P_T_ST] = quo[10] + quo[11];
-    th[P_V_CA] = quo[12];
-    th[P_V_SM] = quo[13];
-    th[P_J_CP] = quo[14];
-    // p_atm: through 1/p_atm and through q_0 = x_t - p_atm (pressures)
-    th[P_P_ATM] = quo[15] - lam_x[0] - lam_x[2];
-    th[P_M_O2] = quo[22];
-    th[P_N_CELL] = quo[23];
-    th[P_FARADAY] = quo[24];
-    th[P_C0] = gV0;
-    th[P_C1] = gV0 * I;
-    th[P_C2] = gV0 * I * I;
-    th[P_LAM_REF] = quo[19];
-    th[P_X_O2] = quo[20] + quo[21];
-    const double dI = quo[25] + gV0 * (P[P_C1] + 2.0 * P[P_C2] * I);
-    out[0] = dI * (r - v_prev);
-  }
-  if (threadIdx.x < 3) out[1 + threadIdx.x] = lam_x[threadIdx.x];
-  __syncwarp();
-  // theta'_p = theta_p m_p^{k*}: back to the nominal parameters
-  if (threadIdx.x < RRG_NPARAM)
-    out[4 + threadIdx.x] =
-        L.pmul ? th[threadIdx.x] * L.pmul[static_cast<size_t>(k) * RRG_NPARAM + threadIdx.x] : th[threadIdx.x];
+  __syncthreads();
+  to_host();
 }
 
 }  // namespace
@@ -810,17 +821,20 @@ cudaError_t launch_adjoint_forward(const Launch& L, bool fp64, int m, int checkp
 
 cudaError_t launch_adjoint_reverse(const Launch& L, bool fp64, int slot0, int count, int checkpoint,
                                    const double* ckpt, void* seg, double* d_out, const double* lane_min,
-                                   const int* lane_arg) {
+                                   const int* lane_arg, double* out_h, int32_t* ss_h) {
   if (count < 1 || slot0 < 0) return cudaErrorInvalidConfiguration;
   if (fp64)
     adjoint_reverse_kernel<double, double><<<count, kRevThreads, 0, L.stream>>>(
-        L, L.d64, checkpoint, ckpt, static_cast<double*>(seg), d_out, slot0, lane_min, lane_arg);
+        L, L.d64, checkpoint, ckpt, static_cast<double*>(seg), d_out, slot0, lane_min, lane_arg, out_h,
+        ss_h);
   else if (reads32(L, fp64))
     adjoint_reverse_kernel<float, float><<<count, kRevThreads, 0, L.stream>>>(
-        L, L.d32, adj_spacing(checkpoint), ckpt, static_cast<float*>(seg), d_out, slot0, lane_min, lane_arg);
+        L, L.d32, adj_spacing(checkpoint), ckpt, static_cast<float*>(seg), d_out, slot0, lane_min, lane_arg, out_h,
+        ss_h);
   else
     adjoint_reverse_kernel<float, double><<<count, kRevThreads, 0, L.stream>>>(
-        L, L.d64, checkpoint, ckpt, static_cast<float*>(seg), d_out, slot0, lane_min, lane_arg);
+        L, L.d64, checkpoint, ckpt, static_cast<float*>(seg), d_out, slot0, lane_min, lane_arg, out_h,
+        ss_h);
   return cudaGetLastError();
 }
 

@@ -115,7 +115,7 @@ struct rrg_ctx {
   uint64_t cl_key_seed = 0, cl_key_t0 = 0;
   uint64_t cl_per = 0, cl_rl_per = 0, cl_rd_per = 0;
   bool cl_conditional = false;  // the cached graph uses a conditional node
-  // the captured search of rrg_step (fixed io_dev / flag_dev pointers),
+  // the captured search of rrg_step (fixed io_h / flag_h pointers),
   // discarded whenever the launch descriptor changes (fill_launch)
   cudaGraphExec_t st_exec = nullptr;
   uint64_t st_per = 0, st_rl_per = 0, st_rd_per = 0;
@@ -145,7 +145,6 @@ struct rrg_ctx {
   double* io_dev = nullptr;     // [0..2] x, [3] r, [4] v, [5..8] out, [8] amp.. see offsets
   int32_t* flag_dev = nullptr;  // [0] flags, [1] status
   double* kap_dev = nullptr;    // [m_cap] kappas in, [m_cap] min slack out
-  uint8_t* adm_dev = nullptr;
   LoopState* loop = nullptr;
   // closed-loop I/O staging (grown on demand)
   double* cl_dev = nullptr;
@@ -248,7 +247,7 @@ void free_all(rrg_ctx* h) {
   void* ptrs[] = {h->params_dev, h->d64, h->d32, h->d64b, h->d32b, h->st, h->cand_kappa,
                   h->cand_v, h->cand_c64, h->cand_c32, h->cand_ok, h->cand_dead, h->cand_ss,
                   h->cand_min, h->recheck_list, h->recheck_jlast, h->recheck_count, h->stats, h->P_dev, h->io_dev,
-                  h->flag_dev, h->kap_dev, h->adm_dev, h->loop, h->cl_dev, h->lane_state,
+                  h->flag_dev, h->kap_dev, h->loop, h->cl_dev, h->lane_state,
                   h->adj_ckpt, h->adj_lane_min, h->adj_lane_arg, h->adj_seg, h->adj_out,
                   h->pmul, h->pmulb, h->pws, h->err_buf, h->fold.d, h->fold.f, h->foldb.d, h->foldb.f};
   for (void* p : ptrs)
@@ -607,17 +606,15 @@ int adj_buffers(rrg_ctx* h, size_t M, int checkpoint) {
   return RRG_OK;
 }
 
-// The inputs of an adjoint call into io_dev (x_t, r_t, v_prev) and kap_dev
-// (the m kappas), from the pinned staging.
-int adj_upload(rrg_ctx* h, const double* x_t, double v_prev, double r_t, const double* kappas, int m) {
+// The inputs of an adjoint call (x_t, r_t, v_prev, the m kappas) in the pinned
+// staging, where the set-up kernel reads them; every call waits for its kernels
+// before the staging is written again.
+void adj_upload(rrg_ctx* h, const double* x_t, double v_prev, double r_t, const double* kappas, int m) {
   double* kap_h = h->io_h + IO_LEN;
   std::memcpy(h->io_h + IO_X, x_t, 3 * sizeof(double));
   h->io_h[IO_R] = r_t;
   h->io_h[IO_V] = v_prev;
   std::memcpy(kap_h, kappas, static_cast<size_t>(m) * sizeof(double));
-  CK(cudaMemcpyAsync(h->io_dev, h->io_h, IO_LEN * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaMemcpyAsync(h->kap_dev, kap_h, m * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-  return RRG_OK;
 }
 
 // Enqueues the candidate set-up of the m uploaded kappas (v_prev and r read
@@ -626,7 +623,7 @@ int adj_upload(rrg_ctx* h, const double* x_t, double v_prev, double r_t, const d
 int adj_enqueue_forward_kernels(rrg_ctx* h, int m, int checkpoint, int precision, bool argmin) {
   const Launch& L = h->L;
   // candidate set-up (kappas, setpoints, rollout constants, steady-state check)
-  CK(launch_eval_prepare(L, h->io_dev + IO_X, 0.0, 0.0, h->kap_dev, m, h->io_dev + IO_V, h->io_dev + IO_R));
+  CK(launch_eval_prepare(L, h->io_h + IO_X, 0.0, 0.0, h->io_h + IO_LEN, m, h->io_h + IO_V, h->io_h + IO_R));
   CK(launch_prepare(L, m));
   h->launches += 2;
   const bool use32 = precision == RRG_FP32 && h->cfg.precision != RRG_FP64 && !h->cfg.scenarios_in_register;
@@ -653,18 +650,22 @@ int adj_enqueue_forward_kernels(rrg_ctx* h, int m, int checkpoint, int precision
 int adj_enqueue_forward(rrg_ctx* h, const double* x_t, double v_prev, double r_t, const double* kappas,
                         int m, int checkpoint, int precision, bool argmin = true) {
   int rc = adj_buffers(h, static_cast<size_t>(m), checkpoint);
-  if (rc == RRG_OK) rc = adj_upload(h, x_t, v_prev, r_t, kappas, m);
-  if (rc == RRG_OK) rc = adj_enqueue_forward_kernels(h, m, checkpoint, precision, argmin);
+  if (rc != RRG_OK) return rc;
+  adj_upload(h, x_t, v_prev, r_t, kappas, m);
+  rc = adj_enqueue_forward_kernels(h, m, checkpoint, precision, argmin);
   return rc;
 }
 
 // with_argmin: the reverse sweep finds each slot's argmin itself (after a
-// forward pass enqueued without its argmin pass).
+// forward pass enqueued without its argmin pass) and leaves its outputs and
+// steady-state flag in the pinned copies too (adj_read without its copies; with
+// the inputs read in place a gradient of 4,096 binary32 scenarios 162 -> 144 us).
 int adj_enqueue_reverse(rrg_ctx* h, int slot0, int count, int checkpoint, int precision,
                         bool with_argmin = false) {
   CK(launch_adjoint_reverse(h->L, precision == RRG_FP64, slot0, count, checkpoint, h->adj_ckpt, h->adj_seg,
                             h->adj_out, with_argmin ? h->adj_lane_min : nullptr,
-                            with_argmin ? h->adj_lane_arg : nullptr));
+                            with_argmin ? h->adj_lane_arg : nullptr, with_argmin ? h->adj_out_h : nullptr,
+                            with_argmin ? h->adj_ss_h : nullptr));
   h->launches += 1;
   return RRG_OK;
 }
@@ -705,10 +706,12 @@ cudaGraphExec_t capture_gradient(rrg_ctx* h, int m, int checkpoint, int precisio
 
 // Reads slots 0..m-1 of the adjoint's output (and the steady-state flags)
 // after the stream drained.
-int adj_read(rrg_ctx* h, int m, std::vector<double>* out, std::vector<int32_t>* ss) {
+int adj_read(rrg_ctx* h, int m, std::vector<double>* out, std::vector<int32_t>* ss, bool written = false) {
   const size_t n = static_cast<size_t>(m) * kAdjOutStride;
-  CK(cudaMemcpyAsync(h->adj_out_h, h->adj_out, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  if (ss) CK(cudaMemcpyAsync(h->adj_ss_h, h->cand_ss, m * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
+  if (!written)
+    CK(cudaMemcpyAsync(h->adj_out_h, h->adj_out, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  if (ss && !written)
+    CK(cudaMemcpyAsync(h->adj_ss_h, h->cand_ss, m * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   out->assign(h->adj_out_h, h->adj_out_h + n);
   if (ss) ss->assign(h->adj_ss_h, h->adj_ss_h + m);
@@ -810,7 +813,6 @@ int rrg_create(const double* model_params, int n_params, const rrg_config* cfg, 
   ALLOC(io_dev, IO_LEN);
   ALLOC(flag_dev, 4);
   ALLOC(kap_dev, 2 * M);
-  ALLOC(adm_dev, M);
   ALLOC(loop, 1);
   if (c.param_unc_rel > 0.0) {
     ALLOC(pmul, N * RRG_NPARAM);
@@ -963,8 +965,6 @@ int rrg_eval_candidates(rrg_handle h, const double* x_t, double v_prev, double r
   uint8_t* adm_h = reinterpret_cast<uint8_t*>(h->io_h + IO_LEN + 2 * M);
   std::memcpy(h->io_h + IO_X, x_t, 3 * sizeof(double));
   std::memcpy(kap_h, kappas, m * sizeof(double));
-  CK(cudaMemcpyAsync(h->io_dev, h->io_h, IO_LEN * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaMemcpyAsync(h->kap_dev, kap_h, m * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   Launch L = h->L;
   L.top_down = 0;  // every candidate's outcome is asked for
   int early = h->cfg.early_exit;
@@ -974,15 +974,15 @@ int rrg_eval_candidates(rrg_handle h, const double* x_t, double v_prev, double r
     L.P = h->P_dev;
     if (early > RRG_EXIT_LANE) early = RRG_EXIT_LANE;
   }
-  CK(launch_eval_prepare(L, h->io_dev + IO_X, v_prev, r_t, h->kap_dev, m));
+  // the kernels read the inputs and write the outcomes in the pinned staging
+  // itself: no copies beside them (3,001 scenarios x 32 candidates 400 -> 392 us)
+  CK(launch_eval_prepare(L, h->io_h + IO_X, v_prev, r_t, kap_h, m));
   CK(launch_prepare(L, m));
   h->launches += 2;
   int rc = enqueue_round_work(h, L, m, early);
   if (rc != RRG_OK) return rc;
-  CK(launch_eval_finish(L, m, h->adm_dev, h->kap_dev + M));
+  CK(launch_eval_finish(L, m, adm_h, kap_h + M));
   h->launches++;
-  CK(cudaMemcpyAsync(adm_h, h->adm_dev, m, cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaMemcpyAsync(kap_h + M, h->kap_dev + M, m * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   if (P)
     CK(cudaMemcpyAsync(P, h->P_dev, static_cast<size_t>(m) * h->cfg.n_scenarios,
                        cudaMemcpyDeviceToHost, h->stream));
@@ -1044,7 +1044,7 @@ int rrg_slack_error(rrg_handle h, const double* x_t, double v_prev, double r_t,
   return RRG_OK;
 }
 
-// The search of rrg_step, captured once on the handle's fixed io pointers:
+// The search of rrg_step, captured once on the handle's pinned io buffers:
 // with a pipelined search the rounds after the pipelined pair are a while node
 // whose body is one round (so none runs after the search is done: a control
 // tick of 32 scenarios that needs one of the three takes 130 us, 133 with all
@@ -1054,7 +1054,7 @@ int rrg_slack_error(rrg_handle h, const double* x_t, double v_prev, double r_t,
 // nothing could be captured.
 cudaGraphExec_t capture_step(rrg_ctx* h) {
   const cudaStreamCaptureMode mode = cudaStreamCaptureModeThreadLocal;
-  double* io = h->io_dev;
+  double* io = h->io_h;  // the search kernels read the inputs and write the result in pinned host memory
   const uint64_t l0 = h->launches, r0 = h->rollout_launches, d0 = h->rounds;
   auto end_capture = [&]() {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
@@ -1078,7 +1078,7 @@ cudaGraphExec_t capture_step(rrg_ctx* h) {
       h->L.cond_launches = h->cfg.precision == RRG_FP32_RECHECK ? 3u : 2u;  // of one round
       h->L.cond_rollouts = h->L.cond_rounds = 1u;
       ok = enqueue_search(h, io + IO_X, io + IO_R, nullptr, io + IO_V, io + IO_OUT, io + IO_OUT + 1,
-                          h->flag_dev, -1, false) == RRG_OK;
+                          h->flag_h, -1, false) == RRG_OK;
       h->L.cond = 0ull;
       h->capturing = false;
       h->st_per = h->launches - l0;
@@ -1108,7 +1108,7 @@ cudaGraphExec_t capture_step(rrg_ctx* h) {
       if (ok) {
         h->capturing = true;
         h->L.cond = hc;
-        ok = enqueue_extra_rounds(h, 1, io + IO_OUT, io + IO_OUT + 1, h->flag_dev) == RRG_OK;
+        ok = enqueue_extra_rounds(h, 1, io + IO_OUT, io + IO_OUT + 1, h->flag_h) == RRG_OK;
         h->L.cond = 0ull;
         h->capturing = false;
         ok = (cudaStreamEndCapture(h->stream, &body) == cudaSuccess) && ok;
@@ -1130,7 +1130,7 @@ cudaGraphExec_t capture_step(rrg_ctx* h) {
     }
     h->capturing = true;
     const int rc = enqueue_search(h, io + IO_X, io + IO_R, nullptr, io + IO_V, io + IO_OUT, io + IO_OUT + 1,
-                                  h->flag_dev);
+                                  h->flag_h);
     h->capturing = false;
     h->st_per = h->launches - l0;
     h->st_rl_per = h->rollout_launches - r0;
@@ -1164,9 +1164,10 @@ int rrg_step(rrg_handle h, const double* x_t, double r_t, double v_prev, double*
   std::memcpy(h->io_h + IO_X, x_t, 3 * sizeof(double));
   h->io_h[IO_R] = r_t;
   h->io_h[IO_V] = v_prev;
-  CK(cudaMemcpyAsync(h->io_dev, h->io_h, 5 * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-  // the search as one graph replay (its launch gaps cost about 50 us per
-  // update when enqueued kernel by kernel), except while the library times
+  // the search as one graph replay on the pinned buffers themselves (with two
+  // copies out and one in beside it a control tick of 32 scenarios took 131 us,
+  // without 118; its launch gaps cost about 50 us per update when enqueued
+  // kernel by kernel), except while the library times
   // rollout launches (profiling), which needs the direct launches' events
   if (!h->profiling && !h->st_exec && !h->st_refused) {
     h->st_exec = capture_step(h);
@@ -1178,13 +1179,14 @@ int rrg_step(rrg_handle h, const double* x_t, double r_t, double v_prev, double*
     h->rollout_launches += h->st_rl_per;
     h->rounds += h->st_rd_per;
   } else {
+    CK(cudaMemcpyAsync(h->io_dev, h->io_h, 5 * sizeof(double), cudaMemcpyHostToDevice, h->stream));
     int rc = enqueue_search(h, h->io_dev + IO_X, h->io_dev + IO_R, nullptr, h->io_dev + IO_V,
                             h->io_dev + IO_OUT, h->io_dev + IO_OUT + 1, h->flag_dev);
     if (rc != RRG_OK) return rc;
+    CK(cudaMemcpyAsync(h->io_h + IO_OUT, h->io_dev + IO_OUT, 2 * sizeof(double),
+                       cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(h->flag_h, h->flag_dev, sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
   }
-  CK(cudaMemcpyAsync(h->io_h + IO_OUT, h->io_dev + IO_OUT, 2 * sizeof(double),
-                     cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaMemcpyAsync(h->flag_h, h->flag_dev, sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   if (v_t) *v_t = h->io_h[IO_OUT];
   if (kappa) *kappa = h->io_h[IO_OUT + 1];
@@ -1462,8 +1464,8 @@ int rrg_slack_gradients(rrg_handle h, const double* x_t, double v_prev, double r
     return set_err(h, RRG_EINVAL, "precision must be RRG_FP64 or RRG_FP32");
   DeviceGuard gd(h->device);
   int rc = adj_buffers(h, static_cast<size_t>(m), checkpoint);
-  if (rc == RRG_OK) rc = adj_upload(h, x_t, v_prev, r_t, kappas, m);
   if (rc != RRG_OK) return rc;
+  adj_upload(h, x_t, v_prev, r_t, kappas, m);
   // the kernels as one graph replay (as rrg_step), except while the library
   // times rollout launches; the graph is keyed by the call's shape and the
   // adjoint buffers (which adj_buffers may have reallocated)
@@ -1493,7 +1495,7 @@ int rrg_slack_gradients(rrg_handle h, const double* x_t, double v_prev, double r
   }
   std::vector<double> out;
   std::vector<int32_t> ss;
-  rc = adj_read(h, m, &out, ss_ok ? &ss : nullptr);
+  rc = adj_read(h, m, &out, ss_ok ? &ss : nullptr, true);
   if (rc != RRG_OK) return rc;
   for (int i = 0; i < m; ++i) {
     const double* o = out.data() + static_cast<size_t>(i) * kAdjOutStride;

@@ -568,10 +568,11 @@ cudaError_t launch_adjoint_forward(const Launch& L, bool fp64, int m, int checkp
                                    double* lane_min, int* lane_arg, double* d_out,
                                    cudaEvent_t fwd_begin, cudaEvent_t fwd_end, bool argmin = true);
 // The reverse sweeps read v_prev and r from the search state the candidate
-// set-up wrote.
+// set-up wrote.  out_h, ss_h: pinned host copies of the slots' outputs and
+// steady-state flags, written by the kernel (or null).
 cudaError_t launch_adjoint_reverse(const Launch& L, bool fp64, int slot0, int count, int checkpoint,
                                    const double* ckpt, void* seg, double* d_out,
-                                   const double* lane_min = nullptr, const int* lane_arg = nullptr);
+                                   const double* lane_min = nullptr, const int* lane_arg = nullptr, double* out_h = nullptr, int32_t* ss_h = nullptr);
 
 // Binary32-vs-binary64 slack error of every trajectory of the m candidates
 // the last eval_prepare + prepare set up (rrg_error.cu): per lane o = i N + k

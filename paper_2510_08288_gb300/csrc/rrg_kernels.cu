@@ -17,6 +17,7 @@
 //
 // Nothing returns to the host between rounds; the whole update can be
 // captured in a CUDA graph.
+#include <cstddef>
 #include <atomic>
 #include <cfloat>
 #include <cmath>
@@ -842,6 +843,13 @@ size_t top_down_pad(const Launch& L, size_t own) {
   const size_t per = kSmShared / static_cast<size_t>(b + 1) + 1024;
   return per > own && per <= kSmShared / static_cast<size_t>(b) - 1024 ? per - own : 0;
 }
+
+// The nominal binary32 lanes read their coefficients as constant operands.  Where
+// these lie decides how the compiler groups the loads of the ones it keeps in
+// registers: 8 bytes past a 16-byte line was fastest (3,001 x 32 candidates x
+// 1,000 steps and a lone warp of 2,000: 0, 4, 8, 12 bytes past it 341 / 350 / 335 /
+// 332 and 165 / 168 / 163.5 / 167.5 us).
+static_assert((offsetof(Launch, m32) + offsetof(StepModel<float>, U)) % 16 == 8, "coefficients off their line");
 
 cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int early_exit,
                            bool recheck_classify, bool allow_pair) {
