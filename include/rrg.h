@@ -389,10 +389,12 @@ RRG_API int rrg_autotune(rrg_handle h, const double *x_t, double r_t, double v_p
  * scenario array (RRG_FP32, RRG_FP32_RECHECK; scenarios_in_register = 0):
  * RRG_PAIR_NEVER, one trajectory per thread; RRG_PAIR_FILLED, two candidates
  * of one scenario per thread (one load of each disturbance, two independent
- * step chains) in register-ring launches large enough that the paired grid
- * fills the SMs at least six times over, one elsewhere (launches that take
- * the TMA ring, rrg_set_tma, stay single: the TMA ring measured faster than
- * either pairing);
+ * step chains) in launches of more than 16 warps per SM (64 with uncertain
+ * parameters) large enough that the paired grid fills the SMs at least six
+ * times over, one elsewhere (launches that take the TMA ring, rrg_set_tma,
+ * stay single: the TMA ring measured faster than either pairing; so do grid
+ * and k-section searches with RRG_EXIT_CANDIDATE, whose candidates run from
+ * the largest down);
  * RRG_PAIR_ALWAYS, two in every launch whose rows are full-horizon segments,
  * on whichever ring the launch takes (the probe and continuation launches of
  * a pipelined search never pair).
@@ -618,7 +620,7 @@ RRG_API int rrg_bisect_decide(rrg_bisect_state *s, const uint8_t *admissible, in
  * cudaDeviceReset, for example, the module and its array are loaded anew);
  * make the first call on a device, and the first after such a change, before
  * any stream capture begins.  The binary64 rollouts evaluate x^e - 1 by the
- * same series as a handle's, so results equal rrg_eval_candidates's on the
+ * same table as a handle's, so results equal rrg_eval_candidates's on the
  * same scenarios bit for bit.  Every call uses the same scratch, which
  * keeps the last call's contents; each call re-initialises everything it
  * reads, but calls that may overlap on the GPU (on different streams, or from
