@@ -57,21 +57,22 @@ RUN_UPDATES = 1000
 # updates before it run untimed (the last W of them are the warm-up).
 WINDOW_START = 115
 PROBE_STEPS = 128
-# algorithmic binary32 flops of one trajectory step, counted from the source
-# of the rollout's right-hand side with its constants multiplied out: 4
-# right-hand sides of 24 (3 MUFU operations counted as one flop each), 3
-# stage points of 6, the RK4 combination of 18, the disturbance add of 3, and
-# output, slack, running min and the finiteness accumulator of 6
+# algorithmic binary32 flops of one trajectory step, counted from the method
+# with the right-hand side's constants multiplied out and held fixed across
+# versions of the code (the folded step executes fewer): 4 right-hand sides of
+# 24 (3 MUFU operations counted as one flop each), 3 stage points of 6, the RK4
+# combination of 18, the disturbance add of 3, and output, slack, running min
+# and the finiteness accumulator of 6
 FLOPS_PER_STEP = 141
 # MUFU operations per binary32 trajectory step: per right-hand side the power
 # term's lg2 and ex2 and the torque term's reciprocal, 4 evaluations per step
 MUFU_PER_STEP = 12
-# instructions a warp issues per trajectory step in the register-ring loop
-# (ncu: instructions executed by the 65,536-scenario sweep's rollout launches
-# at 32,768 scenarios over their lane-steps / 32, parametric and nominal
-# model alike): an issue-bound step reaches at most 141 / (2 x 114) of the
-# derived FP32 peak, which counts every instruction as an FMA
-INSTR_PER_STEP = 114
+# instructions a warp issues per trajectory step on the ring of quads (ncu:
+# instructions executed by a launch of 1,024 scenarios x 16 candidates x 1,000
+# steps without early exit over its lane-steps / 32, nominal model): an
+# issue-bound step reaches at most 141 / (2 x 91) of the derived FP32 peak,
+# which counts every instruction as an FMA
+INSTR_PER_STEP = 91
 ISSUE_CEILING = FLOPS_PER_STEP / (2.0 * INSTR_PER_STEP)
 FP32_LANES_PER_SM = 128
 
@@ -134,9 +135,10 @@ def source_region(rel, begin, end):
 # reads the array once per candidate that is still running (tile-major order;
 # the 3.9 GB array does not fit in L2), up to 16 times the algorithmic bytes.
 SWEEP_TRAFFIC_64K = (7911768832 + 3319040 + 19845668096 + 436992 + 51305741824 + 906496) / 3
-# warp instructions per trajectory-step of the TMA-ring kernel there (22.50 G
-# over 6.56 G lane-steps in the same capture)
-TMA_INSTR_PER_STEP = 110
+# warp instructions per trajectory-step of the TMA-ring kernel (ncu: 728.4 M
+# over the 16,384 scenarios x 16 candidates x 1,000 steps of a nominal launch;
+# the parametric kernel, two multiply-adds per instruction, issues 76)
+TMA_INSTR_PER_STEP = 89
 
 
 # DRAM bytes of one adjoint_forward_kernel<float, float> launch on the adjoint
