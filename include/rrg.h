@@ -420,7 +420,10 @@ RRG_API int rrg_get_pairing(rrg_handle h, int32_t *mode);
  * the TMA for launches of at least 24 warps per SM, where warps compete for
  * issue and the saved load instructions pay, ahead of pairing (which it beat
  * where both apply); below, where a warp running alone would pay the
- * chunk's wait and warp votes on its dependency chain, the per-lane ring;
+ * chunk's wait and warp votes on its dependency chain, and for grid and
+ * k-section searches with uncertain parameters whose launches are held to two
+ * warps per scheduler (RRG_EXIT_CANDIDATE, up to about 35,000 scenarios), the
+ * per-lane ring;
  * RRG_TMA_ALWAYS: the TMA for every such launch.  The results are identical;
  * only the time changes.  The TMA needs stored binary32 scenarios with
  * n_scenarios a multiple of 4 (the tensor map's row stride must be a multiple

@@ -836,10 +836,19 @@ rollout_tma_pair_kernel(const Launch L, const RhsC<float>* __restrict__ cand,
 // scenarios 2.37 / 2.04 / 1.46 ms, 16,384 6.06 / 3.41 / 1.86, 32,768 - / 4.23 /
 // 2.46, 65,536 14.4 / 4.71 / 4.50.
 constexpr size_t kSmShared = 227u << 10;
+long long top_down_blocks(const Launch& L) {
+  const long long need = ((L.N + 31) / 32 * 11LL + 9) / 10;  // warps of a candidate and a tenth
+  return (need + 4LL * L.sms - 1) / (4LL * L.sms);
+}
+// Top-down launches of the parametric model held to at most two warps per
+// scheduler stay on the ring of quads under RRG_TMA_AUTO: rollouts of an update,
+// 16 candidates x 5,000 steps, TMA / quads: 8,192 scenarios 1.75 / 1.53 ms,
+// 16,384 1.84 / 1.66, 32,768 2.48 / 2.26, 49,152 (three warps) 3.18 / 3.28;
+// nominal 16,384 1.60 / 1.65, 32,768 2.16 / 2.15.
+bool top_down_lone(const Launch& L) { return L.top_down == 2 && L.pmul != nullptr && top_down_blocks(L) <= 2; }
 size_t top_down_pad(const Launch& L, size_t own) {
   if (L.top_down != 2) return 0;
-  const long long need = ((L.N + 31) / 32 * 11LL + 9) / 10;  // warps of a candidate and a tenth
-  long long b = (need + 4LL * L.sms - 1) / (4LL * L.sms);
+  const long long b = top_down_blocks(L);
   const size_t per = kSmShared / static_cast<size_t>(b + 1) + 1024;
   return per > own && per <= kSmShared / static_cast<size_t>(b) - 1024 ? per - own : 0;
 }
@@ -896,7 +905,7 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
     }
   } else if (!L.scen_gen && L.tmap != nullptr &&
              (L.tma == RRG_TMA_ALWAYS ||
-              (L.tma == RRG_TMA_AUTO && warps >= static_cast<long long>(RRG_TMA_MIN_WARPS_PER_SM) * sms))) {
+              (L.tma == RRG_TMA_AUTO && !top_down_lone(L) && warps >= static_cast<long long>(RRG_TMA_MIN_WARPS_PER_SM) * sms))) {
     // the TMA ring: one tensor copy per warp and chunk of steps (it takes
     // precedence over the register-ring pairing, which it beat where both
     // apply).  Two candidates per thread on it only with RRG_PAIR_ALWAYS:
