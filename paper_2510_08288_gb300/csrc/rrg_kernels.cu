@@ -834,7 +834,9 @@ rollout_tma_pair_kernel(const Launch L, const RhsC<float>* __restrict__ cand,
 // Rollouts of an update, 16 candidates x 5,000 steps, parametric, all
 // candidates / top-down at full residency / held to one candidate: 4,096
 // scenarios 2.37 / 2.04 / 1.46 ms, 16,384 6.06 / 3.41 / 1.86, 32,768 - / 4.23 /
-// 2.46, 65,536 14.4 / 4.71 / 4.50.
+// 2.46, 65,536 14.4 / 4.71 / 4.50.  It also spreads the survivor's blocks over
+// the SMs; round 1 at full residency, which an update without any admissible
+// candidate would prefer, takes 2.36 instead of 1.66 ms of 16,384 scenarios.
 constexpr size_t kSmShared = 227u << 10;
 long long top_down_blocks(const Launch& L) {
   const long long need = ((L.N + 31) / 32 * 11LL + 9) / 10;  // warps of a candidate and a tenth
@@ -1047,8 +1049,9 @@ bool tma_ring_prepare() {
   const int qs = static_cast<int>(kSmShared - qring_bytes(kRollThreads));
   const bool okq = cudaFuncSetAttribute(rollout_kernel<float, SRC_QRING>, a, qs) == cudaSuccess &&
                    cudaFuncSetAttribute(rollout_pu_kernel<float, SRC_QRING>, a, qs) == cudaSuccess;
+  if (!(ok && okq)) cudaGetLastError();
   state[dev].store(ok && okq ? 1 : 2);
-  return ok;
+  return ok && okq;
 }
 
 bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H) {
