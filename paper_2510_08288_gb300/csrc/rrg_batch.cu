@@ -971,6 +971,7 @@ struct rrg_batch_ctx {
   BState* st = nullptr;
   float* d32 = nullptr;
   CUtensorMap* maps_dev = nullptr;  // [2][S]
+  bool maps_ok = true;         // every instance has its tensor maps
   float* d32b = nullptr;       // second scenario pair, allocated by the first closed loop
   size_t d32_elems = 0;
   cudaStream_t side = nullptr; // draws update t + 1 while update t searches
@@ -1085,12 +1086,18 @@ void bcollect(rrg_batch_ctx* h) {
   h->ev_roll.clear();
 }
 
-// The tensor maps of a pair's scenario arrays (pair 0 or 1).
+// The tensor maps of a pair's scenario arrays (pair 0 or 1).  If one cannot be
+// encoded (encode_scenario_map) the handle has none and every round takes the
+// ring of quads.
 cudaError_t upload_maps(rrg_batch_ctx* h, const float* d32, int pair) {
+  if (!h->maps_ok) return cudaSuccess;
   std::vector<CUtensorMap> m(h->inst.size());
   for (size_t s = 0; s < m.size(); ++s) {
     const BInst& I = h->inst[s];
-    if (!encode_scenario_map(&m[s], d32 + I.off, I.N, I.H)) return cudaErrorNotSupported;
+    if (!encode_scenario_map(&m[s], d32 + I.off, I.N, I.H)) {
+      h->maps_ok = false;
+      return cudaSuccess;
+    }
   }
   return cudaMemcpy(h->maps_dev + static_cast<size_t>(pair) * m.size(), m.data(), m.size() * sizeof(CUtensorMap),
                     cudaMemcpyHostToDevice);
@@ -1121,7 +1128,8 @@ int enqueue_rollout(rrg_batch_ctx* h) {
     if (a && b) BCK(cudaEventRecord(a, h->stream));
   }
   const unsigned long long cand = h->B.c.search == RRG_SEARCH_SPEC_BISECT ? h->B.c.width : h->B.c.M;
-  const int large = h->scen_warps * cand >= static_cast<unsigned long long>(kTmaTileWarps) * h->sms ? 1 : 0;
+  const int large =
+      h->maps_ok && h->scen_warps * cand >= static_cast<unsigned long long>(kTmaTileWarps) * h->sms ? 1 : 0;
   v.kernel[large]<<<h->grid[h->variant][large], block_threads(v.tile), variant_smem(v, large), h->stream>>>(h->B);
   BCK(cudaGetLastError());
   if (timed && a && b) {
