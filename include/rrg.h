@@ -427,8 +427,9 @@ RRG_API int rrg_get_pairing(rrg_handle h, int32_t *mode);
  * RRG_TMA_ALWAYS: the TMA for every such launch.  The results are identical;
  * only the time changes.  The TMA needs stored binary32 scenarios with
  * n_scenarios a multiple of 4 (the tensor map's row stride must be a multiple
- * of 16 bytes) and a driver that encodes the map: without it rrg_get_tma
- * reports RRG_TMA_NEVER and setting another mode returns RRG_EINVAL.  Setting
+ * of 16 bytes) and at most 2^28 (the copy's coordinates are 32-bit), and a
+ * driver that encodes the map: without it rrg_get_tma reports RRG_TMA_NEVER and
+ * setting another mode returns RRG_EINVAL.  Setting
  * waits for the handle's stream and discards the cached closed-loop graph;
  * RRG_EINVAL for a mode outside 0..2. */
 #define RRG_TMA_NEVER 0

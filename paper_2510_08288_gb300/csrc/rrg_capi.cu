@@ -1793,7 +1793,7 @@ int rrg_set_tma(rrg_handle h, int mode) {
   if (mode < RRG_TMA_NEVER || mode > RRG_TMA_ALWAYS)
     return set_err(h, RRG_EINVAL, "TMA mode must be RRG_TMA_NEVER, RRG_TMA_AUTO or RRG_TMA_ALWAYS");
   if (mode != RRG_TMA_NEVER && !h->tma_ok)
-    return set_err(h, RRG_EINVAL, "no TMA ring for this handle (n_scenarios %% 4 != 0, in-register "
+    return set_err(h, RRG_EINVAL, "no TMA ring for this handle (n_scenarios %% 4 != 0 or above 2^28, in-register "
                                   "scenarios, or the driver refused the tensor map)");
   DeviceGuard g(h->device);
   CK(cudaStreamSynchronize(h->stream));

@@ -533,8 +533,12 @@ cudaError_t launch_eval_prepare(const Launch& L, const double* d_x, double v_pre
 cudaError_t launch_eval_finish(const Launch& L, int m, uint8_t* d_adm, double* d_min_slack);
 // Tensor map of a binary32 scenario array in the quad layout for the TMA ring
 // (boxes of 32 scenarios x one chunk of steps x 3 components); false when the
-// driver refuses.  tma_ring_prepare() sets the TMA kernels' shared-memory limit
+// driver refuses, and for more than kTmaMaxScenarios: a box starts at element
+// four times its scenario, a signed 32-bit coordinate, which scenario 2^29 would
+// overflow (the copy then raises an illegal instruction).  Half of that keeps
+// every sum of a coordinate and a box away from the limit.  tma_ring_prepare() sets the TMA kernels' shared-memory limit
 // on the current device (once per device); false if the runtime refuses.
+constexpr int kTmaMaxScenarios = 1 << 28;
 bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H);
 bool tma_ring_prepare();
 // Resident blocks per SM of the two-candidates-per-thread TMA kernel (after

@@ -1055,6 +1055,7 @@ bool tma_ring_prepare() {
 }
 
 bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H) {
+  if (N > kTmaMaxScenarios) return false;
   static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
     void* f = nullptr;
     cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
