@@ -1088,7 +1088,9 @@ void bcollect(rrg_batch_ctx* h) {
 
 // The tensor maps of a pair's scenario arrays (pair 0 or 1).  If one cannot be
 // encoded (encode_scenario_map) the handle has none and every round takes the
-// ring of quads.
+// ring of quads.  Copied on the handle's stream, which orders them before every
+// kernel that reads them (the side stream's forks included): a copy on the legacy
+// stream is not ordered before kernels of a non-blocking one.
 cudaError_t upload_maps(rrg_batch_ctx* h, const float* d32, int pair) {
   if (!h->maps_ok) return cudaSuccess;
   std::vector<CUtensorMap> m(h->inst.size());
@@ -1099,8 +1101,9 @@ cudaError_t upload_maps(rrg_batch_ctx* h, const float* d32, int pair) {
       return cudaSuccess;
     }
   }
-  return cudaMemcpy(h->maps_dev + static_cast<size_t>(pair) * m.size(), m.data(), m.size() * sizeof(CUtensorMap),
-                    cudaMemcpyHostToDevice);
+  const cudaError_t e = cudaMemcpyAsync(h->maps_dev + static_cast<size_t>(pair) * m.size(), m.data(),
+                                        m.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, h->stream);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(h->stream);  // m is this call's
 }
 
 // Rounds of one update's search: 1 for Alg. 3, n_rounds for the k-section;
