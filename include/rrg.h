@@ -673,9 +673,10 @@ RRG_API int rrg_step_latency(rrg_handle h, double v, int steps, double *cycles_p
 #define RRG_BATCH_MAX_INSTANCES 1024
 #define RRG_BATCH_VARIANTS 10  /* rollout variants: lanes per tile {64, 128,
                                   256} x disturbance prefetch depth {8
-                                  (registers), 16 (the per-warp TMA ring's
-                                  chunk)}, then warp tiles (32 lanes, each warp
-                                  takes its own) x {8, 16}, then warp tiles of two
+                                  (registers), 16 (a ring in shared memory, see
+                                  rrg_batch_set_tma)}, then warp tiles (32 lanes,
+                                  each warp takes its own) x {8, 16}, then warp
+                                  tiles of two
                                   candidates per thread (prefetch 8), then warp
                                   tiles of 16 scenarios at two lanes per
                                   trajectory (prefetch 8; tile_lanes reports
@@ -723,6 +724,15 @@ RRG_API int rrg_batch_autotune(rrg_batch_handle h, const double *d_x, const doub
                        int *variant_out, double *ms_out);
 RRG_API int rrg_batch_set_variant(rrg_batch_handle h, int variant);
 RRG_API int rrg_batch_get_variant(rrg_batch_handle h, int *variant, int *tile_lanes, int *prefetch);
+/* The ring of the variants of prefetch depth 16: RRG_TMA_AUTO (the default), the
+ * per-warp TMA ring in rounds of at least 300 warps of tiles per SM and the
+ * per-lane ring of quads below; RRG_TMA_NEVER, RRG_TMA_ALWAYS, one of them in
+ * every round.  The results are identical.  Without the instances' tensor maps
+ * (rrg_set_tma) rrg_batch_get_tma reports RRG_TMA_NEVER and setting another mode
+ * returns RRG_EINVAL.  Setting waits for the handle's stream and discards the
+ * cached closed-loop graph.  rrg_stats.lane_steps_tma counts the TMA ring's. */
+RRG_API int rrg_batch_set_tma(rrg_batch_handle h, int mode);
+RRG_API int rrg_batch_get_tma(rrg_batch_handle h, int32_t *mode);
 /* Width of RRG_SEARCH_SPEC_BISECT batches: the tree nodes each instance
  * evaluates per round, 1..max_candidates (default max_candidates).  Every
  * instance's result is Alg. 1's for every width (the same tree and walk as

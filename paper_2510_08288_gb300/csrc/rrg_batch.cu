@@ -455,6 +455,9 @@ __device__ __forceinline__ void batch_tile(const BLaunch& B, int s, int i, int k
                                             cand_stop ? dead : nullptr, &steps, &end, eps, &jlast, stages, bars,
                                             &B.stats->wait_timeouts);
     if (active) smin = s_out;
+    const unsigned wsteps = __reduce_add_sync(0xffffffffu, steps);
+    if ((threadIdx.x & 31) == 0 && wsteps)
+      atomicAdd(&B.stats->lane_steps_tma, static_cast<unsigned long long>(wsteps));
   } else if (active) {
     const float* d = (st.cur ? B.d32b : B.d32) + I.off;
     if constexpr (FEED == FEED_QRING)
@@ -972,6 +975,7 @@ struct rrg_batch_ctx {
   float* d32 = nullptr;
   CUtensorMap* maps_dev = nullptr;  // [2][S]
   bool maps_ok = true;         // every instance has its tensor maps
+  int tma_mode = RRG_TMA_AUTO;
   float* d32b = nullptr;       // second scenario pair, allocated by the first closed loop
   size_t d32_elems = 0;
   cudaStream_t side = nullptr; // draws update t + 1 while update t searches
@@ -1131,8 +1135,8 @@ int enqueue_rollout(rrg_batch_ctx* h) {
     if (a && b) BCK(cudaEventRecord(a, h->stream));
   }
   const unsigned long long cand = h->B.c.search == RRG_SEARCH_SPEC_BISECT ? h->B.c.width : h->B.c.M;
-  const int large =
-      h->maps_ok && h->scen_warps * cand >= static_cast<unsigned long long>(kTmaTileWarps) * h->sms ? 1 : 0;
+  const bool many = h->scen_warps * cand >= static_cast<unsigned long long>(kTmaTileWarps) * h->sms;
+  const int large = h->maps_ok && (h->tma_mode == RRG_TMA_ALWAYS || (h->tma_mode == RRG_TMA_AUTO && many)) ? 1 : 0;
   v.kernel[large]<<<h->grid[h->variant][large], block_threads(v.tile), variant_smem(v, large), h->stream>>>(h->B);
   BCK(cudaGetLastError());
   if (timed && a && b) {
@@ -1553,6 +1557,28 @@ int rrg_batch_get_variant(rrg_batch_handle h, int* variant, int* tile_lanes, int
   return RRG_OK;
 }
 
+int rrg_batch_set_tma(rrg_batch_handle h, int mode) {
+  if (!h) return RRG_EINVAL;
+  if (mode < RRG_TMA_NEVER || mode > RRG_TMA_ALWAYS)
+    return bset_err(h, RRG_EINVAL, "TMA mode must be RRG_TMA_NEVER, RRG_TMA_AUTO or RRG_TMA_ALWAYS");
+  if (mode != RRG_TMA_NEVER && !h->maps_ok)
+    return bset_err(h, RRG_EINVAL, "no TMA ring for this handle (an instance's tensor map was refused)");
+  BDeviceGuard g(h->device);
+  BCK(cudaStreamSynchronize(h->stream));
+  h->tma_mode = mode;
+  if (h->cl_exec) {  // the cached closed-loop graph holds the old kernels
+    cudaGraphExecDestroy(h->cl_exec);
+    h->cl_exec = nullptr;
+  }
+  return RRG_OK;
+}
+
+int rrg_batch_get_tma(rrg_batch_handle h, int32_t* mode) {
+  if (!h || !mode) return RRG_EINVAL;
+  *mode = h->maps_ok ? h->tma_mode : RRG_TMA_NEVER;
+  return RRG_OK;
+}
+
 int rrg_batch_set_width(rrg_batch_handle h, int width) {
   if (!h) return RRG_EINVAL;
   if (h->cfg.search != RRG_SEARCH_SPEC_BISECT)
@@ -1701,6 +1727,7 @@ int rrg_batch_get_stats(rrg_batch_handle h, rrg_stats* out) {
   out->repairs = 0;
   out->graph_conditional = 0;
   out->wait_timeouts = d.wait_timeouts;
+  out->lane_steps_tma = d.lane_steps_tma;
   return RRG_OK;
 }
 

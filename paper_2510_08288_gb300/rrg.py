@@ -136,6 +136,8 @@ def _load():
                                                     _p, P(ctypes.c_int)]),
         "rrg_batch_set_variant": (ctypes.c_int, [_p, ctypes.c_int]),
         "rrg_batch_get_variant": (ctypes.c_int, [_p, P(ctypes.c_int), P(ctypes.c_int), P(ctypes.c_int)]),
+        "rrg_batch_set_tma": (ctypes.c_int, [_p, ctypes.c_int]),
+        "rrg_batch_get_tma": (ctypes.c_int, [_p, P(ctypes.c_int32)]),
         "rrg_batch_set_profiling": (ctypes.c_int, [_p, ctypes.c_int]),
         "rrg_batch_get_stats": (ctypes.c_int, [_p, P(RrgStats)]),
         "rrg_batch_reset_stats": (ctypes.c_int, [_p]),
@@ -663,6 +665,16 @@ def rrg_batch_get_variant(h):
     return v.value, t.value, f.value
 
 
+def rrg_batch_set_tma(h, mode):
+    _bcheck(lib.rrg_batch_set_tma(h, int(mode)), h)
+
+
+def rrg_batch_get_tma(h) -> int:
+    m = ctypes.c_int32(0)
+    _bcheck(lib.rrg_batch_get_tma(h, ctypes.byref(m)), h)
+    return m.value
+
+
 def rrg_batch_set_profiling(h, on):
     _bcheck(lib.rrg_batch_set_profiling(h, int(bool(on))), h)
 
@@ -769,6 +781,12 @@ class BatchGovernor:
 
     def get_variant(self):
         return rrg_batch_get_variant(self.h)
+
+    def set_tma(self, mode):
+        rrg_batch_set_tma(self.h, mode)
+
+    def get_tma(self):
+        return rrg_batch_get_tma(self.h)
 
     def stats(self):
         return rrg_batch_get_stats(self.h)
