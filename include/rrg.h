@@ -733,6 +733,10 @@ RRG_API int rrg_batch_get_variant(rrg_batch_handle h, int *variant, int *tile_la
  * cached closed-loop graph.  rrg_stats.lane_steps_tma counts the TMA ring's. */
 RRG_API int rrg_batch_set_tma(rrg_batch_handle h, int mode);
 RRG_API int rrg_batch_get_tma(rrg_batch_handle h, int32_t *mode);
+/* As rrg_set_injection.  RRG_INJECT_TMA_NO_COPY: each warp of a round on the TMA
+ * ring times out once; the tile it is on and the tiles it takes afterwards count
+ * as violated. */
+RRG_API int rrg_batch_set_injection(rrg_batch_handle h, int flags);
 /* Width of RRG_SEARCH_SPEC_BISECT batches: the tree nodes each instance
  * evaluates per round, 1..max_candidates (default max_candidates).  Every
  * instance's result is Alg. 1's for every width (the same tree and walk as

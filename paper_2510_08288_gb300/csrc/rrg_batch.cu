@@ -104,6 +104,7 @@ struct BLaunch {
   unsigned long long* t_dev;  // closed-loop update counter
   int32_t* cand_passed;   // trajectories that passed (top_down)
   int top_down;           // grid and k-section with RRG_EXIT_CANDIDATE: as Launch::top_down
+  int inject;             // RRG_INJECT_* test switches (0 in normal use)
 };
 
 // ---------------------------------------------------------------------------
@@ -419,8 +420,13 @@ extern __shared__ __align__(128) unsigned char batch_dyn_smem[];
 // One tile: lanes k of candidate slot (s, i), binary32 rollouts classified
 // for the binary64 recheck, reduced into the candidate's flags.  Called by
 // every thread of the CTA; returns are warp- or CTA-uniform.
+// ring_lost (FEED_TMA; the same for a warp's lanes): the warp gave up on a copy
+// that may still land in its stages (run_lane_tma).  The tile it was on and those
+// it takes afterwards count as violated: nothing is admissible on data that did
+// not arrive.  (Running the later ones without the ring would keep their results,
+// but a second form of the loop beside this one cost 3 % of the rollouts.)
 template <int FEED, int THREADS>
-__device__ __forceinline__ void batch_tile(const BLaunch& B, int s, int i, int k) {
+__device__ __forceinline__ void batch_tile(const BLaunch& B, int s, int i, int k, bool& ring_lost) {
   const BInst I = B.inst[s];
   const size_t slot = static_cast<size_t>(s) * B.c.M + i;
   if (!B.cand_ss[slot]) return;
@@ -450,11 +456,12 @@ __device__ __forceinline__ void batch_tile(const BLaunch& B, int s, int i, int k
     uint64_t* bars = reinterpret_cast<uint64_t*>(batch_dyn_smem + static_cast<size_t>(nw) * 2 * kTmaStageBytes) + 2 * wid;
     const CUtensorMap* tm = B.maps + (st.cur ? B.c.S : 0) + s;
     if ((threadIdx.x & 31) == 0) fence_tensormap(tm);
-    const float s_out = run_lane_tma<false>(U, C, tm, nullptr, k, I.N, I.H, active, 0, I.H, q_ca, w, q_sm, w_abs,
+    if (B.inject & RRG_INJECT_TMA_NO_COPY) tm = nullptr;
+    const float s_out = run_lane_tma<false>(U, C, tm, nullptr, k, I.N, I.H, active && !ring_lost, 0, I.H, q_ca, w, q_sm, w_abs,
                                             inf_v<float>(), thr, cand_stop ? dead : nullptr,
                                             cand_stop ? dead : nullptr, &steps, &end, eps, &jlast, stages, bars,
-                                            &B.stats->wait_timeouts);
-    if (active) smin = s_out;
+                                            &B.stats->wait_timeouts, &ring_lost);
+    if (active) smin = ring_lost ? -inf_v<float>() : s_out;
     const unsigned wsteps = __reduce_add_sync(0xffffffffu, steps);
     if ((threadIdx.x & 31) == 0 && wsteps)
       atomicAdd(&B.stats->lane_steps_tma, static_cast<unsigned long long>(wsteps));
@@ -502,6 +509,7 @@ __global__ void __launch_bounds__(TILE, kBatchThreadsPerSm / TILE) batch_rollout
   __shared__ int sh[3];
   if (blockIdx.x >= B.queue[2]) return;
   const uint32_t total = B.queue[1];
+  bool ring_lost = false;
   for (;;) {
     if (threadIdx.x == 0) {
       const uint32_t t = atomicAdd(B.queue, 1u);
@@ -515,7 +523,7 @@ __global__ void __launch_bounds__(TILE, kBatchThreadsPerSm / TILE) batch_rollout
     const int s = sh[0], i = sh[1], b = sh[2];
     __syncthreads();
     if (s < 0) return;
-    batch_tile<FEED, TILE>(B, s, i, b * TILE + static_cast<int>(threadIdx.x));
+    batch_tile<FEED, TILE>(B, s, i, b * TILE + static_cast<int>(threadIdx.x), ring_lost);
   }
 }
 
@@ -526,6 +534,7 @@ template <int FEED>
 __global__ void __launch_bounds__(128, kBatchThreadsPerSm / 128) batch_rollout_warp_kernel(const BLaunch B) {
   if (blockIdx.x >= B.queue[2]) return;
   const uint32_t total = B.queue[1];
+  bool ring_lost = false;
   const int lane = static_cast<int>(threadIdx.x & 31);
   for (;;) {
     uint32_t t = 0;
@@ -537,7 +546,7 @@ __global__ void __launch_bounds__(128, kBatchThreadsPerSm / 128) batch_rollout_w
     s = __shfl_sync(0xffffffffu, s, 0);
     i = __shfl_sync(0xffffffffu, i, 0);
     b = __shfl_sync(0xffffffffu, b, 0);
-    batch_tile<FEED, 128>(B, s, i, b * 32 + lane);
+    batch_tile<FEED, 128>(B, s, i, b * 32 + lane, ring_lost);
   }
 }
 
@@ -1567,6 +1576,19 @@ int rrg_batch_set_tma(rrg_batch_handle h, int mode) {
   BCK(cudaStreamSynchronize(h->stream));
   h->tma_mode = mode;
   if (h->cl_exec) {  // the cached closed-loop graph holds the old kernels
+    cudaGraphExecDestroy(h->cl_exec);
+    h->cl_exec = nullptr;
+  }
+  return RRG_OK;
+}
+
+int rrg_batch_set_injection(rrg_batch_handle h, int flags) {
+  if (!h) return RRG_EINVAL;
+  if (flags & ~RRG_INJECT_TMA_NO_COPY) return bset_err(h, RRG_EINVAL, "unknown injection flags 0x%x", flags);
+  BDeviceGuard g(h->device);
+  BCK(cudaStreamSynchronize(h->stream));
+  h->B.inject = flags;
+  if (h->cl_exec) {
     cudaGraphExecDestroy(h->cl_exec);
     h->cl_exec = nullptr;
   }

@@ -1007,7 +1007,9 @@ __device__ __forceinline__ void tma_chunk(const void* tmap, uint32_t dst, uint32
       : "memory");
 }
 
-// PACK: rk4_step_packed (the same bits).
+// PACK: rk4_step_packed (the same bits).  Returns *lost = true (if given) when a
+// copy may still be in flight into the warp's stages although the bounded waits
+// ran out: the warp must not use its stages and barriers again.
 template <bool PACK>
 __device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC<float>& C, const void* tmap,
                                               const float* __restrict__ d, int k, int N, int H,
@@ -1016,7 +1018,7 @@ __device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC
                                               const volatile int32_t* dead, volatile int32_t* mark,
                                               unsigned* steps, int* end, float band, int* jlast,
                                               float* stages, uint64_t* bars,
-                                              unsigned long long* timeouts) {
+                                              unsigned long long* timeouts, bool* lost = nullptr) {
   constexpr int T = kTmaChunk;
   const int lane = threadIdx.x & 31;
   float smin = smin_in;
@@ -1059,6 +1061,7 @@ __device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC
     }
     __syncwarp();
     if (lane == 0) {
+      fence_proxy_async_smem();  // the warp may have read these stages for a tile before
       tma_chunk(tmap, st0, bar0, k0, jb);
       if (nchunks > 1) tma_chunk(tmap, st0 + kTmaStageBytes, bar0 + 8u, k0, jb + T);
     }
@@ -1137,6 +1140,7 @@ __device__ __forceinline__ float run_lane_tma(const StepU<float>& K, const StepC
       drained = mbar_wait_bounded(bar0 + 8u * static_cast<uint32_t>(c & 1),
                                   static_cast<uint32_t>((c >> 1) & 1)) && drained;
     drained = __all_sync(0xffffffffu, drained);
+    if (lost != nullptr) *lost = !drained;
     if (timed_out || !drained) {
       if (lane == 0) atomicAdd(timeouts, 1ull);
       if (run) {

@@ -137,6 +137,7 @@ def _load():
         "rrg_batch_set_variant": (ctypes.c_int, [_p, ctypes.c_int]),
         "rrg_batch_get_variant": (ctypes.c_int, [_p, P(ctypes.c_int), P(ctypes.c_int), P(ctypes.c_int)]),
         "rrg_batch_set_tma": (ctypes.c_int, [_p, ctypes.c_int]),
+        "rrg_batch_set_injection": (ctypes.c_int, [_p, ctypes.c_int]),
         "rrg_batch_get_tma": (ctypes.c_int, [_p, P(ctypes.c_int32)]),
         "rrg_batch_set_profiling": (ctypes.c_int, [_p, ctypes.c_int]),
         "rrg_batch_get_stats": (ctypes.c_int, [_p, P(RrgStats)]),
@@ -669,6 +670,10 @@ def rrg_batch_set_tma(h, mode):
     _bcheck(lib.rrg_batch_set_tma(h, int(mode)), h)
 
 
+def rrg_batch_set_injection(h, flags):
+    _bcheck(lib.rrg_batch_set_injection(h, int(flags)), h)
+
+
 def rrg_batch_get_tma(h) -> int:
     m = ctypes.c_int32(0)
     _bcheck(lib.rrg_batch_get_tma(h, ctypes.byref(m)), h)
@@ -787,6 +792,9 @@ class BatchGovernor:
 
     def get_tma(self):
         return rrg_batch_get_tma(self.h)
+
+    def set_injection(self, flags):
+        rrg_batch_set_injection(self.h, flags)
 
     def stats(self):
         return rrg_batch_get_stats(self.h)

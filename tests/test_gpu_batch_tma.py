@@ -85,3 +85,33 @@ def test_rounds_of_many_tiles_take_the_tma_ring(R, orc, params):
     for a, b in out:
         for u, w in zip(a, b):
             np.testing.assert_array_equal(u, w)
+
+
+@pytest.mark.parametrize("variant", RING)
+def test_a_warp_that_gave_up_leaves_the_ring(R, orc, params, variant):
+    """Without copies (RRG_INJECT_TMA_NO_COPY) each warp's wait runs out once: its
+    tile and the many that it takes afterwards count as violated, none of them on
+    the ring again.  Nothing is admissible, and the handle recovers."""
+    import torch
+    warps = 64 * torch.cuda.get_device_properties(0).multi_processor_count
+    cfg = R.rrg_config_default(max_candidates=16, precision=R.FP32_RECHECK, search=R.SEARCH_GRID,
+                               early_exit=R.EXIT_LANE)
+    x, r, vp = _problems(orc, params, 1)
+    with R.BatchGovernor(params, cfg, [64000], [48]) as g:
+        g.set_variant(variant)
+        g.set_tma(R.TMA_ALWAYS)
+        want = g.step(x, r, vp, 21, 5)
+        g.set_injection(R.INJECT_TMA_NO_COPY)
+        g.reset_stats()
+        _, kappa, flags = g.step(x, r, vp, 21, 5)
+        st = g.stats()
+        assert 0 < st["wait_timeouts"] <= warps < 16 * 2000  # once a warp; 2,000 warps of tiles a candidate
+        assert kappa[0] == 0.0 and flags[0] & 1 and want[1][0] > 0.0
+        assert st["lane_steps"] == 0
+        g.set_injection(0)
+        g.reset_stats()
+        for a, b in zip(want, g.step(x, r, vp, 21, 5)):
+            np.testing.assert_array_equal(a, b)
+        assert g.stats()["wait_timeouts"] == 0
+        with pytest.raises(R.RrgError):
+            g.set_injection(2)
