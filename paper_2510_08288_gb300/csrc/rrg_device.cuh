@@ -214,7 +214,7 @@ struct StepU {  // one model's coefficients (per scenario under parametric uncer
   T x2a, x2w, x2s, w2w, w2s, w2n1;
   T x3a, x3w, x3s, x3n1, w3a, w3w, w3s, w3n1, w3n2;
   T x4a, x4w, x4s, x4n1, x4n2, w4a, w4w, w4s, w4n1, w4n2, w4n3;
-  // the step's result (binary32: less the state): cathode pressure, manifold pressure, speed
+  // the step's result: cathode pressure, manifold pressure (fss in binary32: less 1), speed
   T faa, faw, fas, fan1, fan2;
   T fsa, fsw, fss, fsn1, fsn2, fsn3;
   T fwa, fww, fws, fwn1, fwn2, fwn3, fwn4;
@@ -282,16 +282,19 @@ __device__ __forceinline__ double torque(const StepU<double>& U, const PowTable*
   return pow_m1_table(S, x, U.e) * t;
 }
 
-// The step's result from a row's sum r: binary64 rows hold the state's own
-// coefficients (R), binary32 rows the change (R - I), to which the state is added
-// last.  Summed onto the state, each of a row's five to seven terms rounded at the
-// state's magnitude, and R's diagonal, close to 1, lost the digits of the change:
-// the error against binary64 was 20-30 % above that of right-hand sides evaluated
-// stage by stage.  Three additions a step more give, over updates of 1,024
-// scenarios x 2,000 steps (median trajectory, largest of 196,608): stage by stage
-// 2.0e-7, 3.2e-6; summed onto the state 2.5e-7, 4.1e-6; here 1.7e-7, 1.7e-6.
-__device__ __forceinline__ float add_state(float z, float r) { return __fadd_rn(z, r); }
-__device__ __forceinline__ double add_state(double, double r) { return r; }
+// The manifold pressure's result from its row's sum r: a binary64 row holds the
+// pressure's own coefficient, a binary32 row that less 1, so its sum is the change
+// over the step, and the pressure is added last.  Summed onto the pressure, each of
+// the row's seven terms rounded at the pressure's magnitude, and the coefficient,
+// close to 1, lost the digits of the change: the error against binary64 was 20-30 %
+// above that of right-hand sides evaluated stage by stage.  One addition a step more
+// gives, over updates of 1,024 scenarios x 2,000 steps (median trajectory, largest of
+// 196,608): stage by stage 2.0e-7, 3.2e-6; summed onto the pressure 2.5e-7, 4.1e-6;
+// here 1.9e-7, 2.5e-6; the cathode pressure's and the speed's rows so too 1.7e-7,
+// 1.7e-6, for two more additions (16,384 x 16 x 1,000 steps: 730 us with none of
+// them, 737 with this one, 746 with three).
+__device__ __forceinline__ float add_sm(float s, float r) { return __fadd_rn(s, r); }
+__device__ __forceinline__ double add_sm(double, double r) { return r; }
 
 // One RK4 step followed by the disturbance (e_ca, e_w, e_sm) of Eq. 4, in
 // place, on the deviation z = (q_ca, w, q_sm).  w_abs is the absolute speed
@@ -315,15 +318,11 @@ __device__ __forceinline__ void rk4_step_with(const StepU<T>& U, const StepC<T>&
   const T w4 = fma_rn(U.w4n3, n3, fma_rn(U.w4n2, n2, fma_rn(U.w4n1, n1,
                fma_rn(U.w4w, z, fma_rn(U.w4s, s, fma_rn(U.w4a, a, C.w4))))));
   const T n4 = tq(x4, w4);
-  const T r_a = fma_rn(U.fan2, n2, fma_rn(U.fan1, n1, fma_rn(U.faw, z, fma_rn(U.fas, s, fma_rn(U.faa, a, e_ca + C.fa)))));
-  const T r_s = fma_rn(U.fsn3, n3, fma_rn(U.fsn2, n2, fma_rn(U.fsn1, n1,
-                fma_rn(U.fsw, z, fma_rn(U.fss, s, fma_rn(U.fsa, a, e_sm + C.fs))))));
-  const T r_z = fma_rn(U.fwn3, n3, fma_rn(U.fwn2, n2, fma_rn(U.fwn1, n1,
-                fma_rn(U.fww, z, fma_rn(U.fws, s, fma_rn(U.fwa, a, e_w + C.fw))))));
-  // binary32: the sums above are the change over the step (add_state)
-  q_ca = add_state(a, r_a);
-  q_sm = add_state(s, r_s);
-  const T p = add_state(z, r_z);
+  q_ca = fma_rn(U.fan2, n2, fma_rn(U.fan1, n1, fma_rn(U.faw, z, fma_rn(U.fas, s, fma_rn(U.faa, a, e_ca + C.fa)))));
+  q_sm = add_sm(s, fma_rn(U.fsn3, n3, fma_rn(U.fsn2, n2, fma_rn(U.fsn1, n1,
+         fma_rn(U.fsw, z, fma_rn(U.fss, s, fma_rn(U.fsa, a, e_sm + C.fs)))))));
+  const T p = fma_rn(U.fwn3, n3, fma_rn(U.fwn2, n2, fma_rn(U.fwn1, n1,
+              fma_rn(U.fww, z, fma_rn(U.fws, s, fma_rn(U.fwa, a, e_w + C.fw))))));
   w = fma_rn(U.fwn4, n4, p);
   w_abs = fma_rn(U.fwn4, n4, p + C.r_w);
 }
@@ -387,11 +386,9 @@ __device__ __forceinline__ void rk4_step_packed(const StepU<float>& U, const Ste
   const float n3 = tq(x3, w3);
   upk(p4, x4, w4);
   w4 = fma_rn(U.w4n3, n3, w4);
-  float r_a, r_s;
-  upk(pf, r_a, r_s);
-  q_ca = add_state(a, r_a);
-  q_sm = add_state(s, fma_rn(U.fsn3, n3, r_s));
-  p = add_state(z, fma_rn(U.fwn3, n3, p));
+  upk(pf, q_ca, q_sm);
+  q_sm = add_sm(s, fma_rn(U.fsn3, n3, q_sm));
+  p = fma_rn(U.fwn3, n3, p);
   const float n4 = tq(x4, w4);
   w = fma_rn(U.fwn4, n4, p);
 #ifdef RRG_V_WABS1

@@ -424,7 +424,7 @@ __host__ __device__ inline void fold_model(const Fc3K<double>& K, const double* 
 }
 
 // The coefficients rounded once to binary32 (StepU and StepPhi hold nothing
-// but T values), the result's rows less the state (add_state).
+// but T values), fss less 1 (add_sm).
 __host__ __device__ inline void round_model(const StepModel<double>& m, StepModel<float>* out) {
   static_assert(sizeof(StepU<double>) == 2 * sizeof(StepU<float>) &&
                 sizeof(StepPhi<double>) == 2 * sizeof(StepPhi<float>), "arrays of T");
@@ -436,9 +436,7 @@ __host__ __device__ inline void round_model(const StepModel<double>& m, StepMode
 #pragma unroll
 #endif
   for (size_t i = 0; i < sizeof(StepU<float>) / sizeof(float); ++i) uf[i] = static_cast<float>(u[i]);
-  out->U.faa = static_cast<float>(add_rn(m.U.faa, -1.0));
   out->U.fss = static_cast<float>(add_rn(m.U.fss, -1.0));
-  out->U.fww = static_cast<float>(add_rn(m.U.fww, -1.0));
   const double* p = &m.F.h;
   float* pf = &out->F.h;
 #ifdef __CUDA_ARCH__
