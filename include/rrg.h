@@ -443,9 +443,12 @@ RRG_API int rrg_get_tma(rrg_handle h, int32_t *mode);
  * warp's first chunk wait runs out (after at most 0.1 s): the warp counts one
  * timeout in rrg_stats.wait_timeouts, its running lanes report a violation
  * (no candidate is admissible on data that did not arrive), the kernel
- * returns and the handle stays usable.  Waits for the stream and discards the
- * cached closed-loop graph; RRG_EINVAL for unknown flags. */
+ * returns and the handle stays usable.  RRG_INJECT_LAUNCH_ERROR: the rollouts (of
+ * a gradient: the forward pass) are not launched, and the call returns RRG_ECUDA
+ * as if that launch had failed.  Waits for the stream and discards the cached
+ * closed-loop graph; RRG_EINVAL for unknown flags. */
 #define RRG_INJECT_TMA_NO_COPY 1
+#define RRG_INJECT_LAUNCH_ERROR 4
 RRG_API int rrg_set_injection(rrg_handle h, int flags);
 
 /* Times 1 + repeats updates of the handle's search (rrg_autotune's

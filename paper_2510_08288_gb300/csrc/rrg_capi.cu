@@ -354,6 +354,7 @@ cudaEvent_t take_event(rrg_ctx* h) {
 // continuation segments), whose rows cannot share a thread.
 int enqueue_round_work(rrg_ctx* h, const Launch& L, int width, int early_exit, bool recheck = true,
                        bool allow_pair = true) {
+  if (h->inject & RRG_INJECT_LAUNCH_ERROR) return set_err(h, RRG_ECUDA, "injected launch error");
   const bool timed = h->profiling && !h->capturing;
   cudaEvent_t a = nullptr, b = nullptr;
   if (timed) { a = take_event(h); b = take_event(h); }
@@ -574,6 +575,22 @@ cudaError_t grow(T** p, size_t* cap, size_t n) {
 
 namespace {
 
+// A synchronous call's use of the handle's pinned staging, which its kernels and
+// copies read and write: an error return waits for what was queued before the next
+// call may write there (done() after the call's own wait).
+struct StagingUse {
+  rrg_ctx* h;
+  explicit StagingUse(rrg_ctx* ctx) : h(ctx) {}
+  StagingUse(const StagingUse&) = delete;
+  ~StagingUse() {
+    if (h) cudaStreamSynchronize(h->stream);
+  }
+  int done() {
+    h = nullptr;
+    return RRG_OK;
+  }
+};
+
 // Scratch of the adjoint for m kappas (grown on demand; a buffer queued work
 // may still use is freed only after the stream drained).
 int adj_buffers(rrg_ctx* h, size_t M, int checkpoint) {
@@ -626,6 +643,7 @@ int adj_enqueue_forward_kernels(rrg_ctx* h, int m, int checkpoint, int precision
   CK(launch_eval_prepare(L, h->io_h + IO_X, 0.0, 0.0, h->io_h + IO_LEN, m, h->io_h + IO_V, h->io_h + IO_R));
   CK(launch_prepare(L, m));
   h->launches += 2;
+  if (h->inject & RRG_INJECT_LAUNCH_ERROR) return set_err(h, RRG_ECUDA, "injected launch error");
   const bool use32 = precision == RRG_FP32 && h->cfg.precision != RRG_FP64 && !h->cfg.scenarios_in_register;
   if (!use32) {
     CK(launch_materialize64(L));
@@ -651,9 +669,10 @@ int adj_enqueue_forward(rrg_ctx* h, const double* x_t, double v_prev, double r_t
                         int m, int checkpoint, int precision, bool argmin = true) {
   int rc = adj_buffers(h, static_cast<size_t>(m), checkpoint);
   if (rc != RRG_OK) return rc;
+  StagingUse staging(h);
   adj_upload(h, x_t, v_prev, r_t, kappas, m);
   rc = adj_enqueue_forward_kernels(h, m, checkpoint, precision, argmin);
-  return rc;
+  return rc == RRG_OK ? staging.done() : rc;
 }
 
 // with_argmin: the reverse sweep finds each slot's argmin itself (after a
@@ -976,6 +995,7 @@ int rrg_eval_candidates(rrg_handle h, const double* x_t, double v_prev, double r
   }
   // the kernels read the inputs and write the outcomes in the pinned staging
   // itself: no copies beside them (3,001 scenarios x 32 candidates 400 -> 392 us)
+  StagingUse staging(h);
   CK(launch_eval_prepare(L, h->io_h + IO_X, v_prev, r_t, kap_h, m));
   CK(launch_prepare(L, m));
   h->launches += 2;
@@ -989,7 +1009,7 @@ int rrg_eval_candidates(rrg_handle h, const double* x_t, double v_prev, double r
   CK(cudaStreamSynchronize(h->stream));
   std::memcpy(admissible, adm_h, m);
   if (min_slack) std::memcpy(min_slack, kap_h + M, m * sizeof(double));
-  return RRG_OK;
+  return staging.done();
 }
 
 int rrg_slack_error(rrg_handle h, const double* x_t, double v_prev, double r_t,
@@ -1027,6 +1047,7 @@ int rrg_slack_error(rrg_handle h, const double* x_t, double v_prev, double r_t,
   double* kap_h = h->io_h + IO_LEN;
   std::memcpy(h->io_h + IO_X, x_t, 3 * sizeof(double));
   std::memcpy(kap_h, kappas, m * sizeof(double));
+  StagingUse staging(h);
   CK(cudaMemcpyAsync(h->io_dev, h->io_h, IO_LEN * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   CK(cudaMemcpyAsync(h->kap_dev, kap_h, m * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   const Launch& L = h->L;
@@ -1041,7 +1062,7 @@ int rrg_slack_error(rrg_handle h, const double* x_t, double v_prev, double r_t,
   if (unsafe) CK(cudaMemcpyAsync(unsafe, d_bad, lanes * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
   if (ratio) CK(cudaMemcpyAsync(ratio, d_ratio, lanes * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  return RRG_OK;
+  return staging.done();
 }
 
 // The search of rrg_step, captured once on the handle's pinned io buffers:
@@ -1161,6 +1182,7 @@ int rrg_step(rrg_handle h, const double* x_t, double r_t, double v_prev, double*
   if (!x_ok(x_t) || !is_fin(v_prev) || !is_fin(r_t) || !(v_prev > 0.0) || !(r_t > 0.0))
     return set_err(h, RRG_EINVAL, "x_t, v_prev, r_t must be finite and v_prev, r_t > 0");
   DeviceGuard g(h->device);
+  StagingUse staging(h);
   std::memcpy(h->io_h + IO_X, x_t, 3 * sizeof(double));
   h->io_h[IO_R] = r_t;
   h->io_h[IO_V] = v_prev;
@@ -1191,7 +1213,7 @@ int rrg_step(rrg_handle h, const double* x_t, double r_t, double v_prev, double*
   if (v_t) *v_t = h->io_h[IO_OUT];
   if (kappa) *kappa = h->io_h[IO_OUT + 1];
   if (flags) *flags = h->flag_h[0];
-  return RRG_OK;
+  return staging.done();
 }
 
 int rrg_step_dev(rrg_handle h, const double* d_x_t, const double* d_r_t, const double* d_v_prev,
@@ -1465,6 +1487,7 @@ int rrg_slack_gradients(rrg_handle h, const double* x_t, double v_prev, double r
   DeviceGuard gd(h->device);
   int rc = adj_buffers(h, static_cast<size_t>(m), checkpoint);
   if (rc != RRG_OK) return rc;
+  StagingUse staging(h);
   adj_upload(h, x_t, v_prev, r_t, kappas, m);
   // the kernels as one graph replay (as rrg_step), except while the library
   // times rollout launches; the graph is keyed by the call's shape and the
@@ -1507,7 +1530,7 @@ int rrg_slack_gradients(rrg_handle h, const double* x_t, double v_prev, double r
     if (grad) std::memcpy(grad + static_cast<size_t>(i) * (4 + RRG_NPARAM), o + 3, (4 + RRG_NPARAM) * sizeof(double));
     if (ss_ok) ss_ok[i] = ss[i] ? 1 : 0;
   }
-  return RRG_OK;
+  return staging.done();
 }
 
 int rrg_slack_gradient(rrg_handle h, const double* x_t, double v_prev, double r_t, double kappa,
@@ -1808,7 +1831,8 @@ int rrg_set_tma(rrg_handle h, int mode) {
 
 int rrg_set_injection(rrg_handle h, int flags) {
   if (!h) return RRG_EINVAL;
-  if (flags & ~RRG_INJECT_TMA_NO_COPY) return set_err(h, RRG_EINVAL, "unknown injection flags 0x%x", flags);
+  if (flags & ~(RRG_INJECT_TMA_NO_COPY | RRG_INJECT_LAUNCH_ERROR))
+    return set_err(h, RRG_EINVAL, "unknown injection flags 0x%x", flags);
   DeviceGuard g(h->device);
   CK(cudaStreamSynchronize(h->stream));
   h->inject = flags;

@@ -25,6 +25,7 @@ EXIT_NONE, EXIT_LANE, EXIT_CANDIDATE = range(3)
 PAIR_NEVER, PAIR_FILLED, PAIR_ALWAYS = range(3)
 TMA_NEVER, TMA_AUTO, TMA_ALWAYS = range(3)
 INJECT_TMA_NO_COPY = 1
+INJECT_LAUNCH_ERROR = 4
 NPARAM = 27
 MAX_CANDIDATES = 1024
 FLAG_NONE_ADMISSIBLE = 1
