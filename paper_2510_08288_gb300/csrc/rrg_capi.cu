@@ -360,12 +360,13 @@ int enqueue_round_work(rrg_ctx* h, const Launch& L, int width, int early_exit, b
   if (timed) { a = take_event(h); b = take_event(h); }
   if (a && b) CK(cudaEventRecord(a, h->stream));
   const bool fp64 = h->cfg.precision == RRG_FP64;
-  CK(launch_rollout(L, width, fp64, early_exit, h->cfg.precision == RRG_FP32_RECHECK, allow_pair));
+  int kernels = 1;
+  CK(launch_rollout(L, width, fp64, early_exit, h->cfg.precision == RRG_FP32_RECHECK, allow_pair, &kernels));
   if (a && b) {
     CK(cudaEventRecord(b, h->stream));
     h->ev_roll.emplace_back(a, b);
   }
-  h->launches++;
+  h->launches += kernels;
   h->rollout_launches++;
   if (recheck && h->cfg.precision == RRG_FP32_RECHECK) {
     cudaEvent_t c = nullptr, d = nullptr;

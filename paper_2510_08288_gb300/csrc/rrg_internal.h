@@ -94,6 +94,11 @@ struct SearchState {
   int32_t slot_of_node[kMaxTreeNodes];   // bisection tree: heap node -> slot
   int32_t slot_of_node1[kMaxTreeNodes];  // tree of the pipelined second round
   int32_t passed[RRG_MAX_CANDIDATES];  // trajectories that passed, per slot (Launch::top_down)
+  // A round whose launch is held to one candidate's warps (Launch::held): which
+  // launch runs slot i (1, 2; 0: not settled yet), and whether a candidate ran long
+  // before it violated.
+  int32_t row_launch[RRG_MAX_CANDIDATES];
+  int32_t late;
 };
 
 // Device counters of a handle.
@@ -232,6 +237,9 @@ struct Launch {
   // passed stops those below it.  2: the kernels' shared-memory limits are
   // set (top_down_pad).
   int top_down;
+  // Top-down launches in two parts (launch_rollout): 1, the part held to one
+  // candidate's warps, 2, the part that runs what it left; 0: one launch.
+  int held;
 };
 
 // Folds the FC3 parameter vector into the constants the kernels use
@@ -537,8 +545,9 @@ cudaError_t launch_eval_finish(const Launch& L, int m, uint8_t* d_adm, double* d
 // driver refuses, and for more than kTmaMaxScenarios: a box starts at element
 // four times its scenario, a signed 32-bit coordinate, which scenario 2^29 would
 // overflow (the copy then raises an illegal instruction).  Half of that keeps
-// every sum of a coordinate and a box away from the limit.  tma_ring_prepare() sets the TMA kernels' shared-memory limit
-// on the current device (once per device); false if the runtime refuses.
+// every sum of a coordinate and a box away from the limit.
+// tma_ring_prepare() sets the TMA kernels' shared-memory limit on the current
+// device (once per device); false if the runtime refuses.
 constexpr int kTmaMaxScenarios = 1 << 28;
 bool encode_scenario_map(CUtensorMap* m, const float* d32, int N, int H);
 bool tma_ring_prepare();
@@ -550,8 +559,9 @@ int tma_pair_blocks_per_sm(bool pu);
 int pair_blocks_per_sm(bool pu);
 // allow_pair: the round's rows are all full-horizon segments (no pipelined
 // probe), so two candidates may share a thread (Launch::pair).
+// kernels (may be null): receives how many kernels that took.
 cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int early_exit,
-                           bool recheck_classify, bool allow_pair = false);
+                           bool recheck_classify, bool allow_pair = false, int* kernels = nullptr);
 cudaError_t launch_recheck(const Launch& L, int early_exit);
 cudaError_t launch_equilibrium(const Launch& L, double v, double* d_out4, int32_t* d_status);
 cudaError_t launch_step_latency(const Launch& L, double v, int steps, double* d_out2, int32_t* d_status);

@@ -443,6 +443,8 @@ __device__ __forceinline__ void reduce_lane(const Launch& L, int i, int k, int N
   }
 }
 
+constexpr unsigned kLateShare = 32;  // a violation after 1/32 of the horizon is late (Launch::held)
+
 template <typename T, bool PU, int SRC>
 __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restrict__ d_pair0,
                                              const T* __restrict__ d_pair1,
@@ -497,6 +499,21 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
       if (!SH) return;
       idle = true;
       active = false;
+    }
+  }
+  if constexpr (SRC == SRC_QRING || SRC == SRC_TMA) {
+    // a round in two launches: the row's first warp settles which one runs it
+    if (L.held != 0) {
+      int part = 0;
+      if ((threadIdx.x & 31) == 0) {
+        part = *const_cast<volatile int32_t*>(L.st->row_launch + i);
+        if (part == 0 && L.held == 1) {
+          const int now = *const_cast<volatile int32_t*>(&L.st->late) ? 2 : 1;
+          part = atomicCAS(L.st->row_launch + i, 0, now);
+          if (part == 0) part = now;
+        }
+      }
+      if (__shfl_sync(0xffffffffu, part, 0) != L.held) return;
     }
   }
   RhsC<T> R = cand[i];
@@ -594,6 +611,9 @@ __device__ __forceinline__ void rollout_body(const Launch& L, const T* __restric
   }
   if (active && final_lane) {
     if (cand_stop && smin < thr) *dead = 1;
+    if constexpr (SRC == SRC_QRING || SRC == SRC_TMA)
+      if (L.held == 1 && end == LANE_VIOLATED && steps > static_cast<unsigned>(L.H) / kLateShare)
+        *const_cast<volatile int32_t*>(&L.st->late) = 1;
     if (mode == SEG_PROBE) {
       LaneState<T> o;
       o.q[0] = q_ca;
@@ -835,8 +855,8 @@ rollout_tma_pair_kernel(const Launch L, const RhsC<float>* __restrict__ cand,
 // candidates / top-down at full residency / held to one candidate: 4,096
 // scenarios 2.37 / 2.04 / 1.46 ms, 16,384 6.06 / 3.41 / 1.86, 32,768 - / 4.23 /
 // 2.46, 65,536 14.4 / 4.71 / 4.50.  It also spreads the survivor's blocks over
-// the SMs; round 1 at full residency, which an update without any admissible
-// candidate would prefer, takes 2.36 instead of 1.66 ms of 16,384 scenarios.
+// the SMs.  What it costs is an update whose candidates violate late, one after the
+// other on schedulers that hold one warp each (top_down_parts).
 constexpr size_t kSmShared = 227u << 10;
 long long top_down_blocks(const Launch& L) {
   const long long need = ((L.N + 31) / 32 * 11LL + 9) / 10;  // warps of a candidate and a tenth
@@ -849,10 +869,27 @@ long long top_down_blocks(const Launch& L) {
 // nominal 16,384 1.60 / 1.65, 32,768 2.16 / 2.15.
 bool top_down_lone(const Launch& L) { return L.top_down == 2 && L.pmul != nullptr && top_down_blocks(L) <= 2; }
 size_t top_down_pad(const Launch& L, size_t own) {
-  if (L.top_down != 2) return 0;
+  if (L.top_down != 2 || L.held == 2) return 0;
   const long long b = top_down_blocks(L);
   const size_t per = kSmShared / static_cast<size_t>(b + 1) + 1024;
   return per > own && per <= kSmShared / static_cast<size_t>(b) - 1024 ? per - own : 0;
+}
+
+// A held launch is good while the candidates above the result die early.  Once one
+// has run more than 1/32 of the horizon before it violated, the rows that have not
+// begun leave, and a second launch runs them, still from the top, at full residency
+// (what the first one ran, it leaves at once).  An update whose 16 candidates all
+// violate late, 4,000 steps, every candidate at once (stage by stage) / held
+// throughout / in two parts: 8,192 scenarios 0.25 / 0.34 / 0.23 ms, 9,984 0.88 / 1.04
+// / 0.76, 13,000 0.96 / 1.75 / 0.88, 16,384 1.11 / 1.85 / 1.01, 32,768 1.83 / 2.19 /
+// 1.62.  Taken where holding alone loses: not where several candidates are under way
+// in the held launch (7,000: 0.33 / 0.28; 24,576: 1.67 / 1.31) nor from three warps
+// per scheduler on (49,152: 2.33 / 1.86), since the empty blocks of the second launch
+// cost about 10 us a round at 16,384 x 16, 60 us at 65,536 x 16.
+bool top_down_parts(const Launch& L, int rows) {
+  if (rows <= 1 || top_down_pad(L, kTmaSmemBytes) == 0 || L.pair == RRG_PAIR_ALWAYS) return false;
+  const long long b = top_down_blocks(L), warps = (L.N + 31) / 32;
+  return b == 1 ? 2 * warps >= 3LL * L.sms : b == 2 && 10 * warps >= 7 * 8LL * L.sms;
 }
 
 // The nominal binary32 lanes read their coefficients as constant operands.  Where
@@ -862,8 +899,9 @@ size_t top_down_pad(const Launch& L, size_t own) {
 // 332 and 165 / 168 / 163.5 / 167.5 us).
 static_assert((offsetof(Launch, m32) + offsetof(StepModel<float>, U)) % 16 == 8, "coefficients off their line");
 
-cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int early_exit,
-                           bool recheck_classify, bool allow_pair) {
+namespace {
+cudaError_t launch_rollout_part(const Launch& L, int m_launch, bool use_fp64, int early_exit,
+                                bool recheck_classify, bool allow_pair) {
   dim3 grid((L.N + kRollThreads - 1) / kRollThreads, m_launch);
   const int cls = recheck_classify ? 1 : 0;
   // Binary32 lanes on a handle's quads that take neither the TMA ring nor
@@ -972,6 +1010,20 @@ cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int ear
 #undef RRG_ROLLOUT_GEN
 #undef RRG_ROLLOUT
   return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_rollout(const Launch& L, int m_launch, bool use_fp64, int early_exit,
+                           bool recheck_classify, bool allow_pair, int* kernels) {
+  const bool parts = !use_fp64 && !L.scen_gen && top_down_parts(L, m_launch);
+  if (kernels != nullptr) *kernels = parts ? 2 : 1;
+  if (!parts) return launch_rollout_part(L, m_launch, use_fp64, early_exit, recheck_classify, allow_pair);
+  Launch P = L;
+  for (P.held = 1; P.held <= 2; ++P.held) {
+    const cudaError_t e = launch_rollout_part(P, m_launch, use_fp64, early_exit, recheck_classify, allow_pair);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // Binary64 re-run of the trajectories the binary32 pass could not decide,
@@ -1337,7 +1389,11 @@ __device__ void prepare_slot(const Launch& L, int i) {
   L.cand_ss[i] = ok;
   L.cand_dead[i] = ok ? 0 : 1;
   L.cand_min[i] = dkey(inf_v<double>());
-  if (i < RRG_MAX_CANDIDATES) L.st->passed[i] = 0;
+  if (i < RRG_MAX_CANDIDATES) {
+    L.st->passed[i] = 0;
+    L.st->row_launch[i] = 0;
+  }
+  if (i == 0) L.st->late = 0;
 }
 
 // One block per candidate slot of the round the search kernel just set up;
