@@ -795,8 +795,8 @@ cudaError_t launch_adjoint_forward(const Launch& L, bool fp64, int m, int checkp
     const cudaError_t er = cudaEventRecord(fwd_begin, L.stream);
     if (er != cudaSuccess) return er;
   }
-  // four lanes per binary64 trajectory by the rollouts' rule (launch_rollout)
-  const bool coop = fp64 && L.m64.pw != nullptr && static_cast<long long>((L.N + 31) / 32) * m <= 2LL * L.sms;
+  // four lanes per binary64 trajectory by the rollouts' rule
+  const bool coop = fp64 && coop64_fits(L, m);
   if (coop)
     adjoint_forward_coop_kernel<<<dim3((L.N + 7) / 8, m), 32, 0, L.stream>>>(L, L.d64, checkpoint, ckpt, lane_min,
                                                                              lane_arg);

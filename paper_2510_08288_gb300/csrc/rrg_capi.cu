@@ -90,6 +90,7 @@ struct rrg_ctx {
   double* pmul = nullptr;       // parameter multipliers of each pair (parametric uncertainty)
   double* pmulb = nullptr;
   ScenFold fold{}, foldb{};     // the folded models of each pair's scenarios
+  bool own_gamma = false;       // pair 0 has explicit multipliers of gamma other than 1
   cudaStream_t side = nullptr;  // samples update t+1 while update t runs
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool cl_next_ready = false;   // the closed loop's next update is already sampled
@@ -333,8 +334,16 @@ void fill_launch(rrg_ctx* h) {
   L.pmulb = h->pmulb;
   L.fold = h->fold;
   L.foldb = h->foldb;
+  L.own_exponents = h->pmul != nullptr && ((c.param_unc_mask >> P_GAMMA & 1u) != 0 || h->own_gamma);
   L.punc_rho = c.param_unc_rel;
   L.punc_mask = c.param_unc_mask;
+}
+
+// Whether pair 0's multipliers give scenarios exponents of their own.
+void set_own_gamma(rrg_ctx* h, bool own) {
+  if (h->own_gamma == own) return;
+  h->own_gamma = own;
+  fill_launch(h);
 }
 
 cudaEvent_t take_event(rrg_ctx* h) {
@@ -904,6 +913,7 @@ int rrg_sample_scenarios(rrg_handle h, uint64_t seed, uint64_t update_index) {
   if (!h) return RRG_EINVAL;
   DeviceGuard g(h->device);
   h->cl_next_ready = false;  // pair 0 may hold a closed loop's next update
+  set_own_gamma(h, false);
   CK(launch_sample(h->L, seed, update_index, nullptr, h->cfg.dist_amp));
   h->launches += sample_launches(h);
   return RRG_OK;
@@ -944,11 +954,15 @@ int rrg_set_param_multipliers(rrg_handle h, const double* m) {
   if (!m) return set_err(h, RRG_EINVAL, "m is NULL");
   if (!h->pmul) return set_err(h, RRG_EINVAL, "the handle has no parametric uncertainty (param_unc_rel = 0)");
   const size_t n = static_cast<size_t>(h->cfg.n_scenarios) * RRG_NPARAM;
-  for (size_t q = 0; q < n; ++q)
+  bool own_gamma = false;
+  for (size_t q = 0; q < n; ++q) {
     if (!is_fin(m[q]) || !(m[q] > 0.0))
       return set_err(h, RRG_EINVAL, "m[%zu] must be finite and > 0", q);
+    own_gamma |= q % RRG_NPARAM == P_GAMMA && m[q] != 1.0;
+  }
   DeviceGuard g(h->device);
   h->cl_next_ready = false;
+  set_own_gamma(h, own_gamma);
   CK(cudaMemcpyAsync(h->pmul, m, n * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   CK(launch_scenario_fold(h->L, false));
   h->launches++;

@@ -240,7 +240,22 @@ struct Launch {
   // Top-down launches in two parts (launch_rollout): 1, the part held to one
   // candidate's warps, 2, the part that runs what it left; 0: one launch.
   int held;
+  // Scenarios may have exponents of their own, which the binary64 power table does
+  // not hold (pow then).
+  int own_exponents;
 };
+
+// Binary64 rollouts on stored scenarios take four lanes per trajectory (Coop64)
+// while that leaves every scheduler at most two warps (2 x 42 binary64 instructions
+// a step against 110); 500 steps, one lane against four: 1.83 -> 0.96 ms with one
+// warp a scheduler, 1.83 -> 1.40 with two, and a third would cost 2.0.  Where a
+// torque takes pow, which every warp repeats however few of its lanes need it, at
+// most one: 50 steps, one lane against four 0.89 -> 0.78 ms with one warp a
+// scheduler, 0.89 -> 1.46 with two.
+inline bool coop64_fits(const Launch& L, int rows) {
+  const long long lone = static_cast<long long>((L.N + 31) / 32) * rows;  // warps, one lane per trajectory
+  return L.m64.pw != nullptr && lone <= (L.own_exponents ? 1LL : 2LL) * L.sms;
+}
 
 // Folds the FC3 parameter vector into the constants the kernels use
 // (binary64, then rounded once to binary32).  Only products and quotients

@@ -923,12 +923,7 @@ cudaError_t launch_rollout_part(const Launch& L, int m_launch, bool use_fp64, in
 #define RRG_ROLLOUT(KERNEL, T, SRC, D0, D1, CAND, CLS) \
   KERNEL<T, SRC><<<grid, kRollThreads, 0, L.stream>>>(L, D0, D1, CAND, early_exit, CLS)
   if (use_fp64) {
-    // four lanes per trajectory while that leaves every scheduler at most two
-    // warps (2 x 42 binary64 instructions a step against 110); 500 steps, one
-    // lane against four: 1.83 -> 0.96 ms with one warp a scheduler, 1.83 -> 1.40
-    // with two, and a third would cost 2.0
-    const long long warps64 = static_cast<long long>((L.N + 31) / 32) * m_launch;
-    if (!L.scen_gen && L.m64.pw != nullptr && warps64 <= 2LL * sms) {
+    if (!L.scen_gen && coop64_fits(L, m_launch)) {
       const dim3 g4((4 * static_cast<unsigned>(L.N) + kRollThreads - 1) / kRollThreads, m_launch);
       if (L.pmul)
         rollout_pu_kernel<double, SRC_COOP><<<g4, kRollThreads, 0, L.stream>>>(L, L.d64, L.d64b, L.cand_c64,
