@@ -628,9 +628,10 @@ RRG_API int rrg_bisect_decide(rrg_bisect_state *s, const uint8_t *admissible, in
  * make the first call on a device, and the first after such a change, before
  * any stream capture begins.  The binary64 rollouts evaluate x^e - 1 by the
  * same table as a handle's, so results equal rrg_eval_candidates's on the
- * same scenarios bit for bit.  Every call uses the same scratch, which
- * keeps the last call's contents; each call re-initialises everything it
- * reads, but calls that may overlap on the GPU (on different streams, or from
+ * same scenarios bit for bit; the scratch keeps the tables of the first eight
+ * exponents met outside a capture, written by the call that meets one.  Every
+ * call uses the same scratch, which keeps the last call's contents; each call
+ * re-initialises everything else it reads, but calls that may overlap on the GPU (on different streams, or from
  * host threads without ordering between them) race on the scratch and their
  * results are undefined.  Parametric uncertainty is not available here
  * (param_unc_rel != 0: RRG_ENOTIMPL).  Errors: RRG_EINVAL, RRG_ENOTIMPL,

@@ -36,27 +36,31 @@ constexpr size_t kOffCount = kOffMin + align256(kStaticMaxCand * sizeof(unsigned
 constexpr size_t kOffStats = kOffCount + align256(sizeof(uint32_t));
 constexpr size_t kOffList = kOffStats + align256(sizeof(DevStats));
 constexpr size_t kOffJlast = kOffList + align256(kStaticMaxLanes * sizeof(uint32_t));
-constexpr size_t kScratchBytes = kOffJlast + align256(kStaticMaxLanes * sizeof(uint32_t));
+constexpr size_t kOffTables = kOffJlast + align256(kStaticMaxLanes * sizeof(uint32_t));
+constexpr int kTables = 8;  // x^e - 1 tables kept, one per exponent met
+constexpr size_t kScratchBytes = kOffTables + kTables * align256(sizeof(PowTable));
 static_assert(kScratchBytes <= RRG_STATIC_SCRATCH_BYTES, "scratch layout exceeds its stated size");
 
 // The scratch itself: held by every device that loads the library.
 __device__ __align__(256) unsigned char g_rrg_static_scratch[RRG_STATIC_SCRATCH_BYTES];
 
 struct ParamBlock {
-  PowTable pws;   // binary64 x^e - 1 table of the model's exponent (as rrg_create builds it)
   double v[RRG_NPARAM];
 };
-static_assert(sizeof(ParamBlock) + 64 <= 32764, "passed by value to a kernel");
+static_assert(sizeof(PowTable) + 64 <= 32764, "passed by value to a kernel");
 
-// Writes the parameter vector and the x^e - 1 table (passed by value) into
-// the scratch and clears the scratch's step counters.
-__global__ void static_params_kernel(const __grid_constant__ ParamBlock pb, double* params, PowTable* pws,
-                                     DevStats* stats, SearchState* st) {
+// Writes an x^e - 1 table, passed by value, into the scratch.
+__global__ void static_table_kernel(const __grid_constant__ PowTable table, PowTable* out) {
+  const uint4* from = reinterpret_cast<const uint4*>(&table);
+  uint4* to = reinterpret_cast<uint4*>(out);
+  for (unsigned q = threadIdx.x; q < sizeof(PowTable) / sizeof(uint4); q += blockDim.x) to[q] = from[q];
+}
+
+// Writes the parameter vector (passed by value) into the scratch and clears the
+// scratch's step counters.
+__global__ void static_params_kernel(const ParamBlock pb, double* params, DevStats* stats, SearchState* st) {
   const int i = threadIdx.x;
   if (i < RRG_NPARAM) params[i] = pb.v[i];
-  const uint4* from = reinterpret_cast<const uint4*>(&pb.pws);
-  uint4* to = reinterpret_cast<uint4*>(pws);
-  for (unsigned q = i; q < sizeof(PowTable) / sizeof(uint4); q += blockDim.x) to[q] = from[q];
   if (i == 0) {
     st->src[0].d64_valid = 1;  // the caller's binary64 array holds the values
     st->src[1].d64_valid = 1;
@@ -78,6 +82,8 @@ struct ScratchEntry {
   unsigned long long ctx_id;
   unsigned char* ptr;
   int sms;
+  int tables;             // exponents whose tables the scratch holds (at most kTables)
+  double exponent[kTables];
 };
 ScratchEntry g_scratch[kMaxDevices] = {};
 using CtxGetCurrentFn = CUresult (*)(CUcontext*);
@@ -141,10 +147,50 @@ int scratch_for_current_device(unsigned char** out, int* sms) {
     c.ctx_id = ctx;
     c.ptr = static_cast<unsigned char*>(p);
     c.sms = n;
+    c.tables = 0;
   }
   *out = c.ptr;
   *sms = c.sms;
   return RRG_OK;
+}
+
+// The scratch's table of exponent e: one it holds, or one to be written by this
+// call (*write).  A table goes up once per exponent and stays (24 KB by value with
+// every call, and building it whenever the exponent changed, made a call of 32
+// scenarios x 100 steps 6 us slower, 18 us with two models in turn: 55 -> 61 and 73
+// us).  An exponent that finds no place, or is first met while the stream is being
+// captured (the table would only be written by the graph's replays), uses the scratch
+// of the single call.
+PowTable* scratch_table(unsigned char* base, double e, cudaStream_t stream, bool* write) {
+  *write = true;
+  int dev = -1;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) {
+    std::lock_guard<std::mutex> lock(g_mu);
+    ScratchEntry& c = g_scratch[dev];
+    auto at = [&](int q) { return reinterpret_cast<PowTable*>(base + kOffTables + q * align256(sizeof(PowTable))); };
+    for (int q = 0; q < c.tables; ++q)
+      if (c.exponent[q] == e) {
+        *write = false;
+        return at(q);
+      }
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) {
+      cudaGetLastError();
+      capture = cudaStreamCaptureStatusActive;
+    }
+    if (capture == cudaStreamCaptureStatusNone && c.ptr == base && c.tables < kTables) {
+      PowTable t;
+      if (pow_table(e, &t)) {
+        static_table_kernel<<<1, 256, 0, stream>>>(t, at(c.tables));
+        if (cudaGetLastError() == cudaSuccess) {
+          c.exponent[c.tables] = e;
+          *write = false;
+          return at(c.tables++);
+        }
+      }
+    }
+  }
+  return reinterpret_cast<PowTable*>(base + kOffPws);
 }
 
 }  // namespace
@@ -207,9 +253,18 @@ extern "C" int rrg_eval_candidates_static(const double* model_params, int n_para
   fold_constants(model_params, &L.k64, &L.k32);
   // the binary64 rollouts and the recheck evaluate x^e - 1 by the same table
   // as a handle's, so both give the same bits
-  ParamBlock pb;
-  PowTable* const pws = reinterpret_cast<PowTable*>(base + kOffPws);
-  if (pow_table(L.k64.e, &pb.pws)) L.k64.pws = pws;
+  cudaError_t e = cudaSuccess;
+  if (std::fabs(L.k64.e) <= 1.0) {
+    bool write = false;
+    PowTable* const table = scratch_table(base, L.k64.e, L.stream, &write);
+    if (write) {
+      PowTable t;
+      pow_table(L.k64.e, &t);
+      static_table_kernel<<<1, 256, 0, L.stream>>>(t, table);
+      e = cudaGetLastError();
+    }
+    L.k64.pws = table;
+  }
   fold_model(L.k64, model_params, cfg->dt, &L.m64);
   fold_eq(model_params, cfg->y_min, cfg->eps_ss, cfg->y_c, &L.eq);
   round_model(L.m64, &L.m32);
@@ -233,9 +288,12 @@ extern "C" int rrg_eval_candidates_static(const double* model_params, int n_para
   L.sms = sms;
   L.recheck_blocks = 2 * sms;
 
+  ParamBlock pb;
   std::memcpy(pb.v, model_params, sizeof pb.v);
-  static_params_kernel<<<1, 256, 0, L.stream>>>(pb, const_cast<double*>(L.params), pws, L.stats, L.st);
-  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) {
+    static_params_kernel<<<1, 32, 0, L.stream>>>(pb, const_cast<double*>(L.params), L.stats, L.st);
+    e = cudaGetLastError();
+  }
   // the prepare kernel rewrites every per-candidate flag, key and the recheck
   // count, so nothing left in the scratch by an earlier call is read
   if (e == cudaSuccess) e = launch_eval_prepare(L, d_x_t, v_prev, r_t, d_kappas, m);
