@@ -1245,15 +1245,16 @@ int rrg_batch_create(const double* model_params, int n_params, const rrg_config*
     elems += (e + 31ull) & ~31ull;  // 128-byte aligned blocks
     lanes += static_cast<unsigned long long>(M) * static_cast<unsigned long long>(n_scenarios[s]);
   }
-  // the sampler's tiles (32-bit: 2^31 of them would need 50 TB of scenarios)
+  // the sampler's tiles, counted in 32 bits (2^31 of them hold at least 1.6 TB of scenarios)
   std::vector<int32_t> samp_base(static_cast<size_t>(n_instances) + 1, 0);
   unsigned long long tiles = 0;
   for (int s = 0; s < n_instances; ++s) {
     samp_base[s] = static_cast<int32_t>(tiles);
     tiles += static_cast<unsigned long long>(sample_tiles_of(inst[s].N, inst[s].H));
   }
-  samp_base[n_instances] = static_cast<int32_t>(tiles);
   if (lanes >= (1ull << 31)) return bset_err(h, RRG_EINVAL, "sum of max_candidates * n_scenarios >= 2^31");
+  if (tiles >= (1ull << 31)) return bset_err(h, RRG_ENOMEM, "%llu GB of scenarios", elems * sizeof(float) >> 30);
+  samp_base[n_instances] = static_cast<int32_t>(tiles);
 
   h = new (std::nothrow) rrg_batch_ctx();
   if (!h) return bset_err(nullptr, RRG_ENOMEM, "host allocation failed");
