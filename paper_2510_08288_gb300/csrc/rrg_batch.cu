@@ -19,7 +19,6 @@
 //   batch_plant_kernel       simulated plants (closed loop only)
 //
 // The tile queue is one atomic counter; a CTA never waits for another.
-#include <cstddef>
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
@@ -76,6 +75,7 @@ struct BLaunch {
   Fc3K<float> k32;
   EqModel eq;
   StepModel<double> m64;
+  alignas(16) double m32_line;  // as Launch's (16 closed loops: 8 bytes past a line 3.45 ms, on it 3.6)
   StepModel<float> m32;
   const BInst* inst;
   const int32_t* samp_base;  // [S + 1]: sampler tiles before each instance
@@ -204,9 +204,6 @@ __device__ void build_tiles(const BLaunch& B, int tile, int rows) {
     *B.recheck_count = 0u;
   }
 }
-
-// As for Launch (16 closed loops: 8 bytes past a 16-byte line 3.45 ms, 0 bytes 3.6).
-static_assert((offsetof(BLaunch, m32) + offsetof(StepModel<float>, U)) % 16 == 8, "coefficients off their line");
 
 // Speculative bisection per instance: the nodes of the next levels of
 // Alg. 1's bisection tree from the instance's state that fit in `width`

@@ -191,6 +191,7 @@ struct Launch {
   Fc3K<double> k64;             // folded model constants, passed by value
   Fc3K<float> k32;
   StepModel<double> m64;        // the rollout step's coefficients
+  alignas(16) double m32_line;  // m32, and its U, 8 bytes past a 16-byte line (launch_rollout)
   StepModel<float> m32;
   double* d64;                  // scenarios [3][H][N]
   int quads;                    // d32 is in the quad layout (0: the caller's [3][H][N])

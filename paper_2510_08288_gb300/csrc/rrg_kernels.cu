@@ -17,7 +17,6 @@
 //
 // Nothing returns to the host between rounds; the whole update can be
 // captured in a CUDA graph.
-#include <cstddef>
 #include <atomic>
 #include <cfloat>
 #include <cmath>
@@ -94,7 +93,7 @@ cudaError_t launch_step_latency(const Launch& L, double v, int steps, double* d_
 
 // ---------------------------------------------------------------------------
 // Scenario sampling: coalesced over the scenarios k, the step j the same for a
-// whole block (philox_tile).
+// whole block (PhiloxCols).
 //
 // binary64 values: d = a (2u - 1), u = (w >> 11) 2^-53 (bit-exact with the
 // definition in rrg.h).  binary32 copy in the binary32 modes: from the top 24
@@ -896,8 +895,8 @@ bool top_down_parts(const Launch& L, int rows) {
 // these lie decides how the compiler groups the loads of the ones it keeps in
 // registers: 8 bytes past a 16-byte line was fastest (3,001 x 32 candidates x
 // 1,000 steps and a lone warp of 2,000: 0, 4, 8, 12 bytes past it 341 / 350 / 335 /
-// 332 and 165 / 168 / 163.5 / 167.5 us).
-static_assert((offsetof(Launch, m32) + offsetof(StepModel<float>, U)) % 16 == 8, "coefficients off their line");
+// 332 and 165 / 168 / 163.5 / 167.5 us).  Launch::m32_line puts them there.
+
 
 namespace {
 cudaError_t launch_rollout_part(const Launch& L, int m_launch, bool use_fp64, int early_exit,
@@ -1480,8 +1479,6 @@ search_mid_kernel(const Launch L) {
   if (threadIdx.x == 0) {
     int m1 = 0;
     if (s->probe && !s->done) {
-      const int m0 = s->m;
-      (void)m0;
       restore_walk_start(s);
       uint32_t bits;
       int len;
