@@ -473,7 +473,7 @@ RRG_API int rrg_autotune_pairing(rrg_handle h, const double *x_t, double r_t, do
  * reverse
  * pass recomputes trajectory k*'s segments before j* in parallel and then
  * sweeps them backwards; the handle keeps N * (H / checkpoint + 1) * 3 and
- * (H + 1) * 12 doubles of device scratch for them, allocated on first use.
+ * (H + 1) * 3 doubles per kappa of device scratch for them, allocated on first use.
  * Errors: RRG_EINVAL for a null handle or an argument outside its range,
  * RRG_ECUDA (message in rrg_last_error) from the allocation or the
  * launches.  Host in: x_t[3]

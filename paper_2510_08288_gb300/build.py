@@ -25,7 +25,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -ftz=true: the binary32 rollouts never meet subnormal values, and flushing
 # lets lg2/ex2/rcp issue as single MUFU operations on the critical path
 # -ffp-contract=off for the host compiler: host code folds constants the
-# device folds too (fold_rhs) and must not fuse them differently
+# device folds too (fold_model) and must not fuse them differently
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-ftz=true", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
               "-Xcompiler", "-ffp-contract=off",
               "-Xcompiler", "-fvisibility=hidden", "--expt-relaxed-constexpr"]

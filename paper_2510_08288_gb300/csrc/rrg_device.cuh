@@ -1,8 +1,7 @@
 // rrg_device.cuh -- device-side building blocks of the robust reference
 // governor: the FC3 closed-loop right-hand side and output, the RK4 step,
 // the Philox4x64-10 scenario generator and order-preserving keys for
-// atomic minima.  Included by every
-// translation unit with device code.
+// atomic minima.  Included by every translation unit with device code.
 #pragma once
 
 #include <cstdint>
@@ -153,21 +152,6 @@ __device__ __forceinline__ void fc3_rhs(const Fc3K<T>& K, const CandK<T>& C,
 template <typename T>
 __device__ __forceinline__ T fc3_output(const CandK<T>& C, T q_ca, T q_sm) {
   return C.y_scale * (q_sm - q_ca);
-}
-
-// One classical RK4 step of size dt, in place.
-template <typename T>
-__device__ __forceinline__ void rk4_step(const Fc3K<T>& K, const CandK<T>& C, T dt,
-                                         T& q_ca, T& w, T& q_sm) {
-  const T h2 = T(0.5) * dt, h6 = dt / T(6);
-  T a1, b1, c1, a2, b2, c2, a3, b3, c3, a4, b4, c4;
-  fc3_rhs<T>(K, C, q_ca, w, q_sm, a1, b1, c1);
-  fc3_rhs<T>(K, C, q_ca + h2 * a1, w + h2 * b1, q_sm + h2 * c1, a2, b2, c2);
-  fc3_rhs<T>(K, C, q_ca + h2 * a2, w + h2 * b2, q_sm + h2 * c2, a3, b3, c3);
-  fc3_rhs<T>(K, C, q_ca + dt * a3, w + dt * b3, q_sm + dt * c3, a4, b4, c4);
-  q_ca += h6 * ((a1 + a4) + T(2) * (a2 + a3));
-  w += h6 * ((b1 + b4) + T(2) * (b2 + b3));
-  q_sm += h6 * ((c1 + c4) + T(2) * (c2 + c3));
 }
 
 // ---------------------------------------------------------------------------
@@ -391,11 +375,7 @@ __device__ __forceinline__ void rk4_step_packed(const StepU<float>& U, const Ste
   p = fma_rn(U.fwn3, n3, p);
   const float n4 = tq(x4, w4);
   w = fma_rn(U.fwn4, n4, p);
-#ifdef RRG_V_WABS1
-  w_abs = w + C.r_w;
-#else
   w_abs = fma_rn(U.fwn4, n4, p + C.r_w);
-#endif
 }
 
 template <typename T>
