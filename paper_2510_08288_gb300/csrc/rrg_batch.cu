@@ -401,10 +401,10 @@ __device__ __forceinline__ void batch_reduce(const BLaunch& B, size_t slot, int 
 // memory (run_lane_qring); FEED_TMA each warp's ring of 16-step chunks filled
 // by tensor copies (run_lane_tma).  Variants of prefetch depth 16 run the TMA
 // form when a round of every candidate has at least kTmaTileWarps warps of
-// tiles per SM, else the ring of quads, which steps a warp alone on its
-// scheduler faster (177 against 198 cycles) and needs no barriers per tile,
-// while the TMA form issues fewer instructions a step (single problems: 112
-// against 116 cycles a step and scheduler).
+// tiles per SM (or as rrg_batch_set_tma says), else the ring of quads, which steps
+// a warp alone on its scheduler faster (173 against 199 cycles a step) and needs no
+// barriers per tile, while the TMA form issues fewer instructions a step (single
+// problems: 114 against 117 cycles a step and scheduler).
 enum TileFeed : int { FEED_REGS = 0, FEED_QRING = 1, FEED_TMA = 2 };
 constexpr int kTmaTileWarps = 300;
 // Dynamic shared memory of a block of `threads` lanes.

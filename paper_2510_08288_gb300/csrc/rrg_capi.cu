@@ -886,6 +886,7 @@ int rrg_create(const double* model_params, int n_params, const rrg_config* cfg, 
   (void)pair_blocks_per_sm(false);
   (void)pair_blocks_per_sm(true);
   h->smem_ok = tma_ring_prepare();
+  // (n_scenarios % 4: the interface's rule, rrg_set_tma; the map takes any count)
   if (!c.scenarios_in_register && c.n_scenarios % 4 == 0 && h->smem_ok &&
       encode_scenario_map(&h->tmap[0], h->d32, c.n_scenarios, c.horizon)) {
     h->tmap[1] = h->tmap[0];

@@ -176,14 +176,14 @@ __device__ __forceinline__ T fc3_output(const CandK<T>& C, T q_ca, T q_sm) {
 // in binary64 once per model and rounded once.
 //
 // Why: against right-hand sides evaluated stage by stage, a step on the TMA
-// ring takes 89 binary32 instructions instead of 110 (4 torque terms of 7, 53
-// multiply-adds, 3 loads, slack and bookkeeping), and its dependent chain
+// ring takes 90 binary32 instructions instead of 110 (4 torque terms of 7, 53
+// multiply-adds, an addition, 3 loads, slack and bookkeeping), and its dependent chain
 // shortens: x_{i+1} does not depend on N_i (the torque reaches the pressure one
 // stage later), so the power's lg2 and ex2 of a stage overlap the stage
 // before, and the chain through a stage is N_i -> w_{i+1} -> 1 / w -> N_{i+1}.
 // Measured on GB300: one warp's chain 172 -> 145 cycles a step; launches that
-// fill the SMs 2.3e11 -> 3.6e11 steps/s (nominal model, 112 cycles a step and
-// scheduler: 89 issued, and lg2, rcp and ex2 hold their unit for 80).
+// fill the SMs 2.3e11 -> 3.5e11 steps/s (nominal model, 114 cycles a step and
+// scheduler: 90 issued, and lg2, rcp and ex2 hold their unit for 80).
 // In binary64 49 multiply-adds and 4 torque terms of 12 instructions are left
 // (pow_m1_table, rcp_cubic): 257 x 8 trajectories 10.8 -> 3.7 us a step.
 //

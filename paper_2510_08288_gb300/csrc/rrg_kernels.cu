@@ -839,10 +839,10 @@ rollout_tma_pair_kernel(const Launch L, const RhsC<float>* __restrict__ cand,
 // RRG_TMA_AUTO takes the TMA ring for binary32 launches on the stored array
 // of at least this many warps per SM, ahead of pairing; below, the ring of
 // quads.  Measured on GB300 (no early exit, 1,000 steps), TMA against the ring
-// of quads: nominal 16,384 x 16 scenarios 731 against 753 us, 1,024 x 64 (13.5
-// warps per SM) 229 against 234, x 42 176 against 176, one candidate (each warp
+// of quads: nominal 16,384 x 16 scenarios 745 against 761 us, 1,024 x 64 (13.5
+// warps per SM) 234 against 235, x 42 178 against 178, one candidate (each warp
 // alone on its scheduler, where the chunk's wait, votes and refill sit on the
-// chain) 96 against 86; parametric 16,384 x 16 823 against 830.
+// chain) 96 against 84; parametric 16,384 x 16 831 against 837.
 #ifndef RRG_TMA_MIN_WARPS_PER_SM
 #define RRG_TMA_MIN_WARPS_PER_SM 24
 #endif

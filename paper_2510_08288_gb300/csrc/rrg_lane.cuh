@@ -765,7 +765,7 @@ __device__ __forceinline__ float run_lane_ring(const StepU<float>& K, const Step
 // by 16-byte asynchronous copies D quads ahead (each thread copies and reads
 // its own column, so no thread waits for another).  A lone warp's step takes 177
 // cycles, 211 when every value was copied by itself; launches that fill the SMs
-// 116 a step and scheduler.
+// 117 a step and scheduler.
 __device__ __forceinline__ void cp_async16(uint32_t smem_dst, const float4* gmem_src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(gmem_src) : "memory");
 }
