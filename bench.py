@@ -70,9 +70,9 @@ MUFU_PER_STEP = 12
 # instructions a warp issues per trajectory step on the ring of quads (ncu:
 # instructions executed by a launch of 1,024 scenarios x 16 candidates x 1,000
 # steps without early exit over its lane-steps / 32, nominal model): an
-# issue-bound step reaches at most 141 / (2 x 91) of the derived FP32 peak,
+# issue-bound step reaches at most 141 / (2 x 92) of the derived FP32 peak,
 # which counts every instruction as an FMA
-INSTR_PER_STEP = 91
+INSTR_PER_STEP = 92
 ISSUE_CEILING = FLOPS_PER_STEP / (2.0 * INSTR_PER_STEP)
 FP32_LANES_PER_SM = 128
 
@@ -107,14 +107,14 @@ SWEEP_CASE = (100.0, 150.0)     # v_prev, r_t: x_t at the equilibrium of v_prev
 # rollout's sources are the ones profiled: the trajectory loops and model
 # (rrg_lane.cuh, rrg_device.cuh), the rollout kernels and their dispatch in
 # rrg_kernels.cu, and the Launch struct (sha1 of each region)
-TRAFFIC_PER_LAUNCH = (433664 + 24614656 + 35840 + 35584) / 4
+TRAFFIC_PER_LAUNCH = (439040 + 24626944 + 41216 + 41216) / 4
 TRAFFIC_SOURCES = (
-    ("paper_2510_08288_gb300/csrc/rrg_lane.cuh", None, None, "bb86588f91e49ec177d60d8ba804f8f0da51ccab"),
-    ("paper_2510_08288_gb300/csrc/rrg_device.cuh", None, None, "1ef24ed4a16f67f78ee586ee6229fd831974dc8e"),
+    ("paper_2510_08288_gb300/csrc/rrg_lane.cuh", None, None, "f1f8609b0dfb9a2aa7a435f307315a01cce63c59"),
+    ("paper_2510_08288_gb300/csrc/rrg_device.cuh", None, None, "0d9d887b1015e89978cb38ac32b006fda972546d"),
     ("paper_2510_08288_gb300/csrc/rrg_kernels.cu", "// Where a rollout lane takes its disturbances from.",
-     "// Binary64 re-run of the trajectories", "69650da0e7a4601cab97766b63f3c5ad23e6b113"),
+     "// Binary64 re-run of the trajectories", "e1c5f517d2c061ecc2cf234fba6443978fdf073a"),
     ("paper_2510_08288_gb300/csrc/rrg_internal.h", "struct Launch {", "\n};\n",
-     "fb4621135eb51875cc90e855eb357a809ab05b13"),
+     "bb6903ec5b3fc35c796a2ed213ec4789dd57dbb6"),
 )
 
 
@@ -132,13 +132,13 @@ def source_region(rel, begin, end):
 # The sweep's rollout launches at 65,536 scenarios (parametric model, TMA
 # ring): DRAM bytes per launch of one update's three k-section rounds (ncu,
 # one pass over the three launches of the first timed update).  Each round
-# reads the array once per candidate that is still running (tile-major order;
-# the 3.9 GB array does not fit in L2), up to 16 times the algorithmic bytes.
-SWEEP_TRAFFIC_64K = (7911768832 + 3319040 + 19845668096 + 436992 + 51305741824 + 906496) / 3
-# warp instructions per trajectory-step of the TMA-ring kernel (ncu: 728.4 M
+# reads the 3.9 GB array (it does not fit in L2) about 1.5 times: once by the
+# candidate that passes, in part by those above it, which die early.
+SWEEP_TRAFFIC_64K = (5993486080 + 3205120 + 5685671168 + 712448 + 5725633792 + 122368) / 3
+# warp instructions per trajectory-step of the TMA-ring kernel (ncu: 736.7 M
 # over the 16,384 scenarios x 16 candidates x 1,000 steps of a nominal launch;
-# the parametric kernel, two multiply-adds per instruction, issues 76)
-TMA_INSTR_PER_STEP = 89
+# the parametric kernel, two multiply-adds per instruction, issues 77)
+TMA_INSTR_PER_STEP = 90
 
 
 # DRAM bytes of one adjoint_forward_kernel<float, float> launch on the adjoint
@@ -147,13 +147,13 @@ TMA_INSTR_PER_STEP = 89
 # the 3.8 MB of checkpoints and lane minima stay in L2 during the launch),
 # valid while the forward kernel, its launch, the step and the Launch struct
 # are the ones profiled
-ADJ_TRAFFIC_PER_LAUNCH = 49196288 + 3328
+ADJ_TRAFFIC_PER_LAUNCH = 49197056 + 12800
 ADJ_TRAFFIC_SOURCES = (
-    ('paper_2510_08288_gb300/csrc/rrg_adjoint.cu', 'constexpr int kFwdRing = 8;', '__global__ void adjoint_argmin_kernel', 'dd5593761eb2e7fa9699a30371ebecad854ba470'),
-    ('paper_2510_08288_gb300/csrc/rrg_adjoint.cu', 'cudaError_t launch_adjoint_forward(', 'adjoint_argmin_kernel<<<', 'a97cb6582368d4a124a1b7416784f62ca4ea66c5'),
-    ('paper_2510_08288_gb300/csrc/rrg_device.cuh', None, None, '1ef24ed4a16f67f78ee586ee6229fd831974dc8e'),
-    ('paper_2510_08288_gb300/csrc/rrg_lane.cuh', None, None, 'bb86588f91e49ec177d60d8ba804f8f0da51ccab'),
-    ('paper_2510_08288_gb300/csrc/rrg_internal.h', 'struct Launch {', '\n};\n', 'fb4621135eb51875cc90e855eb357a809ab05b13'),
+    ('paper_2510_08288_gb300/csrc/rrg_adjoint.cu', 'constexpr int kFwdRing = 8;', '__global__ void adjoint_argmin_kernel', '26ed80fd4ecf7b43474836b41770ea96b3ff8e90'),
+    ('paper_2510_08288_gb300/csrc/rrg_adjoint.cu', 'cudaError_t launch_adjoint_forward(', 'adjoint_argmin_kernel<<<', 'efd255ab72ceab3dbf842f7564f3eb2edec8541d'),
+    ('paper_2510_08288_gb300/csrc/rrg_device.cuh', None, None, '0d9d887b1015e89978cb38ac32b006fda972546d'),
+    ('paper_2510_08288_gb300/csrc/rrg_lane.cuh', None, None, 'f1f8609b0dfb9a2aa7a435f307315a01cce63c59'),
+    ('paper_2510_08288_gb300/csrc/rrg_internal.h', 'struct Launch {', '\n};\n', 'bb6903ec5b3fc35c796a2ed213ec4789dd57dbb6'),
 )
 
 
